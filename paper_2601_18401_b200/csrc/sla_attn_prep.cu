@@ -1,6 +1,6 @@
 // Work-list construction for the tensor-core span-attention kernel: a counting sort of all pieces
 // (clipped spans) of a chunk of query rows by (batch*Hkv + kv head, 64-key block of the piece's
-// right end, class of blocks covered), and the table of 128-piece tiles cut from the sorted list.
+// right end, class of blocks covered), and the table of 256-piece tiles cut from the sorted list.
 //
 // This is the step Section "Kernel design" describes as grouping (query, span) pairs into buckets by
 // key-block footprint without a global sort.  Each CTA owns a slice of the rows of one
@@ -9,7 +9,7 @@
 //
 //   prep_count       the pieces of every row, parked; histogram of bucket sizes; pieces per row
 //   prep_scan_local  per (batch, kv head): exclusive offsets of its buckets, record and tile totals
-//   prep_scan_global per (batch, kv head): global offsets, tile table entries (a tile = 128 consecutive
+//   prep_scan_global per (batch, kv head): global offsets, tile table entries (a tile = 256 consecutive
 //                    records of the sorted list, whatever end blocks they fall in)
 //   prep_scatter     the parked pieces to their places in the sorted list
 //   prep_tile_bounds per tile: split where neighbouring pieces end far apart; the tile's end block and how
@@ -344,12 +344,13 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scan_global(PrepArgs a) {
     for (int k = tid; k < nk; k += kPrepThreads) cnt[k] += rec_base;
 }
 
-// One warp per tile as cut by prep_scan_global (128 consecutive records).  Where two neighbouring
-// records of the tile end more than kGap key blocks apart the tile is split there (the pieces left of
-// the gap would be walked through it for nothing); the extra tiles are appended to the table.  For
-// every tile: the end block of its last piece (second word) and the number of key blocks from the one
-// its furthest-reaching piece starts in up to that end block (bits 8.. of the last word).
-constexpr int kGap = 2;
+// One warp per tile as cut by prep_scan_global (256 consecutive records).  Where two neighbouring records of the
+// tile end further apart than a span is long the tile is split there: walking the gap would cost more than walking
+// two spans.  (So does a stretch of kMaxStretch blocks, which keeps the block numbers of a tile within 16 bits.)
+// The extra tiles are appended to the table.  For every tile: the end block of its last piece (second word), the
+// number of key blocks from the one its furthest-reaching piece starts in up to that end block (bits 9.. of the last
+// word), and the part of that walk each stream of 128 pieces reaches (`ranges`).
+constexpr int kMaxStretch = 16384;
 __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
     __shared__ int s_eb[8][kRows], s_lo[8][kRows];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -370,23 +371,31 @@ __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
         int seg1 = cnt;
         for (int x0 = seg0 + 1; x0 < cnt && seg1 == cnt; x0 += 32) {
             const int x = x0 + lane;
-            const bool cut = x < cnt && eb[x] - eb[x - 1] > kGap;
+            const bool cut = x < cnt && (eb[x] - eb[x - 1] > a.nb_single || eb[x] - eb[seg0] > kMaxStretch);
             const unsigned m = __ballot_sync(0xffffffffu, cut);
             if (m) seg1 = x0 + __ffs(m) - 1;
         }
-        int lo_min = INT_MAX;
-        for (int x = seg0 + lane; x < seg1; x += 32) lo_min = min(lo_min, lo[x]);
-        lo_min = __reduce_min_sync(0xffffffffu, lo_min);
-        const int eb_last = eb[seg1 - 1];
+        // the two streams of 128 pieces: what each reaches, and the tile's walk that covers both
+        const int mid = min(seg0 + kRows / 2, seg1);
+        int lo_a = INT_MAX, lo_b = INT_MAX;
+        for (int x = seg0 + lane; x < seg1; x += 32) {
+            if (x < mid) lo_a = min(lo_a, lo[x]);
+            else lo_b = min(lo_b, lo[x]);
+        }
+        lo_a = __reduce_min_sync(0xffffffffu, lo_a);
+        lo_b = __reduce_min_sync(0xffffffffu, lo_b);
+        const int eb_last = eb[seg1 - 1], sb = min(lo_a, lo_b) / kBK;
         int idx = t;
         if (n_seg > 0) {
             if (lane == 0) idx = atomicAdd(a.n_tiles, 1);
             idx = __shfl_sync(0xffffffffu, idx, 0);
         }
         if (lane == 0) {
-            if (idx < a.max_tiles)
-                a.tiles[idx] = make_int4(ti.x, eb_last, ti.z + seg0, (seg1 - seg0) | ((eb_last - lo_min / kBK + 1) << 8));
-            else
+            if (idx < a.max_tiles) {
+                a.tiles[idx] = make_int4(ti.x, eb_last, ti.z + seg0, (seg1 - seg0) | ((eb_last - sb + 1) << 9));
+                a.ranges[idx] = make_int2((lo_a / kBK - sb) | ((eb[mid - 1] - sb + 1) << 16),
+                                          mid < seg1 ? (lo_b / kBK - sb) | ((eb_last - sb + 1) << 16) : 0);
+            } else
                 atomicOr(a.status, kStatusBadIndex);   // cannot happen: the table has room for one tile per bucket more
         }
         seg0 = seg1;

@@ -13,9 +13,9 @@
 // rows of one MMA tile must be made to share a key footprint.  Here pieces are grouped by the
 // 64-key block their right end falls in (per batch and KV head) and, inside a group, ordered by how
 // many key blocks they cover, with one counting sort (histogram, prefix sum, scatter) -- no
-// comparison sort of the queries.  A tile is 128 consecutive pieces of the sorted list (of one group,
-// or of neighbouring groups whose end blocks lie next to each other): their Q rows are gathered into
-// shared memory and the tile walks the key blocks they cover from left to right.
+// comparison sort of the queries.  A tile is 256 consecutive pieces of the sorted list (of one group,
+// or of neighbouring groups whose end blocks lie next to each other), two streams of 128: their Q rows are
+// gathered into shared memory and the tile walks the key blocks they cover from left to right.
 //
 //   tc::prepare          the counting sort and the tile table (sla_attn_prep.cu)
 //   tc_attend            persistent CTAs, tile t goes to CTA t mod grid (the table is static once
@@ -25,17 +25,29 @@
 //   tc_merge             per row: log-sum-exp merge of its pieces -> out, lse
 //   tc_merge_gated       per row: A_t = merge(span piece, window piece), O = sum_t alpha_t A_t
 //
-// CTA layout of tc_attend (192 threads, two CTAs per SM): warps 0-3 own one tile row each (TMEM lane
-// = row): Q gather, softmax, epilogue; one thread of warp 4 issues the MMAs; one thread of warp 5
-// issues the TMA loads (K and V as two independent streams).  TMEM: two 64-column S buffers (P aliases
-// the S it came from) and 128 columns of O.  Every wait on an mbarrier is bounded; when one runs out
-// the CTA raises a status bit, drains and leaves.  The kernel is sensitive to its code size (loops
-// over rarely taken paths stay rolled, the spin loops of the waits are not unrolled).
+// CTA layout of tc_attend (512 threads, one CTA per SM): warps 0-3 and 4-7 are the softmax warps of the
+// tile's two streams (one thread per piece, TMEM lane = row); warps 8-11 write the results (and gather the
+// first tile's Q); warps 12 and 13 issue the MMAs of a stream each; warp 14 loads K and V, once for both
+// streams; warp 15 gathers Q for the tiles to come.  TMEM: per stream 128 columns of O and two 64-column S
+// buffers (P aliases the S it came from).  Every wait on an mbarrier is bounded; when one runs out the CTA
+// raises a status bit, drains and leaves.
+//
+// What bounds it: a stream's chain per 64-key block (S ready -> softmax -> P -> PV, S two blocks ahead), the
+// special-function pipe (1024 cycles of exponentials for a block of both streams) and the tensor pipe (1376: an
+// N = 64 S instruction holds it for 52 cycles, not 32, for its operand traffic); it takes about 1950 cycles.
+// Before, two independent CTAs per SM of 128 pieces each, whose row threads also gathered Q and wrote results:
+// 1860 cycles a block in long tiles but 5300 more per tile; now 700 per tile.  Configuration of 65536 tokens, 11
+// blocks per tile: 4.07 -> 3.45 ms; 16384 tokens, 7 blocks: 658 -> 570 us.
+// Two things that the times depend on: the kernel's code has to fit the instruction cache (about 2300
+// instructions; at 3500 the hit rate is 77 % and everything takes a half longer), and the issuing warps have to
+// run converged with one elected lane issuing (see ptx::elect_one): the issuers' time per block bounded the
+// streams at 2500 cycles otherwise.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 #include <limits.h>
 #include <math_constants.h>
+#include <stddef.h>
 
 #include "sla_attn_tc.cuh"
 #include "sla_tc_ptx.cuh"
@@ -47,43 +59,50 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kD = 128;
-using tc::kBK;    // keys per block
+using tc::kBK;    // keys per block of the work list
 using tc::kRows;  // pieces per tile
-constexpr int kThreads = 192;   // 4 row warps, MMA issuer, TMA producer
-constexpr int kTmemCols = 256;
-constexpr int kMaxWalk = 4096;   // most key blocks a tile walks
-constexpr uint32_t kColS = 0;    // S buffers at columns 0 and 64
-constexpr uint32_t kColO = 128;
-constexpr int kQBytes = kRows * kD * 2;      // 32 KiB, two 64-wide halves of 128 rows x 128 B
+constexpr int kHalf = 128;       // pieces per stream: a tile's first and second 128
+constexpr int kThreads = 512;    // 4 row warps per stream, 4 epilogue warps, an MMA issuer per stream, K/V producer, Q gather
+constexpr int kTmemCols = 512;
+constexpr int kMaxWalk = 4096;   // most key blocks a piece covers
+constexpr int kMinTiles = 1024;  // entries of the tile table at least: more than CTAs
+constexpr uint32_t kColO = 0;    // O of the streams at columns 0 and 128
+constexpr uint32_t kColS = 256;  // two S buffers of 64 columns per stream, from columns 256 and 384; P aliases its S
+constexpr int kQBytes = kHalf * kD * 2;      // 32 KiB, two 64-wide halves of 128 rows x 128 B
 constexpr int kKVBytes = kBK * kD * 2;       // 16 KiB, two 64-wide halves of 64 rows x 128 B
-constexpr int kKS = 3;           // K stages (a K block is free again as soon as its S = Q K^T is done)
-constexpr int kVS = 2;           // V stages (and S/P buffers)
+constexpr int kQS = 4;           // Q buffers: the streams of this tile and of the next
+constexpr int kKS = 3;           // K and V stages
 constexpr int kOffQ = 0;
-constexpr int kOffK = kQBytes;
+constexpr int kOffK = kQS * kQBytes;
 constexpr int kOffV = kOffK + kKS * kKVBytes;
-constexpr int kOffMeta = kOffV + kVS * kKVBytes;   // 114688
-constexpr int kMetaBytes = 1024;
-// 113 KiB: two CTAs (plus 1 KiB of system reserve each) fill the 228 KiB of an SM exactly
-constexpr int kSmemBytes = kOffMeta + kMetaBytes;
+constexpr int kOffMeta = kOffV + kKS * kKVBytes;   // 229376
+constexpr int kMetaBytes = 3072;
+constexpr int kSmemBytes = kOffMeta + kMetaBytes;  // 227 KiB: one CTA per SM
 constexpr float kRescaleThreshold = 8.f;     // log2 units: P stays below 2^8
+// registers per thread after the re-split; the sum over the four warpgroups stays within the 4 x 128 of the launch
+constexpr int kRegsRow = 160, kRegsEpi = 96, kRegsIssue = 96;
+static_assert(2 * kRegsRow + kRegsEpi + kRegsIssue <= 4 * 128, "more registers than the block is launched with");
 
 struct Meta {
-    unsigned long long q_full, o_full, o_empty;
-    unsigned long long k_full[kKS], k_empty[kKS], v_full[kVS], v_empty[kVS], s_full[2], p_ready[2];
+    unsigned long long q_full[kQS], q_empty[kQS], kv_full[kKS], kv_empty[2][kKS];
+    unsigned long long s_full[4], p_ready[4], l_full[2], o_full[2], o_empty[2];
     uint32_t tmem_base;
     int abort_flag;
+    float2 stats[kRows];   // {reciprocal denominator, log2-domain log-sum-exp} of the tile's rows, for the epilogue
 };
 static_assert(sizeof(Meta) <= kMetaBytes, "meta block too large");
 
 struct TcParams {
-    const bf16 *q;
-    long long q_sb, q_sh, q_st;
+    const bf16 *q;             // Q as rows at one pitch (in elements), numbered as in its tensor map
+    long long q_pitch;
+    int q_b, q_h, q_t;         // strides of Q in those rows
     int Hq, G, Lc, slots;      // slots: partial results per row (top_k, + 1 with a local window)
-    long long r0;              // first query row of the chunk
+    int r0;                    // first query row of the chunk
     float scale2;              // softmax_scale * log2(e)
     int slot_t, slot_h, slot_b;  // positions of (token, head, batch) among tensor-map coordinates 1..3
     const int4 *recs;          // sorted piece records {row, j, lo, hi}
-    const int4 *tiles;         // {b*Hkv+g, end block, first record, record count | key blocks to walk << 8}
+    const int4 *tiles;         // {b*Hkv+g, end block, first record, record count | key blocks to walk << 9}
+    const int2 *ranges;        // key blocks of the walk a tile's streams take part in: first | end << 16
     const int *n_tiles;
     __half *part_o;            // [rows*slots][128] normalised piece outputs, fp16 with one power-of-two
                                // scale per 32-column chunk (block floating point)
@@ -132,26 +151,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// Gathers one Q row (256 B) into the swizzled A-operand layout with 16-byte async copies; a null
-// source zero-fills the row.  Kept out of line: it runs once per tile from two places, and the
-// kernel's hot loop is faster the less code surrounds it.
-__device__ __noinline__ void gather_q_row(const bf16 *src, uint8_t *q_tile, uint32_t q_row, int tid) {
-    if (src) {
-#pragma unroll
-        for (int cidx = 0; cidx < 16; ++cidx) {
-            const uint32_t dst = q_row + (cidx >> 3) * (kQBytes / 2) + (((cidx & 7) ^ (tid & 7)) << 4);
-            ptx::cp_async16(dst, src + cidx * 8);
-        }
-    } else {
-        uint4 *qdst = reinterpret_cast<uint4 *>(q_tile);
-#pragma unroll
-        for (int cidx = 0; cidx < 16; ++cidx)
-            qdst[(cidx >> 3) * (kQBytes / 32) + tid * 8 + (cidx & 7)] = make_uint4(0, 0, 0, 0);
-    }
-}
-
-__global__ void __launch_bounds__(kThreads, 2)
-tc_attend(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, TcParams p) {
+__global__ void __launch_bounds__(kThreads, 1)
+tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+          const __grid_constant__ CUtensorMap tm_v, TcParams p) {
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t base = ptx::smem_u32(smem);
     Meta *meta = reinterpret_cast<Meta *>(smem + kOffMeta);
@@ -161,337 +163,293 @@ tc_attend(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUte
         if (tid == 0) atomicOr(p.status, kStatusTimeout);
         return;
     }
+    const uint32_t mbase = base + kOffMeta;
+    const uint32_t bar_q_full = mbase + offsetof(Meta, q_full), bar_q_empty = mbase + offsetof(Meta, q_empty);
+    const uint32_t bar_kv_full = mbase + offsetof(Meta, kv_full), bar_kv_empty = mbase + offsetof(Meta, kv_empty);
+    const uint32_t bar_s_full = mbase + offsetof(Meta, s_full), bar_p_ready = mbase + offsetof(Meta, p_ready);
+    const uint32_t bar_l_full = mbase + offsetof(Meta, l_full);
+    const uint32_t bar_o_full = mbase + offsetof(Meta, o_full), bar_o_empty = mbase + offsetof(Meta, o_empty);
 
-    const uint32_t bar_q_full = ptx::smem_u32(&meta->q_full), bar_o_full = ptx::smem_u32(&meta->o_full);
-    const uint32_t bar_o_empty = ptx::smem_u32(&meta->o_empty);
-    const uint32_t bar_k_full = ptx::smem_u32(&meta->k_full[0]), bar_k_empty = ptx::smem_u32(&meta->k_empty[0]);
-    const uint32_t bar_v_full = ptx::smem_u32(&meta->v_full[0]), bar_v_empty = ptx::smem_u32(&meta->v_empty[0]);
-    const uint32_t bar_s_full = ptx::smem_u32(&meta->s_full[0]), bar_p_ready = ptx::smem_u32(&meta->p_ready[0]);
+    // requested before the set-up (the table has an entry for every CTA)
+    const int n_tiles = *p.n_tiles, tile_step = gridDim.x;
+    int tile = blockIdx.x;
+    int4 ti = p.tiles[tile];
 
     if (tid == 0) {
-        ptx::mbar_init(bar_q_full, 4);   // one arrival per row warp
-        ptx::mbar_init(bar_o_full, 1);
-        ptx::mbar_init(bar_o_empty, 4);
-        for (int s = 0; s < kKS; ++s) {
-            ptx::mbar_init(bar_k_full + 8 * s, 1);
-            ptx::mbar_init(bar_k_empty + 8 * s, 1);
+#pragma unroll 1
+        for (int x = 0; x < kQS; ++x) {
+            ptx::mbar_init(bar_q_full + 8 * x, 1);
+            ptx::mbar_init(bar_q_empty + 8 * x, 1);
         }
-        for (int s = 0; s < 2; ++s) {
-            ptx::mbar_init(bar_v_full + 8 * s, 1);
-            ptx::mbar_init(bar_v_empty + 8 * s, 1);
-            ptx::mbar_init(bar_s_full + 8 * s, 1);
-            ptx::mbar_init(bar_p_ready + 8 * s, 4);
+#pragma unroll 1
+        for (int x = 0; x < kKS; ++x) {
+            ptx::mbar_init(bar_kv_full + 8 * x, 1);
+            ptx::mbar_init(bar_kv_empty + 8 * x, 1);
+            ptx::mbar_init(bar_kv_empty + 8 * (kKS + x), 1);
+        }
+#pragma unroll 1
+        for (int x = 0; x < 4; ++x) {
+            ptx::mbar_init(bar_s_full + 8 * x, 1);
+            ptx::mbar_init(bar_p_ready + 8 * x, 4);   // one arrival per row warp
+        }
+#pragma unroll 1
+        for (int x = 0; x < 2; ++x) {
+            ptx::mbar_init(bar_l_full + 8 * x, 4);
+            ptx::mbar_init(bar_o_full + 8 * x, 1);
+            ptx::mbar_init(bar_o_empty + 8 * x, 4);
         }
         meta->abort_flag = 0;
         ptx::fence_barrier_init();
     }
-    if (warp == 5 && lane == 0) {
-        ptx::prefetch_tensormap(&tm_k);
-        ptx::prefetch_tensormap(&tm_v);
-    }
-    if (warp == 4) {
-        ptx::tmem_alloc(ptx::smem_u32(&meta->tmem_base), kTmemCols);
+    if (warp == 12) {
+        ptx::tmem_alloc(mbase + offsetof(Meta, tmem_base), kTmemCols);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = meta->tmem_base;
+    if (tile >= n_tiles) ti = make_int4(0, 0, 0, 0);   // not an entry: nothing below looks records up through it
 
-    constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(kRows, kBK, false, false);   // S = Q K^T, both K-major
-    constexpr uint32_t kIdescO = ptx::idesc_bf16_f32(kRows, kD, false, true);     // O = P V, V is N-major
+    constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(kHalf, kBK, false, false);   // S = Q K^T, both K-major
+    constexpr uint32_t kIdescO = ptx::idesc_bf16_f32(kHalf, kD, false, true);       // O = P V, V is N-major
 
     // Tiles are dealt round-robin: CTA c takes tiles c, c + grid, c + 2 grid, ...  Every role reads its
-    // tile's table entry {b*Hkv+g, end block, first record, count | blocks << 8} straight from global
+    // tile's table entry {b*Hkv+g, end block, first record, count | blocks << 9} straight from global
     // memory, one tile ahead of where it is working, so nothing but mbarriers couples the roles.
-    const int n_tiles = *p.n_tiles;
-    const int tile_step = gridDim.x;
+    auto q_row = [&](int row, int bb) {   // number of a record's row among the rows of Q
+        const int bh = (unsigned)row / (unsigned)p.Lc;
+        return bb * p.q_b + (bh - bb * p.Hq) * p.q_h + (p.r0 + row - bh * p.Lc) * p.q_t;
+    };
+    auto fetch_next = [&]() { return tile + tile_step < n_tiles ? p.tiles[tile + tile_step] : make_int4(0, 0, 0, 0); };
 
-    if (warp == 5 && lane == 0) {
-        // ---------------- TMA producer, event driven: the K blocks and the V blocks of the CTA's tile
-        // sequence are two independent streams, each running as far ahead as its own stages allow (a
-        // K stage frees when its S = Q K^T is done, long before the V stage of the same block).
-        struct Cursor {
-            int tile, j, nblk, sb0, ch, cb;
-            uint32_t n;
-        };
-        auto open_tile = [&](Cursor &cu) {
-            if (cu.tile < n_tiles) {
-                const int4 ti = p.tiles[cu.tile];
-                cu.nblk = ti.w >> 8;
-                cu.sb0 = ti.y - cu.nblk + 1;
-                cu.ch = ti.x % p.Hkv;
-                cu.cb = ti.x / p.Hkv;
-                cu.j = 0;
-            }
-        };
-        auto issue = [&](Cursor &cu, const CUtensorMap *tm, uint32_t bar_full, uint32_t dst) {
-            int c[4];
-            c[1 + p.slot_h] = cu.ch;
-            c[1 + p.slot_b] = cu.cb;
-            c[1 + p.slot_t] = (cu.sb0 + cu.j) * kBK;
-            ptx::mbar_arrive_expect_tx(bar_full, kKVBytes);
-            ptx::tma_load_4d(dst, tm, bar_full, 0, c[1], c[2], c[3]);
-            ptx::tma_load_4d(dst + kKVBytes / 2, tm, bar_full, 64, c[1], c[2], c[3]);
-            ++cu.n;
-            if (++cu.j == cu.nblk) {
-                cu.tile += tile_step;
-                open_tile(cu);
-            }
-        };
-        Cursor ck{(int)blockIdx.x, 0, 0, 0, 0, 0, 0u}, cv{(int)blockIdx.x, 0, 0, 0, 0, 0, 0u};
-        open_tile(ck);
-        cv = ck;
-        uint32_t idle = 0;
-        while (cv.tile < n_tiles) {
-            bool progressed = false;
-            if (ck.tile < n_tiles) {
-                const uint32_t st = ck.n % kKS;
-                if (ptx::mbar_test_wait(bar_k_empty + 8 * st, ((ck.n / kKS) & 1u) ^ 1u)) {
-                    issue(ck, &tm_k, bar_k_full + 8 * st, base + kOffK + st * kKVBytes);
-                    progressed = true;
+    if (warp >= 12) {
+        ptx::setmaxnreg_dec<kRegsIssue>();
+        if (warp < 14) {
+            // ---------------- MMA issuer of stream x: a whole warp, its elected lane issues.  Block after block, across
+            // tile boundaries, S runs two blocks ahead of PV: S(n+2) reuses the buffer of P(n) and is issued right
+            // behind PV(n) (the tensor pipe keeps a thread's order).  The first PV of a tile overwrites O, so it waits
+            // until the epilogue has read the tile before.  Blocks that none of the stream's pieces reach are only
+            // handed on.  Two waits and two commits per block: the issuer's own time per block bounds the stream.
+            const bool leader = ptx::elect_one();
+            const int x = warp - 12;
+            struct Cursor {
+                int tile, j, nblk, nx;
+                int first, end;   // blocks this stream takes part in
+                uint32_t nb;      // of those so far
+            };
+            auto open = [&](Cursor &c) {
+                c.j = 0;
+                if (c.tile < n_tiles) {
+                    const int w = p.tiles[c.tile].w;
+                    c.nblk = w >> 9;
+                    c.nx = (w & 0x1ff) > kHalf ? 2 : 1;
+                    const int rg = x ? p.ranges[c.tile].y : p.ranges[c.tile].x;
+                    c.first = rg & 0xffff;
+                    c.end = rg >> 16;
                 }
-            }
-            {
-                const uint32_t st = cv.n % kVS;
-                if (cv.n < ck.n &&   // K first: V(n) is never requested before K(n)
-                    ptx::mbar_test_wait(bar_v_empty + 8 * st, ((cv.n / kVS) & 1u) ^ 1u)) {
-                    issue(cv, &tm_v, bar_v_full + 8 * st, base + kOffV + st * kKVBytes);
-                    progressed = true;
-                }
-            }
-            if (progressed) {
-                idle = 0;
-            } else if (__nanosleep(40), ++idle > ptx::kSpinLimit || ((idle & 63u) == 0u && *abort_flag)) {
-                *abort_flag = 1;
-                break;
-            }
-        }
-    } else if (warp == 4 && lane == 0) {
-        // ---------------- MMA issuer, event driven: S(j) as soon as K(j) has landed and an S buffer
-        // is free, PV(j) as soon as P(j) and V(j) are there.  S(j+2) reuses the buffer of P(j), so it
-        // is only issued after PV(j); the first PV of a tile overwrites O, so it waits until the row
-        // threads have read the previous tile's O.
-        uint32_t n_kv = 0, T = 0;
-        int tile = blockIdx.x;
-        int nblk = tile < n_tiles ? (p.tiles[tile].w >> 8) : 0;
-        const uint64_t desc_q0 = ptx::smem_desc_sw128(base + kOffQ, 16, 1024);
-        const uint64_t desc_k0 = ptx::smem_desc_sw128(base + kOffK, 16, 1024);
-        const uint64_t desc_v0 = ptx::smem_desc_sw128(base + kOffV, kKVBytes / 2, 1024);
-        for (; tile < n_tiles; tile += tile_step, ++T) {
-            const int nblk_next = tile + tile_step < n_tiles ? (p.tiles[tile + tile_step].w >> 8) : 0;
-            bool ok = ptx::mbar_wait(bar_q_full, T & 1u, abort_flag);
-            ptx::tc_fence_after();
-            int is = 0, ipv = 0;
-            uint32_t idle = 0;
-            while (ok && ipv < nblk) {
-                bool progressed = false;
-                if (is < nblk && is < ipv + 2) {
-                    const uint32_t n = n_kv + is, ks = n % kKS, sbuf = n & 1u;
-                    if (ptx::mbar_test_wait(bar_k_full + 8 * ks, (n / kKS) & 1u)) {
+            };
+            Cursor cs{tile, 0, 0, 0, 0, 0, 0u};
+            open(cs);
+            Cursor cv = cs;
+            const uint32_t s_col = tmem + kColS + x * (2 * kBK), o_col = tmem + kColO + x * kD;
+            uint32_t nq = x, t = 0;
+            const uint64_t desc_q0 = ptx::smem_desc_sw128(base + kOffQ, 16, 1024);
+            const uint64_t desc_k0 = ptx::smem_desc_sw128(base + kOffK, 16, 1024);
+            const uint64_t desc_v0 = ptx::smem_desc_sw128(base + kOffV, kKVBytes / 2, 1024);
+#pragma unroll 1
+            for (uint32_t i = 0; cv.tile < n_tiles; ++i) {
+                if (i >= 2) {
+                    const uint32_t st = (i - 2) % kKS, bar_done = bar_kv_empty + 8 * (x * kKS + st);
+                    const bool last = cv.j == cv.end - 1;
+                    if (cv.j >= cv.first && cv.j < cv.end) {
+                        const uint32_t b = cv.nb & 1u;
+                        if (cv.j == cv.first && t > 0 && !ptx::mbar_wait(bar_o_empty + 8 * x, (t - 1u) & 1u, abort_flag)) break;
+                        if (!ptx::mbar_wait(bar_p_ready + 16 * x + 8 * b, (cv.nb >> 1) & 1u, abort_flag)) break;
                         ptx::tc_fence_after();
-                        const uint32_t d_s = tmem + kColS + sbuf * kBK;
-                        const uint64_t dk = desc_advance(desc_k0, ks * kKVBytes);
+                        const uint64_t dv = desc_advance(desc_v0, st * kKVBytes);
+                        if (leader) {
 #pragma unroll
-                        for (int kk = 0; kk < kD / 16; ++kk) {
-                            const uint32_t half = kk >> 2, inner = (kk & 3) * 32;
-                            ptx::mma_ss(d_s, desc_advance(desc_q0, half * (kQBytes / 2) + inner),
-                                        desc_advance(dk, half * (kKVBytes / 2) + inner), kIdescS, kk > 0);
+                            for (int kk = 0; kk < kBK / 16; ++kk)
+                                ptx::mma_ts(o_col, s_col + b * kBK + kk * 8, desc_advance(dv, kk * 2048), kIdescO, cv.j - cv.first + kk);
+                            ptx::mma_commit(bar_done);
+                            if (last) ptx::mma_commit(bar_o_full + 8 * x);
                         }
-                        ptx::mma_commit(bar_s_full + 8 * sbuf);
-                        ptx::mma_commit(bar_k_empty + 8 * ks);
-                        ++is;
-                        progressed = true;
+                        ++cv.nb;
+                        t += last;
+                    } else if (leader) {
+                        ptx::mbar_arrive(bar_done);
+                    }
+                    if (++cv.j == cv.nblk) {
+                        cv.tile += tile_step;
+                        open(cv);
                     }
                 }
-                if (ipv < is) {
-                    const uint32_t n = n_kv + ipv, vs = n & 1u, ph = (n >> 1) & 1u;
-                    const bool o_free = ipv > 0 || T == 0 || ptx::mbar_test_wait(bar_o_empty, (T - 1u) & 1u);
-                    if (o_free && ptx::mbar_test_wait(bar_p_ready + 8 * vs, ph) && ptx::mbar_test_wait(bar_v_full + 8 * vs, ph)) {
+                if (cs.tile < n_tiles) {
+                    const uint32_t st = i % kKS;
+                    if (!ptx::mbar_wait(bar_kv_full + 8 * st, (i / kKS) & 1u, abort_flag)) break;
+                    const bool last = cs.j == cs.end - 1;
+                    if (cs.j >= cs.first && cs.j < cs.end) {
+                        const uint32_t qs = nq % kQS, b = cs.nb & 1u;
+                        if (cs.j == cs.first && !ptx::mbar_wait(bar_q_full + 8 * qs, (nq / kQS) & 1u, abort_flag)) break;
                         ptx::tc_fence_after();
-                        const uint32_t a_p = tmem + kColS + vs * kBK;   // P aliases S: 64 bf16 = 32 columns
-                        const uint64_t dv = desc_advance(desc_v0, vs * kKVBytes);
+                        const uint64_t dq = desc_advance(desc_q0, qs * kQBytes), dk = desc_advance(desc_k0, st * kKVBytes);
+                        if (leader) {
 #pragma unroll
-                        for (int kk = 0; kk < kBK / 16; ++kk)
-                            ptx::mma_ts(tmem + kColO, a_p + kk * 8, desc_advance(dv, kk * 2048), kIdescO,
-                                        (ipv > 0 || kk > 0) ? 1u : 0u);
-                        ptx::mma_commit(bar_v_empty + 8 * vs);
-                        if (ipv == nblk - 1) ptx::mma_commit(bar_o_full);
-                        ++ipv;
-                        progressed = true;
+                            for (int kk = 0; kk < kD / 16; ++kk)
+                                ptx::mma_ss(s_col + b * kBK, desc_advance(dq, (kk >> 2) * (kQBytes / 2) + (kk & 3) * 32),
+                                            desc_advance(dk, (kk >> 2) * (kKVBytes / 2) + (kk & 3) * 32), kIdescS, kk > 0);
+                            ptx::mma_commit(bar_s_full + 16 * x + 8 * b);
+                            if (last) ptx::mma_commit(bar_q_empty + 8 * qs);
+                        }
+                        ++cs.nb;
+                    }
+                    if (++cs.j == cs.nblk) {
+                        nq += cs.nx;
+                        cs.tile += tile_step;
+                        open(cs);
                     }
                 }
-                if (progressed) {
-                    idle = 0;
-                } else if (__nanosleep(20), ++idle > ptx::kSpinLimit || ((idle & 63u) == 0u && *abort_flag)) {
-                    *abort_flag = 1;
-                    ok = false;
-                }
             }
-            if (!ok) break;
-            n_kv += nblk;
-            nblk = nblk_next;
-        }
-    } else if (warp < 4) {
-        // ---------------- row threads: Q gather, softmax per key block, epilogue
-        const uint32_t lane_addr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-        const uint32_t q_row = base + kOffQ + tid * 128;
-        auto gather_q = [&](bool row_valid, int row) {
-            const bf16 *src = nullptr;
-            if (row_valid) {
-                const int rc = row % p.Lc, bh = row / p.Lc;
-                const int h = bh % p.Hq, bb = bh / p.Hq;
-                src = p.q + bb * p.q_sb + h * p.q_sh + (p.r0 + rc) * p.q_st;
-            }
-            gather_q_row(src, smem + kOffQ, q_row, tid);
-        };
-        uint32_t n_kv = 0, T = 0;
-        int tile = blockIdx.x;
-        int4 ti = tile < n_tiles ? p.tiles[tile] : make_int4(0, 0, 0, 0);
-        int4 rec = make_int4(0, 0, INT_MAX, -1);
-        if (tile < n_tiles) {
-            if (tid < (ti.w & 0xff)) rec = p.recs[ti.z + tid];
-            gather_q(tid < (ti.w & 0xff), rec.x);
-        }
-        // hands the gathered Q tile to the MMA issuer
-        auto publish_q = [&]() {
-            ptx::cp_async_wait_all();
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar_q_full);
-        };
-        if (tile < n_tiles) publish_q();
-        for (; tile < n_tiles; tile += tile_step, ++T) {
-            const int nblk = ti.w >> 8, sb0 = ti.y - nblk + 1, cnt = ti.w & 0xff;
-            const bool valid = tid < cnt;
-            // the next tile: its record is fetched now, its Q row during this tile's last key block
-            const bool has_next = tile + tile_step < n_tiles;
-            const int4 ti_next = has_next ? p.tiles[tile + tile_step] : make_int4(0, 0, 0, 0);
-            const int cnt_next = ti_next.w & 0xff;
-            int4 rec_next = make_int4(0, 0, INT_MAX, -1);
-            if (has_next && tid < cnt_next) rec_next = p.recs[ti_next.z + tid];
-
-            const int lo = rec.z, hi = rec.w;
-            float m_ref = -CUDART_INF_F, l = 0.f;
+        } else if (warp == 14) {
+            // ---------------- K/V producer: K and V of block after block, each as two halves of the head dimension
+            const bool leader = ptx::elect_one();
+            uint32_t n = 0;
             bool ok = true;
-            for (int j = 0; j < nblk && ok; ++j) {
-                const uint32_t n = n_kv + j, st = n & 1u, ph = (n >> 1) & 1u;
-                ok = ptx::mbar_wait_warp(bar_s_full + 8 * st, ph, abort_flag);
+            while (tile < n_tiles && ok) {
+                const int4 ti_next = fetch_next();
+                const int nblk = ti.w >> 9, bb = (unsigned)ti.x / (unsigned)p.Hkv;
+                int c[4];
+                c[1 + p.slot_h] = ti.x - bb * p.Hkv;
+                c[1 + p.slot_b] = bb;
+#pragma unroll 1
+                for (int j = 0; j < nblk; ++j, ++n) {
+                    const uint32_t st = n % kKS, ph = ((n / kKS) & 1u) ^ 1u;
+                    c[1 + p.slot_t] = (ti.y + 1 - nblk + j) * kBK;
+                    ok = ptx::mbar_wait(bar_kv_empty + 8 * st, ph, abort_flag) &&
+                         ptx::mbar_wait(bar_kv_empty + 8 * (kKS + st), ph, abort_flag);
+                    if (!ok) break;
+                    if (leader) {
+                        const uint32_t full = bar_kv_full + 8 * st, dk = base + kOffK + st * kKVBytes, dv = base + kOffV + st * kKVBytes;
+                        ptx::mbar_arrive_expect_tx(full, 2 * kKVBytes);
+                        ptx::tma_load_4d(dk, &tm_k, full, 0, c[1], c[2], c[3]);
+                        ptx::tma_load_4d(dk + kKVBytes / 2, &tm_k, full, 64, c[1], c[2], c[3]);
+                        ptx::tma_load_4d(dv, &tm_v, full, 0, c[1], c[2], c[3]);
+                        ptx::tma_load_4d(dv + kKVBytes / 2, &tm_v, full, 64, c[1], c[2], c[3]);
+                    }
+                }
+                tile += tile_step;
+                ti = ti_next;
+            }
+        } else {
+            // ---------------- Q gather from the CTA's second tile on: the rows of one stream's tile after the other by TMA,
+            // four rows of 64 columns per instruction, a lane four rows, as soon as a Q buffer is free.  The records are
+            // read a stream ahead.  (128 rows take the TMA unit about 4600 cycles: hidden in the tile before.)
+            ptx::prefetch_tensormap(&tm_q);
+            const bool leader = ptx::elect_one();
+            uint32_t nq = (ti.w & 0x1ff) > kHalf ? 2 : 1;
+            int x = 0, rows[4];
+            auto fetch_rows = [&](const int4 &t, int xs) {   // a row beyond the tile's last one: that one again
+                const int last = (t.w & 0x1ff) - 1;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) rows[u] = p.recs[t.z + min(xs * kHalf + 4 * lane + u, last)].x;
+            };
+            tile += tile_step;
+            ti = tile < n_tiles ? p.tiles[tile] : ti;
+            if (tile < n_tiles) fetch_rows(ti, 0);
+            int4 ti_next = fetch_next();
+            while (tile < n_tiles) {
+                const int bb = (unsigned)ti.x / (unsigned)p.Hkv;
+                const uint32_t qs = nq % kQS, full = bar_q_full + 8 * qs;
+                if (!ptx::mbar_wait_warp(bar_q_empty + 8 * qs, ((nq / kQS) & 1u) ^ 1u, abort_flag)) break;
+                if (leader) ptx::mbar_arrive_expect_tx(full, kQBytes);
+                int at[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) at[u] = q_row(rows[u], bb);
+                __syncwarp();
+                const uint32_t dst = base + kOffQ + qs * kQBytes + lane * 512;
+                ptx::tma_gather4(dst, &tm_q, full, 0, at[0], at[1], at[2], at[3]);
+                ptx::tma_gather4(dst + kQBytes / 2, &tm_q, full, 64, at[0], at[1], at[2], at[3]);
+                if (x == 0 && (ti.w & 0x1ff) > kHalf) {
+                    x = 1;
+                } else {
+                    x = 0;
+                    tile += tile_step;
+                    ti = ti_next;
+                    if (tile < n_tiles) ti_next = fetch_next();
+                }
+                if (tile < n_tiles) fetch_rows(ti, x);
+                ++nq;
+            }
+        }
+    } else if (warp >= 8) {
+        // ---------------- epilogue warps: normalised piece outputs and their log-sum-exps, one thread per row
+        ptx::setmaxnreg_dec<kRegsEpi>();
+        const int row = tid & 127;
+        const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        // the Q rows of the CTA's first tile, by 16-byte copies: two rows (16 lanes each) per instruction
+        {
+            const int cnt = ti.w & 0x1ff, chunk = lane & 15, odd = lane >> 4, bb = (unsigned)ti.x / (unsigned)p.Hkv;
+            const uint32_t dst = base + kOffQ + (chunk >> 3) * (kQBytes / 2) + ((warp & 3) * 32 + odd) * 128;
+#pragma unroll 1
+            for (int x = 0; x * kHalf < cnt; ++x) {
+                const int at = q_row(p.recs[ti.z + min(x * kHalf + row, cnt - 1)].x, bb);
+#pragma unroll 4
+                for (int i = 0; i < 16; ++i) {
+                    const int from = __shfl_sync(0xffffffffu, at, 2 * i + odd);
+                    ptx::cp_async16(dst + x * kQBytes + i * 256 + (((chunk & 7) ^ ((2 * i + odd) & 7)) << 4),
+                                    p.q + from * p.q_pitch + chunk * 8);
+                }
+                ptx::cp_async_wait_all();
+                ptx::fence_proxy_async_smem();
+                ptx::bar_sync(1, 128);
+                if (row == 0) ptx::mbar_arrive(bar_q_full + 8 * x);
+            }
+        }
+        uint32_t tx[2] = {0, 0};
+        bool ok = true;
+        while (tile < n_tiles && ok) {
+            const int4 ti_next = fetch_next();
+            const int cnt = ti.w & 0x1ff, nx = cnt > kHalf ? 2 : 1;
+#pragma unroll 1
+            for (int x = 0; x < nx && ok; ++x) {
+                const uint32_t t = x ? tx[1] : tx[0];
+                const int r = x * kHalf + row;
+                const bool valid = r < cnt;
+                const int2 rs = valid ? *reinterpret_cast<const int2 *>(&p.recs[ti.z + r]) : make_int2(0, 0);
+                const long long slot = (long long)rs.x * p.slots + rs.y;
+                __half *dst = p.part_o + slot * kD;
+                ok = ptx::mbar_wait_warp(bar_l_full + 8 * x, t & 1u, abort_flag) &&
+                     ptx::mbar_wait_warp(bar_o_full + 8 * x, t & 1u, abort_flag);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                // S of the last block is done, so nothing reads this tile's Q any more
-                if (j == nblk - 1 && has_next) gather_q(tid < cnt_next, rec_next.x);
-                const uint32_t s_addr = lane_addr + kColS + st * kBK;
-                uint32_t sr[2][32];
-                ptx::tmem_ld32(s_addr, sr[0]);
-                ptx::tmem_ld32(s_addr + 32, sr[1]);
-                ptx::tmem_wait_ld();
-                const int k0 = (sb0 + j) * kBK;
-                const bool any = valid && k0 <= hi && k0 + kBK - 1 >= lo;
-                if (!(any && k0 >= lo && k0 + kBK - 1 <= hi)) {
-                    // bit c of the mask: column c of the block lies inside the piece
-                    const int ca = lo > k0 ? lo - k0 : 0, cb = hi - k0 < kBK - 1 ? hi - k0 : kBK - 1;
-                    const unsigned long long inside = any ? (~0ull >> (63 - (cb - ca))) << ca : 0ull;
-                    const uint32_t in2[2] = {static_cast<uint32_t>(inside), static_cast<uint32_t>(inside >> 32)};
-#pragma unroll
-                    for (int hlf = 0; hlf < 2; ++hlf)
-#pragma unroll
-                        for (int cc = 0; cc < 32; ++cc)
-                            if (!(in2[hlf] & (1u << cc))) sr[hlf][cc] = 0xff800000u;   // -inf
-                }
-                // block maximum on the raw logits (softmax_scale > 0 on this path), four independent chains
-                float bm;
-                {
-                    float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-#pragma unroll
-                    for (int hlf = 0; hlf < 2; ++hlf)
-#pragma unroll
-                        for (int cc = 0; cc < 32; cc += 8)
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                mx[u] = max3(mx[u], __uint_as_float(sr[hlf][cc + 2 * u]), __uint_as_float(sr[hlf][cc + 2 * u + 1]));
-                    bm = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * p.scale2;
-                }
-                // running reference maximum; O is rescaled only when it moves by more than the threshold
-                const bool first = (l == 0.f);   // no key of this row seen so far
-                const bool need = !first && (bm > m_ref + kRescaleThreshold);
-                if (__any_sync(0xffffffffu, need)) {
-                    // PV of the previous block must have landed before O is touched
-                    const uint32_t np = n - 1u;
-                    ok = ptx::mbar_wait_warp(bar_v_empty + 8 * (np & 1u), (np >> 1) & 1u, abort_flag);
-                    if (!ok) break;
-                    ptx::tc_fence_after();
-                    const float f = need ? ex2_approx(m_ref - bm) : 1.f;
-#pragma unroll 1
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t o[32];
-                        ptx::tmem_ld32(lane_addr + kColO + q4 * 32, o);
-                        ptx::tmem_wait_ld();
-#pragma unroll
-                        for (int cc = 0; cc < 32; ++cc) o[cc] = __float_as_uint(__uint_as_float(o[cc]) * f);
-                        ptx::tmem_st32(lane_addr + kColO + q4 * 32, o);
-                    }
-                    if (need) { l *= f; m_ref = bm; }
-                }
-                if (first && bm > -CUDART_INF_F) m_ref = bm;   // first keys of this row
-                uint32_t pk[32];
-                {
-                    // p = 2^(s*scale - m_ref), two columns per packed fp32x2 instruction; masked columns
-                    // hold -inf and give 0 (a row with no key so far has m_ref = -inf: it subtracts 0)
-                    const float neg_m = m_ref > -CUDART_INF_F ? -m_ref : 0.f;
-                    const unsigned long long sc2 = pack2(p.scale2, p.scale2), nm2 = pack2(neg_m, neg_m);
-                    unsigned long long acc2[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) acc2[u] = pack2(0.f, 0.f);
-#pragma unroll
-                    for (int cc = 0; cc < 32; ++cc) {
-                        const int hlf = cc >> 4, c2 = (cc & 15) * 2;
-                        const unsigned long long y = ffma2(
-                            pack2(__uint_as_float(sr[hlf][c2]), __uint_as_float(sr[hlf][c2 + 1])), sc2, nm2);
-                        float y0, y1;
-                        unpack2(y, y0, y1);
-                        const float p0 = ex2_approx(y0), p1 = ex2_approx(y1);
-                        acc2[cc & 3] = fadd2(acc2[cc & 3], pack2(p0, p1));
-                        const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
-                        pk[cc] = *reinterpret_cast<const uint32_t *>(&pp);
-                    }
-                    float s0, s1, s2, s3;
-                    unpack2(fadd2(acc2[0], acc2[1]), s0, s1);
-                    unpack2(fadd2(acc2[2], acc2[3]), s2, s3);
-                    l += (s0 + s1) + (s2 + s3);
-                }
-                ptx::tmem_st32(s_addr, pk);
-                ptx::tmem_wait_st();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_p_ready + 8 * st);
-            }
-            // the next tile's Q rows were requested a block ago: publish them now, so that its first
-            // S = Q K^T runs while this tile drains
-            if (ok && has_next) publish_q();
-            // epilogue: normalised piece output and its log-sum-exp
-            if (ok) ok = ptx::mbar_wait_warp(bar_o_full, T & 1u, abort_flag);
-            if (!ok) break;
-            ptx::tc_fence_after();
-            {
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-                const long long slot = (long long)rec.x * p.slots + rec.y;
-                __half *dst = p.part_o + slot * kD;
+                const float2 stat = meta->stats[r];
                 uint32_t exps = 0;   // biased exponent of each 32-column chunk's largest magnitude
                 // one 32-column chunk: block exponent, fp16 mantissas, two 32-byte stores
-                auto emit = [&](uint32_t (&o)[32], int q4) {
+#pragma unroll 1
+                for (int q4 = 0; q4 < 4; ++q4) {
+                    uint32_t o[32];
+                    ptx::tmem_ld32(lane_addr + kColO + x * kD + q4 * 32, o);
+                    ptx::tmem_wait_ld();
+                    if (q4 == 3) {
+                        // O is in registers: the next tile's first PV may overwrite it
+                        ptx::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(bar_o_empty + 8 * x);
+                    }
                     if (valid) {
-                        float amax = 0.f;
+                        float am[2] = {0.f, 0.f};
 #pragma unroll
-                        for (int cc = 0; cc < 32; ++cc) {
-                            const float x = __uint_as_float(o[cc]) * inv;
-                            o[cc] = __float_as_uint(x);
-                            amax = fmaxf(amax, fabsf(x));
-                        }
+                        for (int cc = 0; cc < 32; cc += 4)
+#pragma unroll
+                            for (int u = 0; u < 2; ++u)
+                                am[u] = max3(am[u], fabsf(__uint_as_float(o[cc + 2 * u])), fabsf(__uint_as_float(o[cc + 2 * u + 1])));
+                        const float amax = fmaxf(am[0], am[1]) * stat.x;
                         uint32_t eb = (__float_as_uint(amax) >> 23) & 0xffu;
                         eb = eb < 1u ? 1u : (eb > 252u ? 252u : eb);
                         exps |= eb << (8 * q4);
-                        const float down = __uint_as_float((253u - eb) << 23);   // 2^(126 - eb): chunk into [-1, 1]
+                        // normalisation and 2^(126 - eb), which brings the chunk into [-1, 1], in one factor
+                        const float down = stat.x * __uint_as_float((253u - eb) << 23);
 #pragma unroll
                         for (int s8 = 0; s8 < 2; ++s8) {
                             uint32_t w[8];
@@ -504,33 +462,140 @@ tc_attend(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUte
                             ptx::st_global_v8(dst + q4 * 32 + s8 * 16, w);
                         }
                     }
-                };
-                // the TMEM read of the next chunk is in flight while this one is converted and stored
-                uint32_t oa[32], ob[32];
-                ptx::tmem_ld32(lane_addr + kColO, oa);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(lane_addr + kColO + 32, ob);
-                emit(oa, 0);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(lane_addr + kColO + 64, oa);
-                emit(ob, 1);
-                ptx::tmem_wait_ld();
-                ptx::tmem_ld32(lane_addr + kColO + 96, ob);
-                emit(oa, 2);
-                ptx::tmem_wait_ld();
-                // O is in registers: the next tile's first PV may overwrite it
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_o_empty);
-                emit(ob, 3);
-                if (valid)
-                    p.part_lse[slot] = make_float2(l > 0.f ? m_ref + log2f(l) : -CUDART_INF_F, __uint_as_float(exps));
+                }
+                if (valid) p.part_lse[slot] = make_float2(stat.y, __uint_as_float(exps));
+                if (x) ++tx[1]; else ++tx[0];
             }
-            n_kv += nblk;
-            rec = rec_next;
+            tile += tile_step;
             ti = ti_next;
         }
-        ptx::cp_async_wait_all();
+    } else {
+        // ---------------- row warps of stream x: softmax per 64-key block, one thread per row
+        ptx::setmaxnreg_inc<kRegsRow>();
+        const int x = warp >> 2, row = tid & 127, r = x * kHalf + row;
+        const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t o_addr = lane_addr + kColO + x * kD, s_col = lane_addr + kColS + x * (2 * kBK);
+        auto interval = [&](const int4 &t) {   // {lo, hi} of this thread's piece
+            return r < (t.w & 0x1ff) ? *reinterpret_cast<const int2 *>(&p.recs[t.z + r].z) : make_int2(INT_MAX, -1);
+        };
+        uint32_t n = 0, na = 0, t = 0;   // blocks and tiles of the stream so far; all blocks of the CTA
+        auto range = [&](int t) { return t < n_tiles ? (x ? p.ranges[t].y : p.ranges[t].x) : 0; };
+        int2 iv = interval(ti);
+        int rg = range(tile);
+        bool ok = true;
+        while (tile < n_tiles && ok) {
+            const int4 ti_next = fetch_next();
+            const int2 iv_next = interval(ti_next);   // requested a tile ahead
+            const int rg_next = range(tile + tile_step);
+            const int nblk = ti.w >> 9, first_block = rg & 0xffff, end_block = rg >> 16;
+            if (first_block < end_block) {
+                const int lo = iv.x, hi = iv.y;
+                int k0 = (ti.y + 1 - nblk + first_block) * kBK;
+                float m_ref = -CUDART_INF_F, l = 0.f;
+#pragma unroll 1
+                for (int j = first_block; j < end_block; ++j, ++n, k0 += kBK) {
+                    const uint32_t b = n & 1u, ph = (n >> 1) & 1u;
+                    ok = ptx::mbar_wait_warp(bar_s_full + 16 * x + 8 * b, ph, abort_flag);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    uint32_t sr[2][32];
+                    ptx::tmem_ld32(s_col + b * kBK, sr[0]);
+                    ptx::tmem_ld32(s_col + b * kBK + 32, sr[1]);
+                    ptx::tmem_wait_ld();
+                    const bool any = k0 <= hi && k0 + kBK - 1 >= lo;
+                    if (!(any && k0 >= lo && k0 + kBK - 1 <= hi)) {
+                        // bit c of the mask: column c of the block lies inside the piece
+                        const int ca = lo > k0 ? lo - k0 : 0, cb = hi - k0 < kBK - 1 ? hi - k0 : kBK - 1;
+                        const unsigned long long inside = any ? (~0ull >> (63 - (cb - ca))) << ca : 0ull;
+                        const uint32_t in2[2] = {static_cast<uint32_t>(inside), static_cast<uint32_t>(inside >> 32)};
+#pragma unroll
+                        for (int hlf = 0; hlf < 2; ++hlf)
+#pragma unroll
+                            for (int cc = 0; cc < 32; ++cc)
+                                if (!(in2[hlf] & (1u << cc))) sr[hlf][cc] = 0xff800000u;   // -inf
+                    }
+                    // block maximum on the raw logits (softmax_scale > 0 on this path), four independent chains
+                    float bm;
+                    {
+                        float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+                        for (int hlf = 0; hlf < 2; ++hlf)
+#pragma unroll
+                            for (int cc = 0; cc < 32; cc += 8)
+#pragma unroll
+                                for (int u = 0; u < 4; ++u)
+                                    mx[u] = max3(mx[u], __uint_as_float(sr[hlf][cc + 2 * u]), __uint_as_float(sr[hlf][cc + 2 * u + 1]));
+                        bm = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * p.scale2;
+                    }
+                    // running reference maximum; O is rescaled only when it moves by more than the threshold
+                    const bool first = (l == 0.f);   // no key of this row seen so far
+                    const bool need = !first && (bm > m_ref + kRescaleThreshold);
+                    if (__any_sync(0xffffffffu, need)) {
+                        // PV of the block before must have landed before O is touched
+                        const uint32_t np = na + j - 1u;
+                        ok = ptx::mbar_wait_warp(bar_kv_empty + 8 * (x * kKS + np % kKS), (np / kKS) & 1u, abort_flag);
+                        if (!ok) break;
+                        ptx::tc_fence_after();
+                        const float f = need ? ex2_approx(m_ref - bm) : 1.f;
+#pragma unroll 1
+                        for (int q8 = 0; q8 < 8; ++q8) {
+                            uint32_t o[16];
+                            ptx::tmem_ld16(o_addr + q8 * 16, o);
+                            ptx::tmem_wait_ld();
+#pragma unroll
+                            for (int cc = 0; cc < 16; ++cc) o[cc] = __float_as_uint(__uint_as_float(o[cc]) * f);
+                            ptx::tmem_st16(o_addr + q8 * 16, o);
+                        }
+                        if (need) { l *= f; m_ref = bm; }
+                    }
+                    if (first && bm > -CUDART_INF_F) m_ref = bm;   // first keys of this row
+                    uint32_t pk[32];
+                    {
+                        // p = 2^(s*scale - m_ref), two columns per packed fp32x2 instruction; masked columns
+                        // hold -inf and give 0 (a row with no key so far has m_ref = -inf: it subtracts 0)
+                        const float neg_m = m_ref > -CUDART_INF_F ? -m_ref : 0.f;
+                        const unsigned long long sc2 = pack2(p.scale2, p.scale2), nm2 = pack2(neg_m, neg_m);
+                        unsigned long long acc2[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) acc2[u] = pack2(0.f, 0.f);
+#pragma unroll
+                        for (int cc = 0; cc < 32; ++cc) {
+                            const int hlf = cc >> 4, c2 = (cc & 15) * 2;
+                            const unsigned long long y = ffma2(
+                                pack2(__uint_as_float(sr[hlf][c2]), __uint_as_float(sr[hlf][c2 + 1])), sc2, nm2);
+                            float y0, y1;
+                            unpack2(y, y0, y1);
+                            const float p0 = ex2_approx(y0), p1 = ex2_approx(y1);
+                            acc2[cc & 3] = fadd2(acc2[cc & 3], pack2(p0, p1));
+                            const __nv_bfloat162 pp = __floats2bfloat162_rn(p0, p1);
+                            pk[cc] = *reinterpret_cast<const uint32_t *>(&pp);
+                        }
+                        float s0, s1, s2, s3;
+                        unpack2(fadd2(acc2[0], acc2[1]), s0, s1);
+                        unpack2(fadd2(acc2[2], acc2[3]), s2, s3);
+                        l += (s0 + s1) + (s2 + s3);
+                    }
+                    ptx::tmem_st32(s_col + b * kBK, pk);
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar_p_ready + 16 * x + 8 * b);
+                }
+                // the epilogue has read the statistics (and O) of the tile before
+                if (ok && t > 0) ok = ptx::mbar_wait_warp(bar_o_empty + 8 * x, (t - 1u) & 1u, abort_flag);
+                ++t;
+                if (ok) {
+                    meta->stats[r] = make_float2(l > 0.f ? 1.f / l : 0.f, l > 0.f ? m_ref + log2f(l) : -CUDART_INF_F);
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar_l_full + 8 * x);
+                }
+            }
+            na += nblk;
+            tile += tile_step;
+            ti = ti_next;
+            iv = iv_next;
+            rg = rg_next;
+        }
     }
 
     // ---- teardown
@@ -540,7 +605,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUte
         __nanosleep(200000);   // let copies and MMAs that may still be in flight land
         __syncthreads();
     }
-    if (warp == 4) {
+    if (warp == 12) {
         __syncwarp();
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, kTmemCols);
@@ -926,19 +991,48 @@ bool make_kv_map(CUtensorMap *tm, const void *ptr, const Call &c, int slot[3]) {
     return r == CUDA_SUCCESS;
 }
 
+// Q as rows of 128 elements at one common pitch (the greatest common divisor of its strides), for the row gather.
+// False when rows at that pitch would overlap: the caller then works on a dense copy of Q.
+long long gcd_ll(long long a, long long b) { while (b) { const long long t = a % b; a = b; b = t; } return a; }
+long long q_pitch(const Call &c) {
+    long long g = c.q_st;
+    if (c.Hq > 1) g = gcd_ll(g, c.q_sh);
+    if (c.B > 1) g = gcd_ll(g, c.q_sb);
+    return g;
+}
+bool q_rows_fit(const Call &c) {
+    const long long g = q_pitch(c);
+    if (g < kD || g >= (1ll << 39)) return false;
+    return ((c.B - 1) * c.q_sb + (c.Hq - 1) * c.q_sh + (c.Lq - 1) * c.q_st) / g < (1ll << 31) - 1;
+}
+bool make_q_map(CUtensorMap *tm, const void *ptr, const Call &c) {
+    auto fn = encode_fn();
+    if (!fn) return false;
+    const long long g = q_pitch(c);
+    cuuint64_t gdim[2] = {(cuuint64_t)kD, (cuuint64_t)(((c.B - 1) * c.q_sb + (c.Hq - 1) * c.q_sh + (c.Lq - 1) * c.q_st) / g + 1)};
+    cuuint64_t gstr[1] = {(cuuint64_t)g * 2};
+    cuuint32_t box[2] = {64, 1}, estr[2] = {1, 1};
+    CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), gdim, gstr, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// out[0] tiles, out[1] pieces, out[2] sum over tiles of (key blocks walked), out[3] sum of pieces x blocks
-__global__ void __launch_bounds__(256) tile_stats(const int4 *__restrict__ tiles, const int *__restrict__ n_tiles,
-                                                  unsigned long long *out) {
+// A stream of up to 128 pieces counts as a tile: out[0] tiles, out[1] pieces, out[2] sum over tiles of (key blocks
+// walked), out[3] sum of pieces x blocks
+__global__ void __launch_bounds__(256) tile_stats(const int4 *__restrict__ tiles, const int2 *__restrict__ ranges,
+                                                  const int *__restrict__ n_tiles, unsigned long long *out) {
     const int n = *n_tiles;
-    unsigned long long a = 0, b = 0, c2 = 0;
+    unsigned long long a = 0, b = 0, c2 = 0, d = 0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const int w = tiles[t].w, cnt = w & 0xff, nblk = w >> 8;
-        a += cnt; b += nblk; c2 += (unsigned long long)cnt * nblk;
+        const int cnt = tiles[t].w & 0x1ff;
+        const int2 r = ranges[t];
+        const int n0 = min(cnt, kHalf), n1 = cnt - n0, w0 = (r.x >> 16) - (r.x & 0xffff), w1 = (r.y >> 16) - (r.y & 0xffff);
+        a += cnt; b += w0 + w1; c2 += (unsigned long long)n0 * w0 + (unsigned long long)n1 * w1; d += 1 + (n1 > 0);
     }
-    atomicAdd(out + 1, a); atomicAdd(out + 2, b); atomicAdd(out + 3, c2);
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = n;
+    atomicAdd(out, d); atomicAdd(out + 1, a); atomicAdd(out + 2, b); atomicAdd(out + 3, c2);
 }
 
 }  // namespace
@@ -946,7 +1040,7 @@ __global__ void __launch_bounds__(256) tile_stats(const int4 *__restrict__ tiles
 cudaError_t launch_tile_stats(const TcLast &last, long long *out4_device, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(out4_device, 0, 4 * sizeof(long long), st);
     if (e != cudaSuccess) return e;
-    tile_stats<<<64, 256, 0, st>>>(last.tiles, last.n_tiles, reinterpret_cast<unsigned long long *>(out4_device));
+    tile_stats<<<64, 256, 0, st>>>(last.tiles, last.ranges, last.n_tiles, reinterpret_cast<unsigned long long *>(out4_device));
     return cudaGetLastError();
 }
 
@@ -1031,6 +1125,7 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     // every (batch, kv head) list is cut every kRows records (one ragged tile each) and split again at
     // gaps between end blocks (fewer than NB per list)
     p.max_tiles = (long long)(slots / kRows) + (long long)p.n_bg * (p.NB + 1) + 1;
+    if (p.max_tiles < kMinTiles) p.max_tiles = kMinTiles;   // every CTA reads its first entry before it knows the count
     size_t off = 0;
     // a region of `size` bytes at the next 256-byte boundary, with a canary gap before it when asked for
     auto take = [&](size_t size) {
@@ -1045,10 +1140,12 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     p.off_key_cursor = p.off_key_count + align256(n_keys * 4);
     p.off_cta_hist = take((size_t)p.ctas_per_bg * n_keys * 4);
     p.off_tiles = take((size_t)p.max_tiles * 16);
+    p.off_ranges = take((size_t)p.max_tiles * 8);
     p.off_recs = take(slots * 16);
     p.off_npieces = take(rows);
     p.off_part_lse = take(slots * 8);
     p.off_part_o = take(slots * kD * 2);
+    p.off_q = take(q_rows_fit(c) ? 0 : rows * kD * 2);
     if (gap) { p.canaries.add(off); off += gap; }
     p.bytes = off;
     return p;
@@ -1068,9 +1165,11 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
     if (plan.bytes > scratch_bytes || !plan.ok) return cudaErrorMemoryAllocation;
     if (plan.max_tiles > (1ll << 30) || (long long)c.B * c.Hq * Lc * plan.slots > (1ll << 31) - 1) return cudaErrorInvalidValue;
 
-    CUtensorMap tm_k, tm_v;
+    CUtensorMap tm_q, tm_k, tm_v;
     int slot[3];
     if (!make_kv_map(&tm_k, k, c, slot) || !make_kv_map(&tm_v, v, c, slot)) return cudaErrorInvalidValue;
+    const bool q_copied = !q_rows_fit(c);
+    if (!q_copied && !make_q_map(&tm_q, q, c)) return cudaErrorInvalidValue;
     // function attributes belong to a device's context: remember them per device, not per process
     static bool attr_set[64] = {};
     int dev = 0;
@@ -1100,6 +1199,7 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         pa.totals = counters + 16;
         pa.n_tiles = counters;
         pa.tiles = (int4 *)(ws + plan.off_tiles);
+        pa.ranges = (int2 *)(ws + plan.off_ranges);
         pa.max_tiles = (int)plan.max_tiles;
         pa.recs = (int4 *)(ws + plan.off_recs);
         // the parked pieces borrow the head of the partial-output buffer, which is written only after them
@@ -1110,17 +1210,35 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         e = tc::prepare(pa, st, launches);
         if (e != cudaSuccess) return e;
         TcParams tp;
-        tp.q = (const bf16 *)q; tp.q_sb = c.q_sb; tp.q_sh = c.q_sh; tp.q_st = c.q_st;
-        tp.Hq = c.Hq; tp.G = c.G; tp.Lc = lc; tp.slots = plan.slots; tp.r0 = r0;
+        if (q_copied) {
+            // strides without a common row pitch: the chunk's rows of Q as a dense [B, Hq, lc, 128] tensor
+            Call d = c;
+            d.Lq = lc; d.q_st = kD; d.q_sh = (long long)lc * kD; d.q_sb = d.q_sh * c.Hq;
+            bf16 *qd = (bf16 *)(ws + plan.off_q);
+            for (int bh = 0; bh < c.B * c.Hq; ++bh) {
+                const bf16 *src = (const bf16 *)q + (bh / c.Hq) * c.q_sb + (bh % c.Hq) * c.q_sh + r0 * c.q_st;
+                e = cudaMemcpy2DAsync(qd + bh * d.q_sh, kD * 2, src, (size_t)c.q_st * 2, kD * 2, lc, cudaMemcpyDeviceToDevice, st);
+                if (e != cudaSuccess) return e;
+            }
+            if (!make_q_map(&tm_q, qd, d)) return cudaErrorInvalidValue;
+            tp.q = qd; tp.q_pitch = kD;
+            tp.q_b = c.Hq * lc; tp.q_h = lc; tp.q_t = 1; tp.r0 = 0;
+        } else {
+            const long long g = q_pitch(c);
+            tp.q = (const bf16 *)q; tp.q_pitch = g;
+            tp.q_b = (int)(c.B > 1 ? c.q_sb / g : 0); tp.q_h = (int)(c.Hq > 1 ? c.q_sh / g : 0); tp.q_t = (int)(c.q_st / g);
+            tp.r0 = (int)r0;
+        }
+        tp.Hq = c.Hq; tp.G = c.G; tp.Lc = lc; tp.slots = plan.slots;
         tp.scale2 = c.softmax_scale * kLog2e;
         tp.slot_t = slot[0]; tp.slot_h = slot[1]; tp.slot_b = slot[2];
-        tp.recs = pa.recs; tp.tiles = pa.tiles;
+        tp.recs = pa.recs; tp.tiles = pa.tiles; tp.ranges = pa.ranges;
         tp.n_tiles = counters;
         tp.part_o = (__half *)(ws + plan.off_part_o); tp.part_lse = (float2 *)(ws + plan.off_part_lse);
         tp.status = c.status; tp.Hkv = c.Hkv;
-        if (last) { last->tiles = pa.tiles; last->n_tiles = counters; }
+        if (last) { last->tiles = pa.tiles; last->ranges = pa.ranges; last->n_tiles = counters; }
         if (timer) timer->begin(st);
-        tc_attend<<<2 * sm_count, kThreads, kSmemBytes, st>>>(tm_k, tm_v, tp);
+        tc_attend<<<sm_count, kThreads, kSmemBytes, st>>>(tm_q, tm_k, tm_v, tp);
         if (timer) timer->end(st);
         const unsigned mblocks = (unsigned)((rows * 16 + 255) / 256);
         if (c.mode == SLA_PER_SPAN && c.top_k <= kGateK)

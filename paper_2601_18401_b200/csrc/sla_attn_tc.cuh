@@ -8,13 +8,13 @@ namespace sla {
 namespace tc {
 
 constexpr int kBK = 64;     // keys per block
-constexpr int kRows = 128;  // pieces per tile
+constexpr int kRows = 256;  // pieces per tile
 
 // Work list of one chunk of query positions, as laid out in the scratch memory:
 //   recs   int4 {row, slot of the row's partial results, lo, hi}: every piece of every row, ordered by
 //          (batch*Hkv + kv head, 64-key block of hi, class of blocks covered)
-//   tiles  int4 {batch*Hkv + kv head, end block of the last record, first record, records | key blocks to walk << 8}:
-//          128 consecutive records, split where neighbouring records end more than a few key blocks apart
+//   tiles  int4 {batch*Hkv + kv head, end block of the last record, first record, records | key blocks to walk << 9}:
+//          256 consecutive records, split where neighbouring records end more than a few key blocks apart
 //   n_tiles, n_pieces[row], and the per-piece partial results
 struct PrepArgs {
     const int32_t *anchor;   // [B,Hq,Lq,top_k]
@@ -36,6 +36,7 @@ struct PrepArgs {
     int *totals;             // [B*Hkv][2]: records and tiles of each (batch, kv head)
     int *n_tiles;            // total number of tiles
     int4 *tiles;
+    int2 *ranges;            // [max_tiles] blocks of the walk the tile's first and second 128 pieces reach: first | end << 16
     int max_tiles;
     int4 *recs;
     int4 *stage;             // [rows][slots] {lo, hi, bucket | slot << 24, ordinal within (CTA, bucket)}: the pieces as

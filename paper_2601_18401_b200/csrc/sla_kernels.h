@@ -53,15 +53,15 @@ struct TcPlan {
     int slots;   // partial results per query row: top_k, plus one for the local window
     bool ok;   // false when the shared-memory histogram of the counting sort cannot hold NB buckets
     long long max_tiles;
-    size_t off_counters, off_key_count, off_key_cursor, off_cta_hist, off_tiles, off_recs, off_npieces, off_part_lse,
-        off_part_o, bytes;
+    size_t off_counters, off_key_count, off_key_cursor, off_cta_hist, off_tiles, off_ranges, off_recs, off_npieces, off_part_lse,
+        off_part_o, off_q, bytes;
     Canaries canaries;
 };
 bool tc_attention_shape_ok(const Call &c, int dtype);  // host-only shape test
 bool tc_attention_supported(const Call &c, int dtype); // shape test + driver entry point present
 TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap = 0);   // gap: bytes of canary between regions
 // Where the tile table of the most recent chunk lives (for sla_attention_tile_stats).
-struct TcLast { const int4 *tiles = nullptr; const int *n_tiles = nullptr; };
+struct TcLast { const int4 *tiles = nullptr; const int2 *ranges = nullptr; const int *n_tiles = nullptr; };
 cudaError_t launch_tile_stats(const TcLast &last, long long *out4_device, cudaStream_t st);
 // Splits the query rows into chunks whose scratch fits `scratch_bytes`; adds its kernel launches to
 // *launches.  Returns cudaErrorMemoryAllocation when not even one query position fits.

@@ -27,3 +27,60 @@ def test_pieces_joined_or_not(sla, handle, rows):
     rows of a whole sequence are joined."""
     w = workload(n_q_heads=8, n_kv_heads=2, seq_len=6144, span_len=70, top_k=8, planted_spans=2)
     run_prefill(sla, handle, w, q_pos0=6144 - 3 * rows, Lq=3 * rows)
+
+
+@pytest.mark.parametrize("seq_len", [127, 128, 129, 255, 256, 257, 384, 385])
+def test_streams_of_a_tile(sla, handle, seq_len):
+    """One piece per row: tiles whose second stream of 128 pieces is missing, has one piece or is full."""
+    run_prefill(sla, handle, workload(n_q_heads=1, n_kv_heads=1, seq_len=seq_len, top_k=1, span_len=40))
+
+
+@pytest.mark.parametrize("span_len", [10, 31, 32, 33, 600])
+def test_walks_of_one_block_and_of_many(sla, handle, span_len):
+    """Spans within a block, over one boundary and over nineteen blocks; two batches, three KV heads."""
+    run_prefill(sla, handle, workload(batch=2, n_q_heads=6, n_kv_heads=3, seq_len=1930, top_k=2, span_len=span_len, seed=78))
+
+
+def test_query_strides_without_a_common_row_pitch(sla, handle):
+    """Heads that start 8 elements after a multiple of the token stride (the rows of Q cannot be numbered at one
+    pitch of 128 elements or more), and token rows of 136 elements: same results as on dense tensors."""
+    import torch
+    from paper_2601_18401_b200 import synth
+    w = workload(batch=2, seq_len=700, span_len=30, top_k=3)
+    x = synth.make_prefill(w, device="cuda:0")
+    B, H, L, D = x["q"].shape
+    params = sla.make_params(w.top_k, w.span_len, head_dim=D)
+    anchor, _ = sla.sla_span_search(handle, x["q_s"], x["k"], params)
+    out, lse = sla.sla_span_attention(handle, x["q"], x["k"], x["v"], anchor, params)
+    for st, sh in ((D, L * D + 8), (D + 8, L * (D + 8) + 8)):
+        q = torch.zeros(B * H * sh, dtype=x["q"].dtype, device="cuda").as_strided((B, H, L, D), (H * sh, sh, st, 1))
+        q.copy_(x["q"])
+        out2, lse2 = sla.sla_span_attention(handle, q, x["k"], x["v"], anchor, params)
+        torch.cuda.synchronize()
+        assert sla.sla_poll_status(handle) == sla.SLA_OK
+        assert torch.equal(out2.contiguous(), out) and torch.equal(lse2, lse)
+
+
+def test_end_blocks_far_apart(sla, handle):
+    """Anchors in two narrow regions and in a few places between them: tiles are cut where neighbouring pieces of
+    the work list end further apart than a span is long, and streams of one tile walk different key blocks."""
+    import parity_util as P
+    import torch
+    from oracle import sla_oracle as O
+    from paper_2601_18401_b200 import synth
+    L, top_k, span_len = 9000, 3, 90
+    w = workload(n_q_heads=2, n_kv_heads=1, seq_len=L, span_len=span_len, top_k=top_k)
+    x = synth.make_prefill(w, device="cuda:0")
+    g = torch.Generator().manual_seed(5)
+    i = torch.arange(L)[None, None, :, None]
+    shape = (1, 2, L, top_k)
+    place = torch.randint(0, 10, shape, generator=g)
+    spot = torch.where(place < 5, torch.randint(300, 420, shape, generator=g), torch.randint(8000, 8100, shape, generator=g))
+    spot = torch.where(place == 9, torch.randint(0, 6, shape, generator=g) * 1000 + 1500, spot)
+    anchor = torch.where(spot <= i, spot, torch.full(shape, -1)).to(torch.int32).cuda()
+    params = sla.make_params(top_k, span_len, head_dim=128)
+    out, lse = sla.sla_span_attention(handle, x["q"], x["k"], x["v"], anchor, params)
+    torch.cuda.synchronize()
+    assert sla.sla_poll_status(handle) == sla.SLA_OK
+    ref = P.oracle_attention_for(P.host_inputs(x), O.BF16, anchor.cpu().numpy(), w)
+    P.compare_attention(out, lse, ref, "bf16")
