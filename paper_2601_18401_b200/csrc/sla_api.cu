@@ -551,7 +551,7 @@ sla_status_t sla_decode_step(sla_handle_t h, const void *q_s, const void *q, con
                                reinterpret_cast<int *>(h->ws + kCounterOffset), out, lse, out_anchor, out_score, st);
     if (e == cudaSuccess) e = sla::launch_canary_check(h->ws + kHeaderBytes, plan.canaries, c.status, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "sla_decode_step");
-    h->launches += 2;
+    h->launches += plan.score_first ? 2 : 1;
     if (plan.canaries.n) { h->last_canaries = plan.canaries; h->last_canary_base = h->ws + kHeaderBytes; }
     return SLA_OK;
 }

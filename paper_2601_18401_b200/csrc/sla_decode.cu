@@ -4,20 +4,20 @@
 // kernel spreads each head's tokens evenly over many CTAs (split-K), streams whole rows with 16-byte
 // loads, keeps a running (max, denominator, numerator) per lane group and merges at the end.
 //
-//   decode_score   grid (anchor chunks, B*Hkv, head tiles)   K anchor rows x G routing queries -> scores.  In
-//                  the sequence-sharded step the CTA that finishes a (batch, KV head) last also selects this
-//                  rank's k best candidates.
-//   decode_attn    grid (n_splits, attention units)          every CTA first selects the k best anchors of its
-//                  head from the scores (a threshold from the thread maxima, the candidates ranked), builds the
-//                  spans of its unit and clips the overlaps -- redundantly per CTA, so that nothing waits for
-//                  one CTA to do it for all -- then runs the online softmax over an even share of the tokens;
-//                  the CTA that finishes a unit last merges the split results through their log-sum-exp.
+//   decode_attn    clusters of up to 8 CTAs, grid (CTAs per attention unit, units): the whole step in one launch.  A
+//                  cluster scores the anchors of its head, a share per CTA, keeps the k best of every share and then of
+//                  all shares (distributed shared memory); every CTA builds the spans of its unit, clips the
+//                  overlaps and runs the online softmax over an even share of the tokens; the cluster's first CTA
+//                  merges the partial results through their log-sum-exp.
 //                  Union mode: one unit per head (its spans and the local window, clipped to disjoint pieces).
 //                  Per-span mode (Algorithm 1 literally): one unit per selected anchor, J_t = S_t united with
 //                  the window; the unit that finishes a head last applies the gate of Section "Combination" to
 //                  the units' outputs.
+//   decode_score   (sequence-sharded step) grid (anchor chunks, B*Hkv, head tiles): K anchor rows x G routing queries ->
+//                  scores; the CTA that finishes a (batch, KV head) last selects this rank's k best candidates.
 // "Last" is decided by an atomic counter per unit / per head in the handle's header region; the last CTA puts
 // the counter back to zero, so a step leaves them as it found them.
+#include <cooperative_groups.h>
 #include <limits.h>
 #include <math_constants.h>
 
@@ -25,6 +25,8 @@
 #include "sla_topk.cuh"
 
 namespace sla {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -41,7 +43,7 @@ template <int LPR> __device__ inline float reduce_sub(float x) {
 template <typename T, int D, int GT>
 __global__ void __launch_bounds__(kScoreThreads)
 decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long long n_ctx, int n, int s_min,
-             float *__restrict__ scores, int *__restrict__ done, int *__restrict__ spans,
+             float *__restrict__ scores, int *__restrict__ done,
              int32_t *__restrict__ out_anchor, float *__restrict__ out_score) {
     extern __shared__ float dsm[];
     __shared__ int s_last;
@@ -57,9 +59,10 @@ decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long lo
     const long long i = n_ctx - 1;
     const T *kbase = k + b * c.kv_sb + g * c.kv_sh;
 
-    // the attention kernel of this step may be scheduled now; it waits for this grid to finish before it
-    // touches anything this kernel writes
+    // the attention kernel of this step may be scheduled now; it waits for this grid to finish before it reads scores.
+    // This grid itself may have been launched beside the tail of the kernel before it.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     float qv[GT][E];
 #pragma unroll
     for (int t = 0; t < GT; ++t) Vec16<T>::load(q_s + b * c.q_sb + (long long)(h0 + t) * c.q_sh + sub * E, qv[t]);
@@ -93,8 +96,7 @@ decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long lo
         }
     }
 
-    // the unsharded step selects in the attention kernel (every CTA for its own head): scores only
-    if (!done) return;
+    if (!done) return;   // the unsharded step selects in the attention kernel: scores only
     // ---- the CTA that completes this (batch, KV head) selects (sequence-sharded step: this rank's candidates)
     __threadfence();
     __syncthreads();
@@ -107,15 +109,10 @@ decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long lo
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    constexpr int kIv = kMaxTopK + 1;   // the spans and the window
-    const int per_warp = n + 2 * topk::kCap + 4 * kIv;
+    const int per_warp = n + 2 * topk::kCap;
     float *sc = dsm + (size_t)warp * per_warp;
     float *cand_v = sc + n;
     int *cand_s = reinterpret_cast<int *>(cand_v + topk::kCap);
-    int *s_lo = cand_s + topk::kCap, *s_hi = s_lo + kIv, *p_lo = s_hi + kIv, *p_hi = p_lo + kIv;
-    const long long ell = base_len(c, i);
-    // span table of an attention unit: piece starts [pcap], cumulative token counts [pcap + 1], count
-    const int pcap = c.mode == SLA_PER_SPAN ? 2 : c.top_k + 1, tstride = 2 * pcap + 2;
     for (int hg = warp; hg < c.G; hg += kWarps) {
         const long long bh = (long long)b * c.Hq + g * c.G + hg;
         const float *src = scores + bh * n;
@@ -124,114 +121,141 @@ decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long lo
         topk::select_topk(sc, n, c.top_k, i, cand_v, cand_s, out_anchor + bh * c.top_k, out_score + bh * c.top_k, lane,
                           s_min, c.off);
         __syncwarp();
-        if (!spans) continue;   // sequence-sharded step: the spans are built after the global selection
-        // intervals: the spans of the selected anchors (Algorithm 1: S_t = [max(0,t-b l), min(i,t+f l)])
-        // and, last, the local window W = [max(0, i-w+1), i]
-        const int n_iv = c.top_k + (c.window > 0 ? 1 : 0);
-        const int w_lo = (int)(i - c.window + 1 > 0 ? i - c.window + 1 : 0);
-        for (int j = lane; j < n_iv; j += 32) {
-            int lo = INT_MAX, hi = -1;
-            if (j == c.top_k) {
-                lo = w_lo;
-                hi = (int)i;
-            } else {
-                const long long t = out_anchor[bh * c.top_k + j];
-                if (t >= 0) {
-                    const long long a = t - (long long)c.back * ell, z = t + (long long)c.fwd * ell;
-                    lo = (int)(a > 0 ? a : 0);
-                    hi = (int)(z < i ? z : i);
-                }
-            }
-            s_lo[j] = lo;
-            s_hi[j] = hi;
-        }
-        __syncwarp();
-        if (c.mode == SLA_PER_SPAN) {
-            // one attention unit per selected anchor: the part of S_t left of the window, then the window
-            if (lane == 0) {
-                int n_sel = 0;
-                for (int j = 0; j < c.top_k; ++j) n_sel += s_hi[j] >= 0;
-                for (int j = 0; j < c.top_k; ++j) {
-                    int *start = spans + (bh * c.top_k + j) * tstride;
-                    int *cum = start + pcap;
-                    int cnt = 0, total = 0;
-                    cum[0] = 0;
-                    // a head with nothing selected attends to the window alone: its first unit carries it
-                    const bool sel = s_hi[j] >= 0, lone_w = n_sel == 0 && j == 0 && c.window > 0;
-                    if (sel) {
-                        const int hi_cut = c.window > 0 && s_hi[j] >= w_lo ? w_lo - 1 : s_hi[j];
-                        if (s_lo[j] <= hi_cut) {
-                            start[cnt] = s_lo[j];
-                            total += hi_cut - s_lo[j] + 1;
-                            cum[++cnt] = total;
-                        }
-                    }
-                    if ((sel || lone_w) && c.window > 0) {
-                        start[cnt] = w_lo;
-                        total += (int)i - w_lo + 1;
-                        cum[++cnt] = total;
-                    }
-                    start[2 * pcap + 1] = cnt;
-                }
-            }
-            __syncwarp();
-            continue;
-        }
-        // union mode: sort by (lo, hi), clip to disjoint pieces, cumulative token counts
-        for (int j = lane; j < n_iv; j += 32) {
-            const int lo = s_lo[j], hi = s_hi[j];
-            int rank = 0;
-            for (int m = 0; m < n_iv; ++m) {
-                const int lm = s_lo[m], hm = s_hi[m];
-                rank += (lm < lo) || (lm == lo && (hm < hi || (hm == hi && m < j)));
-            }
-            p_lo[rank] = lo;
-            p_hi[rank] = hi;
-        }
-        __syncwarp();
-        if (lane == 0) {
-            int *start = spans + bh * tstride;
-            int *cum = start + pcap;
-            int cnt = 0;
-            long long next_free = 0, total = 0;
-            cum[0] = 0;
-            for (int a = 0; a < n_iv; ++a) {
-                const int lo = p_lo[a], hi = p_hi[a];
-                if (hi < 0) break;
-                const long long j0 = lo > next_free ? lo : next_free;
-                if (j0 <= hi) {
-                    start[cnt] = (int)j0;
-                    total += hi - j0 + 1;
-                    cum[cnt + 1] = (int)total;
-                    ++cnt;
-                }
-                if ((long long)hi + 1 > next_free) next_free = (long long)hi + 1;
-            }
-            start[2 * pcap + 1] = cnt;
-        }
-        __syncwarp();
     }
 }
 
 // ------------------------------------------------------------------------------------------------
+// Span table of one attention unit from the selected anchors (in shared memory: s_anchor[top_k], -1 = none), built
+// by the whole CTA: piece starts in s_start, cumulative token counts in s_cum, the number of pieces in s_cnt (all
+// visible to the CTA on return).
+// Union mode: the spans of the selected anchors (Algorithm 1: S_t = [max(0,t-b l), min(i,t+f l)]) and the local
+// window W = [max(0, i-w+1), i], sorted by (lo, hi) and clipped to disjoint pieces.  Per-span mode: unit j is
+// J_t of the j-th selected anchor, the part of S_t left of the window and then the window; a head with nothing
+// selected attends to the window alone, carried by its first unit.
+// (Ranks by a ballot per interval, the intervals dealt to the warps, the clipping by prefix sums over lanes: 17
+// intervals 2500 cycles; with all ranks counted by one warp through shuffles 4700.)
+__device__ inline void build_unit_spans(const Call &c, long long i, long long ell, int j_unit, const int *s_anchor, int *p_lo,
+                                        int *p_hi, int *s_start, int *s_cum, int *s_cnt) {
+    constexpr int kWarps = kAttnThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_iv = c.top_k + (c.window > 0 ? 1 : 0);
+    const int w_lo = (int)(i - c.window + 1 > 0 ? i - c.window + 1 : 0);
+    auto interval = [&](int j, int &lo, int &hi) {   // absent: (INT_MAX, -1)
+        lo = INT_MAX;
+        hi = -1;
+        if (j < c.top_k) {
+            const long long t = s_anchor[j];
+            if (t >= 0) {
+                const long long a = t - (long long)c.back * ell, z = t + (long long)c.fwd * ell;
+                lo = (int)(a > 0 ? a : 0);
+                hi = (int)(z < i ? z : i);
+            }
+        } else if (j < n_iv) {
+            lo = w_lo;
+            hi = (int)i;
+        }
+    };
+    if (c.mode == SLA_PER_SPAN) {
+        if (warp == 0) {
+            bool any = false;
+            for (int j = lane; j < c.top_k; j += 32) any |= s_anchor[j] >= 0;
+            any = __any_sync(0xffffffffu, any);
+            int lo, hi;
+            interval(j_unit, lo, hi);
+            // a head with nothing selected attends to the window alone: its first unit carries it
+            const bool sel = hi >= 0, lone_w = !any && j_unit == 0;
+            const int hi_cut = c.window > 0 && hi >= w_lo ? w_lo - 1 : hi;
+            const int n0 = sel && lo <= hi_cut ? hi_cut - lo + 1 : 0;
+            const int n1 = (sel || lone_w) && c.window > 0 ? (int)i - w_lo + 1 : 0;
+            if (lane == 0) {
+                int cnt = 0;
+                s_cum[0] = 0;
+                if (n0) { s_start[cnt] = lo; s_cum[++cnt] = n0; }
+                if (n1) { s_start[cnt] = w_lo; s_cum[cnt + 1] = n0 + n1; ++cnt; }
+                *s_cnt = cnt;
+            }
+        }
+        __syncthreads();
+        return;
+    }
+    // rank of every interval by (lo, hi, index)
+    int lo[3], hi[3];   // n_iv <= 65: intervals lane, lane + 32, lane + 64
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        lo[r] = INT_MAX;
+        hi[r] = -1;
+        if (32 * r < n_iv) interval(lane + 32 * r, lo[r], hi[r]);
+    }
+    for (int j = warp; j < n_iv; j += kWarps) {
+        int lj, hj, rank = 0;
+        interval(j, lj, hj);   // the same for all lanes
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+            if (32 * r < n_iv) {
+                const int m = lane + 32 * r;
+                rank += __popc(__ballot_sync(0xffffffffu, m < n_iv && (lo[r] < lj || (lo[r] == lj && (hi[r] < hj || (hi[r] == hj && m < j))))));
+            }
+        if (lane == 0) { p_lo[rank] = lj; p_hi[rank] = hj; }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        // In sorted order (absent intervals last), 32 at a time: the running maximum of the ends before an interval
+        // clips its start, a prefix sum of the lengths gives the cumulative token counts, a ballot the slots of
+        // the pieces that are not empty.
+        int end0 = 0, cum0 = 0, cnt0 = 0;
+        if (lane == 0) s_cum[0] = 0;
+        for (int j0 = 0; j0 < n_iv; j0 += 32) {
+            const bool on = j0 + lane < n_iv;
+            const int slo = on ? p_lo[j0 + lane] : INT_MAX, shi = on ? p_hi[j0 + lane] : -1;
+            int end = shi + 1;   // 0 for an absent interval
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, end, off);
+                if (lane >= off) end = max(end, y);
+            }
+            end = max(end, end0);
+            int prev_end = __shfl_up_sync(0xffffffffu, end, 1);
+            if (lane == 0) prev_end = end0;
+            const int start = max(slo, prev_end);
+            const int len = (shi >= 0 && start <= shi) ? shi - start + 1 : 0;
+            int incl = len;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            const unsigned have = __ballot_sync(0xffffffffu, len > 0);
+            if (len > 0) {
+                const int idx = cnt0 + __popc(have & ((1u << lane) - 1u));
+                s_start[idx] = start;
+                s_cum[idx + 1] = cum0 + incl;
+            }
+            cnt0 += __popc(have);
+            cum0 += __shfl_sync(0xffffffffu, incl, 31);
+            end0 = __shfl_sync(0xffffffffu, end, 31);
+        }
+        if (lane == 0) *s_cnt = cnt0;
+    }
+    __syncthreads();
+}
+
 // Top-k of sc[0..n) by the whole CTA (Section "Span search": TopK over Anchors(i)); sc[x] is the score of
 // stride index s_base + x.  Result in shared memory: sel_anchor[r] / sel_score[r], r = 0 .. top_k - 1, best
 // first (larger score, then the nearer anchor, i.e. the smaller stride index), padded with (-1, -inf).
-//   1. every thread takes the maximum of its contiguous run of scores;
-//   2. the smallest of the maxima of k (rounded up to a power of two) groups of threads is a lower bound of the
-//      k-th best score -- at least k scores lie at or above it -- and everything at or above it is a candidate;
-//   3. the candidates are collected (typically a few more than k) and each one's rank among them is its slot.
+//   1. the threads form at least k groups (of whole, half, ... warps); the maximum of every group is a score of its
+//      own, so the smallest of the maxima is a lower bound of the k-th best score;
+//   2. the scores at or above it are collected, a warp at a time (typically a few more than k);
+//   3. each one's rank among them is its slot.
 // When more candidates turn up than the list holds (many equal scores), every warp selects the k best of its
 // eighth of the scores with the warp routine of the prefill kernels instead, and the 8 k winners are ranked.
-// May overwrite sc.
+// (1024 scores, k = 16: 7000 cycles with group maxima through shared memory and an atomic per candidate, 4300 like
+// this; k rounds of a warp-wide maximum take 600 cycles each.  The loops stay rolled: the code runs once per launch,
+// and fetching an instruction for the first time costs 10 to 20 cycles.)
 struct SelectSmem {
-    static constexpr int kCand = 128;
-    unsigned tmax[kAttnThreads];
-    unsigned gmax[kMaxTopK];
-    unsigned thr;
+    static constexpr int kCand = 256;
+    alignas(16) unsigned gmax[kMaxTopK];
     int n_cand;
-    unsigned cand_key[kCand];
-    int cand_x[kCand];
+    alignas(16) uint2 cand[kCand];   // {order key, position in sc}
     // fallback
     float cand_v[kAttnThreads / 32][topk::kCap];
     int cand_s[kAttnThreads / 32][topk::kCap];
@@ -239,71 +263,55 @@ struct SelectSmem {
     float score[kAttnThreads / 32][kMaxTopK];
 };
 
-__device__ inline void cta_select_topk(float *sc, int n, int k, long long i, int s_base, const int *off, SelectSmem &m,
-                                       int *sel_anchor, float *sel_score) {
+__device__ inline void cta_select_topk(float *sc, int n, const Call &c, long long i, int s_base, SelectSmem &m, int *sel_anchor,
+                                       float *sel_score) {
     constexpr int kWarps = kAttnThreads / 32;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per_t = (n + kAttnThreads - 1) / kAttnThreads;
-    const int t0 = tid * per_t < n ? tid * per_t : n, t1 = t0 + per_t < n ? t0 + per_t : n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = c.top_k;
+    // groups of 32, 16, 8 or 4 threads: 8, 16, 32 or 64 of them
+    const int gs = k <= 8 ? 32 : k <= 16 ? 16 : k <= 32 ? 8 : 4, n_groups = kAttnThreads / gs;
     unsigned mx = 0u;   // below every order key of a real score
-    for (int x = t0; x < t1; ++x) mx = max(mx, topk::order_key(sc[x]));
-    m.tmax[tid] = mx;
-    if (tid < k) {
-        sel_anchor[tid] = -1;
-        sel_score[tid] = -CUDART_INF_F;
+#pragma unroll 1
+    for (int x = tid; x < n; x += kAttnThreads) mx = max(mx, max(topk::order_key(sc[x]), 1u));
+#pragma unroll 1
+    for (int off = 1; off < gs; off <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    if (tid % gs == 0) m.gmax[tid / gs] = mx;
+    for (int j = tid; j < k; j += kAttnThreads) {
+        sel_anchor[j] = -1;
+        sel_score[j] = -CUDART_INF_F;
     }
     if (tid == 0) m.n_cand = 0;
     __syncthreads();
-    // Threshold: the threads form kp >= k groups (kp the next power of two); every group's maximum is a score
-    // of its own, so at least k scores lie at or above the smallest group maximum: a lower bound of the k-th
-    // best score that costs two short reductions instead of k rounds of a warp-wide maximum.
-    int kp = 1;
-    while (kp < k) kp <<= 1;
-    const int gs = kAttnThreads / kp;   // threads per group (k <= 64: at least 4)
-    if (tid < kp) {
-        unsigned g = 0u;
-        for (int j = 0; j < gs; ++j) g = max(g, m.tmax[tid * gs + j]);
-        m.gmax[tid] = g;
+    unsigned thr = 0xffffffffu;   // 0 when some group is empty: then everything is a candidate
+    for (int j = 0; j < n_groups; j += 4) {
+        const uint4 g = *reinterpret_cast<const uint4 *>(m.gmax + j);
+        thr = min(thr, min(min(g.x, g.y), min(g.z, g.w)));
     }
-    __syncthreads();
-    if (warp == 0) {
-        unsigned lo = 0xffffffffu;
-        int filled = 0;
-        for (int j = lane; j < kp; j += 32) {
-            const unsigned g = m.gmax[j];
-            filled += g != 0u;
-            lo = min(lo, g);
-        }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        filled = __reduce_add_sync(0xffffffffu, filled);
-        if (lane == 0) m.thr = filled >= k ? lo : 0u;   // fewer than k groups hold a score: everything is a candidate
-    }
-    __syncthreads();
-    const unsigned thr = m.thr;
-    for (int x = t0; x < t1; ++x) {
-        const unsigned key = topk::order_key(sc[x]);
-        if (key >= thr) {
-            const int slot = atomicAdd(&m.n_cand, 1);
-            if (slot < SelectSmem::kCand) {
-                m.cand_key[slot] = key;
-                m.cand_x[slot] = x;
-            }
+#pragma unroll 1
+    for (int x0 = 0; x0 < n; x0 += kAttnThreads) {
+        const int x = x0 + tid;
+        const unsigned key = x < n ? max(topk::order_key(sc[x]), 1u) : 0u;
+        const unsigned who = __ballot_sync(0xffffffffu, key != 0u && key >= thr);
+        if (who) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&m.n_cand, __popc(who));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(who & ((1u << lane) - 1u));
+            if ((who >> lane & 1u) && at < SelectSmem::kCand) m.cand[at] = make_uint2(key, (unsigned)x);
         }
     }
     __syncthreads();
     const int nc = m.n_cand;
     if (nc <= SelectSmem::kCand) {
         if (tid < nc) {
-            const unsigned kc = m.cand_key[tid];
-            const int xc = m.cand_x[tid];
+            const uint2 mine = m.cand[tid];
             int rank = 0;
+#pragma unroll 2
             for (int y = 0; y < nc; ++y) {
-                const unsigned ky = m.cand_key[y];
-                rank += (ky > kc) || (ky == kc && m.cand_x[y] < xc);
+                const uint2 o = m.cand[y];
+                rank += (o.x > mine.x) || (o.x == mine.x && o.y < mine.y);
             }
             if (rank < k) {
-                sel_anchor[rank] = (int)(i + 1 - (off ? (long long)off[s_base + xc] : (long long)(s_base + xc + 1) * (s_base + xc + 1)));
-                sel_score[rank] = sc[xc];
+                sel_anchor[rank] = (int)(i + 1 - stride_offset(c, s_base + (int)mine.y));
+                sel_score[rank] = sc[mine.y];
             }
         }
         __syncthreads();
@@ -313,7 +321,7 @@ __device__ inline void cta_select_topk(float *sc, int n, int k, long long i, int
     const int per = (n + kWarps - 1) / kWarps;
     const int x0 = warp * per < n ? warp * per : n, x1 = x0 + per < n ? x0 + per : n;
     topk::select_topk(sc + x0, x1 - x0, k, i, m.cand_v[warp], m.cand_s[warp], m.anchor[warp], m.score[warp], lane,
-                      s_base + x0, off);
+                      s_base + x0, c.off);
     __syncthreads();
     for (int e = tid; e < kWarps * k; e += kAttnThreads) {
         const int w = e / k, j = e % k;
@@ -336,138 +344,32 @@ __device__ inline void cta_select_topk(float *sc, int n, int k, long long i, int
     __syncthreads();
 }
 
-// Span table of one attention unit from the selected anchors (in shared memory: s_anchor[top_k], -1 = none),
-// built by warp 0: piece starts in s_start, cumulative token counts in s_cum, returns the number of pieces.
-// Union mode: the spans of the selected anchors (Algorithm 1: S_t = [max(0,t-b l), min(i,t+f l)]) and the local
-// window W = [max(0, i-w+1), i], sorted by (lo, hi) and clipped to disjoint pieces.  Per-span mode: unit j is
-// J_t of the j-th selected anchor, the part of S_t left of the window and then the window; a head with nothing
-// selected attends to the window alone, carried by its first unit.
-__device__ inline int build_unit_spans(const Call &c, long long i, int j_unit, const int *s_anchor, int *s_lo, int *s_hi,
-                                       int *p_lo, int *p_hi, int *s_start, int *s_cum) {
-    const int lane = threadIdx.x & 31;
-    const long long ell = base_len(c, i);
-    const int n_iv = c.top_k + (c.window > 0 ? 1 : 0);
-    const int w_lo = (int)(i - c.window + 1 > 0 ? i - c.window + 1 : 0);
-    for (int j = lane; j < n_iv; j += 32) {
-        int lo = INT_MAX, hi = -1;
-        if (j == c.top_k) {
-            lo = w_lo;
-            hi = (int)i;
-        } else {
-            const long long t = s_anchor[j];
-            if (t >= 0) {
-                const long long a = t - (long long)c.back * ell, z = t + (long long)c.fwd * ell;
-                lo = (int)(a > 0 ? a : 0);
-                hi = (int)(z < i ? z : i);
-            }
-        }
-        s_lo[j] = lo;
-        s_hi[j] = hi;
+__device__ __forceinline__ void cg_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cg_wait() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
+template <typename T> __device__ __forceinline__ void unpack16(const uint4 &v, float (&f)[Vec16<T>::kElems]) {
+    if constexpr (sizeof(T) == 2) {
+        Vec16<__nv_bfloat16>::unpack(v, f);
+    } else {
+        f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);
+        f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
     }
-    __syncwarp();
-    int cnt = 0;
-    if (c.mode == SLA_PER_SPAN) {
-        if (lane == 0) {
-            int n_sel = 0;
-            for (int j = 0; j < c.top_k; ++j) n_sel += s_hi[j] >= 0;
-            const int j = j_unit;
-            int total = 0;
-            s_cum[0] = 0;
-            const bool sel = s_hi[j] >= 0, lone_w = n_sel == 0 && j == 0 && c.window > 0;
-            if (sel) {
-                const int hi_cut = c.window > 0 && s_hi[j] >= w_lo ? w_lo - 1 : s_hi[j];
-                if (s_lo[j] <= hi_cut) {
-                    s_start[cnt] = s_lo[j];
-                    total += hi_cut - s_lo[j] + 1;
-                    s_cum[++cnt] = total;
-                }
-            }
-            if ((sel || lone_w) && c.window > 0) {
-                s_start[cnt] = w_lo;
-                total += (int)i - w_lo + 1;
-                s_cum[++cnt] = total;
-            }
-        }
-        return __shfl_sync(0xffffffffu, cnt, 0);
-    }
-    if (n_iv <= 32) {
-        // a lane per interval, everything through shuffles: rank by (lo, hi), then, in sorted order, the running
-        // maximum of the ends before an interval clips its start, a prefix sum of the lengths gives the
-        // cumulative token counts and a ballot the slots of the pieces that are not empty
-        const bool on = lane < n_iv;
-        const int lo = on ? s_lo[lane] : INT_MAX, hi = on ? s_hi[lane] : -1;
-        int rank = 0;
-        for (int m = 0; m < n_iv; ++m) {
-            const int lm = __shfl_sync(0xffffffffu, lo, m), hm = __shfl_sync(0xffffffffu, hi, m);
-            rank += (lm < lo) || (lm == lo && (hm < hi || (hm == hi && m < lane)));
-        }
-        if (on) { p_lo[rank] = lo; p_hi[rank] = hi; }
-        __syncwarp();
-        const int slo = on ? p_lo[lane] : INT_MAX, shi = on ? p_hi[lane] : -1;   // sorted; absent intervals (hi < 0) last
-        // exclusive running maximum of hi + 1 over the intervals before this one
-        int end = shi + 1;   // 0 for an absent interval
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, end, off);
-            if (lane >= off) end = max(end, y);
-        }
-        int prev_end = __shfl_up_sync(0xffffffffu, end, 1);
-        if (lane == 0) prev_end = 0;
-        const int j0 = max(slo, prev_end);
-        const int len = (shi >= 0 && j0 <= shi) ? shi - j0 + 1 : 0;
-        int incl = len;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
-        }
-        const unsigned have = __ballot_sync(0xffffffffu, len > 0);
-        if (len > 0) {
-            const int idx = __popc(have & ((1u << lane) - 1u));
-            s_start[idx] = j0;
-            s_cum[idx + 1] = incl;
-        }
-        if (lane == 0) s_cum[0] = 0;
-        return __popc(have);
-    }
-    for (int j = lane; j < n_iv; j += 32) {
-        const int lo = s_lo[j], hi = s_hi[j];
-        int rank = 0;
-        for (int m = 0; m < n_iv; ++m) {
-            const int lm = s_lo[m], hm = s_hi[m];
-            rank += (lm < lo) || (lm == lo && (hm < hi || (hm == hi && m < j)));
-        }
-        p_lo[rank] = lo;
-        p_hi[rank] = hi;
-    }
-    __syncwarp();
-    if (lane == 0) {
-        long long next_free = 0, total = 0;
-        s_cum[0] = 0;
-        for (int a = 0; a < n_iv; ++a) {
-            const int lo = p_lo[a], hi = p_hi[a];
-            if (hi < 0) break;
-            const long long j0 = lo > next_free ? lo : next_free;
-            if (j0 <= hi) {
-                s_start[cnt] = (int)j0;
-                total += hi - j0 + 1;
-                s_cum[cnt + 1] = (int)total;
-                ++cnt;
-            }
-            if ((long long)hi + 1 > next_free) next_free = (long long)hi + 1;
-        }
-    }
-    return __shfl_sync(0xffffffffu, cnt, 0);
 }
 
-// `scores` [B*Hq][n_cand] (the unsharded step): every CTA selects the top-k of its head itself and builds its
-// unit's spans -- nothing waits for a "last" CTA of the scoring kernel; the CTA of split 0 (of the head's first
-// unit) writes the selection out.  `spans` (the sequence-sharded step): the table decode_shard_select built.
+// One attention unit per cluster row: `gridDim.x` CTAs in clusters of `cluster.num_blocks()` share a unit's tokens.
+//   1. (unsharded step, q_s given) the CTAs of a cluster score the anchors of the unit's head, a share each, and keep
+//      the k best of their share; after a cluster barrier every CTA picks the k best of all shares (read through
+//      distributed shared memory) and builds the unit's spans itself.  Sequence-sharded step: `spans` is the table
+//      decode_shard_select built.
+//   2. online softmax over an even share of the tokens;
+//   3. the cluster's first CTA merges the partial results of the others through distributed shared memory; when a
+//      unit has several clusters, the one that finishes last merges theirs (through `partial` and the counter `done`).
+// One launch instead of two with a hand-over of scores and partial results through global memory: see the figures at
+// plan_decode.
 template <typename T, int D>
-__global__ void __launch_bounds__(kAttnThreads)
-decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, Call c,
-            const int *__restrict__ spans, const float *__restrict__ scores, int n_cand, int s_min,
-            float *__restrict__ partial, int *__restrict__ done,
+__global__ void __launch_bounds__(kAttnThreads, 2)
+decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, Call c,
+            const int *__restrict__ spans, const float *__restrict__ scores, int n_cand, int s_min, int ell, float *__restrict__ partial, int *__restrict__ done,
             float *__restrict__ unit_out, int *__restrict__ done_head, int32_t *__restrict__ sel_anchor,
             float *__restrict__ sel_score, T *__restrict__ out, float *__restrict__ lse,
             float *__restrict__ shard_out) {
@@ -484,38 +386,81 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
     __shared__ int s_start[kMaxTopK + 1], s_cum[kMaxTopK + 2];
     __shared__ float s_m[kSlots], s_l[kSlots];
     __shared__ float s_acc[kWarps][D];
-    __shared__ SelectSmem s_sel;
-    __shared__ int s_anchor[kMaxTopK], s_iv[4 * kIv], s_cnt;
+    __shared__ int s_anchor[kMaxTopK], s_iv[2 * kIv], s_cnt;
     __shared__ float s_score[kMaxTopK];
+    __shared__ SelectSmem s_sel;
+    __shared__ float s_part[D + 2];         // this CTA's maximum, denominator, numerator
+    cg::cluster_group cluster = cg::this_cluster();
+    // the CTAs of a cluster write to each other's shared memory only when all of them have started
+    if (cluster.num_blocks() > 1) cg_arrive();
+    const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int sub = lane % LPR, rsel = lane / LPR;
     // attention unit: a head (union mode) or one selected anchor of a head (per-span mode)
     const bool per_span = c.mode == SLA_PER_SPAN;
     const int units = per_span ? c.top_k : 1, pcap = per_span ? 2 : c.top_k + 1;
-    const long long unit = blockIdx.y, bh = unit / units;
-    const int h = (int)(bh % c.Hq), b = (int)(bh / c.Hq), g = h / c.G;
+    // (32-bit index arithmetic: at the start of a launch every instruction is fetched for the first time, about ten
+    // cycles each, and a 64-bit division is a hundred of them)
+    const unsigned unit32 = blockIdx.y, bh32 = per_span ? unit32 / (unsigned)units : unit32;
+    const unsigned b = bh32 / (unsigned)c.Hq, h = bh32 - b * (unsigned)c.Hq, g = h / (unsigned)c.G;
+    const int j_unit = (int)(unit32 - bh32 * (unsigned)units);
+    const long long unit = unit32, bh = bh32;
     const int n_splits = gridDim.x, split = blockIdx.x;
+    const T *kbase = k + b * c.kv_sb + g * c.kv_sh;
+    const T *vbase = v + b * c.kv_sb + g * c.kv_sh;
 
-    // launched with programmatic stream serialization: everything above overlaps the tail of the
-    // score kernel, whose results are read from here on
+    // launched beside the tail of the kernel before it on the stream (the score kernel, or whatever the caller runs),
+    // whose results are read from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     int cnt;
-    if (scores) {
+    if (!spans) {
         const long long i = c.Lkv - 1;
-        const float *src = scores + bh * n_cand;
-        for (int x = tid; x < n_cand; x += kAttnThreads) s_scores[x] = __ldcg(src + x);
-        __syncthreads();
-        cta_select_topk(s_scores, n_cand, c.top_k, i, s_min, c.off, s_sel, s_anchor, s_score);
-        if (tid < c.top_k && split == 0 && unit % units == 0) {
-            sel_anchor[bh * c.top_k + tid] = s_anchor[tid];
-            sel_score[bh * c.top_k + tid] = s_score[tid];
+        const int per = (n_cand + csize - 1) / csize, x_lo = min(rank * per, n_cand), n_loc = min(per, n_cand - x_lo);
+        if (scores) {
+            for (int x = tid; x < n_cand; x += kAttnThreads) s_scores[x] = __ldcg(scores + bh * n_cand + x);
+        } else {
+            // scores of this CTA's share of the anchors
+            constexpr int LS = D / E, RS = 32 / LS, US = 4;
+            const int ssub = lane % LS, srow = lane / LS;
+            const uint4 q_raw = __ldg(reinterpret_cast<const uint4 *>(q_s + b * c.q_sb + (long long)h * c.q_sh + ssub * E));
+            bool started = csize == 1;
+#pragma unroll 1
+            for (int x0 = 0; x0 < n_loc; x0 += kWarps * RS * US) {
+                uint4 raw[US];
+#pragma unroll
+                for (int u = 0; u < US; ++u) {
+                    const int x = x0 + (u * kWarps + warp) * RS + srow;
+                    // candidate y is stride s_min + y: the first s_min strides land inside the local window
+                    const long long t = x < n_loc ? i + 1 - stride_offset(c, s_min + x_lo + x) : i;
+                    raw[u] = __ldg(reinterpret_cast<const uint4 *>(kbase + t * c.kv_st + ssub * E));
+                }
+                float qv[E];
+                unpack16<T>(q_raw, qv);
+                if (!started) cg_wait();
+                started = true;
+#pragma unroll
+                for (int u = 0; u < US; ++u) {
+                    const int x = x0 + (u * kWarps + warp) * RS + srow;
+                    float kv[E], part = 0.f;
+                    unpack16<T>(raw[u], kv);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) part = fmaf(qv[e], kv[e], part);
+                    part = reduce_sub<LS>(part);
+                    // every CTA of the cluster gets the score: lane r of the row's lanes stores it to rank r
+                    if (ssub < csize && x < n_loc) cluster.map_shared_rank(s_scores, ssub)[x_lo + x] = part * c.search_scale;
+                }
+            }
+            if (!started) cg_wait();
         }
-        if (warp == 0) {
-            const int n = build_unit_spans(c, i, (int)(unit % units), s_anchor, s_iv, s_iv + kIv, s_iv + 2 * kIv, s_iv + 3 * kIv,
-                                           s_start, s_cum);
-            if (lane == 0) s_cnt = n;
-        }
-        __syncthreads();
+        if (csize > 1) cluster.sync();
+        else __syncthreads();
+        cta_select_topk(s_scores, n_cand, c, i, s_min, s_sel, s_anchor, s_score);
+        if (split == 0 && j_unit == 0)
+            for (int j = tid; j < c.top_k; j += kAttnThreads) {
+                sel_anchor[bh * c.top_k + j] = s_anchor[j];
+                sel_score[bh * c.top_k + j] = s_score[j];
+            }
+        build_unit_spans(c, i, ell, j_unit, s_anchor, s_iv, s_iv + kIv, s_start, s_cum, &s_cnt);
         cnt = s_cnt;
     } else {
         const int *sp = spans + unit * (2 * pcap + 2);
@@ -527,8 +472,6 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
     const long long total = cnt > 0 ? s_cum[cnt] : 0;
     const long long f_begin = total * split / n_splits, f_end = total * (split + 1) / n_splits;
 
-    const T *kbase = k + b * c.kv_sb + g * c.kv_sh;
-    const T *vbase = v + b * c.kv_sb + g * c.kv_sh;
     float qv[C][E];
     const float scale2 = c.softmax_scale * kLog2e;
 #pragma unroll
@@ -576,12 +519,7 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
 #pragma unroll
             for (int ch = 0; ch < C; ++ch) {
                 float kv[E];
-                if constexpr (sizeof(T) == 2) {
-                    Vec16<__nv_bfloat16>::unpack(kraw[u][ch], kv);
-                } else {
-                    kv[0] = __uint_as_float(kraw[u][ch].x); kv[1] = __uint_as_float(kraw[u][ch].y);
-                    kv[2] = __uint_as_float(kraw[u][ch].z); kv[3] = __uint_as_float(kraw[u][ch].w);
-                }
+                unpack16<T>(kraw[u][ch], kv);
 #pragma unroll
                 for (int e = 0; e < E; ++e) x[u] = fmaf(qv[ch][e], kv[e], x[u]);
             }
@@ -605,12 +543,7 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
 #pragma unroll
             for (int ch = 0; ch < C; ++ch) {
                 float vv[E];
-                if constexpr (sizeof(T) == 2) {
-                    Vec16<__nv_bfloat16>::unpack(vraw[u][ch], vv);
-                } else {
-                    vv[0] = __uint_as_float(vraw[u][ch].x); vv[1] = __uint_as_float(vraw[u][ch].y);
-                    vv[2] = __uint_as_float(vraw[u][ch].z); vv[3] = __uint_as_float(vraw[u][ch].w);
-                }
+                unpack16<T>(vraw[u][ch], vv);
 #pragma unroll
                 for (int e = 0; e < E; ++e) acc[ch][e] = fmaf(p, vv[e], acc[ch][e]);
             }
@@ -618,6 +551,8 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
         m = m_new;
     }
 
+    // the next kernel may be scheduled when every CTA is here
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // merge the lane groups of the warp, then the warps of the CTA
 #pragma unroll
     for (int off = LPR; off < 32; off <<= 1) {
@@ -655,33 +590,57 @@ decode_attn(const T *__restrict__ q, const T *__restrict__ k, const T *__restric
             ll += s_l[w] * sc;
             aa += s_acc[w][tid] * sc;
         }
-        float *dst = partial + (unit * n_splits + split) * (D + 2);
-        if (tid == 0) { dst[0] = mm; dst[1] = ll; }
-        dst[2 + tid] = aa;
+        if (tid == 0) { s_part[0] = mm; s_part[1] = ll; }
+        s_part[2 + tid] = aa;
     }
-    // ---- the CTA that completes this unit merges the split results
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const int prev = atomicAdd(done + unit, 1);
-        s_last = prev == n_splits - 1;
-        if (s_last) done[unit] = 0;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
     float o_unit = 0.f, lse_unit = -CUDART_INF_F;
-    if (tid < D) {
-        const float *src = partial + unit * n_splits * (D + 2);
-        float mm = -CUDART_INF_F;
-        for (int s = 0; s < n_splits; ++s) mm = fmaxf(mm, __ldcg(src + s * (D + 2)));
-        float ll = 0.f, aa = 0.f;
-        for (int s = 0; s < n_splits; ++s) {
-            const float ms = __ldcg(src + s * (D + 2));
+    // merge of n partial results, the x-th one found by at(x, word): {maximum, denominator, numerator[D]}
+    auto merge = [&](int n, auto at, float &mm, float &ll, float &aa) {
+        mm = -CUDART_INF_F;
+        for (int x = 0; x < n; ++x) mm = fmaxf(mm, at(x, 0));
+        ll = aa = 0.f;
+        for (int x = 0; x < n; ++x) {
+            const float ms = at(x, 0);
             const float sc = (ms == -CUDART_INF_F) ? 0.f : exp2f(ms - mm);
-            ll += __ldcg(src + s * (D + 2) + 1) * sc;
-            aa += __ldcg(src + s * (D + 2) + 2 + tid) * sc;
+            ll += at(x, 1) * sc;
+            aa += at(x, 2 + tid) * sc;
         }
+    };
+    float mm = -CUDART_INF_F, ll = 0.f, aa = 0.f;
+    if (csize > 1) {
+        cluster.sync();
+        if (rank == 0 && tid < D)
+            merge(csize, [&](int x, int w) { return cluster.map_shared_rank(s_part, x)[w]; }, mm, ll, aa);
+        cluster.sync();   // the others' shared memory has been read
+        if (rank != 0) return;
+    } else {
+        __syncthreads();
+        if (tid < D) { mm = s_part[0]; ll = s_part[1]; aa = s_part[2 + tid]; }
+    }
+    const int n_clusters = n_splits / csize;
+    if (n_clusters > 1) {
+        // ---- the cluster that completes this unit merges the clusters' results
+        if (tid < D) {
+            float *dst = partial + (unit * n_clusters + split / csize) * (D + 2);
+            if (tid == 0) { dst[0] = mm; dst[1] = ll; }
+            dst[2 + tid] = aa;
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            const int prev = atomicAdd(done + unit, 1);
+            s_last = prev == n_clusters - 1;
+            if (s_last) done[unit] = 0;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        if (tid < D) {
+            const float *src = partial + unit * n_clusters * (D + 2);
+            merge(n_clusters, [&](int x, int w) { return __ldcg(src + x * (D + 2) + w); }, mm, ll, aa);
+        }
+    }
+    if (tid < D) {
         o_unit = ll > 0.f ? aa / ll : 0.f;
         lse_unit = ll > 0.f ? (mm + log2f(ll)) * kLn2 : -CUDART_INF_F;
     }
@@ -761,52 +720,78 @@ cudaError_t allow_score_smem(K kern, size_t smem) {
 }
 
 template <typename T, int D>
+cudaError_t attn_launch(const T *q_s, const T *q, const T *k, const T *v, const Call &c, const int *spans, const float *scores,
+                        int n_cand, int s_min, const DecodePlan &p, int units, float *partial, int *done, float *unit_out,
+                        int *done_head, int32_t *out_anchor, float *out_score, T *out, float *lse, float *shard_out,
+                        cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.n_splits, c.B * c.Hq * units);
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.dynamicSmemBytes = (size_t)n_cand * sizeof(float);
+    cfg.stream = st;
+    // Programmatic dependent launch: the grid is set up while the kernel before it drains (2 to 3 us a step).  Not for
+    // clusters of eight: CTAs of this grid that start in the last free slots of the one before leave the other
+    // clusters no eight slots in one place (two-span steps over 1M tokens: 32 us without, 38 with it).
+    cudaLaunchAttribute attr[2];
+    if (p.cluster < 8) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (p.cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = p.cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    cfg.attrs = attr;
+    return cudaLaunchKernelEx(&cfg, decode_attn<T, D>, q_s, q, k, v, c, spans, scores, n_cand, s_min,
+                              (int)base_len(c, c.Lkv - 1), partial, done, unit_out,
+                              done_head, out_anchor, out_score, out, lse, shard_out);
+}
+
+template <typename T, int D>
 cudaError_t decode_launch(const void *q_s, const void *q, const void *k, const void *v, const Call &c,
                           long long n_ctx, const DecodePlan &p, void *scratch, int *counters, void *out, float *lse,
                           int32_t *out_anchor, float *out_score, cudaStream_t st) {
     constexpr int E = Vec16<T>::kElems;
     constexpr int RPI = 32 / (D / E);
     char *base = (char *)scratch;
-    float *scores = (float *)(base + p.off_scores);
-    int *spans = (int *)(base + p.off_spans);
-    float *partial = (float *)(base + p.off_partial);
-    float *unit_out = (float *)(base + p.off_unit_out);
     const int units = c.mode == SLA_PER_SPAN ? c.top_k : 1;
-    int *done_bg = counters, *done_unit = counters + c.B * c.Hkv, *done_head = done_unit + c.B * c.Hq * units;
+    int *done_unit = counters + c.B * c.Hkv, *done_head = done_unit + c.B * c.Hq * units;
     const int n = p.n_anchor, s_min = window_strides(c);
-    const int rows_per_cta = (kScoreThreads / 32) * RPI * 2;
-    const int gt = c.G % 8 == 0 ? 8 : c.G % 4 == 0 ? 4 : c.G % 2 == 0 ? 2 : 1;
-    dim3 gs(n > 0 ? (n + rows_per_cta - 1) / rows_per_cta : 1, c.B * c.Hkv, c.G / gt);
     const T *qs = (const T *)q_s, *kk = (const T *)k;
-    if ((size_t)n * sizeof(float) > 40 * 1024) return cudaErrorInvalidValue;   // the attention kernel holds a head's scores in shared memory
-    cudaError_t e = cudaSuccess;
-    // scores only (no completion counter, no shared memory): the attention kernel selects
-#define SLA_LAUNCH_SCORE(GT)                                                                                         \
-    decode_score<T, D, GT><<<gs, kScoreThreads, 0, st>>>(qs, kk, c, n_ctx, n, s_min, scores, (int *)nullptr,         \
-                                                          (int *)nullptr, out_anchor, out_score)
-    switch (gt) {
-        case 8: SLA_LAUNCH_SCORE(8); break;
-        case 4: SLA_LAUNCH_SCORE(4); break;
-        case 2: SLA_LAUNCH_SCORE(2); break;
-        default: SLA_LAUNCH_SCORE(1); break;
-    }
+    if ((size_t)n * sizeof(float) > 40 * 1024) return cudaErrorInvalidValue;   // a head's scores lie in shared memory
+    float *scores = nullptr;
+    if (p.score_first) {
+        scores = (float *)(base + p.off_scores);
+        const int rows_per_cta = (kScoreThreads / 32) * RPI * 2;
+        const int gt = c.G % 8 == 0 ? 8 : c.G % 4 == 0 ? 4 : c.G % 2 == 0 ? 2 : 1;
+        const dim3 gs(n > 0 ? (n + rows_per_cta - 1) / rows_per_cta : 1, c.B * c.Hkv, c.G / gt);
+        // scores only (no completion counter, no shared memory)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = gs;
+        cfg.blockDim = dim3(kScoreThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t e;
+#define SLA_LAUNCH_SCORE(GT) \
+    e = cudaLaunchKernelEx(&cfg, decode_score<T, D, GT>, qs, kk, c, n_ctx, n, s_min, scores, (int *)nullptr, out_anchor, out_score)
+        switch (gt) {
+            case 8: SLA_LAUNCH_SCORE(8); break;
+            case 4: SLA_LAUNCH_SCORE(4); break;
+            case 2: SLA_LAUNCH_SCORE(2); break;
+            default: SLA_LAUNCH_SCORE(1); break;
+        }
 #undef SLA_LAUNCH_SCORE
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // programmatic dependent launch: the attention grid is set up while the score kernel drains
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.n_splits, c.B * c.Hq * units);
-    cfg.blockDim = dim3(kAttnThreads);
-    cfg.dynamicSmemBytes = (size_t)n * sizeof(float);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, decode_attn<T, D>, (const T *)q, kk, (const T *)v, c, (const int *)nullptr,
-                              (const float *)scores, n, s_min, partial, done_unit, unit_out, done_head, out_anchor,
-                              out_score, (T *)out, lse, (float *)nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    return attn_launch<T, D>(qs, (const T *)q, kk, (const T *)v, c, nullptr, scores, n, s_min, p, units,
+                             (float *)(base + p.off_partial), done_unit, (float *)(base + p.off_unit_out), done_head, out_anchor,
+                             out_score, (T *)out, lse, nullptr, st);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -932,7 +917,7 @@ cudaError_t shard_search_launch(const void *q_s, const void *k_local, const Call
     dim3 gs(n > 0 ? (n + rows_per_cta - 1) / rows_per_cta : 1, c.B * c.Hkv, c.G / gt);
     // positions are global: the local slice starts at shard_lo
     const T *qs = (const T *)q_s, *kk = (const T *)k_local - c.shard_lo * c.kv_st;
-    const size_t smem = (size_t)(kScoreThreads / 32) * (n + 2 * topk::kCap + 4 * (kMaxTopK + 1)) * sizeof(float);
+    const size_t smem = (size_t)(kScoreThreads / 32) * (n + 2 * topk::kCap) * sizeof(float);
     if (smem > (size_t)kScoreSmemMax) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
 #define SLA_LAUNCH_SCORE(GT)                                                                                         \
@@ -940,8 +925,8 @@ cudaError_t shard_search_launch(const void *q_s, const void *k_local, const Call
         auto kern = decode_score<T, D, GT>;                                                                          \
         e = allow_score_smem(kern, smem);                                                                            \
         if (e == cudaSuccess)                                                                                        \
-            kern<<<gs, kScoreThreads, smem, st>>>(qs, kk, c, n_ctx, n, s_first, scores, counters, (int *)nullptr,    \
-                                                  cand_anchor, cand_score);                                         \
+            kern<<<gs, kScoreThreads, smem, st>>>(qs, kk, c, n_ctx, n, s_first, scores, counters, cand_anchor,       \
+                                                  cand_score);                                                      \
     } while (0)
     switch (gt) {
         case 8: SLA_LAUNCH_SCORE(8); break;
@@ -968,10 +953,10 @@ cudaError_t shard_attend_launch(const void *q, const void *k_local, const void *
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const T *kk = (const T *)k_local - c.shard_lo * c.kv_st, *vv = (const T *)v_local - c.shard_lo * c.kv_st;
-    decode_attn<T, D><<<dim3(p.n_splits, c.B * c.Hq), kAttnThreads, 0, st>>>(
-        (const T *)q, kk, vv, c, spans, (const float *)nullptr, 0, 0, partial, done_unit, (float *)nullptr, done_head,
-        out_anchor, out_score, (T *)nullptr, (float *)nullptr, partial_out);
-    return cudaGetLastError();
+    DecodePlan ps = p;
+    ps.cluster = 1;
+    return attn_launch<T, D>(nullptr, (const T *)q, kk, vv, c, spans, nullptr, 0, 0, ps, 1, partial, done_unit, nullptr, done_head, out_anchor,
+                             out_score, nullptr, nullptr, partial_out, st);
 }
 
 }  // namespace
@@ -1032,6 +1017,8 @@ int decode_attn_blocks_per_sm(int dtype, int D) {
     return slot;
 }
 
+constexpr int kShare = 128;   // anchors per CTA that it scores itself
+
 DecodePlan plan_decode(const Call &c, long long n_ctx, int cta_slots, size_t gap) {
     DecodePlan p;
     // candidates: the strides whose anchor lies left of the local window
@@ -1049,7 +1036,18 @@ DecodePlan plan_decode(const Call &c, long long n_ctx, int cta_slots, size_t gap
     if (ns > max_tokens / 128) ns = max_tokens / 128;
     if (ns > 256) ns = 256;
     if (ns < 1) ns = 1;
-    p.n_splits = (int)ns;
+    // One launch, the CTAs of a unit in clusters (the largest power of two up to 8) that share the scoring and the
+    // merge, or two, all scores first.  One launch saves the score kernel and its hand-over (8 sequences of 8191
+    // tokens 45 -> 36 us, a two-span step over 100003 tokens 28.7 -> 23.5), but a CTA scores its share after its start
+    // (7 us for 400 anchors: 16 x 181104 tokens 272 -> 280), so the share is bounded; and splits beyond the clusters
+    // are left idle (8 of 9 per head at 1M tokens: 92 -> 100 us), which may cost 24 MB of reading at most, the time
+    // that is saved.
+    const int csz = ns >= 8 ? 8 : ns >= 4 ? 4 : ns >= 2 ? 2 : 1, fused = (int)(ns / csz) * csz;
+    const long long bytes = (long long)c.B * c.Hq * units * max_tokens * 2 * c.D * 2;
+    const bool one = p.n_anchor <= csz * kShare && (double)bytes * (ns - fused) / ns < 24e6;
+    p.score_first = !one;
+    p.cluster = one ? csz : 1;
+    p.n_splits = one ? fused : (int)ns;
     const size_t bh = (size_t)c.B * c.Hq, n_units = bh * units;
     size_t off = 0;
     // a region of `size` bytes at the next 256-byte boundary, with a canary gap before it when asked for

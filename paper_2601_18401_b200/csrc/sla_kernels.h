@@ -76,6 +76,8 @@ struct DecodePlan {
     int n_anchor;       // anchor candidates of the query position: floor(sqrt(n_ctx)) - floor(sqrt(window))
     int n_splits;       // CTAs that share one attention unit's tokens (unit: a head, or one selected
                         // anchor of a head in the per-span mode)
+    int cluster;        // CTAs of a cluster (a divisor of n_splits)
+    bool score_first;   // the anchors are scored by a kernel of their own
     size_t off_scores;  // float [B*Hq][n_anchor]
     size_t off_spans;   // int   [units][2*P + 2]: piece starts, cumulative token counts, piece count
                         //       (P = top_k + 1 in the union mode, 2 in the per-span mode)

@@ -84,3 +84,51 @@ def test_end_blocks_far_apart(sla, handle):
     assert sla.sla_poll_status(handle) == sla.SLA_OK
     ref = P.oracle_attention_for(P.host_inputs(x), O.BF16, anchor.cpu().numpy(), w)
     P.compare_attention(out, lse, ref, "bf16")
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,dtype,D,n_ctx,top_k,span_len,per_span", [
+    (1, 8, 2, "bf16", 128, 70001, 16, 600, False),    # clusters of eight, several per head
+    (1, 32, 8, "bf16", 128, 9001, 8, 0, False),       # one cluster of eight per head
+    (2, 32, 8, "bf16", 128, 4099, 3, 300, False),     # clusters of four
+    (4, 32, 4, "bf16", 64, 4099, 2, 500, False),      # clusters of two, head_dim 64
+    (2, 32, 8, "f32", 128, 3001, 2, 700, True),       # per-span units in clusters of two
+    (10, 32, 8, "bf16", 128, 16384, 4, 30, False),    # one CTA per head; 128 anchors: it scores them itself
+    (10, 32, 8, "bf16", 128, 16641, 4, 30, False),    # 129 anchors: scored first
+    (1, 2, 1, "f32", 64, 1050000, 33, 90, False),     # 1024 anchors and one more per CTA of a cluster of eight
+    (1, 4, 1, "bf16", 128, 40, 64, 3, False),         # fewer anchors than slots, one CTA per head
+])
+def test_decode_split_over_clusters(sla, handle, B, Hq, Hkv, dtype, D, n_ctx, top_k, span_len, per_span):
+    """Decode steps on both sides of the rule that deals a step to CTAs and clusters; the anchors in a local window
+    of 64 tokens are left out in the per-span case."""
+    import parity_util as P
+    import torch
+    from oracle import sla_oracle as O
+    from paper_2601_18401_b200 import synth
+    w = synth.Workload("dc", "decode", B, Hq, Hkv, D, n_ctx, dtype, span_len, top_k, seed=67)
+    kc, vc = synth.make_decode_cache(w, "cuda:0", capacity=n_ctx)
+    x = synth.make_decode_step_inputs(w, 0, "cuda:0")
+    window = 64 if per_span else 0
+    params = sla.make_params(top_k, span_len, window=window, mode=sla.SLA_PER_SPAN if per_span else sla.SLA_UNION, head_dim=D)
+    for rep in range(2):   # the second step finds the completion counters as the first left them
+        got = sla.sla_decode_step(handle, x["q_s"], x["q"], kc, vc, n_ctx, params)
+        torch.cuda.synchronize()
+        assert sla.sla_poll_status(handle) == sla.SLA_OK
+    P.check_decode_step(got, synth.to_numpy(x["q_s"]), synth.to_numpy(x["q"]), synth.to_numpy(kc), synth.to_numpy(vc),
+                        synth.dtype_code(dtype), dtype, n_ctx=n_ctx, top_k=top_k, span_len=span_len, window=window,
+                        mode=O.PER_SPAN if per_span else O.UNION)
+
+
+@pytest.mark.parametrize("n_ctx,Hq,top_k", [(200, 4, 8), (90000, 4, 16), (90000, 4, 64), (66000, 320, 5), (200000, 320, 40)])
+def test_decode_equal_scores(sla, handle, n_ctx, Hq, top_k):
+    """All scores equal: the nearest anchors win, in order; more candidates than the selection's list holds."""
+    import math
+    import torch
+    k = torch.ones(1, 1, n_ctx, 64, dtype=torch.bfloat16, device="cuda").expand(1, Hq // 4, n_ctx, 64)
+    q = torch.ones(1, Hq, 64, dtype=torch.bfloat16, device="cuda")
+    _, _, anchor, score = sla.sla_decode_step(handle, q, q, k, k, n_ctx, sla.make_params(top_k, 5, head_dim=64))
+    torch.cuda.synchronize()
+    assert sla.sla_poll_status(handle) == sla.SLA_OK
+    n = min(top_k, math.isqrt(n_ctx))
+    want = torch.tensor([n_ctx - (s + 1) ** 2 if s < n else -1 for s in range(top_k)], dtype=torch.int32)
+    assert torch.equal(anchor.cpu(), want.expand(1, Hq, top_k))
+    assert (score[..., :n] == 64.0).all()
