@@ -40,7 +40,7 @@ bool search_mma_supported(const Call &c, int dtype);
 cudaError_t launch_search_mma(const void *q_s, const void *k, const Call &c, int32_t *out_anchor, float *out_score,
                               cudaStream_t st, long long *launches);
 
-// ---- span-search with the selection folded into the scoring loop, bf16 / head_dim 128 / groups of four
+// ---- span-search with the selection folded into the scoring loop, bf16 / head_dim 128 / groups of 4, 8 or 16
 // query heads (sla_search_diag.cu)
 bool search_diag_supported(const Call &c, int dtype);
 cudaError_t launch_search_diag(const void *q_s, const void *k, const Call &c, int32_t *out_anchor, float *out_score,

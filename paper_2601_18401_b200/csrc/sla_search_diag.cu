@@ -1,4 +1,4 @@
-// Span-search for bf16, head_dim 128 and groups of four query heads per KV head (Section "Span
+// Span-search for bf16, head_dim 128 and groups of 4, 8 or 16 query heads per KV head (Section "Span
 // search": s_{i,t} = <Q_s(i), K(t)> over the anchors t_s = i + 1 - offset(s), then TopK), with the
 // selection folded into the scoring loop.
 //
@@ -86,11 +86,80 @@ __device__ __forceinline__ void sort_pairs(float (&x)[K], int (&s)[K]) {
             }
 }
 
+// A lane's running top-k: the K best values so far, sorted, in registers, and in shared memory (entry e at lx[32 e],
+// ls[32 e]) every score with its stride index that beat the K-th best when it arrived.
+template <int K>
+struct RunningTop {
+    static constexpr int CAP = ListCap<K>::value;
+    float v[K];
+    int cnt;
+    float *lx;
+    int *ls;
+    __device__ __forceinline__ RunningTop(float *warp_lists, int lane)
+        : cnt(0), lx(warp_lists + lane), ls(reinterpret_cast<int *>(warp_lists + CAP * 32) + lane) {
+#pragma unroll
+        for (int j = 0; j < K; ++j) v[j] = -CUDART_INF_F;
+    }
+    // Drops the list entries that can no longer be among the K best (all lanes, each its own list):
+    // what is left are the entries above the K-th best value and the earliest of those equal to it,
+    // at most K in all, still in stride order.
+    __device__ __forceinline__ void compact() {
+        const float vk = v[K - 1];
+        int allow_eq = K;
+#pragma unroll
+        for (int j = 0; j < K; ++j) allow_eq -= v[j] > vk;
+        int w = 0;
+        for (int e = 0; e < cnt; ++e) {
+            const float x = lx[32 * e];
+            const int s = ls[32 * e];
+            const bool eq = x == vk;
+            if (x > vk || (eq && allow_eq > 0)) {
+                allow_eq -= eq;
+                lx[32 * w] = x;
+                ls[32 * w] = s;
+                ++w;
+            }
+        }
+        cnt = w;
+    }
+    // Two new scores, sa < sb.  Each one that beats the K-th best so far goes to the list; the sorted values take
+    // both in one pass: with hi >= lo the new j-th best is max(v[j], min(v[j-1], hi), min(v[j-2], lo)).
+    __device__ __forceinline__ void offer2(int sa, float xa, int sb, float xb) {
+        if (__any_sync(0xffffffffu, cnt >= CAP - 1)) compact();   // room for both scores
+        const float vk = v[K - 1];
+        if (xa > vk) {
+            lx[32 * cnt] = xa;
+            ls[32 * cnt] = sa;
+            ++cnt;
+        }
+        if (xb > vk) {
+            lx[32 * cnt] = xb;
+            ls[32 * cnt] = sb;
+            ++cnt;
+        }
+        const float hi = fmaxf(xa, xb), lo = fminf(xa, xb);
+#pragma unroll
+        for (int j = K - 1; j >= 2; --j) v[j] = max3(v[j], fminf(v[j - 1], hi), fminf(v[j - 2], lo));
+        if (K >= 2) v[1] = max3(v[1], fminf(v[0], hi), lo);
+        v[0] = fmaxf(v[0], hi);
+    }
+    // The K best with their stride indices, best first; absent entries are (-inf, INT_MAX).
+    __device__ __forceinline__ void finish(float (&x)[K], int (&s)[K]) {
+        compact();
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            const bool on = j < cnt;
+            x[j] = on ? lx[32 * j] : -CUDART_INF_F;
+            s[j] = on ? ls[32 * j] : INT_MAX;
+        }
+        sort_pairs<K>(x, s);
+    }
+};
+
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
             float *__restrict__ out_score) {
-    constexpr int CAP = ListCap<K>::value;
     extern __shared__ float smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r8 = lane >> 2, q = lane & 3;
@@ -98,8 +167,6 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     const long long r0 = ((long long)(gridDim.x - 1 - blockIdx.x) * kWarps + warp) * kQW;
     if (r0 >= c.Lq) return;
     const int bg = blockIdx.y, g = bg % c.Hkv, b = bg / c.Hkv;
-    float *lx = smem + (size_t)warp * (2 * CAP * 32) + lane;                  // list entry e: lx[32 e], ls[32 e]
-    int *ls = reinterpret_cast<int *>(smem + (size_t)warp * (2 * CAP * 32) + CAP * 32) + lane;
 
     const long long last = c.Lq - 1;
     // ---- A operand: rows r8 and r8 + 8 = (position r8>>2, head r8&3) and (position 2 + (r8>>2), head r8&3)
@@ -149,55 +216,7 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         kb[1] = ldg256(row + 64);
     };
 
-    float v[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) v[j] = -CUDART_INF_F;
-    int cnt = 0;
-
-    // Drops the list entries that can no longer be among the K best (all lanes, each its own list):
-    // what is left are the entries above the K-th best value and the earliest of those equal to it,
-    // at most K in all, still in stride order.
-    auto compact = [&]() {
-        const float vk = v[K - 1];
-        int allow_eq = K;
-#pragma unroll
-        for (int j = 0; j < K; ++j) allow_eq -= v[j] > vk;
-        int w = 0;
-        for (int e = 0; e < cnt; ++e) {
-            const float x = lx[32 * e];
-            const int s = ls[32 * e];
-            const bool eq = x == vk;
-            if (x > vk || (eq && allow_eq > 0)) {
-                allow_eq -= eq;
-                lx[32 * w] = x;
-                ls[32 * w] = s;
-                ++w;
-            }
-        }
-        cnt = w;
-    };
-
-    // Two new scores at a time.  Each one that beats the K-th best so far goes to the list; the sorted
-    // values take both in one pass: with hi >= lo the new j-th best is
-    // max(v[j], min(v[j-1], hi), min(v[j-2], lo)).
-    auto offer2 = [&](int sa, float xa, int sb, float xb) {
-        const float vk = v[K - 1];
-        if (xa > vk) {
-            lx[32 * cnt] = xa;
-            ls[32 * cnt] = sa;
-            ++cnt;
-        }
-        if (xb > vk) {
-            lx[32 * cnt] = xb;
-            ls[32 * cnt] = sb;
-            ++cnt;
-        }
-        const float hi = fmaxf(xa, xb), lo = fminf(xa, xb);
-#pragma unroll
-        for (int j = K - 1; j >= 2; --j) v[j] = max3(v[j], fminf(v[j - 1], hi), fminf(v[j - 2], lo));
-        if (K >= 2) v[1] = max3(v[1], fminf(v[0], hi), lo);
-        v[0] = fmaxf(v[0], hi);
-    };
+    RunningTop<K> top(smem + (size_t)warp * (2 * RunningTop<K>::CAP * 32), lane);
     // scores of one B tile (two strides): two independent accumulation chains, added at the end
     auto score = [&](const Words8 (&kb)[2]) -> float {
         float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -210,36 +229,37 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         const float lo = (r8 >> 2) ? a0[1] + a1[1] : a0[0] + a1[0], hi = (r8 >> 2) ? a0[3] + a1[3] : a0[2] + a1[2];
         return ((q & 1) ? hi : lo) * c.search_scale;
     };
-    // four strides (two B tiles): eight 16-byte loads in flight per lane, then two scores per lane
-    auto step = [&](int s0, bool check) {
-        Words8 ka[2], kb[2];
-        fetch(s0, check, ka);
-        fetch(s0 + 2, check, kb);
-        float xa = score(ka), xb = score(kb);
-        if (check) {
-            xa = s0 + u_own < n_own ? xa : -CUDART_INF_F;
-            xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
-        }
-        if (__any_sync(0xffffffffu, cnt >= CAP - 1)) compact();   // room for both scores
-        offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
-    };
+    // two B tiles of two strides, each fetched again as soon as its scores are taken (32768 x 2 positions, K = 2 and
+    // 16384 positions, K = 8: 1.2 to 1.5 % off search and attention together against fetch and use in one step)
+    Words8 ka[2], kb[2];
     int s0 = s_min;
-    for (; s0 + 4 <= n_all; s0 += 4) step(s0, false);
-    for (; s0 < n_max; s0 += 4) step(s0, true);
+    fetch(s0, true, ka);
+    fetch(s0 + 2, true, kb);
+    for (; s0 + 4 <= n_all; s0 += 4) {
+        const float xa = score(ka);
+        fetch(s0 + 4, true, ka);
+        const float xb = score(kb);
+        fetch(s0 + 6, true, kb);
+        top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
+    }
+    for (; s0 < n_max; s0 += 4) {
+        float xa = score(ka), xb = score(kb);
+        xa = s0 + u_own < n_own ? xa : -CUDART_INF_F;
+        xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
+        top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
+        if (s0 + 4 < n_max) {
+            fetch(s0 + 4, true, ka);
+            fetch(s0 + 6, true, kb);
+        }
+    }
 
     // ---- the lane's K best with their stride indices, sorted; then the merge with the lane that holds
     // the pair's other strides (q differs in bit 1): the rank of an entry in the union is its rank here
     // plus the number of the partner's entries that come before it
-    compact();
     float ex[K];
     int es[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const bool on = j < cnt;
-        ex[j] = on ? lx[32 * j] : -CUDART_INF_F;
-        es[j] = on ? ls[32 * j] : INT_MAX;
-    }
-    sort_pairs<K>(ex, es);
+    top.finish(ex, es);
+    const int cnt = top.cnt;
     int rank[K];
 #pragma unroll
     for (int j = 0; j < K; ++j) rank[j] = j;
@@ -266,21 +286,140 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         }
 }
 
+// The same for groups of eight (or sixteen) query heads per KV head: a warp owns one position, the routing queries of
+// eight heads are rows 0..7 of the A operand (rows 8..15 are zero), the columns of B are the keys of eight strides.
+// Lane (r8, q) receives the scores of head r8 at strides s0 + 2q and s0 + 2q + 1, so that four lanes share a head; their
+// sorted lists are merged two at a time.  Every key row is fetched once for eight heads.
+// Bound by the latency of the key rows (a chunk half way through a long context reads them from DRAM) and by issue:
+// 320 instructions per warp and sixteen strides, four lists of K values per head.  4096 positions at 500001, 32/4 heads,
+// K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
+// 484 us here, about 440 us with the tiles fetched a step ahead.
+template <int K>
+__global__ void __launch_bounds__(kWarps * 32, 2)
+search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
+             float *__restrict__ out_score) {
+    extern __shared__ float smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r8 = lane >> 2, q = lane & 3;
+    // the tiles with the most strides (the last positions) start first
+    const long long r = (long long)(gridDim.x - 1 - blockIdx.x) * kWarps + warp;
+    if (r >= c.Lq) return;
+    const int bg = blockIdx.y, g = bg % c.Hkv, b = bg / c.Hkv, h = g * c.G + blockIdx.z * 8 + r8;
+    Words8 qa[2];
+    {
+        const bf16 *base = q_s + b * c.q_sb + (long long)h * c.q_sh + r * c.q_st + 16 * q;
+        qa[0] = ldg256(base);
+        qa[1] = ldg256(base + 64);
+    }
+    const int i = (int)(c.q_pos0 + r);   // positions fit 31 bits
+    const int n = n_strides(c, i);
+    // Algorithm 1: anchors inside the local window are no candidates; t_s lies in W iff offset(s) <= w
+    const int s_min = c.window > 0 ? window_strides(c) : 0;
+    const bf16 *kbase = k + b * c.kv_sb + g * c.kv_sh + 16 * q;
+    const int kv_st = (int)c.kv_st;
+    auto fetch = [&](int s0, bool check, Words8 (&kb)[2]) {   // column r8: the key of stride s0 + r8
+        const int s = s0 + r8;
+        int t = i + 1 - stride_offset(c, s < c.n_off || !c.off ? s : 0);
+        if (check && s >= n) t = i;   // a valid row either way
+        const bf16 *row = kbase + (long long)t * kv_st;
+        kb[0] = ldg256(row);
+        kb[1] = ldg256(row + 64);
+    };
+    RunningTop<K> top(smem + (size_t)warp * (2 * RunningTop<K>::CAP * 32), lane);
+    // two independent accumulation chains, added at the end
+    auto score = [&](const Words8 (&kb)[2], float &x0, float &x1) {
+        float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            mma_bf16_16816(a0, qa[0].w[2 * x], 0u, qa[0].w[2 * x + 1], 0u, kb[0].w[2 * x], kb[0].w[2 * x + 1]);
+            mma_bf16_16816(a1, qa[1].w[2 * x], 0u, qa[1].w[2 * x + 1], 0u, kb[1].w[2 * x], kb[1].w[2 * x + 1]);
+        }
+        x0 = (a0[0] + a1[0]) * c.search_scale;
+        x1 = (a0[1] + a1[1]) * c.search_scale;
+    };
+    // two B tiles of eight strides, each fetched again as soon as its scores are taken
+    Words8 ka[2], kb[2];
+    int s0 = s_min;
+    fetch(s0, true, ka);
+    fetch(s0 + 8, true, kb);
+    for (; s0 + 16 <= n; s0 += 16) {
+        const int s = s0 + 2 * q;
+        float xa, xb;
+        score(ka, xa, xb);
+        fetch(s0 + 16, true, ka);
+        top.offer2(s, xa, s + 1, xb);
+        score(kb, xa, xb);
+        fetch(s0 + 24, true, kb);
+        top.offer2(s + 8, xa, s + 9, xb);
+    }
+    if (s0 < n) {
+        const int s = s0 + 2 * q;
+        float xa, xb;
+        score(ka, xa, xb);
+        top.offer2(s, s < n ? xa : -CUDART_INF_F, s + 1, s + 1 < n ? xb : -CUDART_INF_F);
+        score(kb, xa, xb);
+        top.offer2(s + 8, s + 8 < n ? xa : -CUDART_INF_F, s + 9, s + 9 < n ? xb : -CUDART_INF_F);
+    }
+
+    float ex[K];
+    int es[K];
+    top.finish(ex, es);
+#pragma unroll
+    for (int off = 1; off <= 2; off <<= 1) {
+        // the K best of two sorted lists: the j-th of one against the (K-1-j)-th of the other, then sorted again
+        float px[K];
+        int ps[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            px[j] = __shfl_xor_sync(0xffffffffu, ex[j], off);
+            ps[j] = __shfl_xor_sync(0xffffffffu, es[j], off);
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+            if (beats(px[K - 1 - j], ps[K - 1 - j], ex[j], es[j])) {
+                ex[j] = px[K - 1 - j];
+                es[j] = ps[K - 1 - j];
+            }
+        // what is left is bitonic: log2 K rounds of half-cleaners
+#pragma unroll
+        for (int d = K / 2; d >= 1; d >>= 1)
+#pragma unroll
+            for (int j = 0; j < K; ++j)
+                if ((j & d) == 0) {
+                    const bool sw = beats(ex[j + d], es[j + d], ex[j], es[j]);
+                    const float xa = sw ? ex[j + d] : ex[j], xb = sw ? ex[j] : ex[j + d];
+                    const int sa = sw ? es[j + d] : es[j], sb = sw ? es[j] : es[j + d];
+                    ex[j] = xa; ex[j + d] = xb; es[j] = sa; es[j + d] = sb;
+                }
+    }
+    const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+        if ((j & 3) == q && j < c.top_k) {
+            const bool on = es[j] != INT_MAX;
+            out_anchor[obase + j] = on ? i + 1 - stride_offset(c, es[j]) : -1;
+            out_score[obase + j] = on ? ex[j] : -CUDART_INF_F;
+        }
+}
+
 template <int K>
 cudaError_t launch_k(const bf16 *q_s, const bf16 *k, const Call &c, int32_t *oa, float *os, cudaStream_t st) {
     constexpr size_t smem = (size_t)kWarps * 2 * ListCap<K>::value * 32 * sizeof(float);
-    static bool attr_set[64] = {};
+    const bool four = c.G == kG;
+    void (*kern)(const bf16 *, const bf16 *, Call, int32_t *, float *) = four ? search_diag<K> : search_rows8<K>;
+    static bool attr_set[64][2] = {};
     if (smem > 48 * 1024) {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-        if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(search_diag<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (dev < 0 || dev >= 64 || !attr_set[dev][four]) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) attr_set[dev] = true;
+            if (dev >= 0 && dev < 64) attr_set[dev][four] = true;
         }
     }
-    const dim3 blocks((unsigned)((c.Lq + kWarps * kQW - 1) / (kWarps * kQW)), (unsigned)(c.B * c.Hkv));
-    search_diag<K><<<blocks, kWarps * 32, smem, st>>>(q_s, k, c, oa, os);
+    const int rows = kWarps * (four ? kQW : 1);   // positions per CTA
+    const dim3 blocks((unsigned)((c.Lq + rows - 1) / rows), (unsigned)(c.B * c.Hkv), four ? 1u : (unsigned)(c.G / 8));
+    kern<<<blocks, kWarps * 32, smem, st>>>(q_s, k, c, oa, os);
     return cudaGetLastError();
 }
 
@@ -288,7 +427,7 @@ cudaError_t launch_k(const bf16 *q_s, const bf16 *k, const Call &c, int32_t *oa,
 
 bool search_diag_supported(const Call &c, int dtype) {
     // (the 32-byte loads want 32-byte aligned rows: strides in multiples of 16 elements)
-    return dtype == SLA_BF16 && c.D == 128 && c.G == kG && c.top_k <= 16 && (long long)c.B * c.Hkv <= 65535 &&
+    return dtype == SLA_BF16 && c.D == 128 && (c.G == kG || c.G % 8 == 0) && c.top_k <= 16 && (long long)c.B * c.Hkv <= 65535 &&
            c.kv_st <= INT_MAX && c.q_pos0 + c.Lq <= INT_MAX &&
            (c.q_sb | c.q_sh | c.q_st | c.kv_sb | c.kv_sh | c.kv_st) % 16 == 0;
 }

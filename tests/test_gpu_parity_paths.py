@@ -86,6 +86,26 @@ def test_end_blocks_far_apart(sla, handle):
     P.compare_attention(out, lse, ref, "bf16")
 
 
+@pytest.mark.parametrize("heads,kv_heads,top_k", [(8, 1, 1), (16, 2, 4), (16, 1, 8), (16, 1, 16), (8, 1, 13)])
+def test_search_of_wide_groups(sla, handle, heads, kv_heads, top_k):
+    """Groups of 8 and 16 query heads per KV head, four lanes a head: 1 to 64 strides a row, so that lists of a
+    lane stay empty, short or full and the last step of eight or sixteen strides is ragged; lengths not a multiple
+    of the positions of a block."""
+    import parity_util as P
+    import torch
+    from oracle import sla_oracle as O
+    from paper_2601_18401_b200 import synth
+    for batch, seq_len, pos0 in ((1, 1100, 0), (2, 4103, 4062)):
+        w = workload(batch=batch, n_q_heads=heads, n_kv_heads=kv_heads, seq_len=seq_len, top_k=top_k, span_len=12)
+        x = synth.make_prefill(w, device="cuda:0")
+        q_s = x["q_s"][:, :, pos0:]
+        anchor, score = sla.sla_span_search(handle, q_s, x["k"], sla.make_params(top_k, 12, head_dim=128), q_pos0=pos0)
+        torch.cuda.synchronize()
+        host = P.host_inputs({"q_s": q_s, "k": x["k"]})
+        ref = O.span_search(host["q_s"], host["k"], synth.dtype_code("bf16"), top_k=top_k, q_pos0=pos0, search_scale=1.0)
+        P.compare_search(anchor, score, ref, q_pos0=pos0, q_s=host["q_s"], k=host["k"], search_scale=1.0)
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,dtype,D,n_ctx,top_k,span_len,per_span", [
     (1, 8, 2, "bf16", 128, 70001, 16, 600, False),    # clusters of eight, several per head
     (1, 32, 8, "bf16", 128, 9001, 8, 0, False),       # one cluster of eight per head
