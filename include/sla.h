@@ -45,7 +45,8 @@
  * other supported layout -- fp32, head_dim 64, a stride-0 K/V dimension, a single call over more than
  * about 2.6 million keys -- runs on generic fp32-accumulating kernels with the same results and far
  * lower throughput.  The choice depends on shapes and strides alone, never on the workspace size: a
- * workspace too small for the chosen kernel is SLA_ERR_WORKSPACE.
+ * workspace too small for the chosen kernel is SLA_ERR_WORKSPACE.  (One exception: the generic
+ * span-attention in the union mode needs no workspace, but is faster with what sla_workspace_bytes asks for.)
  *
  * Errors: every call returns an sla_status_t; 0 is success, negative values are errors.  When
  * argument validation fails nothing is launched.  No exception or abort crosses this interface.

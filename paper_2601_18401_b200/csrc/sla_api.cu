@@ -416,6 +416,9 @@ size_t sla_workspace_bytes(const sla_layout_t *l, const sla_params_t *p, int64_t
         // tensor-core span-attention: scratch for chunks of up to 65536 query positions
         const sla::TcPlan tp = sla::plan_attention_tc(c, (int)(Lq < 65536 ? Lq : 65536));
         if (tp.bytes > need) need = tp.bytes;
+    } else if (p->mode == SLA_UNION) {
+        const size_t blocks = sla::attn_blocks_bytes(c, 0);
+        if (blocks > need) need = blocks;
     }
     return need + 4096 + (sla::Canaries::kMax + 1) * sla::Canaries::kBytes;   // slack, and room for debug canaries
 }
@@ -487,6 +490,15 @@ sla_status_t span_attention_impl(sla_handle_t h, const void *q, const void *k, c
                 return fail(h, SLA_ERR_WORKSPACE, "workspace too small for span-attention: ask sla_workspace_bytes%s");
             cudaError_t e = sla::launch_attn_tc(q, k, v, c, anchor, score, out, lse, lse_span, h->ws + kHeaderBytes,
                                                 h->scratch_avail, h->sm_count, st, &h->launches, &h->timer, h->canaries, &h->tc_last);
+            if (e != cudaSuccess) return cuda_fail(h, e, what);
+            return SLA_OK;
+        }
+    }
+    if (sla::attn_blocks_supported(c)) {
+        const long long rows = sla::attn_blocks_rows(c, h->scratch_avail, h->canaries ? sla::Canaries::kBytes : 0);
+        if (rows > 0) {   // a workspace without the room leaves the row kernel, which needs none
+            cudaError_t e = sla::launch_attn_blocks(q, k, v, c, l->dtype, anchor, rows, out, lse,
+                                                    reinterpret_cast<char *>(h->ws) + kHeaderBytes, h->sm_count, h->canaries, st, &h->launches);
             if (e != cudaSuccess) return cuda_fail(h, e, what);
             return SLA_OK;
         }

@@ -12,6 +12,14 @@ cudaError_t launch_attn_simt(const void *q, const void *k, const void *v, const 
                              const int32_t *anchor, const float *score, void *out, float *lse, float *lse_span,
                              cudaStream_t st);
 
+// ---- span-attention of the generic layouts by blocks of keys, union mode (sla_attn_blocks.cu) -----
+bool attn_blocks_supported(const Call &c);
+size_t attn_blocks_bytes(const Call &c, size_t gap);
+long long attn_blocks_rows(const Call &c, size_t avail, size_t gap);
+cudaError_t launch_attn_blocks(const void *q, const void *k, const void *v, const Call &c, int dtype, const int32_t *anchor,
+                               long long step, void *out, float *lse, char *ws, int sm_count, bool canaries, cudaStream_t st,
+                               long long *launches);
+
 // Optional device-side timing of the dominant kernel of a call (CUDA events on the caller's stream).
 struct KernelTimer {
     static constexpr int kMaxPairs = 64;

@@ -1,7 +1,8 @@
 // Generic SIMT kernels of libsla: exact-fp32 span-search and span-attention, one warp per query row.
 //
 // These kernels serve the fp32 path (where tensor-core inputs would lose the precision the 1e-4
-// bound needs) and every shape or parameter set the tensor-core kernels do not cover.  A row of K or
+// bound needs) and every shape or parameter set the tensor-core kernels do not cover; span-attention in the
+// union mode has a kernel by key blocks beside it (sla_attn_blocks.cu).  A row of K or
 // V is read by LPR = D*sizeof(T)/16 adjacent lanes, 16 bytes each, so a warp instruction always
 // fetches whole, consecutive rows.
 #include <limits.h>
@@ -24,6 +25,14 @@ struct RowId {
 };
 __device__ inline RowId decode_row(long long row, const Call &c) {
     RowId o;
+    if ((row | c.Lq) >> 32 == 0) {   // 64-bit divisions are a hundred instructions each
+        const unsigned t1 = (unsigned)row / (unsigned)c.G, bg = t1 / (unsigned)c.Lq;
+        o.r = t1 - bg * (unsigned)c.Lq;
+        o.b = (int)(bg / (unsigned)c.Hkv);
+        o.g = (int)bg - o.b * c.Hkv;
+        o.h = o.g * c.G + (int)((unsigned)row - t1 * (unsigned)c.G);
+        return o;
+    }
     int hg = (int)(row % c.G);
     long long t1 = row / c.G;
     o.r = t1 % c.Lq;
@@ -34,6 +43,20 @@ __device__ inline RowId decode_row(long long row, const Call &c) {
     return o;
 }
 
+// Eight sums over LPR >= 8 adjacent lanes at once: lane sub (sub < 8, or sub % 8) receives the sum of x[sub % 8].
+template <int LPR> __device__ inline float reduce_eight(const float (&x)[8], int sub) {
+    float y[4], z[2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        y[j] = ((sub & 1) ? x[2 * j + 1] : x[2 * j]) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? x[2 * j] : x[2 * j + 1], 1);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        z[j] = ((sub & 2) ? y[2 * j + 1] : y[2 * j]) + __shfl_xor_sync(0xffffffffu, (sub & 2) ? y[2 * j] : y[2 * j + 1], 2);
+    float r = ((sub & 4) ? z[1] : z[0]) + __shfl_xor_sync(0xffffffffu, (sub & 4) ? z[0] : z[1], 4);
+#pragma unroll
+    for (int off = 8; off < LPR; off <<= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    return r;
+}
 template <int LPR> __device__ inline float reduce_sub(float x) {
 #pragma unroll
     for (int off = LPR / 2; off >= 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
@@ -52,7 +75,7 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
     constexpr int E = Vec16<T>::kElems;
     constexpr int LPR = D / E;
     constexpr int RPI = 32 / LPR;
-    constexpr int U = 4;
+    constexpr int U = 8;
     extern __shared__ float smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long row = (long long)blockIdx.x * kWarpsPerBlock + warp;
@@ -60,12 +83,14 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
     const RowId id = decode_row(row, c);
     const long long i = c.q_pos0 + id.r;
     // Algorithm 1: T = Anchors(i) without the window; t_s lies in W exactly when (s+1)^2 <= w
-    const int s_min = window_strides(c);
+    const int s_min = c.window > 0 ? window_strides(c) : 0;
     const int n = n_strides(c, i);
     float *sc = smem + (size_t)warp * n_max;
     const T *qrow = q_s + id.b * c.q_sb + id.h * c.q_sh + id.r * c.q_st;
     const T *kbase = k + id.b * c.kv_sb + id.g * c.kv_sh;
-    const int sub = lane % LPR, rsel = lane / LPR;
+    const int sub = lane % LPR, rsel = lane / LPR, kv_st = (int)c.kv_st;
+    const T *krow = kbase + sub * E;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched beside the tail of the kernel before it
     float qv[E];
     Vec16<T>::load(qrow + sub * E, qv);
 
@@ -77,21 +102,19 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
             const int s = s0 + u * RPI + rsel;
             part[u] = 0.f;
             if (s < n) {
-                const long long t = i + 1 - stride_offset(c, s);
+                const int t = (int)i + 1 - stride_offset(c, s);   // positions fit 31 bits
                 float kv[E];
-                Vec16<T>::load(kbase + t * c.kv_st + sub * E, kv);
+                Vec16<T>::load(krow + (long long)t * kv_st, kv);
 #pragma unroll
                 for (int e = 0; e < E; ++e) part[u] = fmaf(qv[e], kv[e], part[u]);
             }
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const float tot = reduce_sub<LPR>(part[u]);
-            const int s = s0 + u * RPI + rsel;
-            if (sub == 0 && s < n) sc[s] = tot * c.search_scale;
-        }
+        const float tot = reduce_eight<LPR>(part, sub);
+        const int s = s0 + (sub & 7) * RPI + rsel;
+        if (sub < 8 && s < n) sc[s] = tot * c.search_scale;
     }
     __syncwarp();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the attention may be scheduled beside the selection
 
     const long long obase = ((((long long)id.b * c.Hq + id.h) * c.Lq) + id.r) * c.top_k;
     for (int j = 0; j < c.top_k; ++j) {
@@ -381,8 +404,17 @@ cudaError_t search_launch(const void *q_s, const void *k, const Call &c, int32_t
         if (e != cudaSuccess) return e;
     }
     const long long blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    kern<<<(unsigned)blocks, kWarpsPerBlock * 32, smem, st>>>((const T *)q_s, (const T *)k, c, oa, os, n_max);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kWarpsPerBlock * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, (const T *)q_s, (const T *)k, c, oa, os, n_max);
 }
 
 template <typename T, int D>

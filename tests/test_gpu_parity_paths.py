@@ -106,6 +106,40 @@ def test_search_of_wide_groups(sla, handle, heads, kv_heads, top_k):
         P.compare_search(anchor, score, ref, q_pos0=pos0, q_s=host["q_s"], k=host["k"], search_scale=1.0)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(seq_len=1, top_k=6, span_len=300), dict(seq_len=63, top_k=1, span_len=600), dict(seq_len=64, top_k=2, span_len=600),
+    dict(seq_len=65, top_k=64, span_len=2),                                            # every anchor, spans of five keys
+    dict(batch=2, n_q_heads=6, n_kv_heads=2, seq_len=1543, top_k=9, span_len=0),       # lists that fill up several times
+    dict(seq_len=2300, top_k=3, span_len=33, window=200), dict(seq_len=900, top_k=1, span_len=31),   # 199 keys, 64 keys
+    dict(n_q_heads=4, n_kv_heads=4, seq_len=1200, top_k=8, span_len=100),
+])
+@pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128), ("bf16", 64)])
+def test_key_blocks(sla, handle, kw, dtype, D):
+    """The generic span-attention by key blocks: no anchors at all, one block, a block and a key, spans that end on either
+    side of a block edge, a window across spans; and with a workspace that has no room for it, the kernel by rows."""
+    import torch
+    from paper_2601_18401_b200 import synth
+    window = kw.get("window", 0)
+    w = workload(**dict(dict(n_q_heads=2, n_kv_heads=1), **{n: x for n, x in kw.items() if n != "window"}, dtype=dtype, head_dim=D))
+    if not window:
+        run_prefill(sla, handle, w)
+    x = synth.make_prefill(w, device="cuda:0")
+    params = sla.make_params(w.top_k, w.span_len, head_dim=D, window=window)
+    anchor, _ = sla.sla_span_search(handle, x["q_s"], x["k"], params)
+    out, lse = sla.sla_span_attention(handle, x["q"], x["k"], x["v"], anchor, params)
+    small = sla.Handle(0, 1024)
+    out2, lse2 = sla.sla_span_attention(small, x["q"], x["k"], x["v"], anchor, params)
+    torch.cuda.synchronize()
+    assert sla.sla_poll_status(handle) == sla.SLA_OK and sla.sla_poll_status(small) == sla.SLA_OK
+    small.close()
+    # both sum the same products and exponentials in fp32 in other orders: at most (D + n_keys + 30) 2^-24 of a score or a sum
+    # of |scores| < 64, and for bf16 results a rounding of 2^-8 of values < 5 on either side
+    tol = 64 * (D + w.seq_len + 30) * 2.0 ** -24 * 0.25 + (5 * 2.0 ** -8 if dtype == "bf16" else 0.0)
+    fin = torch.isfinite(lse2)
+    assert bool((torch.isfinite(lse) == fin).all())
+    assert float((out.double() - out2.double()).abs().max()) <= tol and bool(((lse - lse2)[fin].abs() <= tol).all())
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,dtype,D,n_ctx,top_k,span_len,per_span", [
     (1, 8, 2, "bf16", 128, 70001, 16, 600, False),    # clusters of eight, several per head
     (1, 32, 8, "bf16", 128, 9001, 8, 0, False),       # one cluster of eight per head
