@@ -140,6 +140,31 @@ def test_key_blocks(sla, handle, kw, dtype, D):
     assert float((out.double() - out2.double()).abs().max()) <= tol and bool(((lse - lse2)[fin].abs() <= tol).all())
 
 
+@pytest.mark.parametrize("seq_len,heads,kv_heads", [(1023, 32, 8), (1024, 32, 8), (1025, 32, 8), (4097, 8, 2), (8193, 16, 4)])
+def test_host_chunks(sla, seq_len, heads, kv_heads):
+    """Prefill through host buffers in chunks that shrink towards the end: one chunk and the first lengths with two, the
+    smallest chunk longer than 512 positions with few heads, quarters of the sequence first."""
+    import parity_util as P
+    import torch
+    from paper_2601_18401_b200 import synth
+    w = workload(seq_len=seq_len, n_q_heads=heads, n_kv_heads=kv_heads, span_len=24, top_k=5)
+    x = synth.make_prefill(w, device="cuda:0")
+    params = sla.make_params(w.top_k, w.span_len, head_dim=128)
+    layout = sla.make_layout(x["q"], x["k"])
+    h = sla.Handle(0, sla.sla_workspace_bytes(layout, params, seq_len, seq_len) + sla.sla_host_staging_bytes(layout, params, seq_len))
+    anchor, score = sla.sla_span_search(h, x["q_s"], x["k"], params)
+    out, lse = sla.sla_span_attention(h, x["q"], x["k"], x["v"], anchor, params)
+    host = {n: t.cpu().pin_memory() for n, t in x.items()}
+    ho, hl, ha, hs = sla.sla_prefill_host(h, host["q_s"], host["q"], host["k"], host["v"], params)
+    assert sla.sla_poll_status(h) == sla.SLA_OK
+    h.close()
+    assert torch.equal(ha, anchor.cpu()) and torch.equal(hs, score.cpu())
+    # either side is within the tolerance of the exact result (touching spans may be joined on one side only)
+    assert (ho.float() - out.cpu().float()).abs().max().item() <= 2 * P.OUT_TOL["bf16"]
+    fin = torch.isfinite(lse.cpu())
+    assert torch.equal(torch.isfinite(hl), fin) and (hl[fin] - lse.cpu()[fin]).abs().max().item() <= 2 * P.LSE_TOL["bf16"]
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,dtype,D,n_ctx,top_k,span_len,per_span", [
     (1, 8, 2, "bf16", 128, 70001, 16, 600, False),    # clusters of eight, several per head
     (1, 32, 8, "bf16", 128, 9001, 8, 0, False),       # one cluster of eight per head
