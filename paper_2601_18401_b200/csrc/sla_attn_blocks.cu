@@ -97,9 +97,8 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     if ((int)blockIdx.z >= n_ctas) return;
     const int n_keys = (int)(c.q_pos0 + r_first + n_rows - k0 < kKeys ? c.q_pos0 + r_first + n_rows - k0 : kKeys);
 
-    // launched beside the tail of the kernel before it; the merge may be scheduled from here on (it waits for this grid)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_wait();
+    chain_release();
     const T *kbase = k + b * c.kv_sb + g * c.kv_sh + (long long)k0 * c.kv_st;
     const T *vbase = v + b * c.kv_sb + g * c.kv_sh + (long long)k0 * c.kv_st;
     for (int x = threadIdx.x; x < kKeys * (D / E); x += kThreads) {
@@ -323,7 +322,7 @@ merge_blocks(Call c, BlockPlan p, int r_first, int n_rows, const int32_t *__rest
         s_b1[warp][j] = hi < 0 ? -1 : hi / kKeys;
     }
     __syncwarp();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_wait();
     const int sub = lane % LPR, half = lane / LPR;
     float M = -CUDART_INF_F, L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -402,23 +401,12 @@ cudaError_t launch_t(const T *q, const T *k, const T *v, const Call &c, const Bl
     const long long ctas = waves * chip - blocks * bg * 6 / 10;
     const int share = (int)(((scanned * bg * c.G + ctas - 1) / ctas + 31) / 32 * 32);
     const long long z = ((long long)n * c.G + share - 1) / share;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, (unsigned)bg, (unsigned)z);
-    cfg.blockDim = dim3(Tile<D>::WARPS * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, q, k, v, c, p, r0, n, share, anchor, ml, part);
+    cudaError_t e = launch_chained(kern, dim3((unsigned)blocks, (unsigned)bg, (unsigned)z), dim3(Tile<D>::WARPS * 32), smem, st, q, k, v, c, p,
+                                   r0, n, share, anchor, ml, part);
     if (e != cudaSuccess) return e;
     const long long rows = (long long)c.B * c.Hq * n;
-    cfg.gridDim = dim3((unsigned)((rows + kMergeWarps - 1) / kMergeWarps));
-    cfg.blockDim = dim3(kMergeWarps * 32);
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, merge_blocks<T, D>, c, p, r0, n, anchor, (const float2 *)ml, (const float *)part, out, lse);
+    return launch_chained(merge_blocks<T, D>, dim3((unsigned)((rows + kMergeWarps - 1) / kMergeWarps)), dim3(kMergeWarps * 32), 0, st, c, p, r0,
+                          n, anchor, (const float2 *)ml, (const float *)part, out, lse);
 }
 
 // Scratch for chunks of at most `rows` query positions; ok = false where the kernel does not apply.

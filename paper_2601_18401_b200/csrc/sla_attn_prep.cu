@@ -7,11 +7,11 @@
 // (batch, kv head), counts its pieces in a shared-memory histogram and touches the global counters
 // once per non-empty bucket, so that global atomics stay far below one per piece.
 //
+//   prep_clear       bucket counts and cursors to zero
 //   prep_count       the pieces of every row, parked; histogram of bucket sizes; pieces per row
-//   prep_scan_local  per (batch, kv head): exclusive offsets of its buckets, record and tile totals
-//   prep_scan_global per (batch, kv head): global offsets, tile table entries (a tile = 256 consecutive
-//                    records of the sorted list, whatever end blocks they fall in)
-//   prep_scatter     the parked pieces to their places in the sorted list
+//   prep_scan        per (batch, kv head): exclusive offsets of its buckets, record and tile totals
+//   prep_scatter     the parked pieces to their places in the sorted list; tile table entries (a tile = 256
+//                    consecutive records of the sorted list, whatever end blocks they fall in)
 //   prep_tile_bounds per tile: split where neighbouring pieces end far apart; the tile's end block and how
 //                    far back its pieces reach (number of key blocks to walk)
 #include <limits.h>
@@ -156,6 +156,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_count(PrepArgs a) {
     for (int x = threadIdx.x; x < nk; x += kPrepThreads) hist[x] = 0;
     for (int x = threadIdx.x; x <= a.nb_max; x += kPrepThreads) cls_tbl[x] = (unsigned char)class_of(x, a);
     __syncthreads();
+    chain_wait();
+    chain_release();
     int lo[KA], hi[KA], slot[KA];
     for (long long q = sh.q0 + threadIdx.x; q < sh.q1; q += kPrepThreads) {
         int h, rc;
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_count(PrepArgs a) {
 }
 
 // Scatter pass: the CTA claims a contiguous range of every bucket it has pieces in (its count is in
-// cta_hist, the bucket's global offset in key_count by now) and moves its parked pieces to their places.
+// cta_hist, the bucket's offset within its (batch, kv head) in key_count by now) and moves its parked pieces to
+// their places.
 __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
     extern __shared__ int hist[];   // [NB * ncls]: first record of this CTA in every bucket
     const int nk = a.NB * a.ncls;
@@ -216,6 +219,22 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
     const int *gcount = a.key_count + (long long)sh.bg * nk;
     int *gcursor = a.key_cursor + (long long)sh.bg * nk;
     const int *mine = a.cta_hist + (long long)blockIdx.x * nk;
+    __shared__ int s_base[2];   // records and tiles of the (batch, kv head)s before this one
+    chain_wait();
+    chain_release();
+    if (threadIdx.x < 32) {
+        int recs = 0, tiles = 0;
+        for (int x = threadIdx.x; x < sh.bg; x += 32) {
+            recs += a.totals[2 * x];
+            tiles += a.totals[2 * x + 1];
+        }
+        recs = __reduce_add_sync(0xffffffffu, recs);
+        tiles = __reduce_add_sync(0xffffffffu, tiles);
+        if (threadIdx.x == 0) {
+            s_base[0] = recs;
+            s_base[1] = tiles;
+        }
+    }
     // four buckets per thread and round, so that the counts, then the claims, are in flight together
     for (int x0 = threadIdx.x; x0 < nk; x0 += 4 * kPrepThreads) {
         int cnt[4], first[4];
@@ -236,6 +255,21 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
         }
     }
     __syncthreads();
+    const int rec_base = s_base[0];
+    if (blockIdx.x == sh.bg * a.ctas_per_bg) {
+        // the first CTA of the (batch, kv head) cuts its part of the sorted list into tiles of kRows records, across end blocks:
+        // entries {batch*Hkv + kv head, (end block: filled in by prep_tile_bounds), first record, records}
+        const int n_recs = a.totals[2 * sh.bg], nt = a.totals[2 * sh.bg + 1], tile_base = s_base[1];
+        for (int t = threadIdx.x; t < nt; t += kPrepThreads) {
+            const int left = n_recs - t * kRows;
+            if (tile_base + t < a.max_tiles)
+                a.tiles[tile_base + t] = make_int4(sh.bg, 0, rec_base + t * kRows, left < kRows ? left : kRows);
+        }
+        if (sh.bg == a.B * a.Hkv - 1 && threadIdx.x == 0) {
+            const int all = tile_base + nt;
+            a.n_tiles[0] = a.n_tiles[1] = all < a.max_tiles ? all : a.max_tiles;   // [1]: the count as cut here
+        }
+    }
     // One thread per parked slot, four slots in flight per thread.  The rows of a (batch, kv head) are
     // consecutive (row = first row + q), so the CTA's slots are one contiguous run of `stage`.
     const unsigned n_el = (unsigned)((sh.q1 - sh.q0) * a.slots);   // rows x slots < 2^31 for the whole chunk
@@ -261,7 +295,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (j[u] < cnt[u])
-                a.recs[hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row[u], pc[u].z >> 24, pc[u].x, pc[u].y);
+                a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row[u], pc[u].z >> 24, pc[u].x, pc[u].y);
     }
 }
 
@@ -292,14 +326,29 @@ __device__ inline int block_excl_scan(int v, int &total, int *warp_sum) {
     return base + x - v;
 }
 
+// The bucket counts and cursors start from zero.
+__global__ void __launch_bounds__(kPrepThreads) prep_clear(PrepArgs a) {
+    const long long n = (long long)a.B * a.Hkv * a.NB * a.ncls;
+    const long long x0 = (long long)blockIdx.x * 4 * kPrepThreads + threadIdx.x;
+    chain_wait();
+    chain_release();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const long long x = x0 + u * kPrepThreads;
+        if (x < n) a.key_count[x] = a.key_cursor[x] = 0;
+    }
+}
+
 // One CTA per (batch, kv head): bucket histogram -> exclusive offsets local to the (batch, kv head),
 // plus how many records and tiles it has.
-__global__ void __launch_bounds__(kPrepThreads) prep_scan_local(PrepArgs a) {
+__global__ void __launch_bounds__(kPrepThreads) prep_scan(PrepArgs a) {
     __shared__ int warp_sum[32];
     const int nk = a.NB * a.ncls, bg = blockIdx.x, tid = threadIdx.x;
     int *cnt = a.key_count + (long long)bg * nk;
     const int per = (nk + kPrepThreads - 1) / kPrepThreads;
     const int k0 = per * tid, k1 = (k0 + per < nk) ? k0 + per : nk;
+    chain_wait();
+    chain_release();
     int local = 0;
     for (int k = k0; k < k1; ++k) local += cnt[k];
     int n_recs;
@@ -316,35 +365,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scan_local(PrepArgs a) {
     }
 }
 
-// One CTA per (batch, kv head): offsets become global, tile table entries are written.
-__global__ void __launch_bounds__(kPrepThreads) prep_scan_global(PrepArgs a) {
-    __shared__ int s_base[2];
-    const int nk = a.NB * a.ncls, bg = blockIdx.x, tid = threadIdx.x, n_bg = a.B * a.Hkv;
-    if (tid == 0) {
-        int rec_base = 0, tile_base = 0;
-        for (int x = 0; x < bg; ++x) { rec_base += a.totals[2 * x]; tile_base += a.totals[2 * x + 1]; }
-        s_base[0] = rec_base;
-        s_base[1] = tile_base;
-        if (bg == n_bg - 1) {
-            const int all = tile_base + a.totals[2 * bg + 1];
-            a.n_tiles[0] = a.n_tiles[1] = all < a.max_tiles ? all : a.max_tiles;   // [1]: the count as cut here
-        }
-    }
-    __syncthreads();
-    const int rec_base = s_base[0], tile_base = s_base[1], n_recs = a.totals[2 * bg];
-    int *cnt = a.key_count + (long long)bg * nk;
-    // tile entries {batch*Hkv + kv head, (end block: filled in by prep_tile_bounds), first record, records}
-    const int nt = (n_recs + kRows - 1) / kRows;
-    for (int t = tid; t < nt; t += kPrepThreads) {
-        const int left = n_recs - t * kRows;
-        if (tile_base + t < a.max_tiles)
-            a.tiles[tile_base + t] = make_int4(bg, 0, rec_base + t * kRows, left < kRows ? left : kRows);
-    }
-    __syncthreads();
-    for (int k = tid; k < nk; k += kPrepThreads) cnt[k] += rec_base;
-}
-
-// One warp per tile as cut by prep_scan_global (256 consecutive records).  Where two neighbouring records of the
+// One warp per tile as cut by prep_scatter (256 consecutive records).  Where two neighbouring records of the
 // tile end further apart than a span is long the tile is split there: walking the gap would cost more than walking
 // two spans.  (So does a stretch of kMaxStretch blocks, which keeps the block numbers of a tile within 16 bits.)
 // The extra tiles are appended to the table.  For every tile: the end block of its last piece (second word), the
@@ -355,6 +376,8 @@ __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
     __shared__ int s_eb[8][kRows], s_lo[8][kRows];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = blockIdx.x * 8 + warp;
+    chain_wait();
+    chain_release();
     if (t >= a.n_tiles[1]) return;
     const int4 ti = a.tiles[t];
     const int cnt = ti.w;
@@ -432,13 +455,17 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
         }
     }
     const unsigned grid = (unsigned)(n_bg * a.ctas_per_bg);
-    k0<<<grid, kPrepThreads, smem, st>>>(a);
-    prep_scan_local<<<n_bg, kPrepThreads, 0, st>>>(a);
-    prep_scan_global<<<n_bg, kPrepThreads, 0, st>>>(a);
-    k1<<<grid, kPrepThreads, smem, st>>>(a);
-    prep_tile_bounds<<<(unsigned)((a.max_tiles + 7) / 8), 256, 0, st>>>(a);
+    // a chain of short kernels: 1999 positions, 32/8 heads, search to merge, 115 us with plain launches, a memset and an
+    // extra kernel for the offsets across (batch, kv head)s, 101 us like this; 16/2 heads, 1590 positions, K = 2 61 and 46 us
+    const long long words = (long long)n_bg * a.NB * a.ncls;
+    const unsigned clear = (unsigned)((words + 4 * kPrepThreads - 1) / (4 * kPrepThreads));
+    cudaError_t e = launch_chained(prep_clear, dim3(clear), dim3(kPrepThreads), 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(k0, dim3(grid), dim3(kPrepThreads), smem, st, a);
+    if (e == cudaSuccess) e = launch_chained(prep_scan, dim3(n_bg), dim3(kPrepThreads), 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(k1, dim3(grid), dim3(kPrepThreads), smem, st, a);
+    if (e == cudaSuccess) e = launch_chained(prep_tile_bounds, dim3((unsigned)((a.max_tiles + 7) / 8)), dim3(256), 0, st, a);
     if (launches) *launches += 5;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace tc

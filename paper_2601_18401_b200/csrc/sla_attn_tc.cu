@@ -170,11 +170,6 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     const uint32_t bar_l_full = mbase + offsetof(Meta, l_full);
     const uint32_t bar_o_full = mbase + offsetof(Meta, o_full), bar_o_empty = mbase + offsetof(Meta, o_empty);
 
-    // requested before the set-up (the table has an entry for every CTA)
-    const int n_tiles = *p.n_tiles, tile_step = gridDim.x;
-    int tile = blockIdx.x;
-    int4 ti = p.tiles[tile];
-
     if (tid == 0) {
 #pragma unroll 1
         for (int x = 0; x < kQS; ++x) {
@@ -205,6 +200,12 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         ptx::tmem_alloc(mbase + offsetof(Meta, tmem_base), kTmemCols);
         ptx::tmem_relinquish();
     }
+    // the set-up above runs beside the kernel before this one
+    chain_wait();
+    chain_release();
+    const int n_tiles = *p.n_tiles, tile_step = gridDim.x;
+    int tile = blockIdx.x;
+    int4 ti = p.tiles[tile];   // the table has an entry for every CTA
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
@@ -622,6 +623,7 @@ tc_merge(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
     const long long row = gid >> 4;
     const int sub = (int)(gid & 15);
     const long long rows = (long long)c.B * c.Hq * Lc;
+    chain_wait();
     if (row >= rows) return;
     const int cnt = n_pieces[row];
     const float2 *pl = part_lse + row * slots;
@@ -706,6 +708,7 @@ tc_merge_gated(const __half *__restrict__ part_o, const float2 *__restrict__ par
     const long long row = gid >> 4;
     const int sub = (int)(gid & 15);
     const long long rows = (long long)c.B * c.Hq * Lc;
+    chain_wait();
     if (row >= rows) return;
     const int rc = (int)((unsigned)row % (unsigned)Lc);   // rows < 2^31
     const int bh = (int)((unsigned)row / (unsigned)Lc);
@@ -810,6 +813,7 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
     const int lane = threadIdx.x & 31;
     const long long row0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
     const long long rows = (long long)c.B * c.Hq * Lc;
+    chain_wait();
     if (row0 >= rows) return;
     const bool has_w = c.window > 0;
     // ---- phase A: lane = row
@@ -1184,8 +1188,7 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
     for (long long r0 = 0; r0 < c.Lq; r0 += Lc) {
         const int lc = (int)((c.Lq - r0 < Lc) ? c.Lq - r0 : Lc);
         const long long rows = (long long)c.B * c.Hq * lc;
-        cudaError_t e = cudaMemsetAsync(ws + plan.off_key_count, 0, 2 * (plan.off_key_cursor - plan.off_key_count), st);
-        if (e != cudaSuccess) return e;
+        cudaError_t e = cudaSuccess;
         if (canaries && (e = launch_canary_fill(ws, plan.canaries, st)) != cudaSuccess) return e;
         tc::PrepArgs pa;
         pa.anchor = anchor; pa.B = c.B; pa.Hq = c.Hq; pa.Hkv = c.Hkv; pa.G = c.G; pa.top_k = c.top_k;
@@ -1238,18 +1241,21 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         tp.status = c.status; tp.Hkv = c.Hkv;
         if (last) { last->tiles = pa.tiles; last->ranges = pa.ranges; last->n_tiles = counters; }
         if (timer) timer->begin(st);
-        tc_attend<<<sm_count, kThreads, kSmemBytes, st>>>(tm_q, tm_k, tm_v, tp);
+        e = launch_chained(tc_attend, dim3(sm_count), dim3(kThreads), kSmemBytes, st, tm_q, tm_k, tm_v, tp);
+        if (e != cudaSuccess) return e;
         if (timer) timer->end(st);
+        // The merges do not release what comes after them: 131072 short CTAs, each with the extra instruction, took 2 % more of
+        // a whole call at 65536 positions.  Nor does the search, whose CTAs are in the way of nothing that could start early.
         const unsigned mblocks = (unsigned)((rows * 16 + 255) / 256);
         if (c.mode == SLA_PER_SPAN && c.top_k <= kGateK)
-            tc_merge_gated_rows<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(tp.part_o, tp.part_lse, anchor, score, c,
-                                                                               plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
+            e = launch_chained(tc_merge_gated_rows, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, (const __half *)tp.part_o,
+                               (const float2 *)tp.part_lse, anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
         else if (c.mode == SLA_PER_SPAN)
-            tc_merge_gated<<<mblocks, 256, 0, st>>>(tp.part_o, tp.part_lse, anchor, score, c, plan.slots, lc, r0,
-                                                    (bf16 *)out, lse, lse_span);
+            e = launch_chained(tc_merge_gated, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
+                               anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
         else
-            tc_merge<<<mblocks, 256, 0, st>>>(tp.part_o, tp.part_lse, pa.n_pieces, c, plan.slots, lc, r0, (bf16 *)out, lse);
-        e = cudaGetLastError();
+            e = launch_chained(tc_merge, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
+                               (const unsigned char *)pa.n_pieces, c, plan.slots, lc, r0, (bf16 *)out, lse);
         if (e != cudaSuccess) return e;
         if (launches) *launches += 2;
         if (canaries && (e = launch_canary_check(ws, plan.canaries, c.status, st)) != cudaSuccess) return e;

@@ -101,6 +101,27 @@ __host__ __device__ inline long long base_len(const Call &c, long long i) {
     return base_len(i, c.span_len, pattern_len(c), c.n_len);
 }
 
+// ---- launches in a chain: a kernel started with launch_chained may be scheduled while the kernel before it on the
+// stream still runs (from the point where all of its CTAs have called chain_release, or have ended).  It calls chain_wait
+// before it touches global memory -- by then the kernel before it, and with it all before that, is complete -- and releases
+// its own successor only after that.
+__device__ inline void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ inline void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ---- element loads: a 16-byte vector of T widened to fp32 ------------------------------------
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {

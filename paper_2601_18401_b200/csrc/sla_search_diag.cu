@@ -171,6 +171,7 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     const long long last = c.Lq - 1;
     // ---- A operand: rows r8 and r8 + 8 = (position r8>>2, head r8&3) and (position 2 + (r8>>2), head r8&3)
     Words8 qa[2], qb[2];
+    chain_wait();
     {
         const long long ra = r0 + (r8 >> 2) < last ? r0 + (r8 >> 2) : last;
         const long long rb = r0 + 2 + (r8 >> 2) < last ? r0 + 2 + (r8 >> 2) : last;
@@ -306,6 +307,7 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     if (r >= c.Lq) return;
     const int bg = blockIdx.y, g = bg % c.Hkv, b = bg / c.Hkv, h = g * c.G + blockIdx.z * 8 + r8;
     Words8 qa[2];
+    chain_wait();
     {
         const bf16 *base = q_s + b * c.q_sb + (long long)h * c.q_sh + r * c.q_st + 16 * q;
         qa[0] = ldg256(base);
@@ -419,8 +421,7 @@ cudaError_t launch_k(const bf16 *q_s, const bf16 *k, const Call &c, int32_t *oa,
     }
     const int rows = kWarps * (four ? kQW : 1);   // positions per CTA
     const dim3 blocks((unsigned)((c.Lq + rows - 1) / rows), (unsigned)(c.B * c.Hkv), four ? 1u : (unsigned)(c.G / 8));
-    kern<<<blocks, kWarps * 32, smem, st>>>(q_s, k, c, oa, os);
-    return cudaGetLastError();
+    return launch_chained(kern, blocks, dim3(kWarps * 32), smem, st, q_s, k, c, oa, os);
 }
 
 }  // namespace

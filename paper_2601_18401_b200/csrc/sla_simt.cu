@@ -90,7 +90,7 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
     const T *kbase = k + id.b * c.kv_sb + id.g * c.kv_sh;
     const int sub = lane % LPR, rsel = lane / LPR, kv_st = (int)c.kv_st;
     const T *krow = kbase + sub * E;
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched beside the tail of the kernel before it
+    chain_wait();
     float qv[E];
     Vec16<T>::load(qrow + sub * E, qv);
 
@@ -114,7 +114,7 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
         if (sub < 8 && s < n) sc[s] = tot * c.search_scale;
     }
     __syncwarp();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the attention may be scheduled beside the selection
+    chain_release();   // the attention may be scheduled beside the selection
 
     const long long obase = ((((long long)id.b * c.Hq + id.h) * c.Lq) + id.r) * c.top_k;
     for (int j = 0; j < c.top_k; ++j) {
@@ -404,17 +404,7 @@ cudaError_t search_launch(const void *q_s, const void *k, const Call &c, int32_t
         if (e != cudaSuccess) return e;
     }
     const long long blocks = (rows + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(kWarpsPerBlock * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, (const T *)q_s, (const T *)k, c, oa, os, n_max);
+    return launch_chained(kern, dim3((unsigned)blocks), dim3(kWarpsPerBlock * 32), smem, st, (const T *)q_s, (const T *)k, c, oa, os, n_max);
 }
 
 template <typename T, int D>
