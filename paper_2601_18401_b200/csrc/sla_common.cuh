@@ -40,6 +40,14 @@ struct Call {
 // floor(sqrt(x)) for 0 <= x < 2^62, exact.
 __host__ __device__ inline long long isqrt_ll(long long x) {
     if (x <= 0) return 0;
+#ifdef __CUDA_ARCH__
+    if (x < (1ll << 31)) {   // a dozen instructions instead of a double-precision root: below 2^31 the rounded float root is
+        unsigned r = (unsigned)__fsqrt_rn((float)x);   // within 46341 * 2^-23 < 0.01 of the true one, so one step mends it
+        if (r * r > (unsigned)x) --r;
+        else if ((r + 1) * (r + 1) <= (unsigned)x) ++r;
+        return r;
+    }
+#endif
     long long r = (long long)sqrt((double)x);
     while (r * r > x) --r;
     while ((r + 1) * (r + 1) <= x) ++r;

@@ -36,7 +36,7 @@ constexpr int kWarps = 8;
 constexpr int kQW = 4;   // query positions per warp
 constexpr int kG = 4;    // query heads per KV head
 
-template <int K> struct ListCap { static constexpr int value = 2 * K + 8; };
+template <int K> struct ListCap { static constexpr int value = (2 * K + 8 + 3) / 4 * 4; };
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                uint32_t b0, uint32_t b1) {
@@ -86,6 +86,35 @@ __device__ __forceinline__ void sort_pairs(float (&x)[K], int (&s)[K]) {
             }
 }
 
+// The K best of this lane's and of lane ^ off's sorted lists, in both lanes: the j-th of one against the (K-1-j)-th of the
+// other leaves them as a bitonic sequence, which log2 K rounds of half-cleaners sort.
+template <int K>
+__device__ __forceinline__ void merge_pairs(float (&x)[K], int (&s)[K], int off) {
+    float px[K];
+    int ps[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        px[j] = __shfl_xor_sync(0xffffffffu, x[j], off);
+        ps[j] = __shfl_xor_sync(0xffffffffu, s[j], off);
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+        if (beats(px[K - 1 - j], ps[K - 1 - j], x[j], s[j])) {
+            x[j] = px[K - 1 - j];
+            s[j] = ps[K - 1 - j];
+        }
+#pragma unroll
+    for (int d = K / 2; d >= 1; d >>= 1)
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+            if ((j & d) == 0) {
+                const bool sw = beats(x[j + d], s[j + d], x[j], s[j]);
+                const float xa = sw ? x[j + d] : x[j], xb = sw ? x[j] : x[j + d];
+                const int sa = sw ? s[j + d] : s[j], sb = sw ? s[j] : s[j + d];
+                x[j] = xa; x[j + d] = xb; s[j] = sa; s[j + d] = sb;
+            }
+}
+
 // A lane's running top-k: the K best values so far, sorted, in registers, and in shared memory (entry e at lx[32 e],
 // ls[32 e]) every score with its stride index that beat the K-th best when it arrived.
 template <int K>
@@ -109,15 +138,23 @@ struct RunningTop {
 #pragma unroll
         for (int j = 0; j < K; ++j) allow_eq -= v[j] > vk;
         int w = 0;
-        for (int e = 0; e < cnt; ++e) {
-            const float x = lx[32 * e];
-            const int s = ls[32 * e];
-            const bool eq = x == vk;
-            if (x > vk || (eq && allow_eq > 0)) {
-                allow_eq -= eq;
-                lx[32 * w] = x;
-                ls[32 * w] = s;
-                ++w;
+        for (int e0 = 0; e0 < cnt; e0 += 4) {   // four loads at a time: the list is as long as a multiple of four
+            float x[4];
+            int s[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x[u] = lx[32 * (e0 + u)];
+                s[u] = ls[32 * (e0 + u)];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool eq = x[u] == vk;
+                if (e0 + u < cnt && (x[u] > vk || (eq && allow_eq > 0))) {
+                    allow_eq -= eq;
+                    lx[32 * w] = x[u];
+                    ls[32 * w] = s[u];
+                    ++w;
+                }
             }
         }
         cnt = w;
@@ -254,36 +291,20 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         }
     }
 
-    // ---- the lane's K best with their stride indices, sorted; then the merge with the lane that holds
-    // the pair's other strides (q differs in bit 1): the rank of an entry in the union is its rank here
-    // plus the number of the partner's entries that come before it
+    // ---- the lane's K best, merged with those of the lane that holds the pair's other strides (q differs in bit 1);
+    // either of the two writes every other slot
     float ex[K];
     int es[K];
     top.finish(ex, es);
-    const int cnt = top.cnt;
-    int rank[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) rank[j] = j;
-#pragma unroll
-    for (int e = 0; e < K; ++e) {
-        const float pv = __shfl_xor_sync(0xffffffffu, ex[e], 2);
-        const int ps = __shfl_xor_sync(0xffffffffu, es[e], 2);
-#pragma unroll
-        for (int j = 0; j < K; ++j) rank[j] += beats(pv, ps, ex[j], es[j]);
-    }
-    const int n_pair = cnt + __shfl_xor_sync(0xffffffffu, cnt, 2);
+    merge_pairs<K>(ex, es, 2);
     if (!row_own) return;
     const long long obase = ((((long long)b * c.Hq + g * kG + hh) * c.Lq) + r0 + jq) * c.top_k;
 #pragma unroll
     for (int j = 0; j < K; ++j)
-        if (j < cnt && rank[j] < c.top_k) {
-            out_anchor[obase + rank[j]] = i_own + 1 - stride_offset(c, es[j]);
-            out_score[obase + rank[j]] = ex[j];
-        }
-    if (u_own == 0)   // fewer candidates than slots: pad
-        for (int j = n_pair; j < c.top_k; ++j) {
-            out_anchor[obase + j] = -1;
-            out_score[obase + j] = -CUDART_INF_F;
+        if ((j & 1) == u_own && j < c.top_k) {
+            const bool on = es[j] != INT_MAX;
+            out_anchor[obase + j] = on ? i_own + 1 - stride_offset(c, es[j]) : -1;
+            out_score[obase + j] = on ? ex[j] : -CUDART_INF_F;
         }
 }
 
@@ -366,34 +387,8 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     float ex[K];
     int es[K];
     top.finish(ex, es);
-#pragma unroll
-    for (int off = 1; off <= 2; off <<= 1) {
-        // the K best of two sorted lists: the j-th of one against the (K-1-j)-th of the other, then sorted again
-        float px[K];
-        int ps[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) {
-            px[j] = __shfl_xor_sync(0xffffffffu, ex[j], off);
-            ps[j] = __shfl_xor_sync(0xffffffffu, es[j], off);
-        }
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-            if (beats(px[K - 1 - j], ps[K - 1 - j], ex[j], es[j])) {
-                ex[j] = px[K - 1 - j];
-                es[j] = ps[K - 1 - j];
-            }
-        // what is left is bitonic: log2 K rounds of half-cleaners
-#pragma unroll
-        for (int d = K / 2; d >= 1; d >>= 1)
-#pragma unroll
-            for (int j = 0; j < K; ++j)
-                if ((j & d) == 0) {
-                    const bool sw = beats(ex[j + d], es[j + d], ex[j], es[j]);
-                    const float xa = sw ? ex[j + d] : ex[j], xb = sw ? ex[j] : ex[j + d];
-                    const int sa = sw ? es[j + d] : es[j], sb = sw ? es[j] : es[j + d];
-                    ex[j] = xa; ex[j + d] = xb; es[j] = sa; es[j + d] = sb;
-                }
-    }
+    merge_pairs<K>(ex, es, 1);
+    merge_pairs<K>(ex, es, 2);
     const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;
 #pragma unroll
     for (int j = 0; j < K; ++j)
