@@ -800,12 +800,16 @@ tc_merge_gated(const __half *__restrict__ part_o, const float2 *__restrict__ par
     if (sub == 0) lse[orow] = lse_first;
 }
 
-// The same for top_k <= 8, arranged so that the per-row arithmetic (gate, log-sum-exp weights, base
+// The same for top_k <= K, K at most 8, arranged so that the per-row arithmetic (gate, log-sum-exp weights, base
 // span length) is done once per row: a warp takes 32 consecutive rows; first every lane works out the
 // coefficients of its own row (weight of every span piece, summed weight of the window piece, the
 // log-sum-exps), then the warp walks its rows two at a time, 16 lanes per row and 8 columns per lane,
 // with the coefficients handed over by shuffles.
+// Bound by the reads of the partial results: with room for eight spans whatever top_k is, 106 registers and the shuffles of
+// absent spans made it 402 us for 32768 positions, 32 heads, two spans and a window (1.1 GB, 2.7 TB/s); with room for two,
+// 48 registers and 213 us.
 constexpr int kGateK = 8;
+template <int K>
 __global__ void __launch_bounds__(256)
 tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
                     const int32_t *__restrict__ anchor, const float *__restrict__ score, Call c, int slots, int Lc,
@@ -817,11 +821,11 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
     if (row0 >= rows) return;
     const bool has_w = c.window > 0;
     // ---- phase A: lane = row
-    float coef[kGateK], cw = 0.f;       // weights of the span pieces and of the window piece
-    uint32_t ex[kGateK], ex_w = 0u;     // their chunk exponents
+    float coef[K], cw = 0.f;       // weights of the span pieces and of the window piece
+    uint32_t ex[K], ex_w = 0u;     // their chunk exponents
     long long out_off = 0;
 #pragma unroll
-    for (int j = 0; j < kGateK; ++j) { coef[j] = 0.f; ex[j] = 0u; }
+    for (int j = 0; j < K; ++j) { coef[j] = 0.f; ex[j] = 0u; }
     {
         const long long row = row0 + lane;
         if (row < rows) {
@@ -839,12 +843,12 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
             const float2 pw = has_w ? __ldg(pl + c.top_k) : make_float2(-CUDART_INF_F, 0.f);
             const float lw = pw.x;
             ex_w = __float_as_uint(pw.y);
-            float scv[kGateK], lj[kGateK];
-            bool sel[kGateK], has_s[kGateK];
+            float scv[K], lj[K];
+            bool sel[K], has_s[K];
             float smax = -CUDART_INF_F;
             int n_sel = 0;
 #pragma unroll
-            for (int j = 0; j < kGateK; ++j) {
+            for (int j = 0; j < K; ++j) {
                 const long long t = j < c.top_k ? an[j] : -1;
                 sel[j] = t >= 0 && t <= i;
                 scv[j] = sel[j] ? sc[j] : -CUDART_INF_F;
@@ -857,7 +861,7 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
             }
             float sden = 0.f;
 #pragma unroll
-            for (int j = 0; j < kGateK; ++j)
+            for (int j = 0; j < K; ++j)
                 if (sel[j]) sden += expf(scv[j] - smax);
             float lse_first = -CUDART_INF_F;
             if (n_sel == 0 && has_w) {   // Algorithm 1, empty selection: the window alone
@@ -866,7 +870,7 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
             }
             bool first = true;
 #pragma unroll
-            for (int j = 0; j < kGateK; ++j) {
+            for (int j = 0; j < K; ++j) {
                 if (j >= c.top_k) break;
                 float l_t = -CUDART_INF_F;
                 if (sel[j]) {
@@ -895,24 +899,24 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
         float acc[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-        float cf[kGateK + 1];
-        uint32_t ee[kGateK + 1];
-        uint4 raw[kGateK + 1];
+        float cf[K + 1];
+        uint32_t ee[K + 1];
+        uint4 raw[K + 1];
 #pragma unroll
-        for (int j = 0; j < kGateK; ++j) {
+        for (int j = 0; j < K; ++j) {
             cf[j] = __shfl_sync(0xffffffffu, coef[j], src);
             ee[j] = __shfl_sync(0xffffffffu, ex[j], src);
         }
-        cf[kGateK] = __shfl_sync(0xffffffffu, cw, src);
-        ee[kGateK] = __shfl_sync(0xffffffffu, ex_w, src);
+        cf[K] = __shfl_sync(0xffffffffu, cw, src);
+        ee[K] = __shfl_sync(0xffffffffu, ex_w, src);
         const long long off = __shfl_sync(0xffffffffu, out_off, src);
 #pragma unroll
-        for (int j = 0; j <= kGateK; ++j) {
-            const int slot = j < kGateK ? j : c.top_k;
+        for (int j = 0; j <= K; ++j) {
+            const int slot = j < K ? j : c.top_k;
             raw[j] = cf[j] != 0.f ? __ldg(reinterpret_cast<const uint4 *>(po + (long long)slot * kD)) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
-        for (int j = 0; j <= kGateK; ++j)
+        for (int j = 0; j <= K; ++j)
             if (cf[j] != 0.f) {
                 const uint32_t eb = (ee[j] >> shift) & 0xffu;
                 const float ws = cf[j] * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
@@ -1248,7 +1252,7 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         // a whole call at 65536 positions.  Nor does the search, whose CTAs are in the way of nothing that could start early.
         const unsigned mblocks = (unsigned)((rows * 16 + 255) / 256);
         if (c.mode == SLA_PER_SPAN && c.top_k <= kGateK)
-            e = launch_chained(tc_merge_gated_rows, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, (const __half *)tp.part_o,
+            e = launch_chained(c.top_k <= 2 ? tc_merge_gated_rows<2> : c.top_k <= 4 ? tc_merge_gated_rows<4> : tc_merge_gated_rows<kGateK>, dim3((unsigned)((rows + 255) / 256)), dim3(256), 0, st, (const __half *)tp.part_o,
                                (const float2 *)tp.part_lse, anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
         else if (c.mode == SLA_PER_SPAN)
             e = launch_chained(tc_merge_gated, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,

@@ -165,6 +165,14 @@ def test_host_chunks(sla, seq_len, heads, kv_heads):
     assert torch.equal(torch.isfinite(hl), fin) and (hl[fin] - lse.cpu()[fin]).abs().max().item() <= 2 * P.LSE_TOL["bf16"]
 
 
+@pytest.mark.parametrize("top_k", [1, 2, 3, 4, 5, 8, 9])
+@pytest.mark.parametrize("window", [0, 40])
+def test_gated_merge_of_each_width(sla, handle, top_k, window):
+    """The per-span merge is built for up to 2, 4 and 8 spans a row; beyond that the general one."""
+    from test_gpu_parity_modes import run_modes
+    run_modes(sla, handle, workload(n_q_heads=2, n_kv_heads=1, seq_len=1100, top_k=top_k, span_len=21), window)
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,dtype,D,n_ctx,top_k,span_len,per_span", [
     (1, 8, 2, "bf16", 128, 70001, 16, 600, False),    # clusters of eight, several per head
     (1, 32, 8, "bf16", 128, 9001, 8, 0, False),       # one cluster of eight per head
