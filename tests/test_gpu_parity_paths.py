@@ -168,7 +168,8 @@ def test_host_chunks(sla, seq_len, heads, kv_heads):
 @pytest.mark.parametrize("top_k", [1, 2, 3, 4, 5, 8, 9])
 @pytest.mark.parametrize("window", [0, 40])
 def test_gated_merge_of_each_width(sla, handle, top_k, window):
-    """The per-span merge is built for up to 2, 4 and 8 spans a row; beyond that the general one."""
+    """The per-span merge is built for up to 2, 4 and 8 spans a row, the counting pass of the work list for up to 5, 9 and
+    17 spans and window together; beyond that the general ones."""
     from test_gpu_parity_modes import run_modes
     run_modes(sla, handle, workload(n_q_heads=2, n_kv_heads=1, seq_len=1100, top_k=top_k, span_len=21), window)
 
