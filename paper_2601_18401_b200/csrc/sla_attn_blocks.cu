@@ -7,7 +7,9 @@
 //           spans (the union is the OR of the spans' masks: no sorting, no clipping); rows with a mask go to a list;
 //   attend  a warp takes LPR lanes x 4 rows per group (32 rows at head_dim 64, 16 at 128): a lane holds 16 dims of four
 //           query rows, reads the same 16 dims of a key as its group's peers (broadcast) and the lanes' sums are exchanged
-//           so that each lane ends up with the score of one row; 32 keys, then the exponentials, then the values;
+//           so that each lane ends up with the score of one row; the 64 keys, then the exponentials, then the values
+//           (every row multiplies all 64, with weight 0 where it did not select the key: an Inf or NaN among them is
+//           zero in shared memory and comes from global memory for the rows that did);
 //   merge   a row has one partial result per key block it touches, at a slot that only the row's own spans determine
 //           (first span that reaches the block, block within that span), combined in slot order.
 // Everything is fp32 FMA (two per instruction), as in the row kernel: bf16 inputs are widened exactly.
@@ -85,6 +87,7 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     float *ks = reinterpret_cast<float *>(smem4), *vs = ks + kKeys * D, *ps = vs + kKeys * D;
     int4 *list = reinterpret_cast<int4 *>(ps + kWarps * ROWS * kPitch);   // row in the chunk, slot, mask
     int *count = reinterpret_cast<int *>(list + kList);
+    unsigned *odd = reinterpret_cast<unsigned *>(count + 1);               // two words: keys whose values are not all finite
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k0 = blockIdx.x * kKeys;
     const int g = blockIdx.y % c.Hkv, b = blockIdx.y / c.Hkv;
@@ -122,7 +125,7 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
             *reinterpret_cast<float4 *>(vs + j * D + d + e) = make_float4(vf[e], vf[e + 1], vf[e + 2], vf[e + 3]);
         }
     }
-    if (threadIdx.x == 0) *count = 0;
+    if (threadIdx.x == 0) *count = odd[0] = odd[1] = 0;
     __syncthreads();
 
     const int sub = lane / NG, grp = lane % NG;
@@ -230,6 +233,23 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
                         }
                     }
             }
+            for (unsigned long long keys = odd[0] | (unsigned long long)odd[1] << 32; keys; keys &= keys - 1) {
+                const int j = __ffsll((long long)keys) - 1;
+                const T *row = vbase + (long long)j * c.kv_st + sub * 4;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int e = e0 + r * NG + grp;
+                    if (e >= n || !(((j < 32 ? (unsigned)list[e].z : (unsigned)list[e].w) >> (j & 31)) & 1u)) continue;
+                    const float w = pw[(r * NG + grp) * kPitch + j];
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        const T *at = row + (x >> 1) * 4 * LPR + (x & 1) * 2;
+                        const float a = (float)at[0], z = (float)at[1];
+                        if (!isfinite(a)) acc[r][x].x = fmaf(w, a, acc[r][x].x);
+                        if (!isfinite(z)) acc[r][x].y = fmaf(w, z, acc[r][x].y);
+                    }
+                }
+            }
             __syncwarp();   // the next scores go to the same place
             if (own < n && sub < 4) ml[mine.y] = make_float2(m, l);
 #pragma unroll
@@ -249,7 +269,7 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     const int n_iv = c.top_k + (c.window > 0 ? 1 : 0);
     const int chunks = (y_end + 31) / 32;
     int ch = blockIdx.z + warp * n_ctas;   // the warp's next chunk
-    bool more;
+    bool more, staged = false;
     do {
         // as many chunks as the list has room for, without a barrier between them
         for (int it = 0; it < kList / kThreads && ch < chunks; ++it, ch += kWarps * n_ctas) {
@@ -284,6 +304,27 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
                     make_int4(hg * n_rows + rc, (int)((row_all * n_rows + rc) * p.slots + slot), (int)(unsigned)mask, (int)(unsigned)(mask >> 32));
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
+        if (!staged) {   // the values this thread brought in: zero times their sum is zero if all are finite
+            staged = true;
+            float4 *mine = reinterpret_cast<float4 *>(vs) + threadIdx.x;
+            constexpr int kMine = kKeys * D / 4 / kThreads;
+            float zero = 0.f;
+#pragma unroll
+            for (int u = 0; u < kMine; ++u) {
+                const float4 w = mine[u * kThreads];
+                zero += w.x * 0.f + w.y * 0.f + (w.z * 0.f + w.w * 0.f);
+            }
+            if (zero != 0.f)
+#pragma unroll 1
+                for (int u = 0; u < kMine; ++u) {
+                    const float4 w = mine[u * kThreads];
+                    if (isfinite(w.x) && isfinite(w.y) && isfinite(w.z) && isfinite(w.w)) continue;
+                    mine[u * kThreads] = make_float4(isfinite(w.x) ? w.x : 0.f, isfinite(w.y) ? w.y : 0.f, isfinite(w.z) ? w.z : 0.f,
+                                                     isfinite(w.w) ? w.w : 0.f);
+                    const int j = (threadIdx.x + u * kThreads) / (D / 4);
+                    atomicOr(odd + j / 32, 1u << (j % 32));
+                }
+        }
         more = __syncthreads_or(ch < chunks);
         attend(*count);
         if (more) {

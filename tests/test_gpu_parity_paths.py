@@ -140,6 +140,45 @@ def test_key_blocks(sla, handle, kw, dtype, D):
     assert float((out.double() - out2.double()).abs().max()) <= tol and bool(((lse - lse2)[fin].abs() <= tol).all())
 
 
+@pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128), ("bf16", 64)])
+def test_values_of_other_rows_do_not_leak(sla, dtype, D):
+    """Inf and NaN among the values reach the rows that selected their key and no others: not those that selected
+    another key of the block, nor those before it.  The kernels by key blocks and by rows agree on every entry."""
+    import math
+    import torch
+    L, top_k, ell = 700, 3, 33
+    g = torch.Generator().manual_seed(11)
+    q, k, v = (torch.randn(1, 2, L, D, generator=g).to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda() for _ in range(3))
+    for at, x in {(0, 333, 5): math.nan, (0, 699, 0): math.inf, (1, 64, D - 1): -math.inf, (1, 64, 2): math.nan, (1, 127, 7): math.inf,
+                  (1, 500, 7): -math.inf}.items():
+        v[(0, *at)] = x
+    params = sla.make_params(top_k, ell, head_dim=D)
+    h, small = sla.Handle(0, sla.sla_workspace_bytes(sla.make_layout(q, k), params, L, L)), sla.Handle(0, 1024)
+    anchor, _ = sla.sla_span_search(h, q, k, params)
+    n0 = sla.sla_kernel_launches(h)
+    out, lse = sla.sla_span_attention(h, q, k, v, anchor, params)
+    assert sla.sla_kernel_launches(h) - n0 == 2   # blocks of keys, merge
+    out2, lse2 = sla.sla_span_attention(small, q, k, v, anchor, params)
+    torch.cuda.synchronize()
+    assert sla.sla_poll_status(h) == sla.SLA_OK and sla.sla_poll_status(small) == sla.SLA_OK
+    h.close()
+    small.close()
+    # entries of the output that a selected key's value makes non-finite
+    i, a = torch.arange(L)[None, None, :, None], anchor.cpu().long()
+    j = torch.arange(L)
+    sel = torch.zeros(1, 2, L, L, dtype=torch.bool)
+    for x in range(top_k):
+        t = a[..., x:x + 1]
+        sel |= (t >= 0) & (j >= t - 2 * ell) & (j <= torch.minimum(t, i))
+    hit = (sel.float() @ (~torch.isfinite(v.cpu())).float()) > 0
+    assert torch.equal(~torch.isfinite(out.cpu()), hit) and hit.any() and not hit.all()
+    assert torch.equal(torch.isnan(out), torch.isnan(out2)) and torch.equal(torch.isposinf(out), torch.isposinf(out2))
+    fin = torch.isfinite(out)
+    # as in test_key_blocks: at most (D + L + 30) 2^-24 of sums of |scores| < 64, a bf16 rounding of values < 5
+    tol = 64 * (D + L + 30) * 2.0 ** -24 * 0.25 + (5 * 2.0 ** -8 if dtype == "bf16" else 0.0)
+    assert (out.double() - out2.double())[fin].abs().max().item() <= tol and (lse - lse2).abs().max().item() <= tol
+
+
 @pytest.mark.parametrize("seq_len,heads,kv_heads", [(1023, 32, 8), (1024, 32, 8), (1025, 32, 8), (4097, 8, 2), (8193, 16, 4)])
 def test_host_chunks(sla, seq_len, heads, kv_heads):
     """Prefill through host buffers in chunks that shrink towards the end: one chunk and the first lengths with two, the
