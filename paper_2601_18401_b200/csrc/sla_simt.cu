@@ -88,7 +88,7 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
     float *sc = smem + (size_t)warp * n_max;
     const T *qrow = q_s + id.b * c.q_sb + id.h * c.q_sh + id.r * c.q_st;
     const T *kbase = k + id.b * c.kv_sb + id.g * c.kv_sh;
-    const int sub = lane % LPR, rsel = lane / LPR, kv_st = (int)c.kv_st;
+    const int sub = lane % LPR, rsel = lane / LPR;
     const T *krow = kbase + sub * E;
     chain_wait();
     float qv[E];
@@ -104,7 +104,7 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
             if (s < n) {
                 const int t = (int)i + 1 - stride_offset(c, s);   // positions fit 31 bits
                 float kv[E];
-                Vec16<T>::load(krow + (long long)t * kv_st, kv);
+                Vec16<T>::load(krow + t * c.kv_st, kv);   // the one search kernel that takes token strides above 31 bits
 #pragma unroll
                 for (int e = 0; e < E; ++e) part[u] = fmaf(qv[e], kv[e], part[u]);
             }

@@ -179,6 +179,24 @@ def test_values_of_other_rows_do_not_leak(sla, dtype, D):
     assert (out.double() - out2.double())[fin].abs().max().item() <= tol and (lse - lse2).abs().max().item() <= tol
 
 
+def test_token_stride_above_31_bits(sla):
+    """Tokens 2^31 + 64 elements apart: search and attention read the same rows as on a dense tensor."""
+    import torch
+    D, L, st = 64, 9, (1 << 31) + 64
+    g = torch.Generator().manual_seed(3)
+    q, k = (torch.randn(1, 2, L, D, generator=g).bfloat16().cuda() for _ in range(2))
+    far = torch.empty((L - 1) * st + 2 * D, dtype=torch.bfloat16, device="cuda").as_strided((1, 2, L, D), (L * st, D, st, 1))
+    far.copy_(k)
+    params = sla.make_params(2, 2, head_dim=D)
+    h = sla.Handle(0, 1 << 20)
+    want, got = (sla.sla_span_search(h, q, x, params) for x in (k, far))
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    want, got = (sla.sla_span_attention(h, q, x, x, want[0], params) for x in (k, far))
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert sla.sla_poll_status(h) == sla.SLA_OK
+    h.close()
+
+
 @pytest.mark.parametrize("seq_len,heads,kv_heads", [(1023, 32, 8), (1024, 32, 8), (1025, 32, 8), (4097, 8, 2), (8193, 16, 4)])
 def test_host_chunks(sla, seq_len, heads, kv_heads):
     """Prefill through host buffers in chunks that shrink towards the end: one chunk and the first lengths with two, the
