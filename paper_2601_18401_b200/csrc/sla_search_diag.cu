@@ -26,6 +26,7 @@
 #include <math_constants.h>
 
 #include "sla_kernels.h"
+#include "sla_topk.cuh"
 
 namespace sla {
 
@@ -316,6 +317,8 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 // 320 instructions per warp and sixteen strides, four lists of K values per head.  4096 positions at 500001, 32/4 heads,
 // K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
 // 484 us here, about 440 us with the tiles fetched a step ahead.
+// The running lists take two scores at a time, neither of them NaN, and only those above -inf.  A warp that met an Inf or NaN
+// among its scores selects again, a pass over the strides per slot: a NaN is no candidate, -inf comes after all others.
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
@@ -363,6 +366,7 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     // two B tiles of eight strides, each fetched again as soon as its scores are taken
     Words8 ka[2], kb[2];
     int s0 = s_min;
+    float zero = 0.f;   // zero times the scores: NaN once one of them is not finite
     fetch(s0, true, ka);
     fetch(s0 + 8, true, kb);
     for (; s0 + 16 <= n; s0 += 16) {
@@ -370,26 +374,65 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
         float xa, xb;
         score(ka, xa, xb);
         fetch(s0 + 16, true, ka);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s, xa, s + 1, xb);
         score(kb, xa, xb);
         fetch(s0 + 24, true, kb);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s + 8, xa, s + 9, xb);
     }
     if (s0 < n) {
         const int s = s0 + 2 * q;
         float xa, xb;
         score(ka, xa, xb);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s, s < n ? xa : -CUDART_INF_F, s + 1, s + 1 < n ? xb : -CUDART_INF_F);
         score(kb, xa, xb);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s + 8, s + 8 < n ? xa : -CUDART_INF_F, s + 9, s + 9 < n ? xb : -CUDART_INF_F);
     }
 
+    const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;
+    if (__any_sync(0xffffffffu, zero != 0.f)) {
+        unsigned taken = 0xffffffffu;   // order key and stride of the score the last slot took
+        int at = -1;
+#pragma unroll 1
+        for (int j = 0; j < c.top_k; ++j) {
+            unsigned best = 0u;         // below every order key of a real score
+            int bs = INT_MAX;
+#pragma unroll 1
+            for (int s1 = s_min; s1 < n; s1 += 8) {
+                float x[2];
+                fetch(s1, true, ka);
+                score(ka, x[0], x[1]);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int s = s1 + 2 * q + u;
+                    const unsigned key = max(topk::order_key(x[u]), 1u);
+                    if (s < n && x[u] == x[u] && (key < taken || (key == taken && s > at)) && key > best) { best = key; bs = s; }
+                }
+            }
+#pragma unroll
+            for (int off = 1; off <= 2; off <<= 1) {
+                const unsigned ob = __shfl_xor_sync(0xffffffffu, best, off);
+                const int os = __shfl_xor_sync(0xffffffffu, bs, off);
+                if (ob > best || (ob == best && os < bs)) { best = ob; bs = os; }
+            }
+            if (q == 0) {
+                const bool on = bs != INT_MAX;
+                out_anchor[obase + j] = on ? i + 1 - stride_offset(c, bs) : -1;
+                out_score[obase + j] = on ? __uint_as_float((best & 0x80000000u) ? (best & 0x7fffffffu) : ~best) : -CUDART_INF_F;
+            }
+            taken = best;
+            at = bs;
+        }
+        return;
+    }
     float ex[K];
     int es[K];
     top.finish(ex, es);
     merge_pairs<K>(ex, es, 1);
     merge_pairs<K>(ex, es, 2);
-    const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;
 #pragma unroll
     for (int j = 0; j < K; ++j)
         if ((j & 3) == q && j < c.top_k) {

@@ -106,6 +106,31 @@ def test_search_of_wide_groups(sla, handle, heads, kv_heads, top_k):
         P.compare_search(anchor, score, ref, q_pos0=pos0, q_s=host["q_s"], k=host["k"], search_scale=1.0)
 
 
+@pytest.mark.parametrize("heads,top_k", [(8, 1), (8, 2), (16, 4), (16, 8), (8, 16)])
+def test_search_of_scores_that_are_not_finite(sla, handle, heads, top_k):
+    """Keys that hold Inf or NaN, groups of 8 and 16 query heads: a NaN score is no candidate and costs no other one its
+    place, -inf comes last, ties go to the nearer anchor."""
+    import torch
+    L = 430
+    g = torch.Generator().manual_seed(13)
+    q, k = ((torch.randn(1, h, L, 128, generator=g) * 64).round() / 64 for h in (heads, 1))
+    k[0, 0, 50::7] = float("nan")
+    k[0, 0, 100, 3], k[0, 0, 200, 9], k[0, 0, 2, 3], k[0, 0, 0, 3] = (float(x) for x in ("-inf", "inf", "inf", "-inf"))
+    anchor, score = sla.sla_span_search(handle, q.bfloat16().cuda(), k.bfloat16().cuda(), sla.make_params(top_k, 8, head_dim=128))
+    torch.cuda.synchronize()
+    anchor, score = anchor.cpu(), score.cpu()
+    q, k = q.bfloat16().double(), k.bfloat16().double()
+    for i in range(L):
+        t = torch.tensor([i + 1 - s * s for s in range(1, i + 2) if s * s <= i + 1])
+        x = torch.einsum("hd,td->ht", q[0, :, i], k[0, 0, t])   # multiples of 2^-12 below 2^9: exact in any order
+        for h in range(heads):
+            keep = ~torch.isnan(x[h])
+            order = torch.sort(x[h][keep], descending=True, stable=True).indices[:top_k]
+            n = len(order)
+            assert torch.equal(anchor[0, h, i, :n].long(), t[keep][order]) and torch.equal(score[0, h, i, :n], x[h][keep][order].float()), (h, i)
+            assert (anchor[0, h, i, n:] == -1).all() and torch.isneginf(score[0, h, i, n:]).all()
+
+
 @pytest.mark.parametrize("kw", [
     dict(seq_len=1, top_k=6, span_len=300), dict(seq_len=63, top_k=1, span_len=600), dict(seq_len=64, top_k=2, span_len=600),
     dict(seq_len=65, top_k=64, span_len=2),                                            # every anchor, spans of five keys
