@@ -692,8 +692,10 @@ sla_status_t sla_prefill_host(sla_handle_t h, const void *q_s_host, const void *
     const size_t qb = (size_t)l->batch * l->n_q_heads * L * l->head_dim * es;
     const size_t kb = (size_t)l->batch * l->n_kv_heads * L * l->head_dim * es;
     const size_t rows = (size_t)l->batch * l->n_q_heads * L;
-    // staging sits at the END of the workspace so that the scratch of the two steps keeps its place
-    char *base = h->ws + h->ws_bytes - stage;
+    // staging sits at the END of the workspace so that the scratch of the two steps keeps its place, on a 256-byte boundary
+    // whatever the handle's size (the scratch has the room: sla_workspace_bytes holds 4096 bytes of slack)
+    const size_t stage_at = (h->ws_bytes - stage) & ~(size_t)255;
+    char *base = h->ws + stage_at;
     auto take = [&base](size_t n) { char *p0 = base; base += (n + 255) & ~(size_t)255; return p0; };
     char *d_qs = take(qb), *d_q = take(qb), *d_out = take(qb), *d_k = take(kb), *d_v = take(kb);
     float *d_lse = (float *)take(rows * 4);
@@ -753,7 +755,7 @@ sla_status_t sla_prefill_host(sla_handle_t h, const void *q_s_host, const void *
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "sla_prefill_host (copy in)");
     const size_t avail_before = h->scratch_avail;
-    h->scratch_avail = h->ws_bytes - kHeaderBytes - stage;   // the staging buffers are not scratch
+    h->scratch_avail = stage_at - kHeaderBytes;   // the staging buffers are not scratch
     sla_status_t s = SLA_OK;
     const size_t k4 = (size_t)p->top_k * 4;
     for (int c = 0; c < n_chunks && s == SLA_OK; ++c) {

@@ -247,6 +247,30 @@ def test_host_chunks(sla, seq_len, heads, kv_heads):
     assert torch.equal(torch.isfinite(hl), fin) and (hl[fin] - lse.cpu()[fin]).abs().max().item() <= 2 * P.LSE_TOL["bf16"]
 
 
+@pytest.mark.parametrize("heads", [1, 2, 4])
+@pytest.mark.parametrize("spare", [4, 1 << 20, (1 << 20) + 12])
+def test_host_staging_in_a_larger_workspace(sla, heads, spare):
+    """A handle with more room than asked for and an odd number of rows: the staging buffers start on an aligned address
+    all the same, and the kernels are those of the exact size (groups of four: the fused selection, launched once)."""
+    import torch
+    from paper_2601_18401_b200 import synth
+    L = 301
+    w = workload(seq_len=L, n_q_heads=heads, n_kv_heads=1, span_len=8, top_k=3)
+    x = synth.make_prefill(w, device="cuda:0")
+    host = {n: t.cpu().pin_memory() for n, t in x.items()}
+    params = sla.make_params(w.top_k, w.span_len, head_dim=128)
+    layout = sla.make_layout(x["q"], x["k"])
+    need = sla.sla_workspace_bytes(layout, params, L, L) + sla.sla_host_staging_bytes(layout, params, L)
+    results, launches = [], []
+    for room in (need, need + spare):
+        h = sla.Handle(0, room)
+        results.append([t.clone() for t in sla.sla_prefill_host(h, host["q_s"], host["q"], host["k"], host["v"], params)])
+        assert sla.sla_poll_status(h) == sla.SLA_OK
+        launches.append(sla.sla_kernel_launches(h))
+        h.close()
+    assert launches[0] == launches[1] and all(torch.equal(a, b) for a, b in zip(*results))
+
+
 @pytest.mark.parametrize("top_k", [1, 2, 3, 4, 5, 8, 9])
 @pytest.mark.parametrize("window", [0, 40])
 def test_gated_merge_of_each_width(sla, handle, top_k, window):
