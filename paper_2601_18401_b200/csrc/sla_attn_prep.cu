@@ -367,20 +367,29 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scan(PrepArgs a) {
 
 // One warp per tile as cut by prep_scatter (256 consecutive records).  Where two neighbouring records of the
 // tile end further apart than a span is long the tile is split there: walking the gap would cost more than walking
-// two spans.  (So does a stretch of kMaxStretch blocks, which keeps the block numbers of a tile within 16 bits.)
+// two spans.  Where few rows look into a long context a tile's records may lie far apart without such a gap, and one CTA
+// would walk them all from end to end: in a list of fewer than kSplitTiles tiles per CTA a tile is also split into
+// stretches of end blocks, a power of two between one and a half and three times a span's length (each part walks a span
+// more; parts of less than 2^kMinStretch blocks would not hide the gather of their Q rows).  In other lists stretches of
+// 2^kMaxStretch blocks keep the block numbers of a tile within 16 bits.
+// Search and attention, without and with that split: 182 rows of 32/8 heads at 123447, one span of 703 keys and a window
+// of 1088 724 and 286 us; 69 rows of 16/8 heads at 195044, four spans of 1765 keys 881 and 368 us; 417 rows of 8/2 heads at 246543,
+// 17 spans of 373 keys 304 and 290 us.
 // The extra tiles are appended to the table.  For every tile: the end block of its last piece (second word), the
 // number of key blocks from the one its furthest-reaching piece starts in up to that end block (bits 9.. of the last
 // word), and the part of that walk each stream of 128 pieces reaches (`ranges`).
-constexpr int kMaxStretch = 16384;
+constexpr int kSplitTiles = 3;
+constexpr int kMinStretch = 4, kMaxStretch = 14;
 __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
     __shared__ int s_eb[8][kRows], s_lo[8][kRows];
+    __shared__ unsigned s_cut[8][kRows / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = blockIdx.x * 8 + warp;
     chain_wait();
     chain_release();
     if (t >= a.n_tiles[1]) return;
     const int4 ti = a.tiles[t];
-    const int cnt = ti.w;
+    const int cnt = ti.w, shift = a.n_tiles[1] < kSplitTiles * a.ctas ? max(kMinStretch, 31 - __clz(3 * a.nb_single)) : kMaxStretch;
     int *eb = s_eb[warp], *lo = s_lo[warp];
     for (int x = lane; x < cnt; x += 32) {
         const int4 rec = a.recs[ti.z + x];
@@ -388,15 +397,33 @@ __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
         lo[x] = rec.z;
     }
     __syncwarp();
-    int seg0 = 0, n_seg = 0;
-    while (seg0 < cnt) {
-        // first record after seg0 that lies beyond a gap (records are ordered by end block)
-        int seg1 = cnt;
-        for (int x0 = seg0 + 1; x0 < cnt && seg1 == cnt; x0 += 32) {
-            const int x = x0 + lane;
-            const bool cut = x < cnt && (eb[x] - eb[x - 1] > a.nb_single || eb[x] - eb[seg0] > kMaxStretch);
+    // the records a part starts at: beyond a gap (records are ordered by end block), or in another stretch than the one
+    // before it; the parts but the first take their places in the table together
+    int n_extra = 0, extra = 0;
+    if (eb[cnt - 1] - eb[0] > a.nb_single) {
+#pragma unroll 1
+        for (int w = 0; w < kRows / 32; ++w) {
+            const int x = 32 * w + lane;
+            const bool cut = x > 0 && x < cnt && (eb[x] - eb[x - 1] > a.nb_single || (eb[x] - eb[0]) >> shift != (eb[x - 1] - eb[0]) >> shift);
             const unsigned m = __ballot_sync(0xffffffffu, cut);
-            if (m) seg1 = x0 + __ffs(m) - 1;
+            if (lane == 0) s_cut[warp][w] = m;
+            n_extra += __popc(m);
+        }
+        __syncwarp();
+        if (n_extra > 0) {
+            if (lane == 0) extra = atomicAdd(a.n_tiles, n_extra);
+            extra = __shfl_sync(0xffffffffu, extra, 0);
+        }
+    }
+    int seg0 = 0, idx = t;
+    while (seg0 < cnt) {
+        int seg1 = cnt;
+        for (int w = (seg0 + 1) / 32; n_extra > 0 && w < kRows / 32; ++w) {
+            const unsigned m = s_cut[warp][w] & (w == (seg0 + 1) / 32 ? ~0u << ((seg0 + 1) % 32) : ~0u);
+            if (m) {
+                seg1 = 32 * w + __ffs(m) - 1;
+                break;
+            }
         }
         // the two streams of 128 pieces: what each reaches, and the tile's walk that covers both
         const int mid = min(seg0 + kRows / 2, seg1);
@@ -408,11 +435,6 @@ __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
         lo_a = __reduce_min_sync(0xffffffffu, lo_a);
         lo_b = __reduce_min_sync(0xffffffffu, lo_b);
         const int eb_last = eb[seg1 - 1], sb = min(lo_a, lo_b) / kBK;
-        int idx = t;
-        if (n_seg > 0) {
-            if (lane == 0) idx = atomicAdd(a.n_tiles, 1);
-            idx = __shfl_sync(0xffffffffu, idx, 0);
-        }
         if (lane == 0) {
             if (idx < a.max_tiles) {
                 a.tiles[idx] = make_int4(ti.x, eb_last, ti.z + seg0, (seg1 - seg0) | ((eb_last - sb + 1) << 9));
@@ -422,7 +444,7 @@ __global__ void __launch_bounds__(256) prep_tile_bounds(PrepArgs a) {
                 atomicOr(a.status, kStatusBadIndex);   // cannot happen: the table has room for one tile per bucket more
         }
         seg0 = seg1;
-        ++n_seg;
+        idx = extra++;
     }
 }
 

@@ -1130,8 +1130,8 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     p.slots = c.top_k + (c.window > 0 ? 1 : 0);
     const size_t slots = rows * p.slots;
     const size_t n_keys = (size_t)p.n_bg * p.NB * p.ncls;
-    // every (batch, kv head) list is cut every kRows records (one ragged tile each) and split again at
-    // gaps between end blocks (fewer than NB per list)
+    // every (batch, kv head) list is cut every kRows records (one ragged tile each) and split again
+    // between end blocks (fewer than NB per list)
     p.max_tiles = (long long)(slots / kRows) + (long long)p.n_bg * (p.NB + 1) + 1;
     if (p.max_tiles < kMinTiles) p.max_tiles = kMinTiles;   // every CTA reads its first entry before it knows the count
     size_t off = 0;
@@ -1205,6 +1205,7 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         pa.key_cursor = (int *)(ws + plan.off_key_cursor);
         pa.totals = counters + 16;
         pa.n_tiles = counters;
+        pa.ctas = sm_count;
         pa.tiles = (int4 *)(ws + plan.off_tiles);
         pa.ranges = (int2 *)(ws + plan.off_ranges);
         pa.max_tiles = (int)plan.max_tiles;

@@ -14,7 +14,8 @@ constexpr int kRows = 256;  // pieces per tile
 //   recs   int4 {row, slot of the row's partial results, lo, hi}: every piece of every row, ordered by
 //          (batch*Hkv + kv head, 64-key block of hi, class of blocks covered)
 //   tiles  int4 {batch*Hkv + kv head, end block of the last record, first record, records | key blocks to walk << 9}:
-//          256 consecutive records, split where neighbouring records end more than a few key blocks apart
+//          256 consecutive records, split where neighbouring records end further apart than a span is long and, in
+//          short lists, after two spans' length of end blocks
 //   n_tiles, n_pieces[row], and the per-piece partial results
 struct PrepArgs {
     const int32_t *anchor;   // [B,Hq,Lq,top_k]
@@ -34,7 +35,8 @@ struct PrepArgs {
     int *key_count;          // [B*Hkv][NB*ncls]: histogram, then exclusive offsets
     int *key_cursor;         // same shape
     int *totals;             // [B*Hkv][2]: records and tiles of each (batch, kv head)
-    int *n_tiles;            // total number of tiles
+    int *n_tiles;            // total number of tiles; the number before they are split
+    int ctas;                // CTAs the tiles are dealt to
     int4 *tiles;
     int2 *ranges;            // [max_tiles] blocks of the walk the tile's first and second 128 pieces reach: first | end << 16
     int max_tiles;

@@ -86,6 +86,17 @@ def test_end_blocks_far_apart(sla, handle):
     P.compare_attention(out, lse, ref, "bf16")
 
 
+@pytest.mark.parametrize("rows,top_k,span_len", [(1, 1, 0), (40, 2, 0), (40, 1, 300), (257, 2, 0), (33, 3, 5)])
+def test_few_rows_far_into_a_context(sla, handle, rows, top_k, span_len):
+    """Pieces that lie far apart without a gap longer than a span: a short list is cut into stretches of end blocks, and no
+    part walks much more than its stretch and a span."""
+    w = workload(n_q_heads=4, n_kv_heads=1, seq_len=60000, top_k=top_k, span_len=span_len)
+    run_prefill(sla, handle, w, q_pos0=60000 - rows, Lq=rows)
+    span = 2 * (span_len or 245) // 64 + 2
+    stats = sla.sla_attention_tile_stats(handle)
+    assert 0 < stats["tile_blocks"] <= (max(16, 3 * span) + span) * stats["tiles"]
+
+
 @pytest.mark.parametrize("heads,kv_heads,top_k", [(8, 1, 1), (16, 2, 4), (16, 1, 8), (16, 1, 16), (8, 1, 13)])
 def test_search_of_wide_groups(sla, handle, heads, kv_heads, top_k):
     """Groups of 8 and 16 query heads per KV head, four lanes a head: 1 to 64 strides a row, so that lists of a
