@@ -494,7 +494,7 @@ sla_status_t span_attention_impl(sla_handle_t h, const void *q, const void *k, c
             return SLA_OK;
         }
     }
-    if (sla::attn_blocks_supported(c)) {
+    if (sla::attn_blocks_supported(c, l->dtype)) {
         const long long rows = sla::attn_blocks_rows(c, h->scratch_avail, h->canaries ? sla::Canaries::kBytes : 0);
         if (rows > 0) {   // a workspace without the room leaves the row kernel, which needs none
             cudaError_t e = sla::launch_attn_blocks(q, k, v, c, l->dtype, anchor, rows, out, lse,

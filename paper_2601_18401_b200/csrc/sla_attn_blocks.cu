@@ -494,20 +494,38 @@ long long target_rows(const Call &c, size_t gap) {
 
 }  // namespace
 
-// The row kernel stays where it is the faster one:
-//   - rows with few keys, whose walk is short (search and attention of 1000 positions, one head, top_k 4, spans of up to 65
-//     keys: 37 us by rows, 29 us by blocks; 400 positions, 41 keys: 24.6 and 26.6 us, the launch of the merge);
-//   - blocks that few of the rows select, so that the scan of the anchors is most of the work, if there are rows enough to
-//     fill the chip (4000 x 2 rows at 200000, four spans of 896 keys: 3105 us by rows, 3311 by blocks; 500 x 2 rows there,
-//     which are one wave of long walks by rows: 1748 and 558 us; 3000 rows at 16384: 160 and 125 us).
-bool attn_blocks_supported(const Call &c) {
+// Which of the two kernels, from what each of them does (microseconds; the factors are fitted to 898 calls of both kernels
+// over rows 1..8000, positions up to 400000, 1..64 spans of 2..3700 keys, and are off by 15 % in the median):
+//   by rows    a warp's walk over its row, one step per span and per two loads of a warp (a row or more of keys each); the
+//              pieces it sorts; the products of selected keys
+//   by blocks  per chunk of rows a launch of two kernels and 64 staged keys and values per CTA, whether any row selects
+//              them or not; the anchors that every CTA scans; the products of whole blocks of selected keys; the slots a
+//              row's merge looks through
+// The blocks have to be a fifth better, which keeps calls with the row kernel where the two estimates lie close.  Over 500
+// other calls that is 2 % above the better kernel in the mean, and 1 call more than 5 % slower than by rows (a rule by the
+// number of rows and slots before it: 105 calls, up to 50 times).  The attention alone by rows and by blocks: 500 x 2 rows at
+// 200000, 128 dims, four spans of 895 keys 1707 and 580 us; 16 x 8 rows at 1000000, four spans of 65 keys 55 and 1110 us;
+// 1 x 8 rows at 300000, 64 dims, the same spans 32 and 180 us; 256 x 4 rows at 60000, two spans of 129 keys 28 and 147 us.
+static bool blocks_are_faster(const Call &c, int dtype, const BlockPlan &p) {
+    const long long i_last = c.q_pos0 + c.Lq - 1, len = (long long)(c.back + c.fwd) * base_len(c, i_last) + 1;
+    const double rows = (double)c.B * c.Hq * c.Lq, blocks = (double)(i_last / kKeys + 1), bg = (double)c.B * c.Hkv;
+    const double strides = n_strides(c, i_last), spans = c.top_k < strides ? c.top_k : strides;
+    const double wanted = (double)c.top_k * len + c.window, keys = wanted < i_last + 1 ? wanted : i_last + 1;
+    const double per_load = 32.0 / (c.D * (dtype == SLA_F32 ? 4 : 2) / 16);   // keys a load of a warp covers
+    const double by_rows = 9 + 0.30 * (spans + keys / (2 * per_load)) + 0.26e-4 * rows * c.top_k + 26e-8 * rows * keys * c.D;
+    const double near = spans * ((len - 1) / (double)kKeys + 1) + (c.window > 0 ? c.window / (double)kKeys + 1 : 0);
+    const double touched = near < blocks ? near : blocks, chunks = (double)((c.Lq + p.Lc - 1) / p.Lc);
+    const double by_blocks = chunks * (16 + 13e-5 * blocks * bg * c.D) +
+                             7.5e-6 * blocks * bg * c.Lq * c.G * (c.top_k + (c.window > 0 ? 1 : 0)) +
+                             5.3e-6 * rows * touched * c.D + 1.5e-3 * p.slots * c.top_k;
+    return by_blocks < 0.8 * by_rows;
+}
+
+bool attn_blocks_supported(const Call &c, int dtype) {
     if (c.mode != SLA_UNION || (c.D != 64 && c.D != 128) || (long long)c.B * c.Hkv > 65535) return false;
     BlockPlan p;
     const long long rows = target_rows(c, 0);
-    if (rows < 1 || !plan(c, rows, 0, p)) return false;
-    const long long i_last = c.q_pos0 + c.Lq - 1, len = (long long)(c.back + c.fwd) * base_len(c, i_last) + 1;
-    if (c.top_k * len + c.window < 192) return false;
-    return 40LL * p.slots >= i_last / kKeys || (long long)c.B * c.Hq * c.Lq < 4096;
+    return rows >= 1 && plan(c, rows, 0, p) && blocks_are_faster(c, dtype, p);
 }
 
 size_t attn_blocks_bytes(const Call &c, size_t gap) {

@@ -13,7 +13,7 @@ cudaError_t launch_attn_simt(const void *q, const void *k, const void *v, const 
                              cudaStream_t st);
 
 // ---- span-attention of the generic layouts by blocks of keys, union mode (sla_attn_blocks.cu) -----
-bool attn_blocks_supported(const Call &c);
+bool attn_blocks_supported(const Call &c, int dtype);   // the kernel applies and is the faster one
 size_t attn_blocks_bytes(const Call &c, size_t gap);
 long long attn_blocks_rows(const Call &c, size_t avail, size_t gap);
 cudaError_t launch_attn_blocks(const void *q, const void *k, const void *v, const Call &c, int dtype, const int32_t *anchor,

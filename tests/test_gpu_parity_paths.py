@@ -142,38 +142,75 @@ def test_search_of_scores_that_are_not_finite(sla, handle, heads, top_k):
             assert (anchor[0, h, i, n:] == -1).all() and torch.isneginf(score[0, h, i, n:]).all()
 
 
-@pytest.mark.parametrize("kw", [
-    dict(seq_len=1, top_k=6, span_len=300), dict(seq_len=63, top_k=1, span_len=600), dict(seq_len=64, top_k=2, span_len=600),
-    dict(seq_len=65, top_k=64, span_len=2),                                            # every anchor, spans of five keys
-    dict(batch=2, n_q_heads=6, n_kv_heads=2, seq_len=1543, top_k=9, span_len=0),       # lists that fill up several times
-    dict(seq_len=2300, top_k=3, span_len=33, window=200), dict(seq_len=900, top_k=1, span_len=31),   # 199 keys, 64 keys
-    dict(n_q_heads=4, n_kv_heads=4, seq_len=1200, top_k=8, span_len=100),
+@pytest.mark.parametrize("by_blocks,kw", [
+    # few keys a row, few rows (at the start, or far into a context), or blocks that few rows select
+    (False, dict(seq_len=1, top_k=6, span_len=300)), (False, dict(seq_len=65, top_k=64, span_len=2)),
+    (False, dict(seq_len=900, top_k=1, span_len=31)), (False, dict(seq_len=60020, q_pos0=60000, span_len=16)),
+    (False, dict(seq_len=9000, q_pos0=8744, top_k=16, span_len=4)),
+    # a last block of 63, 64 keys and one key
+    (True, dict(seq_len=1599, top_k=8, span_len=40)), (True, dict(seq_len=1600, top_k=8, span_len=40)),
+    (True, dict(seq_len=1601, top_k=8, span_len=40)),
+    (True, dict(batch=2, n_q_heads=6, n_kv_heads=2, seq_len=1543, top_k=9, span_len=0)),   # lists that fill up several times
+    (True, dict(seq_len=2300, top_k=6, span_len=33, window=200)), (True, dict(seq_len=3000, q_pos0=2100, top_k=8, span_len=60, window=129)),
+    (True, dict(n_q_heads=4, n_kv_heads=4, seq_len=1200, top_k=8, span_len=100)),
+    (True, dict(seq_len=1000, span_len=600)), (True, dict(seq_len=700, top_k=64, span_len=40)),   # spans cut off at 0; 64 of them
+    (True, dict(seq_len=20000, q_pos0=19301, span_len=0)),
 ])
 @pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128), ("bf16", 64)])
-def test_key_blocks(sla, handle, kw, dtype, D):
-    """The generic span-attention by key blocks: no anchors at all, one block, a block and a key, spans that end on either
-    side of a block edge, a window across spans; and with a workspace that has no room for it, the kernel by rows."""
+def test_key_blocks(sla, handle, by_blocks, kw, dtype, D):
+    """The generic span-attention on both sides of the rule that chooses between the kernels by rows and by blocks of keys,
+    against the oracle; and the two kernels against each other (a workspace without room leaves the one by rows), rows
+    without any anchor among them."""
     import torch
+    from test_gpu_parity_modes import run_modes
     from paper_2601_18401_b200 import synth
-    window = kw.get("window", 0)
-    w = workload(**dict(dict(n_q_heads=2, n_kv_heads=1), **{n: x for n, x in kw.items() if n != "window"}, dtype=dtype, head_dim=D))
-    if not window:
-        run_prefill(sla, handle, w)
+    window, q_pos0 = kw.get("window", 0), kw.get("q_pos0", 0)
+    w = workload(**dict(dict(n_q_heads=2, n_kv_heads=1), **{n: x for n, x in kw.items() if n not in ("window", "q_pos0")}, dtype=dtype, head_dim=D))
+    if window:
+        run_modes(sla, handle, w, window, q_pos0=q_pos0)
+    else:
+        run_prefill(sla, handle, w, q_pos0=q_pos0)
     x = synth.make_prefill(w, device="cuda:0")
+    q_s, q = x["q_s"][:, :, q_pos0:], x["q"][:, :, q_pos0:]
     params = sla.make_params(w.top_k, w.span_len, head_dim=D, window=window)
-    anchor, _ = sla.sla_span_search(handle, x["q_s"], x["k"], params)
-    out, lse = sla.sla_span_attention(handle, x["q"], x["k"], x["v"], anchor, params)
+    anchor, _ = sla.sla_span_search(handle, q_s, x["k"], params, q_pos0=q_pos0)
+    anchor[:, :, 1::5] = -1
     small = sla.Handle(0, 1024)
-    out2, lse2 = sla.sla_span_attention(small, x["q"], x["k"], x["v"], anchor, params)
+    n0, m0 = sla.sla_kernel_launches(handle), sla.sla_kernel_launches(small)
+    out, lse = sla.sla_span_attention(handle, q, x["k"], x["v"], anchor, params, q_pos0=q_pos0)
+    out2, lse2 = sla.sla_span_attention(small, q, x["k"], x["v"], anchor, params, q_pos0=q_pos0)
     torch.cuda.synchronize()
+    # blocks of keys and their merge for every chunk of rows, or the kernel by rows
+    assert (sla.sla_kernel_launches(handle) - n0 > 1) == by_blocks and sla.sla_kernel_launches(small) - m0 == 1
     assert sla.sla_poll_status(handle) == sla.SLA_OK and sla.sla_poll_status(small) == sla.SLA_OK
     small.close()
     # both sum the same products and exponentials in fp32 in other orders: at most (D + n_keys + 30) 2^-24 of a score or a sum
     # of |scores| < 64, and for bf16 results a rounding of 2^-8 of values < 5 on either side
-    tol = 64 * (D + w.seq_len + 30) * 2.0 ** -24 * 0.25 + (5 * 2.0 ** -8 if dtype == "bf16" else 0.0)
+    n_keys = min(w.seq_len, w.top_k * (2 * (w.span_len or 142) + 1) + window)
+    tol = 64 * (D + n_keys + 30) * 2.0 ** -24 * 0.25 + (5 * 2.0 ** -8 if dtype == "bf16" else 0.0)
     fin = torch.isfinite(lse2)
     assert bool((torch.isfinite(lse) == fin).all())
     assert float((out.double() - out2.double()).abs().max()) <= tol and bool(((lse - lse2)[fin].abs() <= tol).all())
+
+
+@pytest.mark.parametrize("rows,pos0,kv_heads,D,top_k,span_len,dtype,most", [
+    (16, 300000, 8, 128, 4, 32, "f32", 1), (1, 300000, 8, 64, 4, 32, "f32", 1), (256, 60000, 4, 64, 2, 64, "bf16", 1),
+    (500, 100000, 2, 128, 4, 447, "f32", 2), (100, 100000, 2, 128, 4, 447, "f32", 2),
+])
+def test_generic_rows_far_into_a_context(sla, rows, pos0, kv_heads, D, top_k, span_len, dtype, most):
+    """A few rows with short spans do not go through all blocks of a long context (they took up to 25 times as long);
+    long spans do."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(9)
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    q, k, v = (torch.empty(1, kv_heads, n, D, dtype=T, device="cuda").normal_(generator=g) for n in (rows, pos0 + rows, pos0 + rows))
+    params = sla.make_params(top_k, span_len, head_dim=D)
+    h = sla.Handle(0, sla.sla_workspace_bytes(sla.make_layout(q, k), params, rows, pos0 + rows))
+    anchor, _ = sla.sla_span_search(h, q, k, params, q_pos0=pos0)
+    n0 = sla.sla_kernel_launches(h)
+    out, _ = sla.sla_span_attention(h, q, k, v, anchor, params, q_pos0=pos0)
+    assert sla.sla_kernel_launches(h) - n0 == most and sla.sla_poll_status(h) == sla.SLA_OK and bool(torch.isfinite(out).all())
+    h.close()
 
 
 @pytest.mark.parametrize("dtype,D", [("f32", 64), ("f32", 128), ("bf16", 64)])
@@ -182,10 +219,10 @@ def test_values_of_other_rows_do_not_leak(sla, dtype, D):
     another key of the block, nor those before it.  The kernels by key blocks and by rows agree on every entry."""
     import math
     import torch
-    L, top_k, ell = 700, 3, 33
+    L, top_k, ell = 1100, 8, 33
     g = torch.Generator().manual_seed(11)
     q, k, v = (torch.randn(1, 2, L, D, generator=g).to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda() for _ in range(3))
-    for at, x in {(0, 333, 5): math.nan, (0, 699, 0): math.inf, (1, 64, D - 1): -math.inf, (1, 64, 2): math.nan, (1, 127, 7): math.inf,
+    for at, x in {(0, 333, 5): math.nan, (0, 1099, 0): math.inf, (1, 64, D - 1): -math.inf, (1, 64, 2): math.nan, (1, 127, 7): math.inf,
                   (1, 500, 7): -math.inf}.items():
         v[(0, *at)] = x
     params = sla.make_params(top_k, ell, head_dim=D)
