@@ -61,6 +61,34 @@ def test_query_strides_without_a_common_row_pitch(sla, handle):
         assert torch.equal(out2.contiguous(), out) and torch.equal(lse2, lse)
 
 
+@pytest.mark.parametrize("batch,heads,kv_heads,L", [(1, 4, 1, 1), (1, 8, 2, 17), (2, 6, 3, 1500), (1, 32, 8, 2600)])
+def test_query_strides_in_chunks(sla, batch, heads, kv_heads, L):
+    """Tokens of all heads side by side with eight elements of padding (no common row pitch): the rows of Q are brought
+    together by one kernel per chunk, in a workspace that takes the call at once and in one that takes 1024 rows."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(21)
+    D, st = 128, heads * 128 + 8
+    q = torch.empty(batch * L * st, dtype=torch.bfloat16, device="cuda").normal_(generator=g).as_strided((batch, heads, L, D), (L * st, D, st, 1))
+    k, v = (torch.empty(batch, kv_heads, L, D, dtype=torch.bfloat16, device="cuda").normal_(generator=g) for _ in range(2))
+    params = sla.make_params(3, 20, head_dim=D)
+    results, launches = [], []
+    dense = q.clone(memory_format=torch.contiguous_format)
+    for x, rows in ((dense, L), (q, L), (dense, min(L, 1024)), (q, min(L, 1024))):
+        h = sla.Handle(0, sla.sla_workspace_bytes(sla.make_layout(x, k), params, rows, L))
+        anchor, _ = sla.sla_span_search(h, x, k, params)
+        n0 = sla.sla_kernel_launches(h)
+        out, lse = sla.sla_span_attention(h, x, k, v, anchor, params)
+        launches.append(sla.sla_kernel_launches(h) - n0)
+        torch.cuda.synchronize()
+        assert sla.sla_poll_status(h) == sla.SLA_OK
+        results.append((out.contiguous(), lse))
+        h.close()
+    for (out, lse), (want, want_lse), n, n_dense in zip(results[1::2], results[::2], launches[1::2], launches[::2]):
+        assert torch.equal(out, want) and torch.equal(lse, want_lse)
+        assert n_dense % 7 == 0 and n == n_dense // 7 * 8
+    assert launches[0] == 7 and (launches[2] > 7) == (L > 1024)
+
+
 def test_end_blocks_far_apart(sla, handle):
     """Anchors in two narrow regions and in a few places between them: tiles are cut where neighbouring pieces of
     the work list end further apart than a span is long, and streams of one tile walk different key blocks."""
