@@ -96,7 +96,7 @@ struct TcParams {
     const bf16 *q;             // Q as rows at one pitch (in elements), numbered as in its tensor map
     long long q_pitch;
     int q_b, q_h, q_t;         // strides of Q in those rows
-    int Hq, G, Lc, slots;      // slots: partial results per row (top_k, + 1 with a local window)
+    int Hq, Lc, slots;         // slots: partial results per row (top_k, + 1 with a local window)
     int r0;                    // first query row of the chunk
     float scale2;              // softmax_scale * log2(e)
     int slot_t, slot_h, slot_b;  // positions of (token, head, batch) among tensor-map coordinates 1..3
@@ -1100,7 +1100,7 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     // joined piece there can be (all spans and the window in one), everything that touches is joined;
     // otherwise the classes are shared between single spans and joined pairs, and a piece stops growing
     // at twice a span (measured on the 262144-token configuration: pairs -4 %, triples +1 %).
-    // Pieces are joined only where the list is dense: joined pieces come in many lengths, and a tile of 128
+    // Pieces are joined only where the list is dense: joined pieces come in many lengths, and a stream of 128
     // pieces can only be filled with one of them when the pieces of one end block and class are about that many.
     // `density` is the most pieces an end block (of one batch and KV head) can have on average.  Joined against not
     // joined: density 67 (4096 rows at position 500000, 16 spans of 2049 keys) walks 204 k key blocks against 141 k,
@@ -1249,7 +1249,7 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
             tp.q_b = (int)(c.B > 1 ? c.q_sb / g : 0); tp.q_h = (int)(c.Hq > 1 ? c.q_sh / g : 0); tp.q_t = (int)(c.q_st / g);
             tp.r0 = (int)r0;
         }
-        tp.Hq = c.Hq; tp.G = c.G; tp.Lc = lc; tp.slots = plan.slots;
+        tp.Hq = c.Hq; tp.Lc = lc; tp.slots = plan.slots;
         tp.scale2 = c.softmax_scale * kLog2e;
         tp.slot_t = slot[0]; tp.slot_h = slot[1]; tp.slot_b = slot[2];
         tp.recs = pa.recs; tp.tiles = pa.tiles; tp.ranges = pa.ranges;

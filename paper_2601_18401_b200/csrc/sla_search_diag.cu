@@ -246,10 +246,10 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 
     const bf16 *kbase = k + b * c.kv_sb + g * c.kv_sh + 16 * q;
     const int kv_st = (int)c.kv_st;
-    auto fetch = [&](int s0, bool check, Words8 (&kb)[2]) {
+    auto fetch = [&](int s0, Words8 (&kb)[2]) {
         const int s = s0 + u_ld;
         int t = i_ld + 1 - stride_offset(c, s < c.n_off || !c.off ? s : 0);
-        if (check && s >= n_ld) t = i_ld;   // a valid row either way
+        if (s >= n_ld) t = i_ld;   // a valid row either way
         const bf16 *row = kbase + (long long)t * kv_st;
         kb[0] = ldg256(row);
         kb[1] = ldg256(row + 64);
@@ -272,13 +272,13 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     // 16384 positions, K = 8: 1.2 to 1.5 % off search and attention together against fetch and use in one step)
     Words8 ka[2], kb[2];
     int s0 = s_min;
-    fetch(s0, true, ka);
-    fetch(s0 + 2, true, kb);
+    fetch(s0, ka);
+    fetch(s0 + 2, kb);
     for (; s0 + 4 <= n_all; s0 += 4) {
         const float xa = score(ka);
-        fetch(s0 + 4, true, ka);
+        fetch(s0 + 4, ka);
         const float xb = score(kb);
-        fetch(s0 + 6, true, kb);
+        fetch(s0 + 6, kb);
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
     }
     for (; s0 < n_max; s0 += 4) {
@@ -287,8 +287,8 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
         if (s0 + 4 < n_max) {
-            fetch(s0 + 4, true, ka);
-            fetch(s0 + 6, true, kb);
+            fetch(s0 + 4, ka);
+            fetch(s0 + 6, kb);
         }
     }
 
@@ -343,10 +343,10 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     const int s_min = c.window > 0 ? window_strides(c) : 0;
     const bf16 *kbase = k + b * c.kv_sb + g * c.kv_sh + 16 * q;
     const int kv_st = (int)c.kv_st;
-    auto fetch = [&](int s0, bool check, Words8 (&kb)[2]) {   // column r8: the key of stride s0 + r8
+    auto fetch = [&](int s0, Words8 (&kb)[2]) {   // column r8: the key of stride s0 + r8
         const int s = s0 + r8;
         int t = i + 1 - stride_offset(c, s < c.n_off || !c.off ? s : 0);
-        if (check && s >= n) t = i;   // a valid row either way
+        if (s >= n) t = i;   // a valid row either way
         const bf16 *row = kbase + (long long)t * kv_st;
         kb[0] = ldg256(row);
         kb[1] = ldg256(row + 64);
@@ -367,17 +367,17 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     Words8 ka[2], kb[2];
     int s0 = s_min;
     float zero = 0.f;   // zero times the scores: NaN once one of them is not finite
-    fetch(s0, true, ka);
-    fetch(s0 + 8, true, kb);
+    fetch(s0, ka);
+    fetch(s0 + 8, kb);
     for (; s0 + 16 <= n; s0 += 16) {
         const int s = s0 + 2 * q;
         float xa, xb;
         score(ka, xa, xb);
-        fetch(s0 + 16, true, ka);
+        fetch(s0 + 16, ka);
         zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s, xa, s + 1, xb);
         score(kb, xa, xb);
-        fetch(s0 + 24, true, kb);
+        fetch(s0 + 24, kb);
         zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s + 8, xa, s + 9, xb);
     }
@@ -403,7 +403,7 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
 #pragma unroll 1
             for (int s1 = s_min; s1 < n; s1 += 8) {
                 float x[2];
-                fetch(s1, true, ka);
+                fetch(s1, ka);
                 score(ka, x[0], x[1]);
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
