@@ -110,9 +110,14 @@ __host__ __device__ inline long long base_len(const Call &c, long long i) {
 }
 
 // ---- launches in a chain: a kernel started with launch_chained may be scheduled while the kernel before it on the
-// stream still runs (from the point where all of its CTAs have called chain_release, or have ended).  It calls chain_wait
-// before it touches global memory -- by then the kernel before it, and with it all before that, is complete -- and releases
-// its own successor only after that.
+// stream still runs (from the point where all of its CTAs have called chain_release, or have ended).  After chain_wait the
+// kernel before it is complete, and with it all before that, since at least one CTA of every kernel of a chain waits
+// before it ends.  What a kernel touches before its chain_wait must be older than the kernel before it:
+//   - a kernel that releases after its own chain_wait lets its successor read, before that one waits, what was complete at
+//     that point (merge_blocks reads the anchors while attend_blocks, which waited for the search, still runs; it may also
+//     set bits of the status word, which no kernel reads);
+//   - a kernel that releases before its chain_wait (decode_score) gives its successor nothing: that one touches no global
+//     memory before its own chain_wait, which returns only when this kernel, its wait included, is complete.
 __device__ inline void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ inline void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>

@@ -4,17 +4,19 @@
 // kernel spreads each head's tokens evenly over many CTAs (split-K), streams whole rows with 16-byte
 // loads, keeps a running (max, denominator, numerator) per lane group and merges at the end.
 //
-//   decode_attn    clusters of up to 8 CTAs, grid (CTAs per attention unit, units): the whole step in one launch.  A
-//                  cluster scores the anchors of its head, a share per CTA, keeps the k best of every share and then of
-//                  all shares (distributed shared memory); every CTA builds the spans of its unit, clips the
-//                  overlaps and runs the online softmax over an even share of the tokens; the cluster's first CTA
-//                  merges the partial results through their log-sum-exp.
+//   decode_attn    grid (CTAs per attention unit, units).  Where the anchors of a head fit a cluster of up to 8 CTAs it is
+//                  the whole step in one launch: each CTA of the cluster scores a share of the anchors and writes the scores to
+//                  all of them (distributed shared memory); otherwise the scores come from decode_score, launched before
+//                  it (plan_decode).  Every CTA then selects the k best of its head itself, builds the spans of its
+//                  unit, clips the overlaps and runs the online softmax over an even share of the tokens; the
+//                  cluster's first CTA merges its partial results through their log-sum-exp, the last cluster of a unit
+//                  those of the clusters.
 //                  Union mode: one unit per head (its spans and the local window, clipped to disjoint pieces).
 //                  Per-span mode (Algorithm 1 literally): one unit per selected anchor, J_t = S_t united with
 //                  the window; the unit that finishes a head last applies the gate of Section "Combination" to
 //                  the units' outputs.
-//   decode_score   (sequence-sharded step) grid (anchor chunks, B*Hkv, head tiles): K anchor rows x G routing queries ->
-//                  scores; the CTA that finishes a (batch, KV head) last selects this rank's k best candidates.
+//   decode_score   grid (anchor chunks, B*Hkv, head tiles): K anchor rows x G routing queries -> scores.  In the
+//                  sequence-sharded step the CTA that finishes a (batch, KV head) last selects this rank's k best candidates.
 // "Last" is decided by an atomic counter per unit / per head in the handle's header region; the last CTA puts
 // the counter back to zero, so a step leaves them as it found them.
 #include <cooperative_groups.h>
@@ -61,8 +63,8 @@ decode_score(const T *__restrict__ q_s, const T *__restrict__ k, Call c, long lo
 
     // the attention kernel of this step may be scheduled now; it waits for this grid to finish before it reads scores.
     // This grid itself may have been launched beside the tail of the kernel before it.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_release();
+    chain_wait();
     float qv[GT][E];
 #pragma unroll
     for (int t = 0; t < GT; ++t) Vec16<T>::load(q_s + b * c.q_sb + (long long)(h0 + t) * c.q_sh + sub * E, qv[t]);
@@ -357,15 +359,13 @@ template <typename T> __device__ __forceinline__ void unpack16(const uint4 &v, f
 }
 
 // One attention unit per cluster row: `gridDim.x` CTAs in clusters of `cluster.num_blocks()` share a unit's tokens.
-//   1. (unsharded step, q_s given) the CTAs of a cluster score the anchors of the unit's head, a share each, and keep
-//      the k best of their share; after a cluster barrier every CTA picks the k best of all shares (read through
-//      distributed shared memory) and builds the unit's spans itself.  Sequence-sharded step: `spans` is the table
-//      decode_shard_select built.
+//   1. (unsharded step) the scores of the unit's head come from decode_score (`scores`), or the CTAs of a cluster score
+//      a share of the anchors each and write every score to all of them; every CTA then picks the k best and builds the
+//      unit's spans itself.  Sequence-sharded step: `spans` is the table decode_shard_select built.
 //   2. online softmax over an even share of the tokens;
 //   3. the cluster's first CTA merges the partial results of the others through distributed shared memory; when a
 //      unit has several clusters, the one that finishes last merges theirs (through `partial` and the counter `done`).
-// One launch instead of two with a hand-over of scores and partial results through global memory: see the figures at
-// plan_decode.
+// One launch or two: see the figures at plan_decode.
 template <typename T, int D>
 __global__ void __launch_bounds__(kAttnThreads, 2)
 decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restrict__ k, const T *__restrict__ v, Call c,
@@ -411,7 +411,7 @@ decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restr
 
     // launched beside the tail of the kernel before it on the stream (the score kernel, or whatever the caller runs),
     // whose results are read from here on
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    chain_wait();
     int cnt;
     if (!spans) {
         const long long i = c.Lkv - 1;
@@ -552,7 +552,7 @@ decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restr
     }
 
     // the next kernel may be scheduled when every CTA is here
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_release();
     // merge the lane groups of the warp, then the warps of the CTA
 #pragma unroll
     for (int off = LPR; off < 32; off <<= 1) {
@@ -768,18 +768,10 @@ cudaError_t decode_launch(const void *q_s, const void *q, const void *k, const v
         const int gt = c.G % 8 == 0 ? 8 : c.G % 4 == 0 ? 4 : c.G % 2 == 0 ? 2 : 1;
         const dim3 gs(n > 0 ? (n + rows_per_cta - 1) / rows_per_cta : 1, c.B * c.Hkv, c.G / gt);
         // scores only (no completion counter, no shared memory)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = gs;
-        cfg.blockDim = dim3(kScoreThreads);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
         cudaError_t e;
 #define SLA_LAUNCH_SCORE(GT) \
-    e = cudaLaunchKernelEx(&cfg, decode_score<T, D, GT>, qs, kk, c, n_ctx, n, s_min, scores, (int *)nullptr, out_anchor, out_score)
+    e = launch_chained(decode_score<T, D, GT>, gs, dim3(kScoreThreads), 0, st, qs, kk, c, n_ctx, n, s_min, scores, (int *)nullptr, \
+                       out_anchor, out_score)
         switch (gt) {
             case 8: SLA_LAUNCH_SCORE(8); break;
             case 4: SLA_LAUNCH_SCORE(4); break;
