@@ -44,9 +44,14 @@
  * run on the tensor-core kernels (span-attention) and the register-MMA kernel (span-search); every
  * other supported layout -- fp32, head_dim 64, a stride-0 K/V dimension, a single call over more than
  * about 2.6 million keys -- runs on generic fp32-accumulating kernels with the same results and far
- * lower throughput.  The choice depends on shapes and strides alone, never on the workspace size: a
- * workspace too small for the chosen kernel is SLA_ERR_WORKSPACE.  (One exception: the generic
- * span-attention in the union mode needs no workspace, but is faster with what sla_workspace_bytes asks for.)
+ * lower throughput.  That choice depends on shapes and strides alone, never on the workspace size: a
+ * workspace too small for the tensor-core kernels is SLA_ERR_WORKSPACE.  The generic span-attention in the
+ * union mode has two kernels, one that goes through blocks of keys and needs scratch memory, and one that
+ * goes by rows and needs none; a workspace of less than about half of what sla_workspace_bytes asks for
+ * leaves the one by rows, also where the other is faster.  Both sum in fp32, in different orders: the last
+ * bits of a result can depend on which one ran, hence on the workspace.  In the same way the workspace, and
+ * the rows of a call, decide which touching spans the tensor-core span-attention attends as one piece; every
+ * result stays within the rounding of its type.
  *
  * Errors: every call returns an sla_status_t; 0 is success, negative values are errors.  When
  * argument validation fails nothing is launched.  No exception or abort crosses this interface.
@@ -328,10 +333,12 @@ sla_status_t sla_decode_shard_merge(sla_handle_t handle, int32_t n_shards, const
 
 /* sla_span_search followed by sla_span_attention on HOST buffers (pinned memory gives the best
  * copy rate): copies q_s, q, k, v to the device, runs both steps, copies out, lse, anchors and
- * scores back, and waits for completion.  Sequences of 4096 tokens and more go through in up to
- * thirty-two chunks of query positions (chunked prefill: a chunk needs the keys up to its own end), with
+ * scores back, and waits for completion.  Sequences of about 1024 tokens and more (twice the smallest chunk:
+ * 512 tokens or 4 MB of copies) go through in up to thirty-two chunks of query positions, a quarter of the
+ * sequence first and half of what is left at the end (chunked prefill: a chunk needs the keys up to its own end), with
  * the copy-in of the next chunk, the kernels of this one and the copy-out of the previous one
- * overlapping on streams the handle owns; results do not depend on the chunking.  Union mode only.
+ * overlapping on streams the handle owns; the selection does not depend on the chunking, outputs only within
+ * the rounding of their type.  Union mode only.
  * All tensors are dense and contiguous
  * ([B,Hq,L,D] / [B,Hkv,L,D], q_pos0 = 0, Lq = Lkv = L); the layout's strides are ignored.  The
  * device staging buffers come out of the handle's workspace, which therefore has to be
