@@ -194,6 +194,28 @@ struct RunningTop {
     }
 };
 
+// The running lists take two scores at a time, neither of them NaN, and only those above -inf.  A warp that met an Inf or
+// NaN among its scores selects again, a pass over the strides per slot: the largest score after the one taken last (smaller
+// stride on ties); a NaN is no candidate, -inf comes after all others.
+struct NextBest {
+    unsigned taken = 0xffffffffu, key = 0u;   // order keys: of the score taken last; of the best after it (0: none)
+    int at = -1, s = INT_MAX;                 // their strides
+    __device__ __forceinline__ void offer(int sx, float x) {
+        const unsigned kx = max(topk::order_key(x), 1u);
+        if (x == x && (kx < taken || (kx == taken && sx > at)) && kx > key) { key = kx; s = sx; }
+    }
+    __device__ __forceinline__ void merge(int off) {
+        const unsigned ok = __shfl_xor_sync(0xffffffffu, key, off);
+        const int os = __shfl_xor_sync(0xffffffffu, s, off);
+        if (ok > key || (ok == key && os < s)) { key = ok; s = os; }
+    }
+    __device__ __forceinline__ bool found() const { return s != INT_MAX; }
+    __device__ __forceinline__ float score() const {
+        return found() ? __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key) : -CUDART_INF_F;
+    }
+    __device__ __forceinline__ void take() { taken = key; at = s; key = 0u; s = INT_MAX; }
+};
+
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
@@ -272,6 +294,7 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     // 16384 positions, K = 8: 1.2 to 1.5 % off search and attention together against fetch and use in one step)
     Words8 ka[2], kb[2];
     int s0 = s_min;
+    float zero = 0.f;   // zero times the scores: NaN once one of them is not finite
     fetch(s0, ka);
     fetch(s0 + 2, kb);
     for (; s0 + 4 <= n_all; s0 += 4) {
@@ -279,10 +302,12 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         fetch(s0 + 4, ka);
         const float xb = score(kb);
         fetch(s0 + 6, kb);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
     }
     for (; s0 < n_max; s0 += 4) {
         float xa = score(ka), xb = score(kb);
+        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         xa = s0 + u_own < n_own ? xa : -CUDART_INF_F;
         xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
@@ -292,6 +317,26 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         }
     }
 
+    const long long obase = ((((long long)b * c.Hq + g * kG + hh) * c.Lq) + r0 + jq) * c.top_k;
+    if (__any_sync(0xffffffffu, zero != 0.f)) {
+        NextBest next;
+#pragma unroll 1
+        for (int j = 0; j < c.top_k; ++j) {
+#pragma unroll 1
+            for (int s1 = s_min; s1 < n_max; s1 += 2) {
+                fetch(s1, ka);
+                const float x = score(ka);
+                if (s1 + u_own < n_own) next.offer(s1 + u_own, x);
+            }
+            next.merge(2);
+            if (row_own && u_own == 0) {
+                out_anchor[obase + j] = next.found() ? i_own + 1 - stride_offset(c, next.s) : -1;
+                out_score[obase + j] = next.score();
+            }
+            next.take();
+        }
+        return;
+    }
     // ---- the lane's K best, merged with those of the lane that holds the pair's other strides (q differs in bit 1);
     // either of the two writes every other slot
     float ex[K];
@@ -299,7 +344,6 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     top.finish(ex, es);
     merge_pairs<K>(ex, es, 2);
     if (!row_own) return;
-    const long long obase = ((((long long)b * c.Hq + g * kG + hh) * c.Lq) + r0 + jq) * c.top_k;
 #pragma unroll
     for (int j = 0; j < K; ++j)
         if ((j & 1) == u_own && j < c.top_k) {
@@ -317,8 +361,6 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 // 320 instructions per warp and sixteen strides, four lists of K values per head.  4096 positions at 500001, 32/4 heads,
 // K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
 // 484 us here, about 440 us with the tiles fetched a step ahead.
-// The running lists take two scores at a time, neither of them NaN, and only those above -inf.  A warp that met an Inf or NaN
-// among its scores selects again, a pass over the strides per slot: a NaN is no candidate, -inf comes after all others.
 template <int K>
 __global__ void __launch_bounds__(kWarps * 32, 2)
 search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
@@ -394,37 +436,25 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
 
     const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;
     if (__any_sync(0xffffffffu, zero != 0.f)) {
-        unsigned taken = 0xffffffffu;   // order key and stride of the score the last slot took
-        int at = -1;
+        NextBest next;
 #pragma unroll 1
         for (int j = 0; j < c.top_k; ++j) {
-            unsigned best = 0u;         // below every order key of a real score
-            int bs = INT_MAX;
 #pragma unroll 1
             for (int s1 = s_min; s1 < n; s1 += 8) {
-                float x[2];
+                const int s = s1 + 2 * q;
+                float xa, xb;
                 fetch(s1, ka);
-                score(ka, x[0], x[1]);
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int s = s1 + 2 * q + u;
-                    const unsigned key = max(topk::order_key(x[u]), 1u);
-                    if (s < n && x[u] == x[u] && (key < taken || (key == taken && s > at)) && key > best) { best = key; bs = s; }
-                }
+                score(ka, xa, xb);
+                if (s < n) next.offer(s, xa);
+                if (s + 1 < n) next.offer(s + 1, xb);
             }
-#pragma unroll
-            for (int off = 1; off <= 2; off <<= 1) {
-                const unsigned ob = __shfl_xor_sync(0xffffffffu, best, off);
-                const int os = __shfl_xor_sync(0xffffffffu, bs, off);
-                if (ob > best || (ob == best && os < bs)) { best = ob; bs = os; }
-            }
+            next.merge(1);
+            next.merge(2);
             if (q == 0) {
-                const bool on = bs != INT_MAX;
-                out_anchor[obase + j] = on ? i + 1 - stride_offset(c, bs) : -1;
-                out_score[obase + j] = on ? __uint_as_float((best & 0x80000000u) ? (best & 0x7fffffffu) : ~best) : -CUDART_INF_F;
+                out_anchor[obase + j] = next.found() ? i + 1 - stride_offset(c, next.s) : -1;
+                out_score[obase + j] = next.score();
             }
-            taken = best;
-            at = bs;
+            next.take();
         }
         return;
     }

@@ -145,9 +145,9 @@ def test_search_of_wide_groups(sla, handle, heads, kv_heads, top_k):
         P.compare_search(anchor, score, ref, q_pos0=pos0, q_s=host["q_s"], k=host["k"], search_scale=1.0)
 
 
-@pytest.mark.parametrize("heads,top_k", [(8, 1), (8, 2), (16, 4), (16, 8), (8, 16)])
+@pytest.mark.parametrize("heads,top_k", [(8, 1), (8, 2), (16, 4), (16, 8), (8, 16), (4, 1), (4, 2), (4, 4), (4, 8), (4, 16)])
 def test_search_of_scores_that_are_not_finite(sla, handle, heads, top_k):
-    """Keys that hold Inf or NaN, groups of 8 and 16 query heads: a NaN score is no candidate and costs no other one its
+    """Keys that hold Inf or NaN, groups of 4, 8 and 16 query heads: a NaN score is no candidate and costs no other one its
     place, -inf comes last, ties go to the nearer anchor."""
     import torch
     L = 430
