@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
         if (sh.bg == a.B * a.Hkv - 1 && threadIdx.x == 0) {
             const int all = tile_base + nt;
             a.n_tiles[0] = a.n_tiles[1] = all < a.max_tiles ? all : a.max_tiles;   // [1]: the count as cut here
+            a.n_tiles[2] = 0;   // tiles claimed by the attention kernel
         }
     }
     // One thread per parked slot, four slots in flight per thread.  The rows of a (batch, kv head) are

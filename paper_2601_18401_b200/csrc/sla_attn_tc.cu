@@ -18,8 +18,8 @@
 // gathered into shared memory and the tile walks the key blocks they cover from left to right.
 //
 //   tc::prepare          the counting sort and the tile table (sla_attn_prep.cu)
-//   tc_attend            persistent CTAs, tile t goes to CTA t mod grid (the table is static once
-//                        built); per tile and key block: S = Q K^T (tcgen05, smem x smem -> TMEM), row
+//   tc_attend            persistent CTAs; tiles are claimed in the order of the table (short lists: tile t
+//                        goes to CTA t mod grid); per tile and key block: S = Q K^T (tcgen05, smem x smem -> TMEM), row
 //                        softmax in registers, P (bf16) back into TMEM, O += P V (tcgen05, TMEM x smem
 //                        -> TMEM); per piece a normalised fp16 block-floating-point partial + lse
 //   tc_merge             per row: log-sum-exp merge of its pieces -> out, lse
@@ -28,7 +28,7 @@
 // CTA layout of tc_attend (512 threads, one CTA per SM): warps 0-3 and 4-7 are the softmax warps of the
 // tile's two streams (one thread per piece, TMEM lane = row); warps 8-11 write the results (and gather the
 // first tile's Q); warps 12 and 13 issue the MMAs of a stream each; warp 14 loads K and V, once for both
-// streams; warp 15 gathers Q for the tiles to come.  TMEM: per stream 128 columns of O and two 64-column S
+// streams; warp 15 claims the tiles to come and gathers their Q.  TMEM: per stream 128 columns of O and two 64-column S
 // buffers (P aliases the S it came from).  Every wait on an mbarrier is bounded; when one runs out the CTA
 // raises a status bit, drains and leaves.
 //
@@ -39,7 +39,7 @@
 // 1860 cycles a block in long tiles but 5300 more per tile; now 700 per tile.  Configuration of 65536 tokens, 11
 // blocks per tile: 4.07 -> 3.45 ms; 16384 tokens, 7 blocks: 658 -> 570 us.
 // Two things that the times depend on: the kernel's code has to fit the instruction cache (about 2300
-// instructions; at 3500 the hit rate is 77 % and everything takes a half longer), and the issuing warps have to
+// instructions, 2700 with the claims; at 3300 the hit rate is 93 %, at 3500 77 % and everything takes a half longer), and the issuing warps have to
 // run converged with one elected lane issuing (see ptx::elect_one): the issuers' time per block bounded the
 // streams at 2500 cycles otherwise.
 #include <cuda.h>
@@ -72,6 +72,14 @@ constexpr int kQBytes = kHalf * kD * 2;      // 32 KiB, two 64-wide halves of 12
 constexpr int kKVBytes = kBK * kD * 2;       // 16 KiB, two 64-wide halves of 64 rows x 128 B
 constexpr int kQS = 4;           // Q buffers: the streams of this tile and of the next
 constexpr int kKS = 3;           // K and V stages
+constexpr int kTS = 4;           // entries of the ring of tiles
+// A list that can have as many tiles per CTA as this (every slot of every row taken) is claimed tile by tile.  Dealt
+// round-robin, the CTAs of a long list end at different times: they were busy for 0.88 of the kernel at 16384 positions, 0.95
+// at 65536 (the kernel: 545 and 3690 us dealt, 515 and 3600 us claimed; two sequences of 262144 positions 71.0 and 67.2 ms).  In a
+// short list a claim comes too late to even anything out, and the ring costs its walks of a few blocks time (1999
+// positions, four spans, at most 7 tiles per CTA: 45.5 us dealt, 49 us claimed).
+constexpr int kClaimTiles = 16;
+constexpr int kTileReaders = 15; // warps that read them: all but the one that claims the tiles
 constexpr int kOffQ = 0;
 constexpr int kOffK = kQS * kQBytes;
 constexpr int kOffV = kOffK + kKS * kKVBytes;
@@ -85,9 +93,11 @@ static_assert(2 * kRegsRow + kRegsEpi + kRegsIssue <= 4 * 128, "more registers t
 
 struct Meta {
     unsigned long long q_full[kQS], q_empty[kQS], kv_full[kKS], kv_empty[2][kKS];
-    unsigned long long s_full[4], p_ready[4], l_full[2], o_full[2], o_empty[2];
+    unsigned long long s_full[4], p_ready[4], l_full[2], o_full[2], o_empty[2], t_full[kTS], t_empty[kTS];
     uint32_t tmem_base;
     int abort_flag;
+    int4 tile[kTS];        // the CTA's tiles: table entry (no records: none is left) and the blocks its streams reach
+    int2 range[kTS];
     float2 stats[kRows];   // {reciprocal denominator, log2-domain log-sum-exp} of the tile's rows, for the epilogue
 };
 static_assert(sizeof(Meta) <= kMetaBytes, "meta block too large");
@@ -103,7 +113,7 @@ struct TcParams {
     const int4 *recs;          // sorted piece records {row, j, lo, hi}
     const int4 *tiles;         // {b*Hkv+g, end block, first record, record count | key blocks to walk << 9}
     const int2 *ranges;        // key blocks of the walk a tile's streams take part in: first | end << 16
-    const int *n_tiles;
+    int *n_tiles;              // number of tiles; [2]: tiles claimed beyond the first two of every CTA
     __half *part_o;            // [rows*slots][128] normalised piece outputs, fp16 with one power-of-two
                                // scale per 32-column chunk (block floating point)
     float2 *part_lse;          // [rows*slots] {log2-domain log-sum-exp of the piece, four chunk exponents}
@@ -151,6 +161,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// kClaim: tiles beyond a CTA's first two are claimed when they are needed, else dealt round-robin.
+template <bool kClaim>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
           const __grid_constant__ CUtensorMap tm_v, TcParams p) {
@@ -169,6 +181,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     const uint32_t bar_s_full = mbase + offsetof(Meta, s_full), bar_p_ready = mbase + offsetof(Meta, p_ready);
     const uint32_t bar_l_full = mbase + offsetof(Meta, l_full);
     const uint32_t bar_o_full = mbase + offsetof(Meta, o_full), bar_o_empty = mbase + offsetof(Meta, o_empty);
+    const uint32_t bar_t_full = mbase + offsetof(Meta, t_full), bar_t_empty = mbase + offsetof(Meta, t_empty);
 
     if (tid == 0) {
 #pragma unroll 1
@@ -186,6 +199,8 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         for (int x = 0; x < 4; ++x) {
             ptx::mbar_init(bar_s_full + 8 * x, 1);
             ptx::mbar_init(bar_p_ready + 8 * x, 4);   // one arrival per row warp
+            ptx::mbar_init(bar_t_full + 8 * x, 1);
+            ptx::mbar_init(bar_t_empty + 8 * x, kTileReaders);
         }
 #pragma unroll 1
         for (int x = 0; x < 2; ++x) {
@@ -203,26 +218,61 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     // the set-up above runs beside the kernel before this one
     chain_wait();
     chain_release();
-    const int n_tiles = *p.n_tiles, tile_step = gridDim.x;
-    int tile = blockIdx.x;
-    int4 ti = p.tiles[tile];   // the table has an entry for every CTA
+    const int n_tiles = *p.n_tiles;
+    // the role's tile; no records when none is left.  (The table has an entry for every CTA.)
+    int4 ti = p.tiles[blockIdx.x];
+    int2 rg;                          // blocks of its walk the streams take part in
+    if (kClaim && tid == 0) {
+        meta->tile[0] = ti;
+        meta->range[0] = p.ranges[blockIdx.x];
+        ptx::mbar_arrive(bar_t_full);
+    }
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = meta->tmem_base;
-    if (tile >= n_tiles) ti = make_int4(0, 0, 0, 0);   // not an entry: nothing below looks records up through it
+    if (blockIdx.x >= n_tiles) ti = make_int4(0, 0, 0, 0);   // not an entry: nothing below looks records up through it
+    auto first_range = [&]() { return ti.w ? (kClaim ? meta->range[0] : p.ranges[blockIdx.x]) : make_int2(0, 0); };
 
     constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(kHalf, kBK, false, false);   // S = Q K^T, both K-major
     constexpr uint32_t kIdescO = ptx::idesc_bf16_f32(kHalf, kD, false, true);       // O = P V, V is N-major
 
-    // Tiles are dealt round-robin: CTA c takes tiles c, c + grid, c + 2 grid, ...  Every role reads its
-    // tile's table entry {b*Hkv+g, end block, first record, count | blocks << 9} straight from global
-    // memory, one tile ahead of where it is working, so nothing but mbarriers couples the roles.
+    // The first two tiles of CTA c are c and c + grid of the table.  Of a long list the warp that gathers Q claims the others, in
+    // the order of the table, and passes each one's entry {b*Hkv+g, end block, first record, count | blocks << 9} on through a
+    // ring in shared memory; a short one is dealt round-robin, and every role reads the table itself.
+    // the claiming kernel has no room in the instruction cache for the longer form of the waits off the critical path
+    auto wait_aside = [&](uint32_t bar, uint32_t parity) {
+        if constexpr (kClaim) return ptx::mbar_wait_short(bar, parity, abort_flag);
+        else return ptx::mbar_wait(bar, parity, abort_flag);
+    };
+    auto read_tile = [&](uint32_t k) {   // the CTA's k-th tile
+        if constexpr (kClaim) {
+            const bool got = __all_sync(0xffffffffu, ptx::mbar_wait_short(bar_t_full + 8 * (k % kTS), (k / kTS) & 1u, abort_flag));
+            ti = meta->tile[k % kTS];
+            rg = meta->range[k % kTS];
+            return got;
+        } else {
+            const int n = blockIdx.x + k * gridDim.x;
+            ti = n < n_tiles ? p.tiles[n] : make_int4(0, 0, 0, 0);
+            rg = n < n_tiles ? p.ranges[n] : make_int2(0, 0);
+            return true;
+        }
+    };
+    auto tile_read = [&](uint32_t k) {   // the warp needs the entry no more
+        if constexpr (kClaim) {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar_t_empty + 8 * (k % kTS));
+        }
+    };
+    auto take_tile = [&](uint32_t k) {
+        const bool got = read_tile(k);
+        tile_read(k);
+        return got;
+    };
     auto q_row = [&](int row, int bb) {   // number of a record's row among the rows of Q
         const int bh = (unsigned)row / (unsigned)p.Lc;
         return bb * p.q_b + (bh - bb * p.Hq) * p.q_h + (p.r0 + row - bh * p.Lc) * p.q_t;
     };
-    auto fetch_next = [&]() { return tile + tile_step < n_tiles ? p.tiles[tile + tile_step] : make_int4(0, 0, 0, 0); };
 
     if (warp >= 12) {
         ptx::setmaxnreg_dec<kRegsIssue>();
@@ -235,31 +285,31 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             const bool leader = ptx::elect_one();
             const int x = warp - 12;
             struct Cursor {
-                int tile, j, nblk, nx;
+                uint32_t k;       // tile
+                int j, nblk, nx;  // nblk 0: no tile left
                 int first, end;   // blocks this stream takes part in
                 uint32_t nb;      // of those so far
             };
-            auto open = [&](Cursor &c) {
+            auto open = [&](Cursor &c) {   // the tile just read
+                const int r = x ? rg.y : rg.x;
                 c.j = 0;
-                if (c.tile < n_tiles) {
-                    const int w = p.tiles[c.tile].w;
-                    c.nblk = w >> 9;
-                    c.nx = (w & 0x1ff) > kHalf ? 2 : 1;
-                    const int rg = x ? p.ranges[c.tile].y : p.ranges[c.tile].x;
-                    c.first = rg & 0xffff;
-                    c.end = rg >> 16;
-                }
+                c.nblk = ti.w >> 9;
+                c.nx = (ti.w & 0x1ff) > kHalf ? 2 : 1;
+                c.first = r & 0xffff;
+                c.end = r >> 16;
             };
-            Cursor cs{tile, 0, 0, 0, 0, 0, 0u};
+            Cursor cs{0u, 0, 0, 0, 0, 0, 0u};
+            rg = first_range();
             open(cs);
             Cursor cv = cs;
+            bool ok = true;
             const uint32_t s_col = tmem + kColS + x * (2 * kBK), o_col = tmem + kColO + x * kD;
             uint32_t nq = x, t = 0;
             const uint64_t desc_q0 = ptx::smem_desc_sw128(base + kOffQ, 16, 1024);
             const uint64_t desc_k0 = ptx::smem_desc_sw128(base + kOffK, 16, 1024);
             const uint64_t desc_v0 = ptx::smem_desc_sw128(base + kOffV, kKVBytes / 2, 1024);
 #pragma unroll 1
-            for (uint32_t i = 0; cv.tile < n_tiles; ++i) {
+            for (uint32_t i = 0; ok && cv.nblk > 0; ++i) {
                 if (i >= 2) {
                     const uint32_t st = (i - 2) % kKS, bar_done = bar_kv_empty + 8 * (x * kKS + st);
                     const bool last = cv.j == cv.end - 1;
@@ -282,11 +332,12 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         ptx::mbar_arrive(bar_done);
                     }
                     if (++cv.j == cv.nblk) {
-                        cv.tile += tile_step;
+                        tile_read(cv.k);
+                        ok = read_tile(++cv.k);   // S has opened it before
                         open(cv);
                     }
                 }
-                if (cs.tile < n_tiles) {
+                if (ok && cs.nblk > 0) {
                     const uint32_t st = i % kKS;
                     if (!ptx::mbar_wait(bar_kv_full + 8 * st, (i / kKS) & 1u, abort_flag)) break;
                     const bool last = cs.j == cs.end - 1;
@@ -307,7 +358,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     }
                     if (++cs.j == cs.nblk) {
                         nq += cs.nx;
-                        cs.tile += tile_step;
+                        ok = read_tile(++cs.k);
                         open(cs);
                     }
                 }
@@ -315,20 +366,20 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         } else if (warp == 14) {
             // ---------------- K/V producer: K and V of block after block, each as two halves of the head dimension
             const bool leader = ptx::elect_one();
-            uint32_t n = 0;
+            uint32_t n = 0, k = 0;
             bool ok = true;
-            while (tile < n_tiles && ok) {
-                const int4 ti_next = fetch_next();
-                const int nblk = ti.w >> 9, bb = (unsigned)ti.x / (unsigned)p.Hkv;
+            tile_read(0);
+            while (ok && ti.w) {
+                const int nblk = ti.w >> 9, bb = (unsigned)ti.x / (unsigned)p.Hkv, t0 = (ti.y + 1 - nblk) * kBK;
                 int c[4];
                 c[1 + p.slot_h] = ti.x - bb * p.Hkv;
                 c[1 + p.slot_b] = bb;
+                ok = take_tile(++k);
 #pragma unroll 1
-                for (int j = 0; j < nblk; ++j, ++n) {
+                for (int j = 0; j < nblk && ok; ++j, ++n) {
                     const uint32_t st = n % kKS, ph = ((n / kKS) & 1u) ^ 1u;
-                    c[1 + p.slot_t] = (ti.y + 1 - nblk + j) * kBK;
-                    ok = ptx::mbar_wait(bar_kv_empty + 8 * st, ph, abort_flag) &&
-                         ptx::mbar_wait(bar_kv_empty + 8 * (kKS + st), ph, abort_flag);
+                    c[1 + p.slot_t] = t0 + j * kBK;
+                    ok = wait_aside(bar_kv_empty + 8 * st, ph) && wait_aside(bar_kv_empty + 8 * (kKS + st), ph);
                     if (!ok) break;
                     if (leader) {
                         const uint32_t full = bar_kv_full + 8 * st, dk = base + kOffK + st * kKVBytes, dv = base + kOffV + st * kKVBytes;
@@ -339,8 +390,6 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         ptx::tma_load_4d(dv + kKVBytes / 2, &tm_v, full, 64, c[1], c[2], c[3]);
                     }
                 }
-                tile += tile_step;
-                ti = ti_next;
             }
         } else {
             // ---------------- Q gather from the CTA's second tile on: the rows of one stream's tile after the other by TMA,
@@ -348,39 +397,61 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             // read a stream ahead.  (128 rows take the TMA unit about 4600 cycles: hidden in the tile before.)
             ptx::prefetch_tensormap(&tm_q);
             const bool leader = ptx::elect_one();
-            uint32_t nq = (ti.w & 0x1ff) > kHalf ? 2 : 1;
-            int x = 0, rows[4];
+            uint32_t k = 0, nq = 0;
+            int n = blockIdx.x + gridDim.x, rows[4];   // the next tile: the second is the CTA's own as well
             auto fetch_rows = [&](const int4 &t, int xs) {   // a row beyond the tile's last one: that one again
                 const int last = (t.w & 0x1ff) - 1;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) rows[u] = p.recs[t.z + min(xs * kHalf + 4 * lane + u, last)].x;
             };
-            tile += tile_step;
-            ti = tile < n_tiles ? p.tiles[tile] : ti;
-            if (tile < n_tiles) fetch_rows(ti, 0);
-            int4 ti_next = fetch_next();
-            while (tile < n_tiles) {
-                const int bb = (unsigned)ti.x / (unsigned)p.Hkv;
-                const uint32_t qs = nq % kQS, full = bar_q_full + 8 * qs;
-                if (!ptx::mbar_wait_warp(bar_q_empty + 8 * qs, ((nq / kQS) & 1u) ^ 1u, abort_flag)) break;
-                if (leader) ptx::mbar_arrive_expect_tx(full, kQBytes);
-                int at[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) at[u] = q_row(rows[u], bb);
-                __syncwarp();
-                const uint32_t dst = base + kOffQ + qs * kQBytes + lane * 512;
-                ptx::tma_gather4(dst, &tm_q, full, 0, at[0], at[1], at[2], at[3]);
-                ptx::tma_gather4(dst + kQBytes / 2, &tm_q, full, 64, at[0], at[1], at[2], at[3]);
-                if (x == 0 && (ti.w & 0x1ff) > kHalf) {
-                    x = 1;
+            // the next tile's entry, passed on to the other warps; the one after it is claimed
+            auto next_tile = [&]() {
+                if constexpr (kClaim) n = __shfl_sync(0xffffffffu, n, 0);
+                const int4 t = n < n_tiles ? p.tiles[n] : make_int4(0, 0, 0, 0);
+                ++k;
+                if constexpr (kClaim) {
+                    const int2 r = n < n_tiles ? p.ranges[n] : make_int2(0, 0);
+                    if (lane == 0) n = atomicAdd(p.n_tiles + 2, 1) + 2 * gridDim.x;
+                    if (!__all_sync(0xffffffffu, wait_aside(bar_t_empty + 8 * (k % kTS), ((k / kTS) & 1u) ^ 1u))) return make_int4(0, 0, 0, 0);
+                    if (leader) {
+                        meta->tile[k % kTS] = t;
+                        meta->range[k % kTS] = r;
+                        ptx::mbar_arrive(bar_t_full + 8 * (k % kTS));
+                    }
                 } else {
-                    x = 0;
-                    tile += tile_step;
-                    ti = ti_next;
-                    if (tile < n_tiles) ti_next = fetch_next();
+                    n += gridDim.x;
                 }
-                if (tile < n_tiles) fetch_rows(ti, x);
-                ++nq;
+                return t;
+            };
+            int4 next = ti;
+            nq = (ti.w & 0x1ff) > kHalf ? 2 : 1;   // the epilogue warps gather the first tile's rows
+            bool first = true, ok = true;
+            while (ok && next.w) {
+                ti = next;
+                next = next_tile();
+                if (first) {
+                    first = false;
+                    if (next.w) fetch_rows(next, 0);
+                    continue;
+                }
+                const int bb = (unsigned)ti.x / (unsigned)p.Hkv, nx = (ti.w & 0x1ff) > kHalf ? 2 : 1;
+#pragma unroll 1
+                for (int x = 0; x < nx; ++x, ++nq) {
+                    const uint32_t qs = nq % kQS, full = bar_q_full + 8 * qs;
+                    ok = __all_sync(0xffffffffu, wait_aside(bar_q_empty + 8 * qs, ((nq / kQS) & 1u) ^ 1u));
+                    if (!ok) break;
+                    if (leader) ptx::mbar_arrive_expect_tx(full, kQBytes);
+                    int at[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) at[u] = q_row(rows[u], bb);
+                    __syncwarp();
+                    const uint32_t dst = base + kOffQ + qs * kQBytes + lane * 512;
+                    ptx::tma_gather4(dst, &tm_q, full, 0, at[0], at[1], at[2], at[3]);
+                    ptx::tma_gather4(dst + kQBytes / 2, &tm_q, full, 64, at[0], at[1], at[2], at[3]);
+                    const bool more = x + 1 < nx;
+                    const int4 t = more ? ti : next;
+                    if (t.w) fetch_rows(t, more);
+                }
             }
         }
     } else if (warp >= 8) {
@@ -388,6 +459,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         ptx::setmaxnreg_dec<kRegsEpi>();
         const int row = tid & 127;
         const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        uint32_t k = 0;
+        bool ok = true;
+        tile_read(0);
         // the Q rows of the CTA's first tile, by 16-byte copies: two rows (16 lanes each) per instruction
         {
             const int cnt = ti.w & 0x1ff, chunk = lane & 15, odd = lane >> 4, bb = (unsigned)ti.x / (unsigned)p.Hkv;
@@ -408,20 +482,18 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             }
         }
         uint32_t tx[2] = {0, 0};
-        bool ok = true;
-        while (tile < n_tiles && ok) {
-            const int4 ti_next = fetch_next();
-            const int cnt = ti.w & 0x1ff, nx = cnt > kHalf ? 2 : 1;
+        while (ok && ti.w) {
+            const int cnt = ti.w & 0x1ff, nx = cnt > kHalf ? 2 : 1, rec0 = ti.z;
+            ok = take_tile(++k);
 #pragma unroll 1
             for (int x = 0; x < nx && ok; ++x) {
                 const uint32_t t = x ? tx[1] : tx[0];
                 const int r = x * kHalf + row;
                 const bool valid = r < cnt;
-                const int2 rs = valid ? *reinterpret_cast<const int2 *>(&p.recs[ti.z + r]) : make_int2(0, 0);
+                const int2 rs = valid ? *reinterpret_cast<const int2 *>(&p.recs[rec0 + r]) : make_int2(0, 0);
                 const long long slot = (long long)rs.x * p.slots + rs.y;
                 __half *dst = p.part_o + slot * kD;
-                ok = ptx::mbar_wait_warp(bar_l_full + 8 * x, t & 1u, abort_flag) &&
-                     ptx::mbar_wait_warp(bar_o_full + 8 * x, t & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, wait_aside(bar_l_full + 8 * x, t & 1u) && wait_aside(bar_o_full + 8 * x, t & 1u));
                 if (!ok) break;
                 ptx::tc_fence_after();
                 const float2 stat = meta->stats[r];
@@ -467,8 +539,6 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 if (valid) p.part_lse[slot] = make_float2(stat.y, __uint_as_float(exps));
                 if (x) ++tx[1]; else ++tx[0];
             }
-            tile += tile_step;
-            ti = ti_next;
         }
     } else {
         // ---------------- row warps of stream x: softmax per 64-key block, one thread per row
@@ -480,18 +550,19 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             return r < (t.w & 0x1ff) ? *reinterpret_cast<const int2 *>(&p.recs[t.z + r].z) : make_int2(INT_MAX, -1);
         };
         uint32_t n = 0, na = 0, t = 0;   // blocks and tiles of the stream so far; all blocks of the CTA
-        auto range = [&](int t) { return t < n_tiles ? (x ? p.ranges[t].y : p.ranges[t].x) : 0; };
-        int2 iv = interval(ti);
-        int rg = range(tile);
+        uint32_t k = 0;
         bool ok = true;
-        while (tile < n_tiles && ok) {
-            const int4 ti_next = fetch_next();
-            const int2 iv_next = interval(ti_next);   // requested a tile ahead
-            const int rg_next = range(tile + tile_step);
-            const int nblk = ti.w >> 9, first_block = rg & 0xffff, end_block = rg >> 16;
+        rg = first_range();
+        tile_read(0);
+        int2 iv = interval(ti);
+        while (ok && ti.w) {
+            const int nblk = ti.w >> 9, range = x ? rg.y : rg.x, first_block = range & 0xffff, end_block = range >> 16;
+            int k0 = (ti.y + 1 - nblk + first_block) * kBK;
+            ok = take_tile(++k);
+            if (!ok) break;
+            const int2 iv_next = interval(ti);   // requested a tile ahead
             if (first_block < end_block) {
                 const int lo = iv.x, hi = iv.y;
-                int k0 = (ti.y + 1 - nblk + first_block) * kBK;
                 float m_ref = -CUDART_INF_F, l = 0.f;
 #pragma unroll 1
                 for (int j = first_block; j < end_block; ++j, ++n, k0 += kBK) {
@@ -592,10 +663,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 }
             }
             na += nblk;
-            tile += tile_step;
-            ti = ti_next;
             iv = iv_next;
-            rg = rg_next;
         }
     }
 
@@ -1197,7 +1265,8 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tc_attend, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(tc_attend<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_attend<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
@@ -1258,7 +1327,8 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         tp.status = c.status; tp.Hkv = c.Hkv;
         if (last) { last->tiles = pa.tiles; last->ranges = pa.ranges; last->n_tiles = counters; }
         if (timer) timer->begin(st);
-        e = launch_chained(tc_attend, dim3(sm_count), dim3(kThreads), kSmemBytes, st, tm_q, tm_k, tm_v, tp);
+        const bool claim = rows * plan.slots >= (long long)kClaimTiles * kRows * sm_count;
+        e = launch_chained(claim ? tc_attend<true> : tc_attend<false>, dim3(sm_count), dim3(kThreads), kSmemBytes, st, tm_q, tm_k, tm_v, tp);
         if (e != cudaSuccess) return e;
         if (timer) timer->end(st);
         // The merges do not release what comes after them: 131072 short CTAs, each with the extra instruction, took 2 % more of

@@ -58,6 +58,16 @@ def run_prefill(sla, handle, w, q_pos0=0, Lq=None, permute=False, softmax_scale=
     return dict(ties=ties, err=err, lerr=lerr, anchor=anchor, out=out, lse=lse, host=host, ref_a=ref_a)
 
 
+# Lists of pieces around the length from which the attention kernel claims its tiles instead of dealing them round-robin
+# (16 tiles of 256 slots for each of 148 SMs = 1184 positions of 32 heads, 16 slots each), spans so short that a tile is
+# walked in one or two blocks, and a list that is claimed in two sequences.
+@pytest.mark.parametrize("kw", [dict(seq_len=1183), dict(seq_len=1184), dict(seq_len=1201, span_len=1, back_factor=0),
+                                dict(seq_len=640, batch=2, span_len=40)])
+def test_claimed_and_dealt_tiles(sla, handle, kw):
+    w = workload(**{**dict(n_q_heads=32, n_kv_heads=8, top_k=16, span_len=9), **kw})
+    run_prefill(sla, handle, w)
+
+
 @pytest.mark.parametrize("kw", [
     dict(),                                                                  # bf16 D128 GQA, ragged L
     dict(dtype="f32"),                                                       # fp32 D128
