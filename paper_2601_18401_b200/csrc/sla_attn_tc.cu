@@ -79,7 +79,10 @@ constexpr int kTS = 4;           // entries of the ring of tiles
 // short list a claim comes too late to even anything out, and the ring costs its walks of a few blocks time (1999
 // positions, four spans, at most 7 tiles per CTA: 45.5 us dealt, 49 us claimed).
 constexpr int kClaimTiles = 16;
-constexpr int kTileReaders = 15; // warps that read them: all but the one that claims the tiles
+// They are read by one lane each of the row and epilogue warps, whose waits are answered for the whole warp, and by every
+// lane of the issuers and of the K/V producer, whose lanes wait each for itself (a vote in each of their waits made the
+// kernel 1 % slower at 16384 positions).
+constexpr int kTileReaders = 12 + 3 * 32;
 constexpr int kOffQ = 0;
 constexpr int kOffK = kQS * kQBytes;
 constexpr int kOffV = kOffK + kKS * kKVBytes;
@@ -245,9 +248,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         if constexpr (kClaim) return ptx::mbar_wait_short(bar, parity, abort_flag);
         else return ptx::mbar_wait(bar, parity, abort_flag);
     };
-    auto read_tile = [&](uint32_t k) {   // the CTA's k-th tile
+    auto read_tile = [&](uint32_t k) {   // the CTA's k-th tile; every lane gets its own answer
         if constexpr (kClaim) {
-            const bool got = __all_sync(0xffffffffu, ptx::mbar_wait_short(bar_t_full + 8 * (k % kTS), (k / kTS) & 1u, abort_flag));
+            const bool got = ptx::mbar_wait_short(bar_t_full + 8 * (k % kTS), (k / kTS) & 1u, abort_flag);
             ti = meta->tile[k % kTS];
             rg = meta->range[k % kTS];
             return got;
@@ -258,15 +261,20 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             return true;
         }
     };
-    auto tile_read = [&](uint32_t k) {   // the warp needs the entry no more
+    auto lane_read = [&](uint32_t k) {   // the lane needs the entry no more
+        if constexpr (kClaim) ptx::mbar_arrive(bar_t_empty + 8 * (k % kTS));
+    };
+    // The same for a whole warp.  Not in the issuers and the K/V producer: there a lane whose wait ran out leaves alone, and
+    // the others would wait for it here without a bound.
+    auto warp_read = [&](uint32_t k) {
         if constexpr (kClaim) {
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar_t_empty + 8 * (k % kTS));
+            if (lane == 0) lane_read(k);
         }
     };
     auto take_tile = [&](uint32_t k) {
-        const bool got = read_tile(k);
-        tile_read(k);
+        const bool got = __all_sync(0xffffffffu, read_tile(k));
+        warp_read(k);
         return got;
     };
     auto q_row = [&](int row, int bb) {   // number of a record's row among the rows of Q
@@ -332,7 +340,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         ptx::mbar_arrive(bar_done);
                     }
                     if (++cv.j == cv.nblk) {
-                        tile_read(cv.k);
+                        lane_read(cv.k);
                         ok = read_tile(++cv.k);   // S has opened it before
                         open(cv);
                     }
@@ -368,13 +376,14 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             const bool leader = ptx::elect_one();
             uint32_t n = 0, k = 0;
             bool ok = true;
-            tile_read(0);
+            lane_read(0);
             while (ok && ti.w) {
                 const int nblk = ti.w >> 9, bb = (unsigned)ti.x / (unsigned)p.Hkv, t0 = (ti.y + 1 - nblk) * kBK;
                 int c[4];
                 c[1 + p.slot_h] = ti.x - bb * p.Hkv;
                 c[1 + p.slot_b] = bb;
-                ok = take_tile(++k);
+                ok = read_tile(++k);
+                lane_read(k);
 #pragma unroll 1
                 for (int j = 0; j < nblk && ok; ++j, ++n) {
                     const uint32_t st = n % kKS, ph = ((n / kKS) & 1u) ^ 1u;
@@ -461,7 +470,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         uint32_t k = 0;
         bool ok = true;
-        tile_read(0);
+        warp_read(0);
         // the Q rows of the CTA's first tile, by 16-byte copies: two rows (16 lanes each) per instruction
         {
             const int cnt = ti.w & 0x1ff, chunk = lane & 15, odd = lane >> 4, bb = (unsigned)ti.x / (unsigned)p.Hkv;
@@ -553,7 +562,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         uint32_t k = 0;
         bool ok = true;
         rg = first_range();
-        tile_read(0);
+        warp_read(0);
         int2 iv = interval(ti);
         while (ok && ti.w) {
             const int nblk = ti.w >> 9, range = x ? rg.y : rg.x, first_block = range & 0xffff, end_block = range >> 16;

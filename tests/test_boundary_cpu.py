@@ -91,3 +91,33 @@ def test_product_path_does_not_touch_the_oracle():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dirpath, f)).read()
                 assert not re.search(r"sla_oracle|from\s+oracle|import\s+oracle|oracle/", text), f
+
+
+def test_roles_that_wait_lane_by_lane_use_no_warp_collective():
+    """The issuers and the K/V producer of the tensor-core attention kernel act on each lane's own answer of a bounded
+    wait.  When one runs out, a lane can leave while its neighbours go on: nothing they reach afterwards may wait for the whole
+    warp, neither in their loops nor in the helpers that these call (a vote there would never end)."""
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(ROOT, "paper_2601_18401_b200", "csrc", "sla_attn_tc.cu")).read())
+    kernel = src[src.index("tc_attend(const __grid_constant__"):]
+    roles = kernel[kernel.index("if (warp < 14)"):kernel.index("ptx::prefetch_tensormap(&tm_q)")]
+    assert roles.count("elect_one()") == 2 and "tma_load_4d" in roles and "mma_ts" in roles
+
+    def body(at):   # the braces that open at or after `at`
+        at = start = kernel.index("{", at)
+        depth = 0
+        while True:
+            depth += {"{": 1, "}": -1}.get(kernel[at], 0)
+            at += 1
+            if depth == 0:
+                return kernel[start:at]
+
+    helpers = {m.group(1): body(m.end()) for m in re.finditer(r"\bauto (\w+) = \[&\]", kernel)}
+    reached, text = set(), roles
+    while True:
+        new = {n for n in re.findall(r"\b(\w+)\(", text) if n in helpers} - reached
+        if not new:
+            break
+        reached |= new
+        text += "".join(helpers[n] for n in new)
+    assert {"read_tile", "wait_aside"} <= reached
+    assert not re.findall(r"__\w+_sync\(|__syncwarp\(|__syncthreads\(|mbar_wait\w*_warp\(|bar_sync\(", text)
