@@ -73,12 +73,22 @@ constexpr int kKVBytes = kBK * kD * 2;       // 16 KiB, two 64-wide halves of 64
 constexpr int kQS = 4;           // Q buffers: the streams of this tile and of the next
 constexpr int kKS = 3;           // K and V stages
 constexpr int kTS = 4;           // entries of the ring of tiles
-// A list that can have as many tiles per CTA as this (every slot of every row taken) is claimed tile by tile.  Dealt
-// round-robin, the CTAs of a long list end at different times: they were busy for 0.88 of the kernel at 16384 positions, 0.95
-// at 65536 (the kernel: 545 and 3690 us dealt, 515 and 3600 us claimed; two sequences of 262144 positions 71.0 and 67.2 ms).  In a
-// short list a claim comes too late to even anything out, and the ring costs its walks of a few blocks time (1999
-// positions, four spans, at most 7 tiles per CTA: 45.5 us dealt, 49 us claimed).
-constexpr int kClaimTiles = 16;
+// A list is claimed tile by tile if it can have kClaimTiles tiles per CTA (every slot of every row taken) and its longest single
+// piece, a span or the window, can cover kClaimBlocks key blocks (kClaimBlocksJoined where touching spans are joined, which
+// makes the walks longer).  Dealt round-robin, the CTAs of a long list end at different times: they were busy for 0.88 of the
+// kernel at 16384 positions, 0.95 at 65536.  Tiles of short walks are over too soon for that, and pass the ring later than the
+// table would have been read.  The kernel, 32/8 heads, eight spans, dealt and claimed, us (runs of one side differ by 1 to 5 %):
+//   joined, from position 0    16384, spans of 65 / 129 / 193 / 257 keys (3 / 4 / 5 / 6 blocks)
+//                                                597, 658 / 590, 628 / 667, 651 / 735, 707
+//                              65536, the same   2529, 2828 / 2752, 2812 / 2950, 2926 / 3593, 3119
+//                              4736, 257 keys 178, 173;  9000, 301 keys 432, 387
+//   not joined, at 90000       12000, spans of 193 / 321 / 385 / 513 keys (5 / 7 / 8 / 10 blocks)
+//                                                551, 642 / 705, 751 / 824, 822 / 977, 920
+//   per span, 32768            four spans of 257 keys, window 256 (6 blocks) 965, 994; spans of 65, window 1088 (18) 1553, 1402
+//   tiles per CTA, at 100000, spans of 635 keys (11 blocks): 5: 183, 185; 7: 200, 206; 12: 245, 241; 16: 302, 282; 40: 593, 589
+// Joined lists have fewer tiles than the slots of their rows suggest.  With walks this long either side wins by the way its
+// tiles happen to fall, up to 18 % (16 spans of 513 keys at 4736, 7 tiles per CTA: 255, 279; eight of them 274, 232).
+constexpr int kClaimTiles = 16, kClaimBlocks = 8, kClaimBlocksJoined = 5;
 // They are read by one lane each of the row and epilogue warps, whose waits are answered for the whole warp, and by every
 // lane of the issuers and of the K/V producer, whose lanes wait each for itself (a vote in each of their waits made the
 // kernel 1 % slower at 16384 positions).
@@ -1336,7 +1346,8 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         tp.status = c.status; tp.Hkv = c.Hkv;
         if (last) { last->tiles = pa.tiles; last->ranges = pa.ranges; last->n_tiles = counters; }
         if (timer) timer->begin(st);
-        const bool claim = rows * plan.slots >= (long long)kClaimTiles * kRows * sm_count;
+        const bool claim = rows * plan.slots >= (long long)kClaimTiles * kRows * sm_count &&
+                           plan.nb_single >= (plan.merge_cap > 0 ? kClaimBlocksJoined : kClaimBlocks);
         e = launch_chained(claim ? tc_attend<true> : tc_attend<false>, dim3(sm_count), dim3(kThreads), kSmemBytes, st, tm_q, tm_k, tm_v, tp);
         if (e != cudaSuccess) return e;
         if (timer) timer->end(st);

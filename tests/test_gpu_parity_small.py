@@ -58,14 +58,70 @@ def run_prefill(sla, handle, w, q_pos0=0, Lq=None, permute=False, softmax_scale=
     return dict(ties=ties, err=err, lerr=lerr, anchor=anchor, out=out, lse=lse, host=host, ref_a=ref_a)
 
 
-# Lists of pieces around the length from which the attention kernel claims its tiles instead of dealing them round-robin
-# (16 tiles of 256 slots for each of 148 SMs = 1184 positions of 32 heads, 16 slots each), spans so short that a tile is
-# walked in one or two blocks, and a list that is claimed in two sequences.
-@pytest.mark.parametrize("kw", [dict(seq_len=1183), dict(seq_len=1184), dict(seq_len=1201, span_len=1, back_factor=0),
-                                dict(seq_len=640, batch=2, span_len=40)])
-def test_claimed_and_dealt_tiles(sla, handle, kw):
-    w = workload(**{**dict(n_q_heads=32, n_kv_heads=8, top_k=16, span_len=9), **kw})
-    run_prefill(sla, handle, w)
+def claimed(call):
+    """Whether the tensor-core attention kernels that `call` launches claim their tiles (one answer per launch)."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    return ["tc_attend<true>" in e.name for e in prof.events() if "tc_attend" in e.name]
+
+
+# Lists of pieces on both sides of the rule by which the attention kernel claims its tiles instead of dealing them round-robin:
+# 16 tiles of 256 slots per SM (here 16 slots in each of 32 heads: 8 positions per SM), and a piece that covers 5 blocks of 64
+# keys in a dense list, where touching spans are joined (193 keys, spans of 96), or 8 in a sparse one (385 keys, spans of 192).
+@pytest.mark.parametrize("more,kw,q_pos0,claims", [
+    (-1, dict(span_len=96), 0, False), (0, dict(span_len=96), 0, True), (17, dict(span_len=95), 0, False), (17, dict(span_len=9), 0, False),
+    (0, dict(span_len=192), 20000, True), (0, dict(span_len=191), 20000, False), (-1, dict(span_len=192), 20000, False),
+])
+def test_claimed_and_dealt_tiles(sla, handle, more, kw, q_pos0, claims):
+    rows = 8 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    w = workload(**{**dict(n_q_heads=32, n_kv_heads=8, top_k=16, seq_len=q_pos0 + rows), **kw})
+    assert claimed(lambda: run_prefill(sla, handle, w, q_pos0=q_pos0, Lq=rows)) == [claims]
+
+
+# SM: the number of multiprocessors; with 32 heads of 16 slots, 8 SM positions are the shortest list that is claimed
+@pytest.mark.parametrize("batch,span_len,back,window,q_pos0,rows,chunk,strided", [
+    (1, 1, 0, 450, 0, "9 * SM + 7", "rows", False),       # per-span mode: spans of one key, most tiles walk one or two blocks
+    (2, 2, 1, 450, 0, "10 * SM + 1", "rows", False),      # the same in two sequences
+    (1, 96, 2, 0, 8000, "18 * SM", "9 * SM", False),      # a workspace that takes half of the rows: the counter starts again
+    (1, 96, 2, 0, 8000, "16 * SM - 1", "8 * SM", False),  # a claimed chunk and a dealt one
+    (2, 100, 2, 0, 6000, "8 * SM", "rows", True),         # rows of Q without a common pitch, gathered first
+])
+def test_claims_of_many_tiles(sla, batch, span_len, back, window, q_pos0, rows, chunk, strided):
+    """Lists of so many tiles that every CTA claims more of them than the ring of tiles has entries, against the oracle."""
+    from paper_2601_18401_b200 import synth
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = eval(rows, dict(SM=sms))
+    chunk = eval(chunk, dict(SM=sms, rows=rows))
+    L, top_k = q_pos0 + rows, 16
+    w = workload(batch=batch, n_q_heads=32, n_kv_heads=8, seq_len=L, top_k=top_k, span_len=span_len, back_factor=back)
+    x = synth.make_prefill(w, device="cuda:0")
+    q_s, q = (x[n][:, :, q_pos0:] for n in ("q_s", "q"))
+    host = P.host_inputs({"q_s": q_s, "q": q, "k": x["k"], "v": x["v"]})
+    code = synth.dtype_code(w.dtype)
+    params = sla.make_params(top_k, span_len, back, head_dim=128, window=window, mode=sla.SLA_PER_SPAN if window else sla.SLA_UNION)
+    ref_s = O.span_search(host["q_s"], host["k"], code, top_k=top_k, q_pos0=q_pos0, window=window)
+    anchor = torch.from_numpy(ref_s["anchor"]).cuda()
+    score = torch.from_numpy(ref_s["score"].astype(np.float32)).cuda()
+    if strided:
+        sh = rows * 128 + 8
+        dense, q = q, torch.zeros(batch * 32 * sh, dtype=q.dtype, device="cuda").as_strided(q.shape, (32 * sh, sh, 128, 1))
+        q.copy_(dense)
+    h = sla.Handle(0, sla.sla_workspace_bytes(sla.make_layout(q, x["k"]), params, chunk, L))
+    res = []
+    if window:
+        routes = claimed(lambda: res.extend(sla.sla_span_attention_gated(h, q, x["k"], x["v"], anchor, score, params)[:2]))
+    else:
+        routes = claimed(lambda: res.extend(sla.sla_span_attention(h, q, x["k"], x["v"], anchor, params, q_pos0=q_pos0)))
+    assert sla.sla_poll_status(h) == sla.SLA_OK
+    assert routes == [n * batch >= 8 * sms for n in [chunk] * (rows // chunk) + [rows % chunk] * (rows % chunk > 0)]
+    stats = sla.sla_attention_tile_stats(h)   # of the last chunk: streams of 128 pieces, two to a tile
+    assert stats["tiles"] > 2 * 6 * sms
+    kw = dict(mode=O.PER_SPAN, score=ref_s["score"], window=window) if window else {}
+    ref = O.span_attention(host["q"], host["k"], host["v"], code, ref_s["anchor"], span_len=span_len, back_factor=back, q_pos0=q_pos0, **kw)
+    P.compare_attention(res[0], res[1], ref, "bf16")
+    h.close()
 
 
 @pytest.mark.parametrize("kw", [
