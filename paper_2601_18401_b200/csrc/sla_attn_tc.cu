@@ -350,7 +350,6 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         ptx::mbar_arrive(bar_done);
                     }
                     if (++cv.j == cv.nblk) {
-                        lane_read(cv.k);
                         ok = read_tile(++cv.k);   // S has opened it before
                         open(cv);
                     }
@@ -380,6 +379,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         open(cs);
                     }
                 }
+                // a tile that PV has left is given back behind the S, which the row warps may be waiting for: 32 arrivals
+                // of a lane each (two sequences of 262144 positions 94.9 ms a call with them before it, 94.5 like this)
+                if (cv.j == 0 && cv.k > 0) lane_read(cv.k - 1);
             }
         } else if (warp == 14) {
             // ---------------- K/V producer: K and V of block after block, each as two halves of the head dimension
