@@ -273,10 +273,13 @@ __device__ inline void cta_select_topk(float *sc, int n, const Call &c, long lon
     const int gs = k <= 8 ? 32 : k <= 16 ? 16 : k <= 32 ? 8 : 4, n_groups = kAttnThreads / gs;
     // The scores are dealt to the groups in turn: no group is empty as soon as there are as many scores, however few.  (With
     // whole groups of neighbours, 90 scores filled three of eight groups, and all of them became candidates: a step of 8
-    // sequences of 8191 tokens, k = 8, 36 to 39 us, and 34 to 35 us like this.)
+    // sequences of 8191 tokens, k = 8, 37.2 to 37.7 us, and 34.4 to 36.7 us like this.)  Each turn starts at another group, so that
+    // the lanes of a warp read different banks (k <= 8; two of the same for k <= 16): without that, steps of 32/4 heads were
+    // up to 0.2 us longer than with neighbours (65536 tokens, k = 4: 13.90 and 13.78 us; 400000, k = 16: 58.2 and 58.1 us).
     unsigned mx = 0u;   // below every order key of a real score
+    const int turn = (tid % gs) * n_groups, of_turn = (tid / gs + turn / 32) % n_groups;
 #pragma unroll 1
-    for (int x = (tid % gs) * n_groups + tid / gs; x < n; x += kAttnThreads) mx = max(mx, max(topk::order_key(sc[x]), 1u));
+    for (int x = turn + of_turn; x < n; x += kAttnThreads) mx = max(mx, max(topk::order_key(sc[x]), 1u));
 #pragma unroll 1
     for (int off = 1; off < gs; off <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     if (tid % gs == 0) m.gmax[tid / gs] = mx;

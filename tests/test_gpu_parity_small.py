@@ -344,6 +344,23 @@ def test_decode_parity(sla, handle, dtype, D, Hq, Hkv):
                             n_ctx=n_ctx, top_k=top_k, span_len=span_len)
 
 
+@pytest.mark.parametrize("top_k", [1, 8, 9, 16, 17, 32, 33, 64])
+def test_decode_selection_edges(sla, handle, top_k):
+    """As many scores as slots, one more and one less, and numbers of scores around whole rounds of the 256 threads that
+    select: groups of threads without any score, with one, and with several."""
+    from paper_2601_18401_b200 import synth
+    w = synth.Workload("d", "decode", 1, 4, 1, 128, 514 * 514, "bf16", 8, top_k, seed=6)
+    kc, vc = synth.make_decode_cache(w, "cuda:0", capacity=w.seq_len)
+    hk, hv = synth.to_numpy(kc), synth.to_numpy(vc)
+    for scores in sorted({max(1, top_k - 1), top_k, top_k + 1, 31, 255, 256, 257, 513}):
+        n_ctx = scores * scores
+        step = synth.make_decode_step_inputs(w, n_ctx, "cuda:0")
+        got = sla.sla_decode_step(handle, step["q_s"], step["q"], kc, vc, n_ctx, sla.make_params(top_k, 8, head_dim=128))
+        torch.cuda.synchronize()
+        P.check_decode_step(got, synth.to_numpy(step["q_s"]), synth.to_numpy(step["q"]), hk, hv, synth.dtype_code("bf16"), "bf16",
+                            n_ctx=n_ctx, top_k=top_k, span_len=8)
+
+
 def test_bounded_wait_expiry_is_reported_and_survivable(sla, handle):
     """A device-side wait that runs out (a barrier nothing arrives on, a bounded number of polls) leaves the
     time-out bit in the status word and returns by itself; the handle reports it once and keeps working."""
