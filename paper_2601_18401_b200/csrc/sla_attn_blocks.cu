@@ -13,8 +13,8 @@
 //   merge   a row has one partial result per key block it touches, at a slot that only the row's own spans determine
 //           (first span that reaches the block, block within that span), combined in slot order.
 // Everything is fp32 FMA (two per instruction), as in the row kernel: bf16 inputs are widened exactly.
-// Bound by the FMA pipe and, at 12 to 16 warps an SM, by the latency of its chains: 105 instructions per key and 32 rows, 64
-// of them f32x2 (issue slots 40 % used; two thirds of the products belong to selected keys).  Search and attention together,
+// Bound by the FMA pipe and, at 12 to 16 warps an SM, by the latency of its chains: 64 f32x2 products per key and 32 rows
+// (issue slots 40 % used; two thirds of the products belong to selected keys).  Search and attention together,
 // row kernel and this one: 4096 positions, one head of 64 dims, top_k 4, spans of 129 keys 88 and 55 us; 3811 positions, one
 // head of 128 dims, top_k 8, spans of up to 125 keys 258 and 100 us; 7343 positions, two heads, 173 keys 479 and 301 us.
 #include <limits.h>

@@ -212,6 +212,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         for (int x = 0; x < 4; ++x) {
             ptx::mbar_init(bar_s_full + 8 * x, 1);
             ptx::mbar_init(bar_p_ready + 8 * x, 4);   // one arrival per row warp
+        }
+#pragma unroll 1
+        for (int x = 0; x < kTS; ++x) {
             ptx::mbar_init(bar_t_full + 8 * x, 1);
             ptx::mbar_init(bar_t_empty + 8 * x, kTileReaders);
         }
@@ -235,8 +238,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     // the role's tile; no records when none is left.  (The table has an entry for every CTA.)
     int4 ti = p.tiles[blockIdx.x];
     int2 rg;                          // blocks of its walk the streams take part in
-    if (kClaim && tid == 0) {
-        meta->tile[0] = ti;
+    if (kClaim && tid == 0) {   // the ring's first entry: every role has read the table's already, and takes the range only
         meta->range[0] = p.ranges[blockIdx.x];
         ptx::mbar_arrive(bar_t_full);
     }
@@ -250,14 +252,14 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     constexpr uint32_t kIdescS = ptx::idesc_bf16_f32(kHalf, kBK, false, false);   // S = Q K^T, both K-major
     constexpr uint32_t kIdescO = ptx::idesc_bf16_f32(kHalf, kD, false, true);       // O = P V, V is N-major
 
-    // The first two tiles of CTA c are c and c + grid of the table.  Of a long list the warp that gathers Q claims the others, in
-    // the order of the table, and passes each one's entry {b*Hkv+g, end block, first record, count | blocks << 9} on through a
-    // ring in shared memory; a short one is dealt round-robin, and every role reads the table itself.
-    // the claiming kernel has no room in the instruction cache for the longer form of the waits off the critical path
+    // Off the critical path the claiming kernel uses the shorter form of the waits, for the instruction cache.
     auto wait_aside = [&](uint32_t bar, uint32_t parity) {
         if constexpr (kClaim) return ptx::mbar_wait_short(bar, parity, abort_flag);
         else return ptx::mbar_wait(bar, parity, abort_flag);
     };
+    // The first two tiles of CTA c are c and c + grid of the table.  Of a long list the warp that gathers Q claims the others, in
+    // the order of the table, and passes each one's entry {b*Hkv+g, end block, first record, count | blocks << 9} on through a
+    // ring in shared memory; a short one is dealt round-robin, and every role reads the table itself.
     auto read_tile = [&](uint32_t k) {   // the CTA's k-th tile; every lane gets its own answer
         if constexpr (kClaim) {
             const bool got = ptx::mbar_wait_short(bar_t_full + 8 * (k % kTS), (k / kTS) & 1u, abort_flag);

@@ -35,8 +35,8 @@ struct PrepArgs {
     int *key_count;          // [B*Hkv][NB*ncls]: histogram, then exclusive offsets
     int *key_cursor;         // same shape
     int *totals;             // [B*Hkv][2]: records and tiles of each (batch, kv head)
-    int *n_tiles;            // total number of tiles; the number before they are split
-    int ctas;                // CTAs the tiles are dealt to
+    int *n_tiles;            // [0] number of tiles, [1] the number before they are split, [2] tiles claimed by tc_attend
+    int ctas;                // CTAs of tc_attend, which the tiles are dealt to or claimed by
     int4 *tiles;
     int2 *ranges;            // [max_tiles] blocks of the walk the tile's first and second 128 pieces reach: first | end << 16
     int max_tiles;

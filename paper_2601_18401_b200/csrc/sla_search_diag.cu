@@ -357,8 +357,8 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 // eight heads are rows 0..7 of the A operand (rows 8..15 are zero), the columns of B are the keys of eight strides.
 // Lane (r8, q) receives the scores of head r8 at strides s0 + 2q and s0 + 2q + 1, so that four lanes share a head; their
 // sorted lists are merged two at a time.  Every key row is fetched once for eight heads.
-// Bound by the latency of the key rows (a chunk half way through a long context reads them from DRAM) and by issue:
-// 320 instructions per warp and sixteen strides, four lists of K values per head.  4096 positions at 500001, 32/4 heads,
+// Bound by the latency of the key rows (a chunk half way through a long context reads them from DRAM) and by issue
+// (four lists of K values per head).  4096 positions at 500001, 32/4 heads,
 // K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
 // 484 us here, about 440 us with the tiles fetched a step ahead.
 template <int K>

@@ -25,7 +25,7 @@ struct RowId {
 };
 __device__ inline RowId decode_row(long long row, const Call &c) {
     RowId o;
-    if ((row | c.Lq) >> 32 == 0) {   // 64-bit divisions are a hundred instructions each
+    if ((row | c.Lq) >> 32 == 0) {   // 64-bit divisions take many times as long
         const unsigned t1 = (unsigned)row / (unsigned)c.G, bg = t1 / (unsigned)c.Lq;
         o.r = t1 - bg * (unsigned)c.Lq;
         o.b = (int)(bg / (unsigned)c.Hkv);
