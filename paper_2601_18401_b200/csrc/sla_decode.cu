@@ -277,7 +277,7 @@ __device__ inline void cta_select_topk(float *sc, int n, const Call &c, long lon
     // the lanes of a warp read different banks (k <= 8; two of the same for k <= 16): without that, steps of 32/4 heads were
     // up to 0.2 us longer than with neighbours (65536 tokens, k = 4: 13.90 and 13.78 us; 400000, k = 16: 58.2 and 58.1 us).
     unsigned mx = 0u;   // below every order key of a real score
-    const int turn = (tid % gs) * n_groups, of_turn = (tid / gs + turn / 32) % n_groups;
+    const int turn = (tid % gs) * n_groups, of_turn = (tid / gs + turn / 32) & (n_groups - 1);
 #pragma unroll 1
     for (int x = turn + of_turn; x < n; x += kAttnThreads) mx = max(mx, max(topk::order_key(sc[x]), 1u));
 #pragma unroll 1
