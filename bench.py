@@ -39,7 +39,7 @@ UNIT = "tokens/s"
 # dram__bytes_read.sum + dram__bytes_write.sum of one tc_attend launch of the default workload
 # (L = 65536): a CONSTANT taken from the one-pass ncu capture of the full-size launch summarised in
 # the profiles folder, not something this run measures
-TC_ATTEND_DRAM_BYTES_PER_LAUNCH = {65536: 4.69e9, 16384: 0.757e9}
+TC_ATTEND_DRAM_BYTES_PER_LAUNCH = {65536: 4.39e9, 16384: 0.734e9}
 TRAFFIC_SOURCE = "constant from the one-pass ncu capture summarised under profiles/, not measured by this run"
 NOMINAL_BF16_TFLOPS = 2250.0   # dense bf16, per GPU
 # the same for one decode_attn launch (the dominant kernel of a decode step), by workload

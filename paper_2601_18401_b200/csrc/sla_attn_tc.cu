@@ -18,8 +18,8 @@
 // gathered into shared memory and the tile walks the key blocks they cover from left to right.
 //
 //   tc::prepare          the counting sort and the tile table (sla_attn_prep.cu)
-//   tc_attend            persistent CTAs; tiles are claimed in the order of the table (short lists: tile t
-//                        goes to CTA t mod grid); per tile and key block: S = Q K^T (tcgen05, smem x smem -> TMEM), row
+//   tc_attend            persistent CTAs; tiles are claimed in the order of the table (short lists and short
+//                        walks: tile t goes to CTA t mod grid); per tile and key block: S = Q K^T (tcgen05, smem x smem -> TMEM), row
 //                        softmax in registers, P (bf16) back into TMEM, O += P V (tcgen05, TMEM x smem
 //                        -> TMEM); per piece a normalised fp16 block-floating-point partial + lse
 //   tc_merge             per row: log-sum-exp merge of its pieces -> out, lse
@@ -38,8 +38,8 @@
 // Before, two independent CTAs per SM of 128 pieces each, whose row threads also gathered Q and wrote results:
 // 1860 cycles a block in long tiles but 5300 more per tile; now 700 per tile.  Configuration of 65536 tokens, 11
 // blocks per tile: 4.07 -> 3.45 ms; 16384 tokens, 7 blocks: 658 -> 570 us.
-// Two things that the times depend on: the kernel's code has to fit the instruction cache (about 2300
-// instructions, 2700 with the claims; at 3300 the hit rate is 93 %, at 3500 77 % and everything takes a half longer), and the issuing warps have to
+// Two things that the times depend on: the kernel's code has to fit the instruction cache (sm__icc_request_hit_rate at 16384
+// positions: 99.8 % dealt, 99.5 % claiming; a larger variant that was 5 % slower had 93 %), and the issuing warps have to
 // run converged with one elected lane issuing (see ptx::elect_one): the issuers' time per block bounded the
 // streams at 2500 cycles otherwise.
 #include <cuda.h>
@@ -75,9 +75,9 @@ constexpr int kKS = 3;           // K and V stages
 constexpr int kTS = 4;           // entries of the ring of tiles
 // A list is claimed tile by tile if it can have kClaimTiles tiles per CTA (every slot of every row taken) and its longest single
 // piece, a span or the window, can cover kClaimBlocks key blocks (kClaimBlocksJoined where touching spans are joined, which
-// makes the walks longer).  Dealt round-robin, the CTAs of a long list end at different times: they were busy for 0.88 of the
-// kernel at 16384 positions, 0.95 at 65536.  Tiles of short walks are over too soon for that, and pass the ring later than the
-// table would have been read.  The kernel, 32/8 heads, eight spans, dealt and claimed, us (runs of one side differ by 1 to 5 %):
+// makes the walks longer).  Dealt round-robin, the CTAs of a long list end at different times: SMs were busy for 0.87 of the
+// kernel at 16384 positions and 0.94 at 65536, and are for 0.95 and 0.97 claimed (553 and 521 us; 3569 and 3491 us).  Tiles of short
+// walks lose more by the claims than by that.  The kernel, 32/8 heads, eight spans, dealt and claimed, us (runs of one side differ by 1 to 5 %):
 //   joined, from position 0    16384, spans of 65 / 129 / 193 / 257 keys (3 / 4 / 5 / 6 blocks)
 //                                                597, 658 / 590, 628 / 667, 651 / 735, 707
 //                              65536, the same   2529, 2828 / 2752, 2812 / 2950, 2926 / 3593, 3119
