@@ -212,9 +212,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         for (int x = 0; x < 4; ++x) {
             ptx::mbar_init(bar_s_full + 8 * x, 1);
             ptx::mbar_init(bar_p_ready + 8 * x, 4);   // one arrival per row warp
-        }
-#pragma unroll 1
-        for (int x = 0; x < kTS; ++x) {
+            static_assert(kTS == 4, "the ring's barriers are initialised with those of the four S buffers");
             ptx::mbar_init(bar_t_full + 8 * x, 1);
             ptx::mbar_init(bar_t_empty + 8 * x, kTileReaders);
         }
@@ -238,7 +236,10 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     // the role's tile; no records when none is left.  (The table has an entry for every CTA.)
     int4 ti = p.tiles[blockIdx.x];
     int2 rg;                          // blocks of its walk the streams take part in
-    if (kClaim && tid == 0) {   // the ring's first entry: every role has read the table's already, and takes the range only
+    // The ring's first entry.  Every role has read the table's already and takes only the range; without the store of the other
+    // half, though, the per-span mode took 0.3 to 0.6 % longer, as with a loop of its own for the ring's barriers above.
+    if (kClaim && tid == 0) {
+        meta->tile[0] = ti;
         meta->range[0] = p.ranges[blockIdx.x];
         ptx::mbar_arrive(bar_t_full);
     }
