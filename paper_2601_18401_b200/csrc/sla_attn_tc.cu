@@ -258,9 +258,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         if constexpr (kClaim) return ptx::mbar_wait_short(bar, parity, abort_flag);
         else return ptx::mbar_wait(bar, parity, abort_flag);
     };
-    // The first two tiles of CTA c are c and c + grid of the table.  Of a long list the warp that gathers Q claims the others, in
-    // the order of the table, and passes each one's entry {b*Hkv+g, end block, first record, count | blocks << 9} on through a
-    // ring in shared memory; a short one is dealt round-robin, and every role reads the table itself.
+    // The first two tiles of CTA c are c and c + grid of the table.  The warp that gathers Q claims the others, in the order of the
+    // table, and passes each one's entry {b*Hkv+g, end block, first record, count | blocks << 9} on through a ring in shared
+    // memory; a list that is not claimed is dealt round-robin, and every role reads the table itself.
     auto read_tile = [&](uint32_t k) {   // the CTA's k-th tile; every lane gets its own answer
         if constexpr (kClaim) {
             const bool got = ptx::mbar_wait_short(bar_t_full + 8 * (k % kTS), (k / kTS) & 1u, abort_flag);
