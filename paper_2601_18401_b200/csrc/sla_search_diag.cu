@@ -33,11 +33,15 @@ namespace sla {
 namespace {
 
 using bf16 = __nv_bfloat16;
-constexpr int kWarps = 8;
+constexpr int kWarps = 4;
 constexpr int kQW = 4;   // query positions per warp
 constexpr int kG = 4;    // query heads per KV head
 
-template <int K> struct ListCap { static constexpr int value = (2 * K + 8 + 3) / 4 * 4; };
+// Entries of a lane's list: of a hundred scores in random order 2 + 2 ln 50 = 10 are among the two best so far, 18, 28 and 45
+// among the four, eight and sixteen best, and a list that runs full costs all lanes of the warp a pass over theirs.  (48 entries
+// for K = 16 are what four CTAs of an SM have room for; with 52, which leave three, 4096 positions at 500001 took 496 us
+// instead of 373.)
+template <int K> struct ListCap { static constexpr int value = K == 2 ? 16 : K == 4 ? 24 : K == 8 ? 32 : 48; };
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                uint32_t b0, uint32_t b1) {
@@ -45,6 +49,14 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// The first of a chain: no accumulators to clear.
+__device__ __forceinline__ void mma_bf16_16816_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                                     uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // 32 bytes per lane in one load: the four lanes of a quad cover a whole 128-byte line of a row, so a warp's
@@ -116,19 +128,25 @@ __device__ __forceinline__ void merge_pairs(float (&x)[K], int (&s)[K], int off)
             }
 }
 
-// A lane's running top-k: the K best values so far, sorted, in registers, and in shared memory (entry e at lx[32 e],
-// ls[32 e]) every score with its stride index that beat the K-th best when it arrived.
+// A lane's running top-k: the K best values so far, sorted, in registers, and in shared memory (entry e at list[32 e]) every
+// score with its stride index that beat the K-th best when it arrived.
 template <int K>
 struct RunningTop {
     static constexpr int CAP = ListCap<K>::value;
     float v[K];
-    int cnt;
-    float *lx;
-    int *ls;
-    __device__ __forceinline__ RunningTop(float *warp_lists, int lane)
-        : cnt(0), lx(warp_lists + lane), ls(reinterpret_cast<int *>(warp_lists + CAP * 32) + lane) {
+    uint32_t list, end;   // shared-memory addresses of the lane's first entry and behind its last; 256 bytes from entry to entry
+    __device__ __forceinline__ RunningTop(float2 *warp_lists, int lane)
+        : list(static_cast<uint32_t>(__cvta_generic_to_shared(warp_lists + lane))), end(list) {
 #pragma unroll
         for (int j = 0; j < K; ++j) v[j] = -CUDART_INF_F;
+    }
+    static __device__ __forceinline__ void put(uint32_t at, float x, int s) {
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(__float_as_int(x)), "r"(s) : "memory");
+    }
+    static __device__ __forceinline__ void get(uint32_t at, float &x, int &s) {
+        int w;
+        asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(w), "=r"(s) : "r"(at) : "memory");
+        x = __int_as_float(w);
     }
     // Drops the list entries that can no longer be among the K best (all lanes, each its own list):
     // what is left are the entries above the K-th best value and the earliest of those equal to it,
@@ -138,42 +156,36 @@ struct RunningTop {
         int allow_eq = K;
 #pragma unroll
         for (int j = 0; j < K; ++j) allow_eq -= v[j] > vk;
-        int w = 0;
-        for (int e0 = 0; e0 < cnt; e0 += 4) {   // four loads at a time: the list is as long as a multiple of four
+        uint32_t w = list;
+        for (uint32_t e = list; e < end; e += 1024) {   // four loads at a time: the list is as long as a multiple of four
             float x[4];
             int s[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                x[u] = lx[32 * (e0 + u)];
-                s[u] = ls[32 * (e0 + u)];
-            }
+            for (int u = 0; u < 4; ++u) get(e + 256 * u, x[u], s[u]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const bool eq = x[u] == vk;
-                if (e0 + u < cnt && (x[u] > vk || (eq && allow_eq > 0))) {
+                if (e + 256 * u < end && (x[u] > vk || (eq && allow_eq > 0))) {
                     allow_eq -= eq;
-                    lx[32 * w] = x[u];
-                    ls[32 * w] = s[u];
-                    ++w;
+                    put(w, x[u], s[u]);
+                    w += 256;
                 }
             }
         }
-        cnt = w;
+        end = w;
     }
     // Two new scores, sa < sb.  Each one that beats the K-th best so far goes to the list; the sorted values take
     // both in one pass: with hi >= lo the new j-th best is max(v[j], min(v[j-1], hi), min(v[j-2], lo)).
     __device__ __forceinline__ void offer2(int sa, float xa, int sb, float xb) {
-        if (__any_sync(0xffffffffu, cnt >= CAP - 1)) compact();   // room for both scores
+        if (__any_sync(0xffffffffu, end - list >= 256 * (CAP - 1))) compact();   // room for both scores
         const float vk = v[K - 1];
         if (xa > vk) {
-            lx[32 * cnt] = xa;
-            ls[32 * cnt] = sa;
-            ++cnt;
+            put(end, xa, sa);
+            end += 256;
         }
         if (xb > vk) {
-            lx[32 * cnt] = xb;
-            ls[32 * cnt] = sb;
-            ++cnt;
+            put(end, xb, sb);
+            end += 256;
         }
         const float hi = fmaxf(xa, xb), lo = fminf(xa, xb);
 #pragma unroll
@@ -186,9 +198,11 @@ struct RunningTop {
         compact();
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const bool on = j < cnt;
-            x[j] = on ? lx[32 * j] : -CUDART_INF_F;
-            s[j] = on ? ls[32 * j] : INT_MAX;
+            get(list + 256 * j, x[j], s[j]);
+            if (list + 256 * j >= end) {
+                x[j] = -CUDART_INF_F;
+                s[j] = INT_MAX;
+            }
         }
         sort_pairs<K>(x, s);
     }
@@ -216,11 +230,53 @@ struct NextBest {
     __device__ __forceinline__ void take() { taken = key; at = s; key = 0u; s = INT_MAX; }
 };
 
-template <int K>
-__global__ void __launch_bounds__(kWarps * 32, 2)
+// What bounds search_diag: the latency of the key rows (L2, a step ahead of their use in 32 registers) and of the step's chains at
+// 16 warps an SM; issue slots 48 % used, L2 at 45 %.  Operations taken out of the step -- accumulators cleared by moves, strides
+// squared and compared per fetch, two stores and 64-bit addresses per list entry -- and CTAs of four warps instead of eight: 16384
+// positions, 32/8 heads, K = 8 250 -> 227 us; 65536 1583 -> 1437; two sequences of 262144, 16/4 heads, K = 16 14.28 -> 12.46 ms;
+// 32768, K = 2 751 -> 673 us.  Five CTAs an SM (96 registers) spill: 240 us for the first of these.
+//
+// The strides a lane fetches, one after another: key positions i + 1 - offset(s), i + 1 - offset(s + step), ...  On the
+// quadratic pattern the distance to the next one, 2 step (s + 1) + step^2, itself grows by 2 step^2.  A position without the
+// stride (s >= n) gets key 0: a valid row either way.
+template <bool kTable>
+struct KeyWalk {
+    const char *base;
+    unsigned pitch;       // bytes
+    int t, d, s, dd;      // kTable: t the query position
+    const int *off;
+    int n;
+    __device__ __forceinline__ KeyWalk(const bf16 *k, const Call &c, int i, int s0, int step, int n_)
+        : base(reinterpret_cast<const char *>(k)), pitch((unsigned)c.kv_st * 2u), off(c.off), n(n_) {
+        if constexpr (kTable) {
+            t = i; s = s0; d = step;
+        } else {
+            t = s0 < n ? i + 1 - (s0 + 1) * (s0 + 1) : -1;   // (the square of a stride that exists fits 31 bits)
+            d = step * (2 * (s0 + 1) + step);
+            dd = 2 * step * step;
+        }
+    }
+    __device__ __forceinline__ void next(Words8 (&kb)[2]) {
+        unsigned at;
+        if constexpr (kTable) {
+            at = s < n ? (unsigned)(t + 1 - off[s]) : 0u;
+            s += d;
+        } else {
+            at = (unsigned)max(t, 0);
+            t -= d;
+            d += dd;
+        }
+        const char *row = base + (unsigned long long)at * pitch;
+        kb[0] = ldg256(row);
+        kb[1] = ldg256(row + 128);
+    }
+};
+
+template <int K, bool kTable>
+__global__ void __launch_bounds__(kWarps * 32, 4)
 search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
             float *__restrict__ out_score) {
-    extern __shared__ float smem[];
+    extern __shared__ float2 smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r8 = lane >> 2, q = lane & 3;
     // the tiles with the most strides (the last positions) start first
@@ -266,23 +322,16 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     const int n_max = full_group ? n_at(i0 + kQW - 1) : n_at((int)(c.q_pos0 + last));
     const int n_all = full_group ? n0 : s_min;   // strides below n_all exist for every position of the warp
 
-    const bf16 *kbase = k + b * c.kv_sb + g * c.kv_sh + 16 * q;
-    const int kv_st = (int)c.kv_st;
-    auto fetch = [&](int s0, Words8 (&kb)[2]) {
-        const int s = s0 + u_ld;
-        int t = i_ld + 1 - stride_offset(c, s < c.n_off || !c.off ? s : 0);
-        if (s >= n_ld) t = i_ld;   // a valid row either way
-        const bf16 *row = kbase + (long long)t * kv_st;
-        kb[0] = ldg256(row);
-        kb[1] = ldg256(row + 64);
-    };
+    KeyWalk<kTable> walk(k + b * c.kv_sb + g * c.kv_sh + 16 * q, c, i_ld, s_min + u_ld, 2, n_ld);
 
-    RunningTop<K> top(smem + (size_t)warp * (2 * RunningTop<K>::CAP * 32), lane);
+    RunningTop<K> top(smem + (size_t)warp * (RunningTop<K>::CAP * 32), lane);
     // scores of one B tile (two strides): two independent accumulation chains, added at the end
     auto score = [&](const Words8 (&kb)[2]) -> float {
-        float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+        float a0[4], a1[4];
+        mma_bf16_16816_first(a0, qa[0].w[0], qb[0].w[0], qa[0].w[1], qb[0].w[1], kb[0].w[0], kb[0].w[1]);
+        mma_bf16_16816_first(a1, qa[1].w[0], qb[1].w[0], qa[1].w[1], qb[1].w[1], kb[1].w[0], kb[1].w[1]);
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
+        for (int x = 1; x < 4; ++x) {
             mma_bf16_16816(a0, qa[0].w[2 * x], qb[0].w[2 * x], qa[0].w[2 * x + 1], qb[0].w[2 * x + 1], kb[0].w[2 * x], kb[0].w[2 * x + 1]);
             mma_bf16_16816(a1, qa[1].w[2 * x], qb[1].w[2 * x], qa[1].w[2 * x + 1], qb[1].w[2 * x + 1], kb[1].w[2 * x], kb[1].w[2 * x + 1]);
         }
@@ -295,13 +344,13 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
     Words8 ka[2], kb[2];
     int s0 = s_min;
     float zero = 0.f;   // zero times the scores: NaN once one of them is not finite
-    fetch(s0, ka);
-    fetch(s0 + 2, kb);
+    walk.next(ka);
+    walk.next(kb);
     for (; s0 + 4 <= n_all; s0 += 4) {
         const float xa = score(ka);
-        fetch(s0 + 4, ka);
+        walk.next(ka);
         const float xb = score(kb);
-        fetch(s0 + 6, kb);
+        walk.next(kb);
         zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
     }
@@ -312,8 +361,8 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
         if (s0 + 4 < n_max) {
-            fetch(s0 + 4, ka);
-            fetch(s0 + 6, kb);
+            walk.next(ka);
+            walk.next(kb);
         }
     }
 
@@ -324,7 +373,7 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         for (int j = 0; j < c.top_k; ++j) {
 #pragma unroll 1
             for (int s1 = s_min; s1 < n_max; s1 += 2) {
-                fetch(s1, ka);
+                KeyWalk<kTable>(k + b * c.kv_sb + g * c.kv_sh + 16 * q, c, i_ld, s1 + u_ld, 2, n_ld).next(ka);
                 const float x = score(ka);
                 if (s1 + u_own < n_own) next.offer(s1 + u_own, x);
             }
@@ -360,12 +409,14 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 // Bound by the latency of the key rows (a chunk half way through a long context reads them from DRAM) and by issue
 // (four lists of K values per head).  4096 positions at 500001, 32/4 heads,
 // K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
-// 484 us here, about 440 us with the tiles fetched a step ahead.
-template <int K>
-__global__ void __launch_bounds__(kWarps * 32, 2)
+// 484 us here, about 440 us with the tiles fetched a step ahead, 373 us (from 407 on the same GPU) with the shorter step.
+// Half of the A operand is zero, so that five CTAs fit an SM up to K = 8 with few spills (28 bytes at K = 8): 16384 positions, 32/4
+// heads, K = 8 253 us with four CTAs, 234 with five; 2048 at 300000 141 and 120; K = 2 152 and 140, 123 and 102.
+template <int K, bool kTable>
+__global__ void __launch_bounds__(kWarps * 32, K <= 8 ? 5 : 4)
 search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, int32_t *__restrict__ out_anchor,
              float *__restrict__ out_score) {
-    extern __shared__ float smem[];
+    extern __shared__ float2 smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r8 = lane >> 2, q = lane & 3;
     // the tiles with the most strides (the last positions) start first
@@ -384,21 +435,15 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     // Algorithm 1: anchors inside the local window are no candidates; t_s lies in W iff offset(s) <= w
     const int s_min = c.window > 0 ? window_strides(c) : 0;
     const bf16 *kbase = k + b * c.kv_sb + g * c.kv_sh + 16 * q;
-    const int kv_st = (int)c.kv_st;
-    auto fetch = [&](int s0, Words8 (&kb)[2]) {   // column r8: the key of stride s0 + r8
-        const int s = s0 + r8;
-        int t = i + 1 - stride_offset(c, s < c.n_off || !c.off ? s : 0);
-        if (s >= n) t = i;   // a valid row either way
-        const bf16 *row = kbase + (long long)t * kv_st;
-        kb[0] = ldg256(row);
-        kb[1] = ldg256(row + 64);
-    };
-    RunningTop<K> top(smem + (size_t)warp * (2 * RunningTop<K>::CAP * 32), lane);
+    KeyWalk<kTable> walk(kbase, c, i, s_min + r8, 8, n);   // column r8: the keys of strides s_min + r8, + 8, ...
+    RunningTop<K> top(smem + (size_t)warp * (RunningTop<K>::CAP * 32), lane);
     // two independent accumulation chains, added at the end
     auto score = [&](const Words8 (&kb)[2], float &x0, float &x1) {
-        float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+        float a0[4], a1[4];
+        mma_bf16_16816_first(a0, qa[0].w[0], 0u, qa[0].w[1], 0u, kb[0].w[0], kb[0].w[1]);
+        mma_bf16_16816_first(a1, qa[1].w[0], 0u, qa[1].w[1], 0u, kb[1].w[0], kb[1].w[1]);
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
+        for (int x = 1; x < 4; ++x) {
             mma_bf16_16816(a0, qa[0].w[2 * x], 0u, qa[0].w[2 * x + 1], 0u, kb[0].w[2 * x], kb[0].w[2 * x + 1]);
             mma_bf16_16816(a1, qa[1].w[2 * x], 0u, qa[1].w[2 * x + 1], 0u, kb[1].w[2 * x], kb[1].w[2 * x + 1]);
         }
@@ -409,17 +454,17 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     Words8 ka[2], kb[2];
     int s0 = s_min;
     float zero = 0.f;   // zero times the scores: NaN once one of them is not finite
-    fetch(s0, ka);
-    fetch(s0 + 8, kb);
+    walk.next(ka);
+    walk.next(kb);
     for (; s0 + 16 <= n; s0 += 16) {
         const int s = s0 + 2 * q;
         float xa, xb;
         score(ka, xa, xb);
-        fetch(s0 + 16, ka);
+        walk.next(ka);
         zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s, xa, s + 1, xb);
         score(kb, xa, xb);
-        fetch(s0 + 24, kb);
+        walk.next(kb);
         zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
         top.offer2(s + 8, xa, s + 9, xb);
     }
@@ -443,7 +488,7 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
             for (int s1 = s_min; s1 < n; s1 += 8) {
                 const int s = s1 + 2 * q;
                 float xa, xb;
-                fetch(s1, ka);
+                KeyWalk<kTable>(kbase, c, i, s1 + r8, 8, n).next(ka);
                 score(ka, xa, xb);
                 if (s < n) next.offer(s, xa);
                 if (s + 1 < n) next.offer(s + 1, xb);
@@ -476,15 +521,17 @@ template <int K>
 cudaError_t launch_k(const bf16 *q_s, const bf16 *k, const Call &c, int32_t *oa, float *os, cudaStream_t st) {
     constexpr size_t smem = (size_t)kWarps * 2 * ListCap<K>::value * 32 * sizeof(float);
     const bool four = c.G == kG;
-    void (*kern)(const bf16 *, const bf16 *, Call, int32_t *, float *) = four ? search_diag<K> : search_rows8<K>;
-    static bool attr_set[64][2] = {};
+    const bool table = c.off != nullptr;
+    void (*kern)(const bf16 *, const bf16 *, Call, int32_t *, float *) =
+        four ? (table ? search_diag<K, true> : search_diag<K, false>) : table ? search_rows8<K, true> : search_rows8<K, false>;
+    static bool attr_set[64][4] = {};
     if (smem > 48 * 1024) {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-        if (dev < 0 || dev >= 64 || !attr_set[dev][four]) {
+        if (dev < 0 || dev >= 64 || !attr_set[dev][2 * four + table]) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) attr_set[dev][four] = true;
+            if (dev >= 0 && dev < 64) attr_set[dev][2 * four + table] = true;
         }
     }
     const int rows = kWarps * (four ? kQW : 1);   // positions per CTA

@@ -170,6 +170,30 @@ def test_search_of_scores_that_are_not_finite(sla, handle, heads, top_k):
             assert (anchor[0, h, i, n:] == -1).all() and torch.isneginf(score[0, h, i, n:]).all()
 
 
+@pytest.mark.parametrize("window", [0, 1, 24, 25, 400, 2**31 - 1])
+@pytest.mark.parametrize("heads", [4, 8, 16])
+def test_search_walk_of_strides(sla, handle, heads, window):
+    """Groups of 4, 8 and 16 query heads at lengths around the positions of a warp and of a block, windows that leave all,
+    some or no strides (the largest has a stride whose square exceeds 31 bits); scores exact in any order of summation."""
+    import torch
+    g = torch.Generator().manual_seed(29)
+    for L, pos0, top_k in ((1, 0, 1), (3, 0, 2), (5, 0, 8), (15, 2, 4), (17, 0, 16), (33, 30, 8), (402, 380, 4), (1100, 1059, 16)):
+        q, k = ((torch.randn(1, h, n, 128, generator=g) * 64).round() / 64 for h, n in ((heads, L - pos0), (1, L)))
+        q, k = q.bfloat16(), k.bfloat16()
+        params = sla.make_params(top_k, 8, window=window, head_dim=128)
+        anchor, score = sla.sla_span_search(handle, q.cuda(), k.cuda(), params, q_pos0=pos0)
+        torch.cuda.synchronize()
+        anchor, score, q, k = anchor.cpu(), score.cpu(), q.double(), k.double()
+        for i in range(pos0, L):
+            t = torch.tensor([i + 1 - s * s for s in range(1, i + 2) if window < s * s <= i + 1], dtype=torch.long)
+            x = torch.einsum("hd,td->ht", q[0, :, i - pos0], k[0, 0, t])
+            order = torch.sort(x, dim=1, descending=True, stable=True).indices[:, :top_k]
+            n = order.shape[1]
+            a, v = anchor[0, :, i - pos0], score[0, :, i - pos0]
+            assert torch.equal(a[:, :n].long(), t[order]) and torch.equal(v[:, :n], x.gather(1, order).float()), (L, i)
+            assert (a[:, n:] == -1).all() and torch.isneginf(v[:, n:]).all()
+
+
 @pytest.mark.parametrize("by_blocks,kw", [
     # few keys a row, few rows (at the start, or far into a context), or blocks that few rows select
     (False, dict(seq_len=1, top_k=6, span_len=300)), (False, dict(seq_len=65, top_k=64, span_len=2)),
