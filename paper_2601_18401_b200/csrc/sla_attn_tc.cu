@@ -720,73 +720,132 @@ copy_q_rows(const bf16 *__restrict__ q, Call c, long long r0, int Lc, bf16 *__re
     *reinterpret_cast<uint4 *>(dst + row * kD + sub * 8) = __ldg(reinterpret_cast<const uint4 *>(src));
 }
 
-// Per row: merge the normalised piece outputs through their log-sum-exp.  16 threads per row.
-__global__ void __launch_bounds__(256)
+// Per row: merge the normalised piece outputs through their log-sum-exp.  A warp takes per_warp consecutive rows (a power of
+// two, 2 to 32): first 32 / per_warp lanes each work out a row's weights and write its lse, then every half of the warp adds up
+// every other row's pieces, 8 columns per lane, four pieces at a time with the next four already requested.  The last rows come
+// first: their partial results were written last, and what the L2 still holds of them is read from there.
+// Bound by the reads of the partial results (3.2 GB at 65536 positions, 32 heads, eight spans: 6.6 TB/s).  With 16 lanes that
+// all worked out their row's weights, issue slots were 72 % used and the loads of a row waited for the sum of the one before:
+// 637 us, and 480 like this; 16384 positions 152 and 114 us, 1999 positions, four spans 19.6 and 15.7 (ncu).
+// Rows of a warp: up to kMergePieces slots -- fewer pieces in a row cost more for the weights, more make the last warps' turn
+// long -- and as many warps as keep the loads going.  16 and 8 rows of 16 slots: 131072 rows 101 and 97 us (93 before); 32 and 16 rows of 2
+// slots: 960000 rows 123 and 129 us (207 before); 16, 8 and 4 rows of 8 slots: 128000 rows 40, 44 and 46 us (47 before), 16000 rows
+// 16.0, 12.0 and 10.4 (10.2 before).
+constexpr int kMergeWarps = 4;      // of a CTA
+constexpr int kMergePieces = 128;   // slots a warp takes at most, with two rows or more
+constexpr int kMergeFill = 19;      // warps an SM at least, down to two rows a warp
+__global__ void __launch_bounds__(kMergeWarps * 32, 8)
 tc_merge(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
-         const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0,
+         const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0, int per_warp,
          bf16 *__restrict__ out, float *__restrict__ lse) {
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long row = gid >> 4;
-    const int sub = (int)(gid & 15);
+    extern __shared__ float2 s_weight[];   // [rows of the CTA][slots, an odd number] {weight, chunk exponents; 0: no part in the result}
+    const int lane = threadIdx.x & 31;
+    const long long row0 = ((long long)(gridDim.x - 1 - blockIdx.x) * kMergeWarps + (threadIdx.x >> 5)) * per_warp;
     const long long rows = (long long)c.B * c.Hq * Lc;
     chain_wait();
-    if (row >= rows) return;
-    const int cnt = n_pieces[row];
-    const float2 *pl = part_lse + row * slots;
-    const __half *po = part_o + row * slots * kD + sub * 8;
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    // running maximum and denominator (log2 domain); the pieces come four at a time so that their
-    // loads are in flight together
-    float mx = -CUDART_INF_F, den = 0.f;
-    for (int j0 = 0; j0 < cnt; j0 += 4) {
-        float2 pj[4];
-        uint4 raw[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool on = j0 + u < cnt;
-            pj[u] = on ? __ldg(pl + j0 + u) : make_float2(-CUDART_INF_F, 0.f);
-            raw[u] = on ? __ldg(reinterpret_cast<const uint4 *>(po + (long long)(j0 + u) * kD)) : make_uint4(0, 0, 0, 0);
+    if (row0 >= rows) return;
+    // ---- weights: 32 / per_warp lanes per row
+    const int lanes = 32 / per_warp, pitch = slots | 1;   // odd: the lanes' rows start in different banks
+    __shared__ int4 s_row[kMergeWarps][32];   // {offset of the row in `out` (two words), reciprocal denominator, pieces}
+    int4 *rows_of = s_row[threadIdx.x >> 5];
+    float2 *sw = s_weight + (threadIdx.x >> 5) * per_warp * pitch;
+    {
+        const int own = lane / lanes, first = lane % lanes;
+        const long long row = row0 + own < rows ? row0 + own : rows - 1;   // rows past the last: that one again
+        const int cnt = n_pieces[row];
+        const float2 *pl = part_lse + row * slots;
+        float2 *mine = sw + own * pitch;
+        float mx = -CUDART_INF_F, den = 0.f;
+#pragma unroll 4
+        for (int j = first; j < cnt; j += lanes) {
+            const float2 pj = __ldg(pl + j);
+            mine[j] = pj;
+            mx = fmaxf(mx, pj.x);
         }
-        float bm = fmaxf(fmaxf(pj[0].x, pj[1].x), fmaxf(pj[2].x, pj[3].x));
-        if (bm > mx) {
-            const float r = mx == -CUDART_INF_F ? 0.f : exp2f(mx - bm);
-            den *= r;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] *= r;
-            mx = bm;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (pj[u].x == -CUDART_INF_F) continue;
-            const float w = exp2f(pj[u].x - mx);
+        for (int o = 1; o < lanes; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        for (int j = first; j < cnt; j += lanes) {
+            const float2 pj = mine[j];
+            const bool on = pj.x != -CUDART_INF_F;
+            const float w = on ? exp2f(pj.x - mx) : 0.f;
             den += w;
-            const uint32_t eb = (__float_as_uint(pj[u].y) >> (8 * (sub >> 2))) & 0xffu;
-            const float ws = w * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
+            mine[j] = make_float2(w, on ? pj.y : 0.f);
+        }
+        for (int o = 1; o < lanes; o <<= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+        const int rc = (int)((unsigned)row % (unsigned)Lc);   // rows < 2^31
+        const int bh = (int)((unsigned)row / (unsigned)Lc);
+        const int h = bh % c.Hq, b = bh / c.Hq;
+        const long long r = r0 + rc, off = b * c.q_sb + h * c.q_sh + r * c.q_st;
+        if (first == 0) {
+            rows_of[own] = make_int4((int)off, (int)(off >> 32), __float_as_int(den > 0.f ? 1.f / den : 0.f), cnt);
+            lse[((long long)b * c.Hq + h) * c.Lq + r] = den > 0.f ? (mx + log2f(den)) * kLn2 : -CUDART_INF_F;
+        }
+    }
+    __syncwarp();
+    // ---- 16 lanes per row: its pieces four at a time, the next four (of this row or of the next but one) requested before the
+    // ones in hand are added up
+    const int sub = lane & 15, shift = 8 * (sub >> 2);
+    const int last = (int)(rows - 1 - row0 < per_warp - 1 ? rows - 1 - row0 : per_warp - 1);
+    const __half *po = part_o + row0 * slots * kD + sub * 8;
+    auto load = [&](uint4 (&raw)[4], int row, int j, int n) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (j + u < n) raw[u] = __ldg(reinterpret_cast<const uint4 *>(po + (long long)(row * slots + j + u) * kD));
+    };
+    unsigned long long acc[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[e] = pack2(0.f, 0.f);
+    auto add = [&](const uint4 (&raw)[4], int row, int j, int n) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j + u >= n) break;
+            const float2 w = sw[row * pitch + j + u];
+            const uint32_t exps = __float_as_uint(w.y);
+            if (exps == 0u) continue;
+            const float ws = w.x * __uint_as_float((((exps >> shift) & 0xffu) + 1u) << 23);   // weight x 2^(eb - 126)
+            const unsigned long long ww = pack2(ws, ws);
             const uint32_t rw[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rw[e]));
-                acc[2 * e] = fmaf(ws, f.x, acc[2 * e]);
-                acc[2 * e + 1] = fmaf(ws, f.y, acc[2 * e + 1]);
+                acc[e] = ffma2(pack2(f.x, f.y), ww, acc[e]);
             }
         }
-    }
-    const float inv = den > 0.f ? 1.f / den : 0.f;
-    const int rc = (int)((unsigned)row % (unsigned)Lc);   // rows < 2^31
-    const int bh = (int)((unsigned)row / (unsigned)Lc);
-    const int h = bh % c.Hq, b = bh / c.Hq;
-    const long long r = r0 + rc;
-    uint32_t w[4];
+    };
+    int row = lane >> 4, j = 0, n = row <= last ? rows_of[row].w : 0;
+    uint4 raw[2][4];
+    load(raw[0], row, j, n);
+    for (;;) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const __nv_bfloat162 pp = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
-        w[e] = *reinterpret_cast<const uint32_t *>(&pp);
+        for (int y = 0; y < 2; ++y) {
+            int row2 = row, j2 = j + 4, n2 = n;
+            if (j2 >= n) {
+                row2 = row + 2;
+                j2 = 0;
+                n2 = row2 <= last ? rows_of[row2].w : 0;
+            }
+            load(raw[y ^ 1], row2, j2, n2);
+            add(raw[y], row, j, n);
+            if (row2 != row) {
+                if (row <= last) {
+                    const int4 ri = rows_of[row];
+                    const float f = __int_as_float(ri.z);
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float a0, a1;
+                        unpack2(acc[e], a0, a1);
+                        const __nv_bfloat162 pp = __floats2bfloat162_rn(a0 * f, a1 * f);
+                        w[e] = *reinterpret_cast<const uint32_t *>(&pp);
+                        acc[e] = pack2(0.f, 0.f);
+                    }
+                    const long long off = (long long)(((unsigned long long)(unsigned)ri.y << 32) | (unsigned)ri.x);
+                    *reinterpret_cast<uint4 *>(out + off + sub * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            row = row2; j = j2; n = n2;
+        }
+        if (!__any_sync(0xffffffffu, row <= last)) break;
     }
-    *reinterpret_cast<uint4 *>(out + b * c.q_sb + h * c.q_sh + r * c.q_st + sub * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-    if (sub == 0)
-        lse[((long long)b * c.Hq + h) * c.Lq + r] = den > 0.f ? (mx + log2f(den)) * kLn2 : -CUDART_INF_F;
 }
 
 // Per row, per-span mode (Algorithm 1 with the gate of Section "Combination"): slot j holds the
@@ -921,7 +980,7 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
                     const int32_t *__restrict__ anchor, const float *__restrict__ score, Call c, int slots, int Lc,
                     long long r0, bf16 *__restrict__ out, float *__restrict__ lse, float *__restrict__ lse_span) {
     const int lane = threadIdx.x & 31;
-    const long long row0 = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const long long row0 = ((long long)(gridDim.x - 1 - blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
     const long long rows = (long long)c.B * c.Hq * Lc;
     chain_wait();
     if (row0 >= rows) return;
@@ -1366,8 +1425,14 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
             e = launch_chained(tc_merge_gated, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
                                anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
         else
-            e = launch_chained(tc_merge, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
-                               (const unsigned char *)pa.n_pieces, c, plan.slots, lc, r0, (bf16 *)out, lse);
+        {
+            int per_warp = 32;
+            while (per_warp > 2 && (per_warp * plan.slots > kMergePieces || rows < (long long)kMergeFill * sm_count * per_warp)) per_warp /= 2;
+            const int per_cta = per_warp * kMergeWarps;
+            e = launch_chained(tc_merge, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(32 * kMergeWarps),
+                               (size_t)per_cta * (plan.slots | 1) * sizeof(float2), st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
+                               (const unsigned char *)pa.n_pieces, c, plan.slots, lc, r0, per_warp, (bf16 *)out, lse);
+        }
         if (e != cudaSuccess) return e;
         if (launches) *launches += 2;
         if (canaries && (e = launch_canary_check(ws, plan.canaries, c.status, st)) != cudaSuccess) return e;

@@ -170,6 +170,22 @@ def test_search_of_scores_that_are_not_finite(sla, handle, heads, top_k):
             assert (anchor[0, h, i, n:] == -1).all() and torch.isneginf(score[0, h, i, n:]).all()
 
 
+@pytest.mark.parametrize("heads,kv_heads,seq_len,top_k,window", [
+    (32, 8, 2877, 2, 0), (32, 8, 1473, 8, 0), (32, 8, 773, 16, 0),   # 32, 16 and 8 rows a warp, the last warp's cut off
+    (32, 8, 417, 6, 40), (16, 4, 417, 4, 0), (1, 1, 101, 3, 0), (2, 1, 579, 64, 100),
+])
+def test_merge_of_pieces(sla, handle, heads, kv_heads, seq_len, top_k, window):
+    """Rows of a warp from 2 to 32, rows that fill no whole block, 2 to 65 slots a row and rows of a single piece.  (From position
+    64 on: a row of a handful of keys may be off by 2^-9 (|out| + max |v|), the roundings of the result and of its weights,
+    which is more than the tolerance where both are near 4.)"""
+    from test_gpu_parity_modes import run_modes
+    w = workload(n_q_heads=heads, n_kv_heads=kv_heads, seq_len=seq_len, top_k=top_k, span_len=7)
+    if window:
+        run_modes(sla, handle, w, window, q_pos0=64)
+    else:
+        run_prefill(sla, handle, w, q_pos0=64)
+
+
 @pytest.mark.parametrize("window", [0, 1, 24, 25, 400, 2**31 - 1])
 @pytest.mark.parametrize("heads", [4, 8, 16])
 def test_search_walk_of_strides(sla, handle, heads, window):
