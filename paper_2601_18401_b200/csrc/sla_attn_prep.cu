@@ -140,6 +140,14 @@ __device__ __forceinline__ int row_of(const PrepArgs &a, const Share &s, long lo
     return (int)(((long long)s.b * a.Hq + h) * a.Lc + rc);
 }
 
+// Where a CTA parks the n-th piece of its row q: all first pieces, then all second ones, ...  A warp's rows are neighbours, so that
+// it writes and reads whole sectors, and the slots that no row fills are never touched.  65536 positions, 32/8 heads, eight spans:
+// counting pass 162 us with a row's pieces side by side, 95 like this, scatter pass 172 and 147; 16384 33 and 25, 27 and 24 (ncu).
+__device__ __forceinline__ int4 *parked(const PrepArgs &a, const Share &s, long long q, int n) {
+    const long long row0 = ((long long)s.b * a.Hq + s.g * a.G) * a.Lc + s.q0;   // the CTA's rows are consecutive
+    return a.stage + row0 * a.slots + n * (s.q1 - s.q0) + (q - s.q0);
+}
+
 // Counting pass.  Every piece of the CTA's rows is built once, counted in the CTA's shared-memory
 // histogram (the value the atomic returns is the piece's ordinal within its bucket and CTA) and parked
 // in `stage`; the histogram goes to the global bucket counts and, whole, to cta_hist.
@@ -167,13 +175,14 @@ __global__ void __launch_bounds__(kPrepThreads) prep_count(PrepArgs a) {
         const long long ell = base_len(i, a.span_len, a.len_first, a.n_len);
         if constexpr (K > 0) {
             if (a.mode == SLA_UNION) {
-                int4 *st = a.stage + (long long)row * a.slots;
+                int4 *st = parked(a, sh, q, 0);
+                const long long pitch = sh.q1 - sh.q0;
                 const int n = union_pieces_stream<KA>(an, a.top_k, (int)i, ell, a.back, a.fwd, a.window, a.merge_cap, a.status,
                                                       [&](int l0, int h0, int ordinal) {
                                                           const int eb = h0 / kBK, len = eb - l0 / kBK;
                                                           const int bucket = bucket_at(eb, cls_tbl[len < a.nb_max ? len : a.nb_max], a);
                                                           const int ord = atomicAdd(&hist[bucket], 1);
-                                                          st[ordinal] = make_int4(l0, h0, bucket | (ordinal << 24), ord);
+                                                          st[ordinal * pitch] = make_int4(l0, h0, bucket | (ordinal << 24), ord);
                                                       });
                 a.n_pieces[row] = (unsigned char)n;
                 continue;
@@ -185,11 +194,12 @@ __global__ void __launch_bounds__(kPrepThreads) prep_count(PrepArgs a) {
         else
             cnt = row_pieces(an, a.top_k, i, ell, a.back, a.fwd, a.window, a.mode, a.merge_cap, lo, hi, slot, a.status);
         a.n_pieces[row] = (unsigned char)cnt;
-        int4 *st = a.stage + (long long)row * a.slots;
+        int4 *st = parked(a, sh, q, 0);
+        const long long pitch = sh.q1 - sh.q0;
         auto park = [&](int j) {
             const int bucket = bucket_of(lo[j], hi[j], a);
             const int ord = atomicAdd(&hist[bucket], 1);
-            st[j] = make_int4(lo[j], hi[j], bucket | (slot[j] << 24), ord);
+            st[j * pitch] = make_int4(lo[j], hi[j], bucket | (slot[j] << 24), ord);
         };
         if constexpr (K > 0) {
 #pragma unroll
@@ -271,32 +281,27 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
             a.n_tiles[2] = 0;   // tiles claimed by the attention kernel
         }
     }
-    // One thread per parked slot, four slots in flight per thread.  The rows of a (batch, kv head) are
-    // consecutive (row = first row + q), so the CTA's slots are one contiguous run of `stage`.
-    const unsigned n_el = (unsigned)((sh.q1 - sh.q0) * a.slots);   // rows x slots < 2^31 for the whole chunk
-    const long long row_base = ((long long)sh.b * a.Hq + sh.g * a.G) * a.Lc + sh.q0;
-    const int4 *st = a.stage + row_base * a.slots;
+    // One thread per row, four pieces in flight per thread; the last rows first, whose pieces the L2 still holds.
     constexpr int U = 4;
-    for (unsigned e0 = threadIdx.x; e0 < n_el; e0 += U * kPrepThreads) {
-        int4 pc[U];
-        int row[U], cnt[U], j[U];
-        // all loads first (a slot beyond the row's count holds stale bytes that are not looked at)
+    const int n_rows = (int)(sh.q1 - sh.q0);
+    const int row_base = (int)(((long long)sh.b * a.Hq + sh.g * a.G) * a.Lc + sh.q0);   // rows x slots < 2^31 for the whole chunk
+    const int4 *st = parked(a, sh, sh.q0, 0);
+    int ql = n_rows - 1 - (int)threadIdx.x;
+    int cnt = ql >= 0 ? a.n_pieces[row_base + ql] : 0;
+    for (; ql >= 0;) {
+        const int next = ql - kPrepThreads, next_cnt = next >= 0 ? a.n_pieces[row_base + next] : 0;
+        for (int j0 = 0; j0 < cnt; j0 += U) {
+            int4 pc[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const unsigned e = e0 + u * kPrepThreads;
-            const unsigned ql = e / (unsigned)a.slots;
-            j[u] = (int)(e - ql * (unsigned)a.slots);
-            row[u] = (int)(row_base + ql);
-            cnt[u] = 0;
-            if (e < n_el) {
-                cnt[u] = a.n_pieces[row[u]];
-                pc[u] = __ldg(st + e);
-            }
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < cnt) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < cnt)
+                    a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j[u] < cnt[u])
-                a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row[u], pc[u].z >> 24, pc[u].x, pc[u].y);
+        ql = next;
+        cnt = next_cnt;
     }
 }
 
@@ -341,23 +346,37 @@ __global__ void __launch_bounds__(kPrepThreads) prep_clear(PrepArgs a) {
 }
 
 // One CTA per (batch, kv head): bucket histogram -> exclusive offsets local to the (batch, kv head),
-// plus how many records and tiles it has.
+// plus how many records and tiles it has.  Many buckets lie in shared memory meanwhile: read and written whole lines at a time, an
+// odd number per thread, so that the threads of a warp read different banks.  Each thread's own straight from global memory, and
+// like this (ncu): 14336 buckets 23.8 and 12.4 us, 40960 41.7 and 13.3, but 8192 6.4 and 7.5.
+constexpr int kScanDirect = 8;   // buckets per thread that are read straight from global memory
+template <bool kShared>
 __global__ void __launch_bounds__(kPrepThreads) prep_scan(PrepArgs a) {
+    extern __shared__ int hist[];   // [NB * ncls]
     __shared__ int warp_sum[32];
     const int nk = a.NB * a.ncls, bg = blockIdx.x, tid = threadIdx.x;
-    int *cnt = a.key_count + (long long)bg * nk;
-    const int per = (nk + kPrepThreads - 1) / kPrepThreads;
-    const int k0 = per * tid, k1 = (k0 + per < nk) ? k0 + per : nk;
+    int *cnt = a.key_count + (long long)bg * nk, *at = kShared ? hist : cnt;
+    const int most = (nk + kPrepThreads - 1) / kPrepThreads, per = kShared ? most | 1 : most;
+    const int k0 = per * tid < nk ? per * tid : nk, k1 = (k0 + per < nk) ? k0 + per : nk;
     chain_wait();
     chain_release();
+    if constexpr (kShared) {
+#pragma unroll 8
+        for (int k = tid; k < nk; k += kPrepThreads) hist[k] = cnt[k];
+        __syncthreads();
+    }
     int local = 0;
-    for (int k = k0; k < k1; ++k) local += cnt[k];
+    for (int k = k0; k < k1; ++k) local += at[k];
     int n_recs;
     int run = block_excl_scan(local, n_recs, warp_sum);
     for (int k = k0; k < k1; ++k) {
-        const int c = cnt[k];
-        cnt[k] = run;
+        const int c = at[k];
+        at[k] = run;
         run += c;
+    }
+    if constexpr (kShared) {
+        __syncthreads();
+        for (int k = tid; k < nk; k += kPrepThreads) cnt[k] = hist[k];
     }
     // tiles: the sorted list of the (batch, kv head) is cut every kRows records, across end blocks
     if (tid == 0) {
@@ -461,8 +480,9 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
     const int variant = n_iv <= 5 ? 3 : n_iv <= 9 ? 0 : n_iv <= 17 ? 1 : 2;
     void (*k0)(PrepArgs) = variant == 3 ? prep_count<5> : variant == 0 ? prep_count<9> : variant == 1 ? prep_count<17> : prep_count<0>;
     void (*k1)(PrepArgs) = prep_scatter;
+    const bool many = a.NB * a.ncls > kScanDirect * kPrepThreads;
     // function attributes belong to a device's context: remember the largest size set per device
-    static size_t attr_bytes[64][5] = {};   // the four counting kernels and the scatter kernel
+    static size_t attr_bytes[64][6] = {};   // the four counting kernels, the scatter kernel and the scan
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     const bool known = dev >= 0 && dev < 64;
@@ -477,6 +497,11 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
             if (e != cudaSuccess) return e;
             if (known) attr_bytes[dev][4] = smem;
         }
+        if (many && (!known || smem > attr_bytes[dev][5])) {
+            cudaError_t e = cudaFuncSetAttribute(prep_scan<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            if (known) attr_bytes[dev][5] = smem;
+        }
     }
     const unsigned grid = (unsigned)(n_bg * a.ctas_per_bg);
     // a chain of short kernels: 1999 positions, 32/8 heads, search to merge, 115 us with plain launches, a memset and an
@@ -485,7 +510,7 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
     const unsigned clear = (unsigned)((words + 4 * kPrepThreads - 1) / (4 * kPrepThreads));
     cudaError_t e = launch_chained(prep_clear, dim3(clear), dim3(kPrepThreads), 0, st, a);
     if (e == cudaSuccess) e = launch_chained(k0, dim3(grid), dim3(kPrepThreads), smem, st, a);
-    if (e == cudaSuccess) e = launch_chained(prep_scan, dim3(n_bg), dim3(kPrepThreads), 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(many ? prep_scan<true> : prep_scan<false>, dim3(n_bg), dim3(kPrepThreads), many ? smem : 0, st, a);
     if (e == cudaSuccess) e = launch_chained(k1, dim3(grid), dim3(kPrepThreads), smem, st, a);
     if (e == cudaSuccess) e = launch_chained(prep_tile_bounds, dim3((unsigned)((a.max_tiles + 7) / 8)), dim3(256), 0, st, a);
     if (launches) *launches += 5;

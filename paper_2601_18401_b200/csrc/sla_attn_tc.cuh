@@ -41,7 +41,7 @@ struct PrepArgs {
     int2 *ranges;            // [max_tiles] blocks of the walk the tile's first and second 128 pieces reach: first | end << 16
     int max_tiles;
     int4 *recs;
-    int4 *stage;             // [rows][slots] {lo, hi, bucket | slot << 24, ordinal within (CTA, bucket)}: the pieces as
+    int4 *stage;             // per CTA [slots][its rows] {lo, hi, bucket | slot << 24, ordinal within (CTA, bucket)}: the pieces as
                              // the counting pass found them, so that the scatter pass need not build them again
     int slots;               // partial results (and staged pieces) per row
     int *cta_hist;           // [CTAs][NB*ncls]: every CTA's bucket counts

@@ -186,6 +186,13 @@ def test_merge_of_pieces(sla, handle, heads, kv_heads, seq_len, top_k, window):
         run_prefill(sla, handle, w, q_pos0=64)
 
 
+@pytest.mark.parametrize("seq_len", [174720, 174721])
+def test_buckets_of_the_sort(sla, handle, seq_len):
+    """Spans of 81 keys, three length classes: 8190 and 8193 buckets, on both sides of the scan's way of reading them; rows
+    that fill no warp of the passes over the pieces."""
+    run_prefill(sla, handle, workload(n_q_heads=4, n_kv_heads=2, seq_len=seq_len, top_k=5, span_len=40), q_pos0=seq_len - 301, Lq=301)
+
+
 @pytest.mark.parametrize("window", [0, 1, 24, 25, 400, 2**31 - 1])
 @pytest.mark.parametrize("heads", [4, 8, 16])
 def test_search_walk_of_strides(sla, handle, heads, window):
