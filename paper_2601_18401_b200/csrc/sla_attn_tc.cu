@@ -27,8 +27,8 @@
 //
 // CTA layout of tc_attend (512 threads, one CTA per SM): warps 0-3 and 4-7 are the softmax warps of the
 // tile's two streams (one thread per piece, TMEM lane = row); warps 8-11 write the results (and gather the
-// first tile's Q); warps 12 and 13 issue the MMAs of a stream each; warp 14 loads K and V, once for both
-// streams; warp 15 claims the tiles to come and gathers their Q.  TMEM: per stream 128 columns of O and two 64-column S
+// first tile's Q and, where the tiles are dealt, the second stream's); warps 12 and 13 issue the MMAs of a stream each; warp 14
+// loads K and V, once for both streams; warp 15 claims the tiles to come and gathers their Q.  TMEM: per stream 128 columns of O and two 64-column S
 // buffers (P aliases the S it came from).  Every wait on an mbarrier is bounded; when one runs out the CTA
 // raises a status bit, drains and leaves.
 //
@@ -70,7 +70,7 @@ constexpr uint32_t kColO = 0;    // O of the streams at columns 0 and 128
 constexpr uint32_t kColS = 256;  // two S buffers of 64 columns per stream, from columns 256 and 384; P aliases its S
 constexpr int kQBytes = kHalf * kD * 2;      // 32 KiB, two 64-wide halves of 128 rows x 128 B
 constexpr int kKVBytes = kBK * kD * 2;       // 16 KiB, two 64-wide halves of 64 rows x 128 B
-constexpr int kQS = 4;           // Q buffers: the streams of this tile and of the next
+constexpr int kQS = 4;           // Q buffers: two per stream, in turn (buffer 2 * (n & 1) + x for the n-th tile of stream x)
 constexpr int kKS = 3;           // K and V stages
 constexpr int kTS = 4;           // entries of the ring of tiles
 // A list is claimed tile by tile if it can have kClaimTiles tiles per CTA (every slot of every row taken) and its longest single
@@ -199,7 +199,8 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     if (tid == 0) {
 #pragma unroll 1
         for (int x = 0; x < kQS; ++x) {
-            ptx::mbar_init(bar_q_full + 8 * x, 1);
+            // an arrival of each epilogue warp, or that of the gather and three of the same lane beside it
+            ptx::mbar_init(bar_q_full + 8 * x, 4);
             ptx::mbar_init(bar_q_empty + 8 * x, 1);
         }
 #pragma unroll 1
@@ -307,7 +308,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             const int x = warp - 12;
             struct Cursor {
                 uint32_t k;       // tile
-                int j, nblk, nx;  // nblk 0: no tile left
+                int j, nblk;      // nblk 0: no tile left
                 int first, end;   // blocks this stream takes part in
                 uint32_t nb;      // of those so far
             };
@@ -315,17 +316,16 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 const int r = x ? rg.y : rg.x;
                 c.j = 0;
                 c.nblk = ti.w >> 9;
-                c.nx = (ti.w & 0x1ff) > kHalf ? 2 : 1;
                 c.first = r & 0xffff;
                 c.end = r >> 16;
             };
-            Cursor cs{0u, 0, 0, 0, 0, 0, 0u};
+            Cursor cs{0u, 0, 0, 0, 0, 0u};
             rg = first_range();
             open(cs);
             Cursor cv = cs;
             bool ok = true;
             const uint32_t s_col = tmem + kColS + x * (2 * kBK), o_col = tmem + kColO + x * kD;
-            uint32_t nq = x, t = 0;
+            uint32_t nq = 0, t = 0;   // tiles of the stream that S and PV are through with
             const uint64_t desc_q0 = ptx::smem_desc_sw128(base + kOffQ, 16, 1024);
             const uint64_t desc_k0 = ptx::smem_desc_sw128(base + kOffK, 16, 1024);
             const uint64_t desc_v0 = ptx::smem_desc_sw128(base + kOffV, kKVBytes / 2, 1024);
@@ -362,8 +362,8 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     if (!ptx::mbar_wait(bar_kv_full + 8 * st, (i / kKS) & 1u, abort_flag)) break;
                     const bool last = cs.j == cs.end - 1;
                     if (cs.j >= cs.first && cs.j < cs.end) {
-                        const uint32_t qs = nq % kQS, b = cs.nb & 1u;
-                        if (cs.j == cs.first && !ptx::mbar_wait(bar_q_full + 8 * qs, (nq / kQS) & 1u, abort_flag)) break;
+                        const uint32_t qs = 2 * (nq & 1u) + x, b = cs.nb & 1u;
+                        if (cs.j == cs.first && !ptx::mbar_wait(bar_q_full + 8 * qs, (nq >> 1) & 1u, abort_flag)) break;
                         ptx::tc_fence_after();
                         const uint64_t dq = desc_advance(desc_q0, qs * kQBytes), dk = desc_advance(desc_k0, st * kKVBytes);
                         if (leader) {
@@ -375,9 +375,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                             if (last) ptx::mma_commit(bar_q_empty + 8 * qs);
                         }
                         ++cs.nb;
+                        nq += last;
                     }
                     if (++cs.j == cs.nblk) {
-                        nq += cs.nx;
                         ok = read_tile(++cs.k);
                         open(cs);
                     }
@@ -421,7 +421,7 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             // read a stream ahead.  (128 rows take the TMA unit about 4600 cycles: hidden in the tile before.)
             ptx::prefetch_tensormap(&tm_q);
             const bool leader = ptx::elect_one();
-            uint32_t k = 0, nq = 0;
+            uint32_t k = 0, nq[2] = {1u, (ti.w & 0x1ff) > kHalf ? 1u : 0u};   // the epilogue warps gather the first tile's rows
             int n = blockIdx.x + gridDim.x, rows[4];   // the next tile: the second is the CTA's own as well
             auto fetch_rows = [&](const int4 &t, int xs) {   // a row beyond the tile's last one: that one again
                 const int last = (t.w & 0x1ff) - 1;
@@ -448,7 +448,6 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 return t;
             };
             int4 next = ti;
-            nq = (ti.w & 0x1ff) > kHalf ? 2 : 1;   // the epilogue warps gather the first tile's rows
             bool first = true, ok = true;
             while (ok && next.w) {
                 ti = next;
@@ -458,13 +457,18 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     if (next.w) fetch_rows(next, 0);
                     continue;
                 }
-                const int bb = (unsigned)ti.x / (unsigned)p.Hkv, nx = (ti.w & 0x1ff) > kHalf ? 2 : 1;
+                const int bb = (unsigned)ti.x / (unsigned)p.Hkv, nx = kClaim && (ti.w & 0x1ff) > kHalf ? 2 : 1;   // (dealt: the epilogue warps take the second stream's)
 #pragma unroll 1
-                for (int x = 0; x < nx; ++x, ++nq) {
-                    const uint32_t qs = nq % kQS, full = bar_q_full + 8 * qs;
-                    ok = __all_sync(0xffffffffu, wait_aside(bar_q_empty + 8 * qs, ((nq / kQS) & 1u) ^ 1u));
+                for (int x = 0; x < nx; ++x) {
+                    const uint32_t turn = x ? nq[1]++ : nq[0]++, qs = 2 * (turn & 1u) + x, full = bar_q_full + 8 * qs;
+                    ok = __all_sync(0xffffffffu, wait_aside(bar_q_empty + 8 * qs, ((turn >> 1) & 1u) ^ 1u));
                     if (!ok) break;
-                    if (leader) ptx::mbar_arrive_expect_tx(full, kQBytes);
+                    if (leader) {
+                        ptx::mbar_arrive_expect_tx(full, kQBytes);
+                        ptx::mbar_arrive(full);
+                        ptx::mbar_arrive(full);
+                        ptx::mbar_arrive(full);
+                    }
                     int at[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) at[u] = q_row(rows[u], bb);
@@ -486,29 +490,54 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         uint32_t k = 0;
         bool ok = true;
         warp_read(0);
-        // the Q rows of the CTA's first tile, by 16-byte copies: two rows (16 lanes each) per instruction
-        {
-            const int cnt = ti.w & 0x1ff, chunk = lane & 15, odd = lane >> 4, bb = (unsigned)ti.x / (unsigned)p.Hkv;
-            const uint32_t dst = base + kOffQ + (chunk >> 3) * (kQBytes / 2) + ((warp & 3) * 32 + odd) * 128;
-#pragma unroll 1
-            for (int x = 0; x * kHalf < cnt; ++x) {
-                const int at = q_row(p.recs[ti.z + min(x * kHalf + row, cnt - 1)].x, bb);
+        // Q rows of a stream's tile by 16-byte copies, two rows (16 lanes each) per instruction
+        auto copy_rows = [&](const int4 &t, int x, uint32_t buf) {
+            const int cnt = t.w & 0x1ff, chunk = lane & 15, odd = lane >> 4, bb = (unsigned)t.x / (unsigned)p.Hkv;
+            const uint32_t dst = base + kOffQ + buf * kQBytes + (chunk >> 3) * (kQBytes / 2) + ((warp & 3) * 32 + odd) * 128;
+            const int at = q_row(p.recs[t.z + min(x * kHalf + row, cnt - 1)].x, bb);
 #pragma unroll 4
-                for (int i = 0; i < 16; ++i) {
-                    const int from = __shfl_sync(0xffffffffu, at, 2 * i + odd);
-                    ptx::cp_async16(dst + x * kQBytes + i * 256 + (((chunk & 7) ^ ((2 * i + odd) & 7)) << 4),
-                                    p.q + from * p.q_pitch + chunk * 8);
-                }
-                ptx::cp_async_wait_all();
-                ptx::fence_proxy_async_smem();
-                ptx::bar_sync(1, 128);
-                if (row == 0) ptx::mbar_arrive(bar_q_full + 8 * x);
+            for (int i = 0; i < 16; ++i) {
+                const int from = __shfl_sync(0xffffffffu, at, 2 * i + odd);
+                ptx::cp_async16(dst + i * 256 + (((chunk & 7) ^ ((2 * i + odd) & 7)) << 4), p.q + from * p.q_pitch + chunk * 8);
             }
+        };
+        auto rows_copied = [&](uint32_t buf) {   // (no barrier among the four warps: one whose wait ran out would leave them there)
+            ptx::cp_async_wait_all();
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar_q_full + 8 * buf);
+        };
+        // the CTA's first tile
+#pragma unroll 1
+        for (int x = 0; x * kHalf < (ti.w & 0x1ff); ++x) {
+            copy_rows(ti, x, x);
+            rows_copied(x);
         }
+        // Where the tiles are dealt their walks may be shorter than the gather of their rows by TMA (4600 cycles a stream): the
+        // second stream's rows are copied here, two tiles ahead, behind the tile whose buffer they take, and handed over before
+        // the next one's results.  1999 positions, 32/8 heads, four spans (walks of two to three blocks): kernel 47.3 -> 41.5 us.
+        uint32_t nq = (ti.w & 0x1ff) > kHalf ? 1u : 0u;
+        int copied = -1;   // buffer
+        auto copy_ahead = [&](int n) {
+            const int4 t = n < n_tiles ? p.tiles[n] : make_int4(0, 0, 0, 0);
+            if ((t.w & 0x1ff) > kHalf) {
+                copied = 2 * (nq & 1u) + 1;
+                const bool got = __all_sync(0xffffffffu, wait_aside(bar_q_empty + 8 * copied, ((nq >> 1) & 1u) ^ 1u));
+                ++nq;
+                if (!got) return false;
+                copy_rows(t, 1, copied);
+            }
+            return true;
+        };
+        if constexpr (!kClaim) ok = copy_ahead(blockIdx.x + gridDim.x);
         uint32_t tx[2] = {0, 0};
         while (ok && ti.w) {
             const int cnt = ti.w & 0x1ff, nx = cnt > kHalf ? 2 : 1, rec0 = ti.z;
             ok = take_tile(++k);
+            if constexpr (!kClaim) {
+                if (copied >= 0) rows_copied(copied);
+                copied = -1;
+            }
 #pragma unroll 1
             for (int x = 0; x < nx && ok; ++x) {
                 const uint32_t t = x ? tx[1] : tx[0];
@@ -562,6 +591,9 @@ tc_attend(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 }
                 if (valid) p.part_lse[slot] = make_float2(stat.y, __uint_as_float(exps));
                 if (x) ++tx[1]; else ++tx[0];
+            }
+            if constexpr (!kClaim) {
+                if (ok) ok = copy_ahead(blockIdx.x + (k + 1) * gridDim.x);
             }
         }
     } else {

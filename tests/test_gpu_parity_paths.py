@@ -35,6 +35,14 @@ def test_streams_of_a_tile(sla, handle, seq_len):
     run_prefill(sla, handle, workload(n_q_heads=1, n_kv_heads=1, seq_len=seq_len, top_k=1, span_len=40))
 
 
+@pytest.mark.parametrize("seq_len", [364, 434, 664, 964, 1264])
+def test_tiles_dealt_to_a_block(sla, handle, seq_len):
+    """Short walks, up to four tiles a block on 148 multiprocessors, each (batch, KV head) ending in a ragged tile: rows of the
+    second stream that are copied one and two tiles ahead, or are not there.  (Several spans, from position 64 on: rows of a
+    handful of keys may be further off than the tolerance, see test_merge_of_pieces.)"""
+    run_prefill(sla, handle, workload(n_q_heads=32, n_kv_heads=8, seq_len=seq_len, top_k=4, span_len=9, seed=79), q_pos0=64)
+
+
 @pytest.mark.parametrize("span_len", [10, 31, 32, 33, 600])
 def test_walks_of_one_block_and_of_many(sla, handle, span_len):
     """Spans within a block, over one boundary and over nineteen blocks; two batches, three KV heads."""
