@@ -5,7 +5,7 @@
 // keeps 64 keys and values in shared memory and serves every query row of its share that selected any of them:
 //   scan    each thread reads the anchors of a row and forms the 64-bit mask of the block's keys that lie in the row's
 //           spans (the union is the OR of the spans' masks: no sorting, no clipping); rows with a mask go to a list;
-//   attend  a warp takes LPR lanes x 4 rows per group (32 rows at head_dim 64, 16 at 128): a lane holds 16 dims of four
+//   attend  a warp takes LPR lanes x up to 4 rows per group (32 rows at head_dim 64, 16 at 128): a lane holds 16 dims of four
 //           query rows, reads the same 16 dims of a key as its group's peers (broadcast) and the lanes' sums are exchanged
 //           so that each lane ends up with the score of one row; the 64 keys, then the exponentials, then the values
 //           (every row multiplies all 64, with weight 0 where it did not select the key: an Inf or NaN among them is
@@ -15,10 +15,12 @@
 // Everything is fp32 FMA (two per instruction), as in the row kernel: bf16 inputs are widened exactly.
 // Bound by the FMA pipe and, at 12 to 16 warps an SM, by the latency of its chains: 64 f32x2 products per key and 32 rows
 // (issue slots 40 % used; two thirds of the products belong to selected keys).  Search and attention together,
-// row kernel and this one: 4096 positions, one head of 64 dims, top_k 4, spans of 129 keys 88 and 55 us; 3811 positions, one
+// row kernel and this one: 4096 positions, one head of 64 dims, top_k 4, spans of 129 keys 88 and 52 us; 3811 positions, one
 // head of 128 dims, top_k 8, spans of up to 125 keys 258 and 100 us; 7343 positions, two heads, 173 keys 479 and 301 us.
 #include <limits.h>
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "sla_kernels.h"
 
@@ -133,135 +135,157 @@ attend_blocks(const T *__restrict__ q, const T *__restrict__ k, const T *__restr
     float *pw = ps + warp * ROWS * kPitch;
     const float *kl = ks + sub * 4, *vl = vs + sub * 4;
 
-    auto attend = [&](int n) {
-        for (int e0 = warp * ROWS; e0 < n; e0 += kWarps * ROWS) {
-            // the lane's own row (the one whose scores it receives): row sub & 3 of its group
-            const int own = e0 + (sub & 3) * NG + grp;
-            int4 mine = make_int4(0, 0, 0, 0);
-            if (own < n) mine = list[own];
-            const T *qrow[4];
-            float2 qv[4][8];
+    // one pass of the warp over the block: R rows per group, entries e0 + r NG + grp of the list
+    auto pass = [&](auto rows_per_group, int e0, int n) {
+        constexpr int R = decltype(rows_per_group)::value;
+        // the lane's own row (the one whose scores it receives): row sub & 3 of its group
+        const int own = (sub & 3) < R ? e0 + (sub & 3) * NG + grp : n;
+        int4 mine = make_int4(0, 0, 0, 0);
+        if (own < n) mine = list[own];
+        const T *qrow[R];
+        float2 qv[R][8];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int e = e0 + r * NG + grp;
-                const int row = list[e < n ? e : n - 1].x, rc = row % n_rows, hg = row / n_rows;
-                qrow[r] = q + b * c.q_sb + (long long)(g * c.G + hg) * c.q_sh + (long long)(r_first + rc) * c.q_st + sub * 4;
+        for (int r = 0; r < R; ++r) {
+            const int e = e0 + r * NG + grp;
+            const int row = list[e < n ? e : n - 1].x, rc = row % n_rows, hg = row / n_rows;
+            qrow[r] = q + b * c.q_sb + (long long)(g * c.G + hg) * c.q_sh + (long long)(r_first + rc) * c.q_st + sub * 4;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                float f[4];
+                if constexpr (sizeof(T) == 4) {
+                    const float4 w = __ldg(reinterpret_cast<const float4 *>(qrow[r] + x * 4 * LPR));
+                    f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
+                } else {
+                    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(qrow[r] + x * 4 * LPR));
+                    f[0] = __uint_as_float(w.x << 16); f[1] = __uint_as_float(w.x & 0xffff0000u);
+                    f[2] = __uint_as_float(w.y << 16); f[3] = __uint_as_float(w.y & 0xffff0000u);
+                }
+                qv[r][2 * x] = make_float2(f[0] * scale2, f[1] * scale2);
+                qv[r][2 * x + 1] = make_float2(f[2] * scale2, f[3] * scale2);
             }
+        // scores of the 64 keys, masked, to shared memory
+        float m = -CUDART_INF_F, l = 0.f;
+#pragma unroll 1
+        for (int j = 0; j < kKeys; j += 4) {
+            const unsigned mask = (j < 32 ? (unsigned)mine.z : (unsigned)mine.w) >> (j & 31);
+            float s[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int u = 0; u < 4; ++u) {
+                float2 t[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) t[r] = make_float2(0.f, 0.f);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    float f[4];
-                    if constexpr (sizeof(T) == 4) {
-                        const float4 w = __ldg(reinterpret_cast<const float4 *>(qrow[r] + x * 4 * LPR));
-                        f[0] = w.x; f[1] = w.y; f[2] = w.z; f[3] = w.w;
-                    } else {
-                        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(qrow[r] + x * 4 * LPR));
-                        f[0] = __uint_as_float(w.x << 16); f[1] = __uint_as_float(w.x & 0xffff0000u);
-                        f[2] = __uint_as_float(w.y << 16); f[3] = __uint_as_float(w.y & 0xffff0000u);
+                    const float4 w = *reinterpret_cast<const float4 *>(kl + (j + u) * D + x * 4 * LPR);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        t[r] = fma2(qv[r][2 * x], make_float2(w.x, w.y), t[r]);
+                        t[r] = fma2(qv[r][2 * x + 1], make_float2(w.z, w.w), t[r]);
                     }
-                    qv[r][2 * x] = make_float2(f[0] * scale2, f[1] * scale2);
-                    qv[r][2 * x + 1] = make_float2(f[2] * scale2, f[3] * scale2);
                 }
-            // scores of the 64 keys, masked, to shared memory
-            float m = -CUDART_INF_F, l = 0.f;
-#pragma unroll 1
-            for (int j = 0; j < kKeys; j += 4) {
-                const unsigned mask = (j < 32 ? (unsigned)mine.z : (unsigned)mine.w) >> (j & 31);
-                float s[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float2 t[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) t[r] = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const float4 w = *reinterpret_cast<const float4 *>(kl + (j + u) * D + x * 4 * LPR);
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            t[r] = fma2(qv[r][2 * x], make_float2(w.x, w.y), t[r]);
-                            t[r] = fma2(qv[r][2 * x + 1], make_float2(w.z, w.w), t[r]);
-                        }
-                    }
-                    const float t0 = t[0].x + t[0].y, t1 = t[1].x + t[1].y, t2 = t[2].x + t[2].y, t3 = t[3].x + t[3].y;
-                    const float ya = ((sub & 1) ? t1 : t0) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? t0 : t1, NG);
-                    const float yb = ((sub & 1) ? t3 : t2) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? t2 : t3, NG);
-                    float z = ((sub & 2) ? yb : ya) + __shfl_xor_sync(0xffffffffu, (sub & 2) ? ya : yb, 2 * NG);
-                    if (LPR == 8) z += __shfl_xor_sync(0xffffffffu, z, 4 * NG);
-                    s[u] = (mask >> u) & 1u ? z : -CUDART_INF_F;
-                    m = fmaxf(m, s[u]);
-                }
-                if (sub < 4) *reinterpret_cast<float4 *>(pw + lane * kPitch + j) = make_float4(s[0], s[1], s[2], s[3]);
+                const float t0 = t[0].x + t[0].y, t1 = t[1].x + t[1].y, t2 = t[2].x + t[2].y, t3 = t[3].x + t[3].y;
+                const float ya = ((sub & 1) ? t1 : t0) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? t0 : t1, NG);
+                const float yb = ((sub & 1) ? t3 : t2) + __shfl_xor_sync(0xffffffffu, (sub & 1) ? t2 : t3, NG);
+                float z = ((sub & 2) ? yb : ya) + __shfl_xor_sync(0xffffffffu, (sub & 2) ? ya : yb, 2 * NG);
+                if (LPR == 8) z += __shfl_xor_sync(0xffffffffu, z, 4 * NG);
+                s[u] = (mask >> u) & 1u ? z : -CUDART_INF_F;
+                m = fmaxf(m, s[u]);
             }
-            // exponentials of the lane's own row
-            const float ref = m == -CUDART_INF_F ? 0.f : m;
-            if (sub < 4) {
+            if (sub < 4) *reinterpret_cast<float4 *>(pw + lane * kPitch + j) = make_float4(s[0], s[1], s[2], s[3]);
+        }
+        // exponentials of the lane's own row
+        const float ref = m == -CUDART_INF_F ? 0.f : m;
+        if (sub < 4) {
 #pragma unroll 2
-                for (int j = 0; j < kKeys; j += 4) {
-                    float4 *w = reinterpret_cast<float4 *>(pw + lane * kPitch + j);
-                    float4 x = *w;
-                    x.x = exp2f(x.x - ref); x.y = exp2f(x.y - ref); x.z = exp2f(x.z - ref); x.w = exp2f(x.w - ref);
-                    l += (x.x + x.y) + (x.z + x.w);
-                    *w = x;
-                }
-            }
-            __syncwarp();
-            // values
-            float2 acc[4][8];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int x = 0; x < 8; ++x) acc[r][x] = make_float2(0.f, 0.f);
-#pragma unroll 1
             for (int j = 0; j < kKeys; j += 4) {
-                float pr[4][4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float4 w = *reinterpret_cast<const float4 *>(pw + (r * NG + grp) * kPitch + j);
-                    pr[r][0] = w.x; pr[r][1] = w.y; pr[r][2] = w.z; pr[r][3] = w.w;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const float4 w = *reinterpret_cast<const float4 *>(vl + (j + u) * D + x * 4 * LPR);
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const float2 pp = make_float2(pr[r][u], pr[r][u]);
-                            acc[r][2 * x] = fma2(pp, make_float2(w.x, w.y), acc[r][2 * x]);
-                            acc[r][2 * x + 1] = fma2(pp, make_float2(w.z, w.w), acc[r][2 * x + 1]);
-                        }
-                    }
+                float4 *w = reinterpret_cast<float4 *>(pw + lane * kPitch + j);
+                float4 x = *w;
+                x.x = exp2f(x.x - ref); x.y = exp2f(x.y - ref); x.z = exp2f(x.z - ref); x.w = exp2f(x.w - ref);
+                l += (x.x + x.y) + (x.z + x.w);
+                *w = x;
             }
-            for (unsigned long long keys = odd[0] | (unsigned long long)odd[1] << 32; keys; keys &= keys - 1) {
-                const int j = __ffsll((long long)keys) - 1;
-                const T *row = vbase + (long long)j * c.kv_st + sub * 4;
+        }
+        __syncwarp();
+        // values
+        float2 acc[R][8];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int e = e0 + r * NG + grp;
-                    if (e >= n || !(((j < 32 ? (unsigned)list[e].z : (unsigned)list[e].w) >> (j & 31)) & 1u)) continue;
-                    const float w = pw[(r * NG + grp) * kPitch + j];
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        const T *at = row + (x >> 1) * 4 * LPR + (x & 1) * 2;
-                        const float a = (float)at[0], z = (float)at[1];
-                        if (!isfinite(a)) acc[r][x].x = fmaf(w, a, acc[r][x].x);
-                        if (!isfinite(z)) acc[r][x].y = fmaf(w, z, acc[r][x].y);
+            for (int x = 0; x < 8; ++x) acc[r][x] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int j = 0; j < kKeys; j += 4) {
+            float pr[R][4];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 w = *reinterpret_cast<const float4 *>(pw + (r * NG + grp) * kPitch + j);
+                pr[r][0] = w.x; pr[r][1] = w.y; pr[r][2] = w.z; pr[r][3] = w.w;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float4 w = *reinterpret_cast<const float4 *>(vl + (j + u) * D + x * 4 * LPR);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float2 pp = make_float2(pr[r][u], pr[r][u]);
+                        acc[r][2 * x] = fma2(pp, make_float2(w.x, w.y), acc[r][2 * x]);
+                        acc[r][2 * x + 1] = fma2(pp, make_float2(w.z, w.w), acc[r][2 * x + 1]);
                     }
                 }
-            }
-            __syncwarp();   // the next scores go to the same place
-            if (own < n && sub < 4) ml[mine.y] = make_float2(m, l);
+        }
+        for (unsigned long long keys = odd[0] | (unsigned long long)odd[1] << 32; keys; keys &= keys - 1) {
+            const int j = __ffsll((long long)keys) - 1;
+            const T *row = vbase + (long long)j * c.kv_st + sub * 4;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
+            for (int r = 0; r < R; ++r) {
                 const int e = e0 + r * NG + grp;
-                if (e < n) {
-                    float *o = part + (size_t)list[e].y * D + sub * 4;
+                if (e >= n || !(((j < 32 ? (unsigned)list[e].z : (unsigned)list[e].w) >> (j & 31)) & 1u)) continue;
+                const float w = pw[(r * NG + grp) * kPitch + j];
 #pragma unroll
-                    for (int x = 0; x < 4; ++x)
-                        *reinterpret_cast<float4 *>(o + x * 4 * LPR) =
-                            make_float4(acc[r][2 * x].x, acc[r][2 * x].y, acc[r][2 * x + 1].x, acc[r][2 * x + 1].y);
+                for (int x = 0; x < 8; ++x) {
+                    const T *at = row + (x >> 1) * 4 * LPR + (x & 1) * 2;
+                    const float a = (float)at[0], z = (float)at[1];
+                    if (!isfinite(a)) acc[r][x].x = fmaf(w, a, acc[r][x].x);
+                    if (!isfinite(z)) acc[r][x].y = fmaf(w, z, acc[r][x].y);
                 }
+            }
+        }
+        __syncwarp();   // the next scores go to the same place
+        if (own < n && sub < 4) ml[mine.y] = make_float2(m, l);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int e = e0 + r * NG + grp;
+            if (e < n) {
+                float *o = part + (size_t)list[e].y * D + sub * 4;
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    *reinterpret_cast<float4 *>(o + x * 4 * LPR) =
+                        make_float4(acc[r][2 * x].x, acc[r][2 * x].y, acc[r][2 * x + 1].x, acc[r][2 * x + 1].y);
+            }
+        }
+    };
+    // The list in as few passes as four rows per group allow, its rows shared out evenly among the warps, the passes nearly equal:
+    // a list of 92 rows is three rows per group in all four warps instead of four in three of them, one of 136 rows two passes of
+    // three and two.  Search and attention: 4096 positions, one head, four spans 56.5 and 52.6 us; 8000, four heads 452 and 422; bf16,
+    // 8192, four heads 428 and 388.  (At head_dim 128 the registers do not suffice: 3811 positions, eight spans 101 and 104 us.)
+    auto attend = [&](int n) {
+        if constexpr (D == 128) {
+            for (int e0 = warp * ROWS; e0 < n; e0 += kWarps * ROWS) pass(std::integral_constant<int, 4>(), e0, n);
+        } else {
+            int units = (n + kWarps * NG - 1) / (kWarps * NG);   // rows per group still to come
+            for (int passes = (units + 3) / 4, e0 = 0; passes > 0; --passes) {
+                const int rows = (units + passes - 1) / passes, at = e0 + warp * NG * rows;
+                if (at < n) {
+                    if (rows == 4) pass(std::integral_constant<int, 4>(), at, n);
+                    else if (rows == 3) pass(std::integral_constant<int, 3>(), at, n);
+                    else if (rows == 2) pass(std::integral_constant<int, 2>(), at, n);
+                    else pass(std::integral_constant<int, 1>(), at, n);
+                }
+                units -= rows;
+                e0 += kWarps * NG * rows;
             }
         }
     };

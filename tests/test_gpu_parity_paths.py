@@ -234,6 +234,8 @@ def test_search_walk_of_strides(sla, handle, heads, window):
     (True, dict(seq_len=1599, top_k=8, span_len=40)), (True, dict(seq_len=1600, top_k=8, span_len=40)),
     (True, dict(seq_len=1601, top_k=8, span_len=40)),
     (True, dict(batch=2, n_q_heads=6, n_kv_heads=2, seq_len=1543, top_k=9, span_len=0)),   # lists that fill up several times
+    # lists of less than a row per group and warp up to more than four: one to four rows per group, one pass and two
+    (True, dict(n_q_heads=1, seq_len=4099, top_k=4, span_len=64)), (True, dict(seq_len=2600, top_k=4, span_len=40)),
     (True, dict(seq_len=2300, top_k=6, span_len=33, window=200)), (True, dict(seq_len=3000, q_pos0=2100, top_k=8, span_len=60, window=129)),
     (True, dict(n_q_heads=4, n_kv_heads=4, seq_len=1200, top_k=8, span_len=100)),
     (True, dict(seq_len=1000, span_len=600)), (True, dict(seq_len=700, top_k=64, span_len=40)),   # spans cut off at 0; 64 of them
