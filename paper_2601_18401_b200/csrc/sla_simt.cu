@@ -9,6 +9,7 @@
 #include <math_constants.h>
 
 #include "sla_kernels.h"
+#include "sla_topk.cuh"
 
 namespace sla {
 
@@ -124,14 +125,14 @@ search_rows_simt(const T *__restrict__ q_s, const T *__restrict__ k, Call c,
             const float v = sc[s];
             if (v > bv) { bv = v; bs = s; }
         }
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-            const int os = __shfl_xor_sync(0xffffffffu, bs, off);
-            if (ov > bv || (ov == bv && os < bs)) { bv = ov; bs = os; }
-        }
+        // the largest of the lanes' best, of equal ones the smallest stride (0 and -0 are equal).  Two reductions of the warp
+        // instead of five exchanges of both: 3811 positions, two heads of 128 dims, K = 8 29.4 -> 26.8 us; 2000, eight heads, K = 16
+        // 64.6 -> 53.3.
+        const unsigned key = bs != INT_MAX ? topk::order_key(bv + 0.f) : 0u, top = __reduce_max_sync(0xffffffffu, key);
+        bs = (int)__reduce_min_sync(0xffffffffu, key == top ? (unsigned)bs : (unsigned)INT_MAX);
         if (lane == 0) {
             if (bs != INT_MAX) {
+                bv = sc[bs];
                 out_anchor[obase + j] = (int32_t)(i + 1 - stride_offset(c, bs));
                 out_score[obase + j] = bv;
                 sc[bs] = -CUDART_INF_F;

@@ -225,6 +225,28 @@ def test_search_walk_of_strides(sla, handle, heads, window):
             assert (a[:, n:] == -1).all() and torch.isneginf(v[:, n:]).all()
 
 
+@pytest.mark.parametrize("dtype,top_k", [("f32", 1), ("f32", 9), ("bf16", 64)])
+def test_generic_search_of_equal_scores(sla, handle, dtype, top_k):
+    """Small whole numbers, zeros of both signs among the products: many equal scores, the nearer anchor first, for fewer and
+    more strides than lanes."""
+    import torch
+    L, g = 1700, torch.Generator().manual_seed(31)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    q, k = (torch.zeros(1, 1, L, 64) for _ in range(2))
+    q[..., :3], k[..., :3] = (torch.randint(-1, 2, (1, 1, L, 3), generator=g).float() for _ in range(2))
+    k[:, :, ::5] = -0.0
+    anchor, score = sla.sla_span_search(handle, q.to(dt).cuda(), k.to(dt).cuda(), sla.make_params(top_k, 8, head_dim=64))
+    torch.cuda.synchronize()
+    anchor, score = anchor.cpu()[0, 0], score.cpu()[0, 0]
+    for i in range(0, L, 7):
+        t = torch.tensor([i + 1 - s * s for s in range(1, i + 2) if s * s <= i + 1])
+        x = k[0, 0, t] @ q[0, 0, i]
+        order = torch.sort(x, descending=True, stable=True).indices[:top_k]
+        n = len(order)
+        assert torch.equal(anchor[i, :n].long(), t[order]) and torch.equal(score[i, :n], x[order]), i
+        assert (anchor[i, n:] == -1).all() and torch.isneginf(score[i, n:]).all()
+
+
 @pytest.mark.parametrize("by_blocks,kw", [
     # few keys a row, few rows (at the start, or far into a context), or blocks that few rows select
     (False, dict(seq_len=1, top_k=6, span_len=300)), (False, dict(seq_len=65, top_k=64, span_len=2)),
