@@ -1004,10 +1004,11 @@ tc_merge_gated(const __half *__restrict__ part_o, const float2 *__restrict__ par
 // with the coefficients handed over by shuffles.
 // Bound by the reads of the partial results: with room for eight spans whatever top_k is, 106 registers and the shuffles of
 // absent spans made it 402 us for 32768 positions, 32 heads, two spans and a window (1.1 GB, 2.7 TB/s); with room for two,
-// 48 registers and 213 us.
+// 48 registers and 213 us; with the next two rows' pieces requested ahead 64 registers and 170 us (6.4 TB/s).  Eight spans 993 and 581 us,
+// five 723 and 493, but four 265 and 281 (122 registers, two CTAs an SM): built for four it requests them in the same step.
 constexpr int kGateK = 8;
 template <int K>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, K <= 2 ? 4 : 1)
 tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
                     const int32_t *__restrict__ anchor, const float *__restrict__ score, Call c, int slots, int Lc,
                     long long r0, bf16 *__restrict__ out, float *__restrict__ lse, float *__restrict__ lse_span) {
@@ -1088,17 +1089,13 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
     // ---- phase B: two rows per step, 16 lanes per row
     const int sub = lane & 15, hi = lane >> 4;
     const int shift = 8 * (sub >> 2);
-#pragma unroll 4
-    for (int rr = 0; rr < 16; ++rr) {
+    constexpr bool kAhead = K != 4;   // a step's pieces are requested before the sums of the one before
+    float cf[2][K + 1];
+    uint32_t ee[2][K + 1];
+    uint4 raw[2][K + 1];
+    auto fetch = [&](int rr, float (&cf)[K + 1], uint32_t (&ee)[K + 1], uint4 (&raw)[K + 1]) {
         const int src = 2 * rr + hi;
-        const long long row = row0 + src;
-        const __half *po = part_o + row * slots * kD + sub * 8;
-        float acc[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-        float cf[K + 1];
-        uint32_t ee[K + 1];
-        uint4 raw[K + 1];
+        const __half *po = part_o + (row0 + src) * slots * kD + sub * 8;
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             cf[j] = __shfl_sync(0xffffffffu, coef[j], src);
@@ -1106,18 +1103,31 @@ tc_merge_gated_rows(const __half *__restrict__ part_o, const float2 *__restrict_
         }
         cf[K] = __shfl_sync(0xffffffffu, cw, src);
         ee[K] = __shfl_sync(0xffffffffu, ex_w, src);
-        const long long off = __shfl_sync(0xffffffffu, out_off, src);
 #pragma unroll
-        for (int j = 0; j <= K; ++j) {
-            const int slot = j < K ? j : c.top_k;
-            raw[j] = cf[j] != 0.f ? __ldg(reinterpret_cast<const uint4 *>(po + (long long)slot * kD)) : make_uint4(0, 0, 0, 0);
+        for (int j = 0; j <= K; ++j)
+            if (cf[j] != 0.f) raw[j] = __ldg(reinterpret_cast<const uint4 *>(po + (long long)(j < K ? j : c.top_k) * kD));
+    };
+    if constexpr (kAhead) fetch(0, cf[0], ee[0], raw[0]);
+#pragma unroll (kAhead ? 2 : 4)
+    for (int rr = 0; rr < 16; ++rr) {
+        const int now = kAhead ? rr & 1 : 0;
+        const int src = 2 * rr + hi;
+        const long long row = row0 + src;
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        const long long off = __shfl_sync(0xffffffffu, out_off, src);
+        if constexpr (kAhead) {
+            if (rr + 1 < 16) fetch(rr + 1, cf[now ^ 1], ee[now ^ 1], raw[now ^ 1]);
+        } else {
+            fetch(rr, cf[0], ee[0], raw[0]);
         }
 #pragma unroll
         for (int j = 0; j <= K; ++j)
-            if (cf[j] != 0.f) {
-                const uint32_t eb = (ee[j] >> shift) & 0xffu;
-                const float ws = cf[j] * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
-                const uint32_t rw[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
+            if (cf[now][j] != 0.f) {
+                const uint32_t eb = (ee[now][j] >> shift) & 0xffu;
+                const float ws = cf[now][j] * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
+                const uint32_t rw[4] = {raw[now][j].x, raw[now][j].y, raw[now][j].z, raw[now][j].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rw[e]));
