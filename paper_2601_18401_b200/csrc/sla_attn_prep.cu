@@ -24,6 +24,10 @@ namespace tc {
 namespace {
 
 constexpr int kPrepThreads = 1024;
+// Without being asked the runtime gives a kernel 48 KB of shared memory, its own arrays included (128 bytes at most beside a histogram).
+constexpr size_t kPlainSmem = 47 * 1024;
+constexpr size_t kMostSmem = kHistBytes + kMaxWalk + 16;   // histogram and class table of the longest list
+static_assert(kMostSmem <= 226 * 1024, "a CTA has 227 KB");
 
 // Bucket of a piece: its end block and the class of the number of blocks it covers.  Classes are even
 // steps over [0, nb_single) (a single span) and, for joined pieces, over [nb_single, nb_max).
@@ -352,7 +356,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_clear(PrepArgs a) {
 constexpr int kScanDirect = 8;   // buckets per thread that are read straight from global memory
 template <bool kShared>
 __global__ void __launch_bounds__(kPrepThreads) prep_scan(PrepArgs a) {
-    extern __shared__ int hist[];   // [NB * ncls]
+    extern __shared__ int hist[];   // kShared: [NB * ncls]
     __shared__ int warp_sum[32];
     const int nk = a.NB * a.ncls, bg = blockIdx.x, tid = threadIdx.x;
     int *cnt = a.key_count + (long long)bg * nk, *at = kShared ? hist : cnt;
@@ -481,36 +485,31 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
     void (*k0)(PrepArgs) = variant == 3 ? prep_count<5> : variant == 0 ? prep_count<9> : variant == 1 ? prep_count<17> : prep_count<0>;
     void (*k1)(PrepArgs) = prep_scatter;
     const bool many = a.NB * a.ncls > kScanDirect * kPrepThreads;
-    // function attributes belong to a device's context: remember the largest size set per device
-    static size_t attr_bytes[64][6] = {};   // the four counting kernels, the scatter kernel and the scan
+    const size_t scan_smem = many ? (size_t)a.NB * a.ncls * sizeof(int) : 0;
+    // Function attributes belong to a device's context: remembered per device.  A kernel is given the most that any list takes, so that
+    // no later call or other thread has to raise it, or lowers it.
+    static bool allowed[64][6] = {};   // the four counting kernels, the scatter kernel and the scan
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     const bool known = dev >= 0 && dev < 64;
-    if (smem > 48 * 1024) {
-        if (!known || smem > attr_bytes[dev][variant]) {
-            cudaError_t e = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            if (known) attr_bytes[dev][variant] = smem;
-        }
-        if (!known || smem > attr_bytes[dev][4]) {
-            cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            if (known) attr_bytes[dev][4] = smem;
-        }
-        if (many && (!known || smem > attr_bytes[dev][5])) {
-            cudaError_t e = cudaFuncSetAttribute(prep_scan<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            if (known) attr_bytes[dev][5] = smem;
-        }
-    }
+    auto allow = [&](void (*kern)(PrepArgs), int which, size_t bytes) -> cudaError_t {
+        if (bytes <= kPlainSmem || (known && allowed[dev][which])) return cudaSuccess;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostSmem);
+        if (e == cudaSuccess && known) allowed[dev][which] = true;
+        return e;
+    };
+    cudaError_t e = allow(k0, variant, smem);
+    if (e == cudaSuccess) e = allow(k1, 4, smem);
+    if (e == cudaSuccess) e = allow(prep_scan<true>, 5, scan_smem);
+    if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(n_bg * a.ctas_per_bg);
     // a chain of short kernels: 1999 positions, 32/8 heads, search to merge, 115 us with plain launches, a memset and an
     // extra kernel for the offsets across (batch, kv head)s, 101 us like this; 16/2 heads, 1590 positions, K = 2 61 and 46 us
     const long long words = (long long)n_bg * a.NB * a.ncls;
     const unsigned clear = (unsigned)((words + 4 * kPrepThreads - 1) / (4 * kPrepThreads));
-    cudaError_t e = launch_chained(prep_clear, dim3(clear), dim3(kPrepThreads), 0, st, a);
+    e = launch_chained(prep_clear, dim3(clear), dim3(kPrepThreads), 0, st, a);
     if (e == cudaSuccess) e = launch_chained(k0, dim3(grid), dim3(kPrepThreads), smem, st, a);
-    if (e == cudaSuccess) e = launch_chained(many ? prep_scan<true> : prep_scan<false>, dim3(n_bg), dim3(kPrepThreads), many ? smem : 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(many ? prep_scan<true> : prep_scan<false>, dim3(n_bg), dim3(kPrepThreads), scan_smem, st, a);
     if (e == cudaSuccess) e = launch_chained(k1, dim3(grid), dim3(kPrepThreads), smem, st, a);
     if (e == cudaSuccess) e = launch_chained(prep_tile_bounds, dim3((unsigned)((a.max_tiles + 7) / 8)), dim3(256), 0, st, a);
     if (launches) *launches += 5;

@@ -61,10 +61,10 @@ using bf16 = __nv_bfloat16;
 constexpr int kD = 128;
 using tc::kBK;    // keys per block of the work list
 using tc::kRows;  // pieces per tile
+using tc::kMaxWalk;
 constexpr int kHalf = 128;       // pieces per stream: a tile's first and second 128
 constexpr int kThreads = 512;    // 4 row warps per stream, 4 epilogue warps, an MMA issuer per stream, K/V producer, Q gather
 constexpr int kTmemCols = 512;
-constexpr int kMaxWalk = 4096;   // most key blocks a piece covers
 constexpr int kMinTiles = 1024;  // entries of the tile table at least: more than CTAs
 constexpr uint32_t kColO = 0;    // O of the streams at columns 0 and 128
 constexpr uint32_t kColS = 256;  // two S buffers of 64 columns per stream, from columns 256 and 384; P aliases its S
@@ -1302,9 +1302,8 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     // 5 % shorter without joining at density 417, 2 % at 512 and longer from 2048 on.
     constexpr long long kJoinDensity = 384;
     const long long density = (long long)c.G * Lc * (c.top_k + (c.window > 0 ? 1 : 0)) / p.NB;
-    const size_t hist_cap = 160 * 1024;
     constexpr int kJoinWidth = 3;
-    const int ncls_avail = (int)(hist_cap / ((size_t)p.NB * 4));
+    const int ncls_avail = (int)(tc::kHistBytes / ((size_t)p.NB * 4));
     p.ncls1 = p.nb_single < 8 ? p.nb_single : 8;
     while (p.ncls1 > 1 && p.ncls1 > ncls_avail) p.ncls1 /= 2;
     int ncls2 = 0;
@@ -1329,7 +1328,7 @@ TcPlan plan_attention_tc(const Call &c, int Lc, size_t gap) {
     }
     p.merge_cap = ncls2 > 0 ? (p.nb_max - 2) * kBK : 0;   // a piece of T tokens covers at most (T-1)/64 + 2 blocks
     p.ncls = p.ncls1 + ncls2;
-    p.ok = (size_t)p.NB * p.ncls * 4 <= hist_cap;
+    p.ok = (size_t)p.NB * p.ncls * 4 <= tc::kHistBytes;
     // the work-list kernels hold one CTA per SM (their histogram fills the shared memory): no more CTAs
     // than SMs, or the last few would run as a second wave
     p.ctas_per_bg = 148 / p.n_bg > 1 ? 148 / p.n_bg : 1;

@@ -9,6 +9,8 @@ namespace tc {
 
 constexpr int kBK = 64;     // keys per block
 constexpr int kRows = 256;  // pieces per tile
+constexpr int kMaxWalk = 4096;                  // most key blocks a piece covers
+constexpr size_t kHistBytes = 160 * 1024;       // most counters of the sort that a CTA holds, in bytes
 
 // Work list of one chunk of query positions, as laid out in the scratch memory:
 //   recs   int4 {row, slot of the row's partial results, lo, hi}: every piece of every row, ordered by

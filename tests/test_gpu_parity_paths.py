@@ -201,6 +201,30 @@ def test_buckets_of_the_sort(sla, handle, seq_len):
     run_prefill(sla, handle, workload(n_q_heads=4, n_kv_heads=2, seq_len=seq_len, top_k=5, span_len=40), q_pos0=seq_len - 301, Lq=301)
 
 
+def test_lists_around_the_plain_shared_memory():
+    """Eight length classes and 1531 to 1536 key blocks: histograms of 48992 to 49168 bytes (with the class table), around the 48 KB
+    that a kernel has without asking, of which its own arrays are a part.  In a process of its own, the smallest first: what a
+    longer list was allowed before would hide a size that is not asked for."""
+    import os
+    import subprocess
+    import sys
+    code = """if True:
+        import paper_2601_18401_b200 as sla
+        from test_gpu_parity_modes import run_modes
+        from test_gpu_parity_small import run_prefill, workload
+        h = sla.Handle(0, 256 << 20)
+        sla.sla_set_debug_canaries(h, True)
+        for L in (97984, 97985, 98240, 98241):
+            w = workload(n_q_heads=4, n_kv_heads=1, seq_len=L, top_k=8, span_len=0)
+            run_prefill(sla, h, w, q_pos0=L - 301)
+            run_modes(sla, h, w.scaled(top_k=2, back_factor=4, fwd_factor=2), 1088, q_pos0=L - 301)
+        """
+    here = os.path.dirname(os.path.abspath(__file__))
+    path = os.pathsep.join([here, os.path.dirname(here), os.environ.get("PYTHONPATH", "")])
+    r = subprocess.run([sys.executable, "-c", code], env=dict(os.environ, PYTHONPATH=path), capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
 @pytest.mark.parametrize("window", [0, 1, 24, 25, 400, 2**31 - 1])
 @pytest.mark.parametrize("heads", [4, 8, 16])
 def test_search_walk_of_strides(sla, handle, heads, window):
