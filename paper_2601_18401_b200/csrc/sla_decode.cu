@@ -709,14 +709,14 @@ decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restr
     }
 }
 
-// Dynamic shared memory above 48 KiB has to be allowed per kernel and device context.  The score kernel
+// Shared memory above 48 KiB, a kernel's own 16 bytes included, has to be allowed per kernel and device context.  The score kernel
 // is given the largest size it can ever be launched with, once per (device, instantiation): later steps
 // then launch without touching function attributes, whatever the context length.
 constexpr int kScoreSmemMax = 200 * 1024;
 template <typename K>
 cudaError_t allow_score_smem(K kern, size_t smem) {
     static bool done[64] = {};
-    if (smem <= 48 * 1024) return cudaSuccess;
+    if (smem <= 47 * 1024) return cudaSuccess;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;

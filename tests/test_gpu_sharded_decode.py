@@ -82,6 +82,26 @@ def test_sharded_step_equals_unsharded(sla, world, n_ctx0, span_len, top_k, dtyp
     handle.close()
 
 
+def test_shard_of_as_many_candidates_as_plain_shared_memory_takes(sla):
+    """1407 to 1409 candidates in one shard: 49120 to 49184 bytes of scores, around the 48 KB that a kernel has without asking, of
+    which its own arrays are a part.  The smallest first: what a longer context was allowed before would hide it."""
+    from paper_2601_18401_b200 import sharded
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q_s, q = (torch.empty(1, 1, 128, dtype=torch.bfloat16, device="cuda").normal_(generator=g) for _ in range(2))
+    kc, vc = (torch.empty(1, 1, 1409 ** 2 + 1, 128, dtype=torch.bfloat16, device="cuda").normal_(generator=g) for _ in range(2))
+    handle = sla.Handle(0, 64 << 20)
+    params = sla.make_params(8, 100, head_dim=128)
+    for n in (1407, 1408, 1409):
+        n_ctx = n * n + 1
+        out, lse, anchor, score = sharded.decode_step_sharded(handle, q_s, q, kc, vc, 0, n_ctx, params, shard_len=kc.shape[2])
+        ref_out, ref_lse, ref_anchor, ref_score = sla.sla_decode_step(handle, q_s, q, kc, vc, n_ctx, params)
+        torch.cuda.synchronize()
+        assert sla.sla_poll_status(handle) == sla.SLA_OK
+        assert torch.equal(anchor, ref_anchor) and torch.equal(score, ref_score)
+        assert (out.float() - ref_out.float()).abs().max().item() <= 2.0 ** -6 and (lse - ref_lse).abs().max().item() <= 1e-4
+    handle.close()
+
+
 def _rank_main(rank, world, port, n_ctx0, out_q):
     """One rank of the two-process run: its own process, CUDA context and handle on device 0."""
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
