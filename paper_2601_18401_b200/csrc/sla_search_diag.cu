@@ -355,11 +355,10 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
         top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
     }
     for (; s0 < n_max; s0 += 4) {
-        float xa = score(ka), xb = score(kb);
-        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
-        xa = s0 + u_own < n_own ? xa : -CUDART_INF_F;
-        xb = s0 + 2 + u_own < n_own ? xb : -CUDART_INF_F;
-        top.offer2(s0 + u_own, xa, s0 + 2 + u_own, xb);
+        const float xa = score(ka), xb = score(kb);
+        const bool on_a = s0 + u_own < n_own, on_b = s0 + 2 + u_own < n_own;   // (key 0 stands in for the key of an absent stride)
+        zero = fmaf(on_a ? xa : 0.f, 0.f, fmaf(on_b ? xb : 0.f, 0.f, zero));
+        top.offer2(s0 + u_own, on_a ? xa : -CUDART_INF_F, s0 + 2 + u_own, on_b ? xb : -CUDART_INF_F);
         if (s0 + 4 < n_max) {
             walk.next(ka);
             walk.next(kb);
@@ -471,12 +470,14 @@ search_rows8(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, i
     if (s0 < n) {
         const int s = s0 + 2 * q;
         float xa, xb;
+        auto offer_present = [&](int s) {   // (key 0 stands in for the key of an absent stride)
+            zero = fmaf(s < n ? xa : 0.f, 0.f, fmaf(s + 1 < n ? xb : 0.f, 0.f, zero));
+            top.offer2(s, s < n ? xa : -CUDART_INF_F, s + 1, s + 1 < n ? xb : -CUDART_INF_F);
+        };
         score(ka, xa, xb);
-        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
-        top.offer2(s, s < n ? xa : -CUDART_INF_F, s + 1, s + 1 < n ? xb : -CUDART_INF_F);
+        offer_present(s);
         score(kb, xa, xb);
-        zero = fmaf(xa, 0.f, fmaf(xb, 0.f, zero));
-        top.offer2(s + 8, s + 8 < n ? xa : -CUDART_INF_F, s + 9, s + 9 < n ? xb : -CUDART_INF_F);
+        offer_present(s + 8);
     }
 
     const long long obase = (((long long)b * c.Hq + h) * c.Lq + r) * c.top_k;

@@ -201,6 +201,37 @@ def test_buckets_of_the_sort(sla, handle, seq_len):
     run_prefill(sla, handle, workload(n_q_heads=4, n_kv_heads=2, seq_len=seq_len, top_k=5, span_len=40), q_pos0=seq_len - 301, Lq=301)
 
 
+@pytest.mark.parametrize("heads,top_k", [(4, 2), (4, 16), (8, 16), (16, 16)])
+def test_search_beside_a_first_key_that_is_not_finite(sla, handle, heads, top_k):
+    """Positions with 131 strides, none of which reaches key 0: an Inf there, with which strides that a position does not have are
+    padded, changes nothing and sends no row through the selection pass by pass (four searches 0.1 ms, 0.24 to 1.6 ms where all
+    rows took that)."""
+    import torch
+    L, pos0 = 17423, 131 * 131
+    g = torch.Generator(device="cuda").manual_seed(17)
+    q, k = (torch.empty(1, h, n, 128, dtype=torch.bfloat16, device="cuda").normal_(generator=g) for h, n in ((heads, L - pos0), (1, L)))
+    odd = k.clone()
+    odd[:, :, 0, 5] = float("inf")
+    params = sla.make_params(top_k, 8, head_dim=128)
+
+    def search(keys):
+        times = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                got = sla.sla_span_search(handle, q, keys, params, q_pos0=pos0)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return got, min(times)
+
+    (anchor, score), t = search(k)
+    (anchor2, score2), t2 = search(odd)
+    assert torch.equal(anchor, anchor2) and torch.equal(score, score2)
+    assert t2 < 1.5 * t, (t, t2)
+
+
 def test_lists_around_the_plain_shared_memory():
     """Eight length classes and 1531 to 1536 key blocks: histograms of 48992 to 49168 bytes (with the class table), around the 48 KB
     that a kernel has without asking, of which its own arrays are a part.  In a process of its own, the smallest first: what a
