@@ -287,23 +287,36 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
     }
     // One thread per row, four pieces in flight per thread; the last rows first, whose pieces the L2 still holds.
     constexpr int U = 4;
-    const int n_rows = (int)(sh.q1 - sh.q0);
+    const int n_rows = (int)(sh.q1 - sh.q0), tid = threadIdx.x;
     const int row_base = (int)(((long long)sh.b * a.Hq + sh.g * a.G) * a.Lc + sh.q0);   // rows x slots < 2^31 for the whole chunk
     const int4 *st = parked(a, sh, sh.q0, 0);
-    int ql = n_rows - 1 - (int)threadIdx.x;
+    auto move = [&](int ql, int j0, int end, int cnt) {   // pieces j0 to j0 + 3 of row ql
+        int4 pc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u < end) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u < cnt)
+                a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
+    };
+    if (n_rows <= kPrepThreads / 2) {
+        // Few rows: as many threads as there are for each, and a slot is read along with the number of pieces (one beyond it holds
+        // stale bytes that are not looked at).  Sixteen positions of 32/8 heads, 64 spans: 12.3 us with a thread per row, 5.5
+        // like this; 300 positions, 8/2 heads 14.6 and 6.3 us (ncu).
+        if (n_rows == 0) return;
+        const int sharers = kPrepThreads / n_rows, part = tid / n_rows, ql = n_rows - 1 - (tid - part * n_rows);
+        if (part >= sharers) return;
+        const int cnt = a.n_pieces[row_base + ql];
+        move(ql, part * U, a.slots, cnt);
+        for (int j0 = (part + sharers) * U; j0 < cnt; j0 += sharers * U) move(ql, j0, cnt, cnt);
+        return;
+    }
+    int ql = n_rows - 1 - tid;
     int cnt = ql >= 0 ? a.n_pieces[row_base + ql] : 0;
-    for (; ql >= 0;) {
+    while (ql >= 0) {
         const int next = ql - kPrepThreads, next_cnt = next >= 0 ? a.n_pieces[row_base + next] : 0;
-        for (int j0 = 0; j0 < cnt; j0 += U) {
-            int4 pc[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (j0 + u < cnt) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (j0 + u < cnt)
-                    a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
-        }
+        for (int j0 = 0; j0 < cnt; j0 += U) move(ql, j0, cnt, cnt);
         ql = next;
         cnt = next_cnt;
     }

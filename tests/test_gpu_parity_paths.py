@@ -201,6 +201,14 @@ def test_buckets_of_the_sort(sla, handle, seq_len):
     run_prefill(sla, handle, workload(n_q_heads=4, n_kv_heads=2, seq_len=seq_len, top_k=5, span_len=40), q_pos0=seq_len - 301, Lq=301)
 
 
+@pytest.mark.parametrize("heads,kv_heads,rows,q_pos0,top_k,span_len", [
+    (8, 2, 3, 9000, 64, 40), (32, 8, 37, 9000, 64, 40), (8, 1, 1, 9000, 40, 20),   # a few rows a block, some blocks without any
+])
+def test_rows_of_many_pieces_moved_by_several_threads(sla, handle, heads, kv_heads, rows, q_pos0, top_k, span_len):
+    """Rows whose pieces several threads of the list's last pass move, up to 64 pieces a row."""
+    run_prefill(sla, handle, workload(n_q_heads=heads, n_kv_heads=kv_heads, seq_len=q_pos0 + rows, top_k=top_k, span_len=span_len), q_pos0=q_pos0)
+
+
 @pytest.mark.parametrize("heads,top_k", [(4, 2), (4, 16), (8, 16), (16, 16)])
 def test_search_beside_a_first_key_that_is_not_finite(sla, handle, heads, top_k):
     """Positions with 131 strides, none of which reaches key 0: an Inf there, with which strides that a position does not have are
