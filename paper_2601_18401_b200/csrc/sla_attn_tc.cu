@@ -752,8 +752,85 @@ copy_q_rows(const bf16 *__restrict__ q, Call c, long long r0, int Lc, bf16 *__re
     *reinterpret_cast<uint4 *>(dst + row * kD + sub * 8) = __ldg(reinterpret_cast<const uint4 *>(src));
 }
 
+// dst += w x (eight columns of a piece's block-floating-point output; `exps` holds the chunk exponents)
+__device__ __forceinline__ void add_piece(const uint4 &raw, float exps, int sub, float w, float (&dst)[8]) {
+    const uint32_t eb = (__float_as_uint(exps) >> (8 * (sub >> 2))) & 0xffu;
+    const float ws = w * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
+    const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rw[e]));
+        dst[2 * e] = fmaf(ws, f.x, dst[2 * e]);
+        dst[2 * e + 1] = fmaf(ws, f.y, dst[2 * e + 1]);
+    }
+}
+
+// Per row: merge the normalised piece outputs through their log-sum-exp, for few rows.  16 lanes per row, 8 columns each; every lane
+// works out the row's weights.
+// Bound by a row's chain of loads, which tc_merge below makes longer.  100, 150 and 300 positions, 32 heads, eight spans: tc_merge 5.2, 5.2
+// and 6.5 us, this 4.5, 4.5 and 6.0; sixty-four spans over 16384 keys, 300 positions 38.6 and 32.1; 16000 rows of eight 7.0 and 6.8,
+// 32000 11.1 and 11.3, of sixty-four 47.9 and 51.4 (ncu).
+__global__ void __launch_bounds__(256)
+tc_merge_few(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
+             const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0,
+             bf16 *__restrict__ out, float *__restrict__ lse) {
+    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long row = gid >> 4;
+    const int sub = (int)(gid & 15);
+    const long long rows = (long long)c.B * c.Hq * Lc;
+    chain_wait();
+    if (row >= rows) return;
+    const int cnt = n_pieces[row];
+    const float2 *pl = part_lse + row * slots;
+    const __half *po = part_o + row * slots * kD + sub * 8;
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    // running maximum and denominator (log2 domain); the pieces come four at a time so that their loads are in flight together
+    float mx = -CUDART_INF_F, den = 0.f;
+    for (int j0 = 0; j0 < cnt; j0 += 4) {
+        float2 pj[4];
+        uint4 raw[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool on = j0 + u < cnt;
+            pj[u] = on ? __ldg(pl + j0 + u) : make_float2(-CUDART_INF_F, 0.f);
+            raw[u] = on ? __ldg(reinterpret_cast<const uint4 *>(po + (long long)(j0 + u) * kD)) : make_uint4(0, 0, 0, 0);
+        }
+        const float bm = fmaxf(fmaxf(pj[0].x, pj[1].x), fmaxf(pj[2].x, pj[3].x));
+        if (bm > mx) {
+            const float r = mx == -CUDART_INF_F ? 0.f : exp2f(mx - bm);
+            den *= r;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] *= r;
+            mx = bm;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (pj[u].x == -CUDART_INF_F) continue;
+            const float w = exp2f(pj[u].x - mx);
+            den += w;
+            add_piece(raw[u], pj[u].y, sub, w, acc);
+        }
+    }
+    const float inv = den > 0.f ? 1.f / den : 0.f;
+    const int rc = (int)((unsigned)row % (unsigned)Lc);   // rows < 2^31
+    const int bh = (int)((unsigned)row / (unsigned)Lc);
+    const int h = bh % c.Hq, b = bh / c.Hq;
+    const long long r = r0 + rc;
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 pp = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+        w[e] = *reinterpret_cast<const uint32_t *>(&pp);
+    }
+    *reinterpret_cast<uint4 *>(out + b * c.q_sb + h * c.q_sh + r * c.q_st + sub * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+    if (sub == 0)
+        lse[((long long)b * c.Hq + h) * c.Lq + r] = den > 0.f ? (mx + log2f(den)) * kLn2 : -CUDART_INF_F;
+}
+
 // Per row: merge the normalised piece outputs through their log-sum-exp.  A warp takes per_warp consecutive rows (a power of
-// two, 2 to 32): first 32 / per_warp lanes each work out a row's weights and write its lse, then every half of the warp adds up
+// two, kMergeLeast to 32): first 32 / per_warp lanes each work out a row's weights and write its lse, then every half of the warp adds up
 // every other row's pieces, 8 columns per lane, four pieces at a time with the next four already requested.  The last rows come
 // first: their partial results were written last, and what the L2 still holds of them is read from there.
 // Bound by the reads of the partial results (3.2 GB at 65536 positions, 32 heads, eight spans: 6.6 TB/s).  With 16 lanes that
@@ -762,10 +839,12 @@ copy_q_rows(const bf16 *__restrict__ q, Call c, long long r0, int Lc, bf16 *__re
 // Rows of a warp: up to kMergePieces slots -- fewer pieces in a row cost more for the weights, more make the last warps' turn
 // long -- and as many warps as keep the loads going.  16 and 8 rows of 16 slots: 131072 rows 101 and 97 us (93 before); 32 and 16 rows of 2
 // slots: 960000 rows 123 and 129 us (207 before); 16, 8 and 4 rows of 8 slots: 128000 rows 40, 44 and 46 us (47 before), 16000 rows
-// 16.0, 12.0 and 10.4 (10.2 before).
+// 16.0, 12.0 and 10.4 (10.2 before).  Never two: 64000 rows of 64 slots, a piece or two in most, 24.0 and with four 15.6 (15.1 with
+// tc_merge_few), 256000 rows 179 and 156 (160).  The same four are not enough for 9600 rows of 64 pieces: 39 us, tc_merge_few 32.
 constexpr int kMergeWarps = 4;      // of a CTA
-constexpr int kMergePieces = 128;   // slots a warp takes at most, with two rows or more
-constexpr int kMergeFill = 19;      // warps an SM at least, down to two rows a warp
+constexpr int kMergePieces = 128;   // slots a warp takes at most, with more than kMergeLeast rows
+constexpr int kMergeFill = 19;      // warps an SM at least; fewer rows than kMergeLeast in each: tc_merge_few
+constexpr int kMergeLeast = 4;
 __global__ void __launch_bounds__(kMergeWarps * 32, 8)
 tc_merge(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
          const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0, int per_warp,
@@ -884,19 +963,6 @@ tc_merge(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
 // attention over the part of S_t left of the window, slot top_k the attention over the window; A_t
 // merges the two through their log-sum-exp, and O = sum_t alpha_t A_t with alpha = softmax of the
 // selected anchors' search scores.  16 threads per row, 8 columns each.
-// dst += w x (eight columns of a piece's block-floating-point output; `exps` holds the chunk exponents)
-__device__ __forceinline__ void add_piece(const uint4 &raw, float exps, int sub, float w, float (&dst)[8]) {
-    const uint32_t eb = (__float_as_uint(exps) >> (8 * (sub >> 2))) & 0xffu;
-    const float ws = w * __uint_as_float((eb + 1u) << 23);   // weight x 2^(eb - 126)
-    const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&rw[e]));
-        dst[2 * e] = fmaf(ws, f.x, dst[2 * e]);
-        dst[2 * e + 1] = fmaf(ws, f.y, dst[2 * e + 1]);
-    }
-}
-
 __global__ void __launch_bounds__(256)
 tc_merge_gated(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
                const int32_t *__restrict__ anchor, const float *__restrict__ score, Call c, int slots, int Lc,
@@ -1465,10 +1531,12 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         else if (c.mode == SLA_PER_SPAN)
             e = launch_chained(tc_merge_gated, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
                                anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
-        else
-        {
+        else if (rows < (long long)kMergeFill * sm_count * kMergeLeast)
+            e = launch_chained(tc_merge_few, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
+                               (const unsigned char *)pa.n_pieces, c, plan.slots, lc, r0, (bf16 *)out, lse);
+        else {
             int per_warp = 32;
-            while (per_warp > 2 && (per_warp * plan.slots > kMergePieces || rows < (long long)kMergeFill * sm_count * per_warp)) per_warp /= 2;
+            while (per_warp > kMergeLeast && (per_warp * plan.slots > kMergePieces || rows < (long long)kMergeFill * sm_count * per_warp)) per_warp /= 2;
             const int per_cta = per_warp * kMergeWarps;
             e = launch_chained(tc_merge, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(32 * kMergeWarps),
                                (size_t)per_cta * (plan.slots | 1) * sizeof(float2), st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,

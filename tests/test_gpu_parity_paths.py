@@ -310,6 +310,13 @@ def test_generic_search_of_equal_scores(sla, handle, dtype, top_k):
         assert (anchor[i, n:] == -1).all() and torch.isneginf(score[i, n:]).all()
 
 
+@pytest.mark.parametrize("heads,kv_heads,seq_len,top_k", [(32, 8, 415, 4), (32, 8, 416, 4), (32, 8, 416, 64), (2, 1, 164, 64)])
+def test_merge_of_few_rows(sla, handle, heads, kv_heads, seq_len, top_k):
+    """Rows on both sides of the number from which a warp merges several (11248 on 148 multiprocessors), four rows a warp, up to 64 slots a row.  (From
+    position 64 on, see test_merge_of_pieces.)"""
+    run_prefill(sla, handle, workload(n_q_heads=heads, n_kv_heads=kv_heads, seq_len=seq_len, top_k=top_k, span_len=7), q_pos0=64)
+
+
 @pytest.mark.parametrize("by_blocks,kw", [
     # few keys a row, few rows (at the start, or far into a context), or blocks that few rows select
     (False, dict(seq_len=1, top_k=6, span_len=300)), (False, dict(seq_len=65, top_k=64, span_len=2)),
