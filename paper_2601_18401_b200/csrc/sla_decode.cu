@@ -710,11 +710,11 @@ decode_attn(const T *__restrict__ q_s, const T *__restrict__ q, const T *__restr
 }
 
 // Shared memory above 48 KiB, a kernel's own 16 bytes included, has to be allowed per kernel and device context.  The score kernel
-// is given the largest size it can ever be launched with, once per (device, instantiation): later steps
+// is given the largest size it can ever be launched with, once per (device, kernel): later steps
 // then launch without touching function attributes, whatever the context length.
 constexpr int kScoreSmemMax = 200 * 1024;
-template <typename K>
-cudaError_t allow_score_smem(K kern, size_t smem) {
+template <auto kern>   // (by the kernel, not its type: those of all head sizes and group sizes have the same)
+cudaError_t allow_score_smem(size_t smem) {
     static bool done[64] = {};
     if (smem <= 47 * 1024) return cudaSuccess;
     int dev = 0;
@@ -920,8 +920,8 @@ cudaError_t shard_search_launch(const void *q_s, const void *k_local, const Call
     cudaError_t e = cudaSuccess;
 #define SLA_LAUNCH_SCORE(GT)                                                                                         \
     do {                                                                                                             \
-        auto kern = decode_score<T, D, GT>;                                                                          \
-        e = allow_score_smem(kern, smem);                                                                            \
+        constexpr auto kern = decode_score<T, D, GT>;                                                                \
+        e = allow_score_smem<kern>(smem);                                                                            \
         if (e == cudaSuccess)                                                                                        \
             kern<<<gs, kScoreThreads, smem, st>>>(qs, kk, c, n_ctx, n, s_first, scores, counters, cand_anchor,       \
                                                   cand_score);                                                      \

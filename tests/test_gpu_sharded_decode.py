@@ -102,6 +102,27 @@ def test_shard_of_as_many_candidates_as_plain_shared_memory_takes(sla):
     handle.close()
 
 
+@pytest.mark.parametrize("head_dim,dtype", [(64, torch.bfloat16), (128, torch.bfloat16), (64, torch.float32)])
+def test_shards_of_many_candidates_for_every_group_size(sla, head_dim, dtype):
+    """1450 candidates in one shard, more than plain shared memory takes, one after another for groups of 1, 2, 4 and 8 query heads: the
+    kernel of each asks for its own."""
+    from paper_2601_18401_b200 import sharded
+    g = torch.Generator(device="cuda").manual_seed(4)
+    n_ctx = 1450 ** 2 + 1
+    kc, vc = (torch.empty(1, 1, n_ctx, head_dim, dtype=dtype, device="cuda").normal_(generator=g) for _ in range(2))
+    handle = sla.Handle(0, 64 << 20)
+    params = sla.make_params(8, 100, head_dim=head_dim)
+    for heads in (1, 2, 4, 8):
+        q_s, q = (torch.empty(1, heads, head_dim, dtype=dtype, device="cuda").normal_(generator=g) for _ in range(2))
+        out, lse, anchor, score = sharded.decode_step_sharded(handle, q_s, q, kc, vc, 0, n_ctx, params, shard_len=n_ctx)
+        ref_out, ref_lse, ref_anchor, ref_score = sla.sla_decode_step(handle, q_s, q, kc, vc, n_ctx, params)
+        torch.cuda.synchronize()
+        assert sla.sla_poll_status(handle) == sla.SLA_OK
+        assert torch.equal(anchor, ref_anchor) and torch.equal(score, ref_score)
+        assert (out.float() - ref_out.float()).abs().max().item() <= 2.0 ** -6 and (lse - ref_lse).abs().max().item() <= 1e-4
+    handle.close()
+
+
 def _rank_main(rank, world, port, n_ctx0, out_q):
     """One rank of the two-process run: its own process, CUDA context and handle on device 0."""
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
