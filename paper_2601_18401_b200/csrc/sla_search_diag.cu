@@ -525,16 +525,7 @@ cudaError_t launch_k(const bf16 *q_s, const bf16 *k, const Call &c, int32_t *oa,
     const bool table = c.off != nullptr;
     void (*kern)(const bf16 *, const bf16 *, Call, int32_t *, float *) =
         four ? (table ? search_diag<K, true> : search_diag<K, false>) : table ? search_rows8<K, true> : search_rows8<K, false>;
-    static bool attr_set[64][4] = {};
-    if (smem > 48 * 1024) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-        if (dev < 0 || dev >= 64 || !attr_set[dev][2 * four + table]) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) attr_set[dev][2 * four + table] = true;
-        }
-    }
+    static_assert(smem <= 48 * 1024, "what a kernel without arrays of its own has without asking");
     const int rows = kWarps * (four ? kQW : 1);   // positions per CTA
     const dim3 blocks((unsigned)((c.Lq + rows - 1) / rows), (unsigned)(c.B * c.Hkv), four ? 1u : (unsigned)(c.G / 8));
     return launch_chained(kern, blocks, dim3(kWarps * 32), smem, st, q_s, k, c, oa, os);
