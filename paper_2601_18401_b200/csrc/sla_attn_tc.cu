@@ -765,11 +765,13 @@ __device__ __forceinline__ void add_piece(const uint4 &raw, float exps, int sub,
     }
 }
 
-// Per row: merge the normalised piece outputs through their log-sum-exp, for few rows.  16 lanes per row, 8 columns each; every lane
-// works out the row's weights.
-// Bound by a row's chain of loads, which tc_merge below makes longer.  100, 150 and 300 positions, 32 heads, eight spans: tc_merge 5.2, 5.2
-// and 6.5 us, this 4.5, 4.5 and 6.0; sixty-four spans over 16384 keys, 300 positions 38.6 and 32.1; 16000 rows of eight 7.0 and 6.8,
-// 32000 11.1 and 11.3, of sixty-four 47.9 and 51.4 (ncu).
+// Per row: merge the normalised piece outputs through their log-sum-exp, for few rows or many slots.  16 lanes per row, 8 columns
+// each; every lane works out the row's weights.
+// Bound by a row's chain of loads, which tc_merge below makes longer.  Few rows, this and tc_merge (ncu): 100, 150 and 300 positions, 32 heads,
+// eight spans 4.5, 4.5 and 6.0 us, 5.2, 5.2 and 7.8; 500 positions 6.8 and 7.0, 1000 11.3 and 11.1.  Many slots, this and tc_merge with four and with two
+// rows a warp: 64 spans over 16384 keys, 600, 1200, 1800 and 4500 positions 34, 61, 85 and 199 us, 36, 63, 91 and 208, 33, 59, 82 and 201; from the
+// start, a piece or two in most rows, 1800 and 4500 positions 14 and 33 us, 14 and 32, 22 and 52.  With 32 spans four rows a warp are
+// ahead where rows have many pieces: 1000, 1400 and 4500 positions 40, 52 and 145 us, 36, 49 and 138.
 __global__ void __launch_bounds__(256)
 tc_merge_few(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
              const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0,
@@ -839,12 +841,11 @@ tc_merge_few(const __half *__restrict__ part_o, const float2 *__restrict__ part_
 // Rows of a warp: up to kMergePieces slots -- fewer pieces in a row cost more for the weights, more make the last warps' turn
 // long -- and as many warps as keep the loads going.  16 and 8 rows of 16 slots: 131072 rows 101 and 97 us (93 before); 32 and 16 rows of 2
 // slots: 960000 rows 123 and 129 us (207 before); 16, 8 and 4 rows of 8 slots: 128000 rows 40, 44 and 46 us (47 before), 16000 rows
-// 16.0, 12.0 and 10.4 (10.2 before).  Never two: 64000 rows of 64 slots, a piece or two in most, 24.0 and with four 15.6 (15.1 with
-// tc_merge_few), 256000 rows 179 and 156 (160).  The same four are not enough for 9600 rows of 64 pieces: 39 us, tc_merge_few 32.
+// 16.0, 12.0 and 10.4 (10.2 before).
 constexpr int kMergeWarps = 4;      // of a CTA
-constexpr int kMergePieces = 128;   // slots a warp takes at most, with more than kMergeLeast rows
-constexpr int kMergeFill = 19;      // warps an SM at least; fewer rows than kMergeLeast in each: tc_merge_few
-constexpr int kMergeLeast = 4;
+constexpr int kMergePieces = 128;   // slots a warp takes at most
+constexpr int kMergeFill = 19;      // warps an SM at least
+constexpr int kMergeLeast = 4;      // rows a warp takes at least; where the two above allow fewer: tc_merge_few
 __global__ void __launch_bounds__(kMergeWarps * 32, 8)
 tc_merge(const __half *__restrict__ part_o, const float2 *__restrict__ part_lse,
          const unsigned char *__restrict__ n_pieces, Call c, int slots, int Lc, long long r0, int per_warp,
@@ -1531,12 +1532,12 @@ cudaError_t launch_attn_tc(const void *q, const void *k, const void *v, const Ca
         else if (c.mode == SLA_PER_SPAN)
             e = launch_chained(tc_merge_gated, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
                                anchor, score, c, plan.slots, lc, r0, (bf16 *)out, lse, lse_span);
-        else if (rows < (long long)kMergeFill * sm_count * kMergeLeast)
+        else if (rows < (long long)kMergeFill * sm_count * kMergeLeast || plan.slots * kMergeLeast > kMergePieces)
             e = launch_chained(tc_merge_few, dim3(mblocks), dim3(256), 0, st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,
                                (const unsigned char *)pa.n_pieces, c, plan.slots, lc, r0, (bf16 *)out, lse);
         else {
             int per_warp = 32;
-            while (per_warp > kMergeLeast && (per_warp * plan.slots > kMergePieces || rows < (long long)kMergeFill * sm_count * per_warp)) per_warp /= 2;
+            while (per_warp * plan.slots > kMergePieces || rows < (long long)kMergeFill * sm_count * per_warp) per_warp /= 2;
             const int per_cta = per_warp * kMergeWarps;
             e = launch_chained(tc_merge, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(32 * kMergeWarps),
                                (size_t)per_cta * (plan.slots | 1) * sizeof(float2), st, (const __half *)tp.part_o, (const float2 *)tp.part_lse,

@@ -310,10 +310,11 @@ def test_generic_search_of_equal_scores(sla, handle, dtype, top_k):
         assert (anchor[i, n:] == -1).all() and torch.isneginf(score[i, n:]).all()
 
 
-@pytest.mark.parametrize("heads,kv_heads,seq_len,top_k", [(32, 8, 415, 4), (32, 8, 416, 4), (32, 8, 416, 64), (2, 1, 164, 64)])
+@pytest.mark.parametrize("heads,kv_heads,seq_len,top_k", [
+    (32, 8, 415, 4), (32, 8, 416, 4), (32, 8, 416, 32), (32, 8, 416, 33), (32, 8, 416, 64), (2, 1, 164, 64)])
 def test_merge_of_few_rows(sla, handle, heads, kv_heads, seq_len, top_k):
-    """Rows on both sides of the number from which a warp merges several (11248 on 148 multiprocessors), four rows a warp, up to 64 slots a row.  (From
-    position 64 on, see test_merge_of_pieces.)"""
+    """Rows and slots on both sides of the numbers up to which a warp merges several rows (11248 rows on 148 multiprocessors, 32 slots), four rows a
+    warp.  (From position 64 on, see test_merge_of_pieces.)"""
     run_prefill(sla, handle, workload(n_q_heads=heads, n_kv_heads=kv_heads, seq_len=seq_len, top_k=top_k, span_len=7), q_pos0=64)
 
 
