@@ -226,6 +226,13 @@ __global__ void __launch_bounds__(kPrepThreads) prep_count(PrepArgs a) {
 // Scatter pass: the CTA claims a contiguous range of every bucket it has pieces in (its count is in
 // cta_hist, the bucket's offset within its (batch, kv head) in key_count by now) and moves its parked pieces to
 // their places.
+// kFewRows: at most kFewScatter rows a CTA, several threads a row.  With a thread a row few threads went through up to 65 pieces each and the
+// others had none: 16 positions of 32/8 heads, 64 spans 12.2 and 5.7 us; 300 positions, 8/2 heads 14.8 and 6.3; 1200 (267 rows a CTA) 19.2
+// and 17.4 (ncu).  Not where a thread moves a row's pieces in one step, nor with two threads a row: 2000 positions, 64 spans 5.4 and 6.4 us.
+// (An instantiation of its own: in one kernel the other lists' pass took 48 registers instead of 32 and 1999 positions, four spans 0.2 to 0.4 us more.)
+constexpr int kScatterStep = 4;   // pieces a thread has in flight
+constexpr int kFewScatter = kPrepThreads / 3;   // three threads a row at least
+template <bool kFewRows>
 __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
     extern __shared__ int hist[];   // [NB * ncls]: first record of this CTA in every bucket
     const int nk = a.NB * a.ncls;
@@ -286,37 +293,43 @@ __global__ void __launch_bounds__(kPrepThreads) prep_scatter(PrepArgs a) {
         }
     }
     // One thread per row, four pieces in flight per thread; the last rows first, whose pieces the L2 still holds.
-    constexpr int U = 4;
-    const int n_rows = (int)(sh.q1 - sh.q0), tid = threadIdx.x;
+    constexpr int U = kScatterStep;
+    const int n_rows = (int)(sh.q1 - sh.q0);
     const int row_base = (int)(((long long)sh.b * a.Hq + sh.g * a.G) * a.Lc + sh.q0);   // rows x slots < 2^31 for the whole chunk
     const int4 *st = parked(a, sh, sh.q0, 0);
-    auto move = [&](int ql, int j0, int end, int cnt) {   // pieces j0 to j0 + 3 of row ql
-        int4 pc[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j0 + u < end) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (j0 + u < cnt)
-                a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
-    };
-    if (n_rows <= kPrepThreads / 2) {
-        // Few rows: as many threads as there are for each, and a slot is read along with the number of pieces (one beyond it holds
-        // stale bytes that are not looked at).  Sixteen positions of 32/8 heads, 64 spans: 12.3 us with a thread per row, 5.5
-        // like this; 300 positions, 8/2 heads 14.6 and 6.3 us (ncu).
+    if constexpr (kFewRows) {
+        // as many threads as there are for each row, the slots read along with the number of pieces (one beyond it holds stale bytes
+        // that are not looked at)
         if (n_rows == 0) return;
-        const int sharers = kPrepThreads / n_rows, part = tid / n_rows, ql = n_rows - 1 - (tid - part * n_rows);
+        const int sharers = kPrepThreads / n_rows, part = (int)threadIdx.x / n_rows, ql = n_rows - 1 - ((int)threadIdx.x - part * n_rows);
         if (part >= sharers) return;
         const int cnt = a.n_pieces[row_base + ql];
-        move(ql, part * U, a.slots, cnt);
-        for (int j0 = (part + sharers) * U; j0 < cnt; j0 += sharers * U) move(ql, j0, cnt, cnt);
+        for (int j0 = part * U, end = a.slots; j0 < end; j0 += sharers * U, end = cnt) {
+            int4 pc[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < end) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < cnt)
+                    a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
+        }
         return;
     }
-    int ql = n_rows - 1 - tid;
+    int ql = n_rows - 1 - (int)threadIdx.x;
     int cnt = ql >= 0 ? a.n_pieces[row_base + ql] : 0;
-    while (ql >= 0) {
+    for (; ql >= 0;) {
         const int next = ql - kPrepThreads, next_cnt = next >= 0 ? a.n_pieces[row_base + next] : 0;
-        for (int j0 = 0; j0 < cnt; j0 += U) move(ql, j0, cnt, cnt);
+        for (int j0 = 0; j0 < cnt; j0 += U) {
+            int4 pc[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < cnt) pc[u] = __ldg(st + (long long)(j0 + u) * n_rows + ql);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u < cnt)
+                    a.recs[rec_base + hist[pc[u].z & 0xffffff] + pc[u].w] = make_int4(row_base + ql, pc[u].z >> 24, pc[u].x, pc[u].y);
+        }
         ql = next;
         cnt = next_cnt;
     }
@@ -496,12 +509,13 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
     const int n_iv = a.top_k + (a.window > 0 ? 1 : 0);
     const int variant = n_iv <= 5 ? 3 : n_iv <= 9 ? 0 : n_iv <= 17 ? 1 : 2;
     void (*k0)(PrepArgs) = variant == 3 ? prep_count<5> : variant == 0 ? prep_count<9> : variant == 1 ? prep_count<17> : prep_count<0>;
-    void (*k1)(PrepArgs) = prep_scatter;
+    const bool few = a.slots > kScatterStep && ((long long)a.G * a.Lc + a.ctas_per_bg - 1) / a.ctas_per_bg <= kFewScatter;
+    void (*k1)(PrepArgs) = few ? prep_scatter<true> : prep_scatter<false>;
     const bool many = a.NB * a.ncls > kScanDirect * kPrepThreads;
     const size_t scan_smem = many ? (size_t)a.NB * a.ncls * sizeof(int) : 0;
     // Function attributes belong to a device's context: remembered per device.  A kernel is given the most that any list takes, so that
     // no later call or other thread has to raise it, or lowers it.
-    static bool allowed[64][6] = {};   // the four counting kernels, the scatter kernel and the scan
+    static bool allowed[64][7] = {};   // the four counting kernels, the two scatter kernels and the scan
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
     const bool known = dev >= 0 && dev < 64;
@@ -512,8 +526,8 @@ cudaError_t prepare(const PrepArgs &a, cudaStream_t st, long long *launches) {
         return e;
     };
     cudaError_t e = allow(k0, variant, smem);
-    if (e == cudaSuccess) e = allow(k1, 4, smem);
-    if (e == cudaSuccess) e = allow(prep_scan<true>, 5, scan_smem);
+    if (e == cudaSuccess) e = allow(k1, 4 + few, smem);
+    if (e == cudaSuccess) e = allow(prep_scan<true>, 6, scan_smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(n_bg * a.ctas_per_bg);
     // a chain of short kernels: 1999 positions, 32/8 heads, search to merge, 115 us with plain launches, a memset and an

@@ -203,6 +203,8 @@ def test_buckets_of_the_sort(sla, handle, seq_len):
 
 @pytest.mark.parametrize("heads,kv_heads,rows,q_pos0,top_k,span_len", [
     (8, 2, 3, 9000, 64, 40), (32, 8, 37, 9000, 64, 40), (8, 1, 1, 9000, 40, 20),   # a few rows a block, some blocks without any
+    (32, 8, 37, 9000, 4, 40), (32, 8, 37, 9000, 5, 40),   # pieces that one thread moves in a step, and one more
+    (32, 8, 1534, 9000, 5, 40), (32, 8, 1535, 9000, 5, 40),   # 341 and 342 rows a block on 148 multiprocessors
 ])
 def test_rows_of_many_pieces_moved_by_several_threads(sla, handle, heads, kv_heads, rows, q_pos0, top_k, span_len):
     """Rows whose pieces several threads of the list's last pass move, up to 64 pieces a row."""
