@@ -519,7 +519,8 @@ long long target_rows(const Call &c, size_t gap) {
 }  // namespace
 
 // Which of the two kernels, from what each of them does (microseconds; the factors are fitted to 898 calls of both kernels
-// over rows 1..8000, positions up to 400000, 1..64 spans of 2..3700 keys, and are off by 15 % in the median):
+// over rows 1..8000, positions up to 400000, 1..64 spans of 2..3700 keys, and are off by 15 % in the median; the calls were timed
+// before a list's rows were shared out evenly among the warps, which took 7 to 10 % off the blocks at head_dim 64):
 //   by rows    a warp's walk over its row, one step per span and per two loads of a warp (a row or more of keys each); the
 //              pieces it sorts; the products of selected keys
 //   by blocks  per chunk of rows a launch of two kernels and 64 staged keys and values per CTA, whether any row selects

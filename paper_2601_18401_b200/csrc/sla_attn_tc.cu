@@ -1072,7 +1072,9 @@ tc_merge_gated(const __half *__restrict__ part_o, const float2 *__restrict__ par
 // Bound by the reads of the partial results: with room for eight spans whatever top_k is, 106 registers and the shuffles of
 // absent spans made it 402 us for 32768 positions, 32 heads, two spans and a window (1.1 GB, 2.7 TB/s); with room for two,
 // 48 registers and 213 us; with the next two rows' pieces requested ahead 64 registers and 170 us (6.4 TB/s).  Eight spans 993 and 581 us,
-// five 723 and 493, but four 265 and 281 (122 registers, two CTAs an SM): built for four it requests them in the same step.
+// five 723 and 493, but four 265 and 281 (122 registers, two CTAs an SM): built for four it requests them in the same step, 270 us with 72
+// registers.  (With 64, four CTAs an SM, 255 us, but search to merge of 500 positions at 16384, three and four spans, takes 138 and 154 us
+// instead of 127 and 144.)
 constexpr int kGateK = 8;
 template <int K>
 __global__ void __launch_bounds__(256, K <= 2 ? 4 : 1)

@@ -409,7 +409,7 @@ search_diag(const bf16 *__restrict__ q_s, const bf16 *__restrict__ k, Call c, in
 // (four lists of K values per head).  4096 positions at 500001, 32/4 heads,
 // K = 16: 1515 us with a warp per position and selection from shared memory (the kernel of the other group sizes),
 // 484 us here, about 440 us with the tiles fetched a step ahead, 373 us (from 407 on the same GPU) with the shorter step.
-// Half of the A operand is zero, so that five CTAs fit an SM up to K = 8 with few spills (28 bytes at K = 8): 16384 positions, 32/4
+// Half of the A operand is zero, so that five CTAs fit an SM up to K = 8 with few spills (24 bytes at K = 8, 44 with a table): 16384 positions, 32/4
 // heads, K = 8 253 us with four CTAs, 234 with five; 2048 at 300000 141 and 120; K = 2 152 and 140, 123 and 102.
 template <int K, bool kTable>
 __global__ void __launch_bounds__(kWarps * 32, K <= 8 ? 5 : 4)
